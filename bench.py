@@ -119,8 +119,8 @@ class ClockSampler:
 #       -c 20 --csv --log-file launches.csv python bench.py --profile --steps 1 --warmup 0 --no-cpu-baseline
 # A changed kernel has no entry, and the line then reports null.
 FILTER_TRAFFIC = {
-    ("ac16c6118738c34c92934d753be73dd680a508500a2e32bf5f83788584569732",
-     "19da060f812c9aa7e1bdab083bd343179dc94de2746a1a1f3fa7d22a8f801d02"): 0.988e9 + 0.031e9,
+    ("6bd769946ab94e7f10cea56098c556932ad8d70a6ece13860732d85d7dbb645e",
+     "63c9dbc321616d713b944b8786da0ab400f22c2b9e448d1eecf7242991f45025"): 0.989e9 + 0.031e9,
 }
 
 
@@ -144,11 +144,11 @@ def stage_bytes(P, n_batch, resident, frame, csize, ntiles):
     """Algorithmic HBM bytes of each stage (each operand read or written once).
     csize: stored colour bytes (16 FP32 / 8 16-bit). A buffered sample is
     x, y, mx, my (16 B), t (4), depth (4), seq (4) and its colour; a frame
-    record is x', y', a^2, bin column (16 B), its colour and seq (4)."""
+    record is 32 bytes (x', y', a^2, bin, r, g, b, seq)."""
     ingest = n_batch * (16 + csize + 8) + resident * (16 + 4 + 4 + 4 + csize) + P * 8
     grads = resident * (4 + 4 + csize) + P * (4 + 4 + 16 + 4 + 16) + ntiles * 64
-    reproj = resident * (16 + 4 + 4 + csize) + frame * (16 + csize + 4) + P * 12
-    recon = frame * (16 + csize) + P * (16 + 8 + 4 + 8 + 16)
+    reproj = resident * (16 + 4 + 4 + csize) + frame * 32 + P * 12
+    recon = frame * 32 + P * (16 + 8 + 4 + 8 + 16)
     feedback = ntiles * (64 + 32)
     return {"ingest": ingest, "gradients": grads, "reproject": reproj, "reconstruct": recon, "feedback": feedback}
 

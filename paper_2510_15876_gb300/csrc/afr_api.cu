@@ -60,7 +60,7 @@ cudaError_t dalloc(T **p, size_t n) {
 void free_all(AfrContext *c) {
     void *ptrs[] = {c->r_xy, c->r_mo, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->bucket, c->fifo_flag, c->fifo_rank, c->fifo_scan,
                     c->ccnt, c->coff, c->ccur, c->lbar, c->grad, c->pstat, c->sigma, c->tile_terms, c->fconst, c->cov_r[0], c->cov_r[1], c->cov_n, c->amin2, c->tiles, c->fcnt,
-                    c->foff, c->fpos, c->fcol, c->fseq, c->flist, c->flseq, c->q_xy, c->q_mo, c->q_t, c->q_seq, c->q_col, c->q_total, c->q_world, c->r_world, c->scan_tmp, c->scan_tmp_in, c->bgrad, c->bparam, c->dcount, c->derr};
+                    c->foff, c->frec, c->sbin, c->flist, c->flseq, c->q_xy, c->q_mo, c->q_t, c->q_seq, c->q_col, c->q_total, c->q_world, c->r_world, c->scan_tmp, c->scan_tmp_in, c->bgrad, c->bparam, c->dcount, c->derr};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -231,9 +231,8 @@ AfrStatus afr_create(const AfrConfig *cfg, AfrContext **out) {
         AFR_ALLOC(c->q_total, 1);
         if (e == cudaSuccess) e = cudaMemset(c->q_total, 0, sizeof(uint32_t));
     }
-    AFR_ALLOC(c->fpos, c->frame_cap);
-    if (e == cudaSuccess) e = dmalloc(&c->fcol, c->frame_cap * c->csize);
-    AFR_ALLOC(c->fseq, c->frame_cap);
+    AFR_ALLOC(c->frec, c->frame_cap + afr::kFramePad);
+    AFR_ALLOC(c->sbin, c->frame_cap);
     AFR_ALLOC(c->flist, c->frame_cap);
     AFR_ALLOC(c->flseq, c->frame_cap);
     AFR_ALLOC(c->scan_tmp, c->scan_tmp_n);
@@ -603,20 +602,18 @@ AfrStatus afr_export_frame(AfrContext *c, uint32_t *off_host, float *rec_host, u
     if (e != cudaSuccess) return cuda_fail(c, e, "afr_export_frame");
     size_t n = off_host[c->P];
     if (n > cap) return fail(c, AFR_ERR_INVALID_ARG, "afr_export_frame: capacity too small");
-    std::vector<float4> pos(n ? n : 1);
-    std::vector<unsigned char> col((n ? n : 1) * c->csize);
-    if (n) {
-        e = cudaMemcpy(pos.data(), c->fpos, n * 16, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(col.data(), c->fcol, n * c->csize, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(seq_host, c->fseq, n * 4, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(c, e, "afr_export_frame");
-    }
+    std::vector<afr::FrameRec> rec(n);
+    if (n) e = cudaMemcpy(rec.data(), c->frec, n * sizeof(afr::FrameRec), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(c, e, "afr_export_frame");
     for (size_t i = 0; i < n; ++i) {
         float *o = rec_host + i * 6;
-        o[0] = pos[i].x;
-        o[1] = pos[i].y;
-        o[2] = pos[i].z;
-        widen_colors(c->ct, col.data(), i, o + 3);
+        o[0] = rec[i].p.x;
+        o[1] = rec[i].p.y;
+        o[2] = rec[i].p.z;
+        o[3] = rec[i].c.x;
+        o[4] = rec[i].c.y;
+        o[5] = rec[i].c.z;
+        std::memcpy(seq_host + i, &rec[i].c.w, 4);
     }
     return AFR_OK;
 }
@@ -900,8 +897,7 @@ AfrStatus afr_batch_reconstruct(AfrBatch *b, float t_now, const AfrParams *param
         x.fconst = c->fconst;
         x.amin2 = c->amin2;
         x.foff = c->foff;
-        x.fpos = c->fpos;
-        x.fcol = c->fcol;
+        x.frec = c->frec;
         x.out = reinterpret_cast<float4 *>(o);
         x.derr = c->derr;
         x.fcap = (uint32_t)c->frame_cap;

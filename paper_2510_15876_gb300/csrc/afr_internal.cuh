@@ -18,6 +18,8 @@ constexpr float kAgeDecay = 3.47f;               // section 4: exp(-3.47 a)
 constexpr float kLumR = 0.2126f, kLumG = 0.7152f, kLumB = 0.0722f;  // Rec. 709
 constexpr float kSigmaSMin = 0.5f, kSigmaTMin = 0.05f;
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kPitch = 18;                       // frame records carry their bin as row * kPitch + column (below)
+constexpr int kFramePad = 32;                    // records past frame_cap that the filter may read (never sums)
 constexpr int kSortedBinMax = 4096;              // frame bins ordered by seq up to this size
 
 // device counters (unsigned long long)
@@ -64,6 +66,14 @@ struct Camera {
     float m[12];
 };
 
+// One record of the frame view, 32 bytes (one sector), in bin order. The
+// colour is widened to FP32 whatever the storage type of the queues, so that
+// the filter reads a record with one 256-bit load and converts nothing.
+struct alignas(32) FrameRec {
+    float4 p;   // x', y', a^2, bin row * kPitch + column as int bits (bin_place)
+    float4 c;   // r, g, b, sequence number as uint32 bits
+};
+
 // Per-context record of a batched launch (device memory).
 struct BatchCtx {
     int W, H, R, S, ntx, tbx, th, ntiles_x;
@@ -75,8 +85,7 @@ struct BatchCtx {
     float4 *fconst;
     const uint32_t *amin2;
     const uint32_t *foff;
-    const float4 *fpos;
-    const void *fcol;
+    const FrameRec *frec;
     float4 *out;
     uint32_t *derr;
     uint32_t fcap;      // frame-view record capacity (checks)
@@ -142,9 +151,8 @@ struct AfrContext {
     // frame view
     uint32_t *fcnt = nullptr;     // [P]
     uint32_t *foff = nullptr;     // [P+1]
-    float4 *fpos = nullptr;       // [frame_cap] (x', y', a^2, bin column as int bits)
-    void *fcol = nullptr;         // [frame_cap]
-    uint32_t *fseq = nullptr;     // [frame_cap] sequence numbers
+    afr::FrameRec *frec = nullptr;  // [frame_cap + kFramePad]
+    uint32_t *sbin = nullptr;     // [frame_cap] each source slot's bin (reprojection scratch)
     uint32_t *flist = nullptr;    // [frame_cap] each bin's source slots, unordered (reprojection scratch)
     uint32_t *flseq = nullptr;    // [frame_cap] their sequence numbers
     size_t frame_cap = 0;
@@ -220,6 +228,27 @@ template <> struct ColorStore<AFR_BF16> {
 
 __device__ __forceinline__ float luminance(float3 c) {
     return fmaf(kLumB, c.z, fmaf(kLumG, c.y, kLumR * c.x));
+}
+
+// A frame record's bin, in its p.w. The filter subtracts the place of
+// its footprint's corner to index a table of the footprint box (at most
+// kPitch columns wide), so the record carries one number for both.
+__device__ __forceinline__ float bin_place(float xp, float yp) {
+    return __int_as_float((int)floorf(yp) * kPitch + (int)floorf(xp));
+}
+
+// 256-bit accesses of a frame record (read-only path for the load)
+__device__ __forceinline__ FrameRec load_rec(const FrameRec *r) {
+    FrameRec v;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v.p.x), "=f"(v.p.y), "=f"(v.p.z), "=f"(v.p.w), "=f"(v.c.x), "=f"(v.c.y), "=f"(v.c.z), "=f"(v.c.w)
+        : "l"(r));
+    return v;
+}
+__device__ __forceinline__ void store_rec(FrameRec *r, const FrameRec &v) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(r), "f"(v.p.x), "f"(v.p.y),
+                 "f"(v.p.z), "f"(v.p.w), "f"(v.c.x), "f"(v.c.y), "f"(v.c.z), "f"(v.c.w)
+                 : "memory");
 }
 
 // ---- double-float arithmetic ------------------------------------------------

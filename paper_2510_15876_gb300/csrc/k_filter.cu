@@ -11,6 +11,8 @@
 // for every sample and E - m <= ((R+1)^2 - R^2 + ...) ks stays small for
 // the sample that attains the bound, so the normalised colour is exact up to
 // rounding whatever the ages; W is reported as S * 2^-m.
+#include <type_traits>
+
 #include "afr_internal.cuh"
 
 namespace afr {
@@ -41,10 +43,13 @@ __device__ __forceinline__ float tile_volume(int x, int y, int W, int H, int S, 
     return n > 0.f ? A * window / n : A * window;
 }
 
+// floor(sqrt(R^2 - dy^2)), |dy| <= R <= 8: the radicand is an integer, so half
+// a unit added before the root keeps the approximation's error away from the
+// integers.
 __device__ __forceinline__ int half_width(int R, int dy) {
-    int h = 0;
-    while ((h + 1) * (h + 1) + dy * dy <= R * R) ++h;
-    return h;
+    float h;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"((float)(R * R - dy * dy) + 0.5f));
+    return (int)h;
 }
 
 __device__ __forceinline__ float bin_gap(int d) {   // nearest distance from a pixel centre to a bin d away
@@ -173,17 +178,30 @@ __global__ void k_coverage_init(int P, float r0, float *__restrict__ r, int32_t 
 // discs is, row by row of bins, one contiguous run of columns, and the frame
 // view stores the records of consecutive bins of a row contiguously; so the
 // union's records are (2R + 2) contiguous index ranges. Lanes enumerate the
-// rows (range and count), a warp scan lays them out in one flat index space,
-// and the gather runs a flat loop over it: lane l takes flat indices l,
-// l + 32, ... (two independent streams per iteration), following its row with
-// a cursor, so loads are coalesced and every lane runs the same trip count
-// whatever the bin occupancy. A table in shared memory gives, for each
-// (row, column) of the union box, the exponent shift of each of the four
-// pixels, or -inf (weight 0) where the bin lies outside that pixel's disc;
-// a record's column is stored with it. The arithmetic runs on pixel pairs
-// (same row) with paired FP32 instructions. Each lane accumulates the four
-// pixels; the warp reduces them at the end. The per-pixel constants (-ks,
-// -kt, shift) come from k_sigma.
+// rows (range and count, from the tile's bin offsets in shared memory), a warp
+// scan lays them out in one flat index space, and the gather runs a flat loop
+// over it: lane l takes flat indices l, l + 32, ..., following its row with a
+// cursor, so loads are coalesced and every lane runs the same trip count
+// whatever the bin occupancy; a record is one 256-bit load, and the next one
+// is loaded while the current one is summed. Which of the four discs hold a
+// record's bin depends only on the bin's place in the union box and R: a table
+// (0 in the disc, -inf outside, per pixel), shared by every block, is indexed
+// by the place that the record carries (row * kPitch + column, less the place
+// of the box's corner). The arithmetic runs on pixel pairs (same row) with
+// paired FP32 instructions. Each lane accumulates the four pixels; the warp
+// reduces them at the end. The per-pixel constants (-ks, -kt, shift) come from
+// k_sigma.
+//
+// Bound: instruction issue and L1 (one launch at 960x540x16: 59% of issue
+// slots, 66% of the L1 data pipe, 1588 warp instructions a block of which 31
+// iterations take 44 each; 24 of the 44 are arithmetic). Records and row
+// offsets in one place each, the shared disc table and the prefetch took the
+// launch at 1920x1080x16 from 1600 to 1115 us (FP32 colours), 1280x720x8 with
+// R = 5 from 607 to 409 us and 640x480x8 in FP16 from 185 to 128 us. The shift
+// table per block (disc + shift, no addition per record) measured 1655 us, its
+// shared memory taken from L1; four CTAs a SM (64 registers, spills) 1183 us;
+// a prefetch two records deep 1413 us (spills); CTAs of 12 or 24 warps
+// 1317-1500 us.
 constexpr int kMaxRows = 2 * 8 + 2;   // union rows (and columns) for R <= 8
 constexpr int kWarps = 8;
 constexpr int kMaxBatch = 64;         // contexts per batched launch
@@ -265,42 +283,39 @@ __device__ __forceinline__ float warp_reduce16(float (&v)[16]) {
     return v[0];
 }
 
-// Pixel pair j (pixels (0, j) and (1, j)) constants and accumulators.
+// Constants and accumulators of the block's pixel pairs: pair j holds pixels
+// (0, j) and (1, j).
 struct PairConsts {
-    f2 cx;         // (cx0, cx1)
-    f2 cy;         // (cy0, cy1): row centres
-    f2 nks[2], nkt[2];
+    f2 cx;               // (cx0, cx1)
+    f2 cy[2];            // (cy_j, cy_j): row centres
+    f2 nks[2], nkt[2], m[2];
 };
 struct PairAcc {
     f2 S[2], C[2], r[2], g[2], b[2];
 };
 
-// sh: the exponent shifts of the four pixels for the record's bin (-inf
-// outside a pixel's disc), pixel k = 2 j + column in component k.
+// in: 0 for each pixel whose disc holds the record's bin, else -inf; pixel
+// k = 2 j + column in component k.
 template <bool KAHAN>
-__device__ __forceinline__ void accumulate(const PairConsts &pc, float4 sh, float4 rec, float3 c, PairAcc &A) {
-    const f2 dx = sub2(pk(rec.x, rec.x), pc.cx);
+__device__ __forceinline__ void accumulate(const PairConsts &pc, float4 in, const FrameRec &q, PairAcc &A) {
+    const f2 dx = sub2(pk(q.p.x, q.p.x), pc.cx);
     const f2 sx = mul2(dx, dx);
-    const f2 dy = sub2(pk(rec.y, rec.y), pc.cy);
-    const f2 sy = mul2(dy, dy);
-    float sy0, sy1;
-    upk(sy, sy0, sy1);
-    const f2 a2 = pk(rec.z, rec.z);
-    const f2 cr = pk(c.x, c.x), cg = pk(c.y, c.y), cb = pk(c.z, c.z);
-    const f2 m[2] = {pk(sh.x, sh.y), pk(sh.z, sh.w)};
+    const f2 y = pk(q.p.y, q.p.y), a2 = pk(q.p.z, q.p.z);
+    const f2 cr = pk(q.c.x, q.c.x), cg = pk(q.c.y, q.c.y), cb = pk(q.c.z, q.c.z);
+    const f2 t[2] = {pk(in.x, in.y), pk(in.z, in.w)};
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-        const float syj = j ? sy1 : sy0;
-        const f2 d2 = add2(sx, pk(syj, syj));
-        const f2 e = fma2(d2, pc.nks[j], fma2(a2, pc.nkt[j], m[j]));
+        const f2 dy = sub2(y, pc.cy[j]);
+        const f2 d2 = fma2(dy, dy, sx);
+        const f2 e = fma2(d2, pc.nks[j], fma2(a2, pc.nkt[j], add2(pc.m[j], t[j])));
         float e0, e1;
         upk(e, e0, e1);
         const f2 w = pk(ex2(e0), ex2(e1));
         if (KAHAN) {
-            const f2 y = sub2(w, A.C[j]);
-            const f2 t = add2(A.S[j], y);
-            A.C[j] = sub2(sub2(t, A.S[j]), y);
-            A.S[j] = t;
+            const f2 v = sub2(w, A.C[j]);
+            const f2 n = add2(A.S[j], v);
+            A.C[j] = sub2(sub2(n, A.S[j]), v);
+            A.S[j] = n;
         } else {
             A.S[j] = add2(A.S[j], w);
         }
@@ -310,157 +325,248 @@ __device__ __forceinline__ void accumulate(const PairConsts &pc, float4 sh, floa
     }
 }
 
-// Per-warp shared memory of one 2x2 block.
-struct QuadSmem {
-    float4 shift[kMaxRows * kMaxRows];   // per (row, column) of the union box
-    uint32_t rstart[kMaxRows + 1];       // flat index of each row's first record; rstart[nv] = total
-    uint32_t rbase[kMaxRows];            // record index minus flat index within the row
+// Discs of the union box of a 2x2 block at footprint radius R: entry
+// (v, u) = bin row by - R + v, column bx - R + u.
+struct DiscTable {
+    float4 in[kMaxRows * kPitch];
 };
 
-// Row cursor of one gather stream: flat index j lies in union row v.
-struct Cursor {
-    int v, tb;            // row, shift-table offset of column 0 of the image
-    uint32_t end, base;   // flat end of row v, record index - flat index
-};
-
-__device__ __forceinline__ void advance(Cursor &k, uint32_t j, const QuadSmem &sm, int span, int colofs) {
-    while (j >= k.end) {
-        ++k.v;
-        k.end = sm.rstart[k.v + 1];
-        k.base = sm.rbase[k.v];
-        k.tb = k.v * span + colofs;
+__device__ __forceinline__ void fill_discs(DiscTable &t, int R) {
+    for (int i = threadIdx.x; i < (2 * R + 2) * kPitch; i += blockDim.x) {
+        const int v = i / kPitch - R, u = i % kPitch - R;
+        float s[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int du = u - (k & 1), dv = v - (k >> 1);
+            s[k] = du * du + dv * dv <= R * R ? 0.f : -INFINITY;
+        }
+        t.in[i] = make_float4(s[0], s[1], s[2], s[3]);
     }
 }
 
-// One 2x2 pixel block (top-left pixel bx, by) by one warp.
+// A value in a register that the assembler cannot compute again from
+// parameters and special registers inside a loop (a shuffle is opaque to it).
+__device__ __forceinline__ uint32_t keep(uint32_t v) {
+    asm volatile("shfl.sync.bfly.b32 %0, %0, 0, 0x1f, 0xffffffff;" : "+r"(v));
+    return v;
+}
+template <typename T>
+__device__ __forceinline__ T *keep(T *v) {
+    const unsigned long long u = reinterpret_cast<unsigned long long>(v);
+    const uint32_t lo = keep((uint32_t)u), hi = keep((uint32_t)(u >> 32));
+    return reinterpret_cast<T *>(((unsigned long long)hi << 32) | lo);
+}
+
+// p + i as one multiply-add
+template <typename T>
+__device__ __forceinline__ const T *element(const T *p, int i) {
+    unsigned long long a;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(a) : "r"(i), "n"((int)sizeof(T)), "l"(p));
+    return reinterpret_cast<const T *>(a);
+}
+
+__device__ __forceinline__ uint32_t smem_at(const void *p) { return keep((uint32_t)__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ float4 lds4(uint32_t at) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at));
+    return v;
+}
+__device__ __forceinline__ uint2 lds2(uint32_t at) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(at));
+    return v;
+}
+
+// Row cursor of one lane of the gather: at is the shared address of the row
+// table's entry (flat end, record index - flat index) for the row that holds
+// the lane's flat index j + lane; end and base are that entry with the lane
+// taken off.
+struct Cursor {
+    uint32_t at;
+    int end, base;
+};
+
+__device__ __forceinline__ void step(Cursor &k, int j, int lane) {   // at most one row on
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ge.s32 p, %3, %1;\n\t"
+        "@p add.u32 %0, %0, 8;\n\t"
+        "@p ld.shared.v2.b32 {%1, %2}, [%0];\n\t"
+        "@p sub.s32 %1, %1, %4;\n\t}"
+        : "+r"(k.at), "+r"(k.end), "+r"(k.base) : "r"(j), "r"(lane));
+}
+
+template <bool ONE>
+__device__ __forceinline__ void advance(Cursor &k, int j, int lane) {
+    do step(k, j, lane);
+    while (!ONE && __any_sync(0xffffffffu, j >= k.end));
+}
+
+// What the blocks of a CTA's tile share, loaded once: the gather constants of
+// its pixels, and the bin offsets of every row of the tile and its halo, so
+// that a block's row ranges cost two shared loads instead of a chain of global
+// ones.
+constexpr int kTilePixels = 128;              // (2 tbx) x (64 / tbx)
+constexpr int kTileOffsets = 1008;            // the most of (64 / tbx + 2R) x (2 tbx + 2R + 1): tbx 2, R 8
+struct TileSmem {
+    float4 fc[kTilePixels];
+    uint32_t off[kTileOffsets];
+    uint2 rows[kWarps][kMaxRows];
+};
+
+// Offsets of the bins of rows y0 - R .. y0 + th + R - 1 at columns x0 - R ..
+// x0 + tw + R (clamped to the row's first and last; rows outside the image
+// are empty).
+__device__ __forceinline__ void load_offsets(TileSmem &t, int W, int H, int R, int x0, int y0, int tw, int th,
+                                             const uint32_t *__restrict__ foff) {
+    const int cols = tw + 2 * R + 1;
+    for (int r = threadIdx.x >> 5; r < th + 2 * R; r += kWarps) {
+        const int row = y0 - R + r;
+        for (int c = threadIdx.x & 31; c < cols; c += 32) {
+            uint32_t v = 0;
+            if (row >= 0 && row < H) v = __ldg(foff + (size_t)row * W + min(max(x0 - R + c, 0), W));
+            t.off[r * cols + c] = v;
+        }
+    }
+}
+
+// Pixels past the right or bottom edge repeat the edge pixel (never stored).
+__device__ __forceinline__ float4 load_const(int i, int W, int H, int x0, int y0, int tw,
+                                             const float4 *__restrict__ fconst) {
+    return __ldg(fconst + (size_t)min(y0 + i / tw, H - 1) * W + min(x0 + i % tw, W - 1));
+}
+
+// One 2x2 pixel block by one warp: the block (lx, ly) of the tile at (x0, y0),
+// tw pixels wide, whose offsets were loaded for footprints up to Rt.
 // VAR: each pixel's footprint radius is read from its gather constants
-// (adaptive footprints); otherwise every pixel uses Rfix.
-template <int CT, bool KAHAN, bool VAR>
-__device__ __forceinline__ void filter_block(int W, int H, int Rfix, int bx, int by, const float4 *__restrict__ fconst,
-                                             const uint32_t *__restrict__ foff, const float4 *__restrict__ fpos,
-                                             const void *__restrict__ fcol, float4 *__restrict__ out,
-                                             QuadSmem &sm, const DebugCheck &dc) {
-    using CS = ColorStore<CT>;
+// (adaptive footprints); otherwise every pixel uses Rt. table: the warp's own
+// discs (VAR; held says for which radius it was filled last) or the CTA's, at
+// shared address table_at. frec: the frame view from this lane's record on.
+template <bool KAHAN, bool VAR>
+__device__ __forceinline__ void filter_block(int W, int H, int Rt, int x0, int y0, int tw, int lx, int ly,
+                                             const FrameRec *frec, float4 *__restrict__ out, const TileSmem &ts,
+                                             DiscTable *table, uint32_t table_at, int &held, uint2 *rows,
+                                             uint32_t rows_at, const DebugCheck &dc) {
     const int lane = threadIdx.x & 31;
-    float4 fc = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));   // -1: no pixel
-    if (lane < 4) {
-        const int x = bx + (lane & 1), y = by + (lane >> 1);
-        if (x < W && y < H) fc = __ldg(fconst + (size_t)y * W + x);
-    }
-    float nks[4], nkt[4], mk[4];
-    int Rk[4];   // footprint radius of each pixel, -1 outside the image
+    const int bx = x0 + 2 * lx, by = y0 + 2 * ly;
+    float4 fc[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        nks[k] = __shfl_sync(0xffffffffu, fc.x, k);
-        nkt[k] = __shfl_sync(0xffffffffu, fc.y, k);
-        mk[k] = __shfl_sync(0xffffffffu, fc.z, k);
-        if (VAR) Rk[k] = __shfl_sync(0xffffffffu, __float_as_int(fc.w), k);
-        else Rk[k] = (bx + (k & 1) < W && by + (k >> 1) < H) ? Rfix : -1;
+    for (int k = 0; k < 4; ++k) fc[k] = ts.fc[(2 * ly + (k >> 1)) * tw + 2 * lx + (k & 1)];
+    int R = Rt;
+    bool same = true;
+    if (VAR) {
+        const int R0 = __float_as_int(fc[0].w), R1 = __float_as_int(fc[1].w), R2 = __float_as_int(fc[2].w),
+                  R3 = __float_as_int(fc[3].w);
+        R = max(max(R0, R1), max(R2, R3));   // the block's largest footprint
+        same = min(min(R0, R1), min(R2, R3)) == R;
     }
-    const int R = VAR ? max(max(Rk[0], Rk[1]), max(Rk[2], Rk[3])) : Rfix;   // the block's largest footprint
-    const int span = 2 * R + 2, nv = span;
-    // union rows: lane v (< nv) takes bin row by + v - R; the union of the
-    // four discs' rows is one run of columns [bx + lo, bx + hi]
+    // union rows: lane v (< 2R + 2) takes bin row by - R + v; the union of the
+    // four discs' rows is one run of columns [bx - lo, bx + 1 + hi]
     uint32_t cnt = 0, first = 0;
-    if (lane < nv) {
-        const int v = lane - R, row = by + v;
-        int lo = 1 << 20, hi = -(1 << 20);
-        if (VAR) {
+    if (lane < 2 * R + 2) {
+        const int v = lane - R;
+        int lo, hi;
+        if (!VAR || same) {   // of the two pixel rows, the nearer has the wider run
+            lo = hi = half_width(R, v > 0 ? v - 1 : v);
+        } else {
+            lo = hi = -2;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int dv = v - (k >> 1);
-                if (Rk[k] >= 0 && dv >= -Rk[k] && dv <= Rk[k]) {
-                    const int h = half_width(Rk[k], dv);
-                    lo = min(lo, (k & 1) - h);
-                    hi = max(hi, (k & 1) + h);
+                const int dv = v - (k >> 1), Rk = __float_as_int(fc[k].w);
+                if (dv >= -Rk && dv <= Rk) {
+                    const int h = half_width(Rk, dv);
+                    lo = max(lo, h - (k & 1));
+                    hi = max(hi, h + (k & 1) - 1);
                 }
             }
-        } else {
-            // two pixel rows, one radius: the union row spans the wider half-width
-            const bool col1 = bx + 1 < W, row1 = by + 1 < H;
-            const int h0 = (v >= -R && v <= R) ? half_width(R, v) : -1;
-            const int h1 = (row1 && v - 1 >= -R && v - 1 <= R) ? half_width(R, v - 1) : -1;
-            const int hm = max(h0, h1);
-            if (hm >= 0) {
-                lo = -hm;
-                hi = (col1 ? 1 : 0) + hm;
-            }
         }
-        if (lo <= hi && row >= 0 && row < H) {
-            const int c0 = max(0, bx + lo), c1 = min(W - 1, bx + hi);
-            const size_t q = (size_t)row * W;
-            first = __ldg(foff + q + c0);
-            cnt = __ldg(foff + q + c1 + 1) - first;
-            if (!AFR_CHECK(__ldg(foff + q + c1 + 1) >= first && cnt <= dc.cap, dc.derr)) cnt = 0;
+        if (lo + hi >= -1) {
+            const uint32_t *o = ts.off + (2 * ly + v + Rt) * (tw + 2 * Rt + 1) + 2 * lx + Rt;
+            first = o[-lo];
+            const uint32_t last = o[hi + 2];
+            cnt = last - first;
+            if (!AFR_CHECK(last >= first && cnt <= dc.cap, dc.derr)) cnt = 0;
         }
     }
     const uint32_t incl = warp_incl_scan_u(cnt);
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-    if (lane < nv) {
-        sm.rstart[lane + 1] = incl;
-        sm.rbase[lane] = first - (incl - cnt);
-    }
-    if (lane == 0) sm.rstart[0] = 0;
-    // shift table: entry (v, u) of pixel k = (kx, ky) is its shift if
-    // (u - kx)^2 + (v - ky)^2 <= R_k^2 (the pixel's own disc; none outside
-    // the image)
-    for (int t = lane; t < nv * span; t += 32) {
-        const int v = t / span - R, u = t % span - R;
-        float s4[4];
+    if (lane < 2 * R + 2) rows[lane] = make_uint2(lane == 2 * R + 1 ? 0x7fffffffu : incl, first - (incl - cnt));
+    // rows of 32 records or more between the first and the last: an iteration moves a lane at most one row on
+    const bool one = __all_sync(0xffffffffu, cnt >= 32u || lane == 0 || lane >= 2 * R + 1);
+    if (VAR && (!same || held != R)) {   // most neighbouring footprints have settled at one radius
+        for (int t = lane; t < (2 * R + 2) * kPitch; t += 32) {
+            const int v = t / kPitch - R, u = t % kPitch - R;
+            float s[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int du = u - (k & 1), dv = v - (k >> 1);
-            s4[k] = (Rk[k] >= 0 && du * du + dv * dv <= Rk[k] * Rk[k]) ? mk[k] : -INFINITY;
+            for (int k = 0; k < 4; ++k) {
+                const int du = u - (k & 1), dv = v - (k >> 1), Rk = __float_as_int(fc[k].w);
+                s[k] = du * du + dv * dv <= Rk * Rk ? 0.f : -INFINITY;
+            }
+            table->in[t] = make_float4(s[0], s[1], s[2], s[3]);
         }
-        sm.shift[t] = make_float4(s4[0], s4[1], s4[2], s4[3]);
+        held = same ? R : -1;
     }
     __syncwarp();
     PairConsts pc;
     pc.cx = pk((float)bx + 0.5f, (float)bx + 1.5f);
-    pc.cy = pk((float)by + 0.5f, (float)by + 1.5f);
-    pc.nks[0] = pk(nks[0], nks[1]);
-    pc.nks[1] = pk(nks[2], nks[3]);
-    pc.nkt[0] = pk(nkt[0], nkt[1]);
-    pc.nkt[1] = pk(nkt[2], nkt[3]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float cy = (float)(by + j) + 0.5f;
+        pc.cy[j] = pk(cy, cy);
+        pc.nks[j] = pk(fc[2 * j].x, fc[2 * j + 1].x);
+        pc.nkt[j] = pk(fc[2 * j].y, fc[2 * j + 1].y);
+        pc.m[j] = pk(fc[2 * j].z, fc[2 * j + 1].z);
+    }
     PairAcc A;
 #pragma unroll
     for (int j = 0; j < 2; ++j) A.S[j] = A.C[j] = A.r[j] = A.g[j] = A.b[j] = 0ull;
-    const int colofs = R - bx;   // table column of image column qx: qx + colofs
-    Cursor ka{-1, 0, 0u, 0u}, kb{-1, 0, 0u, 0u};
-    uint32_t j = lane;
-    for (; j + 32 < total; j += 64) {
-        advance(ka, j, sm, span, colofs);
-        advance(kb, j + 32, sm, span, colofs);
-        uint32_t ia = j + ka.base, ib = j + 32 + kb.base;
-        const bool va = AFR_CHECK(ia < dc.cap, dc.derr), vb = AFR_CHECK(ib < dc.cap, dc.derr);
-        if (!va) ia = 0;   // skipped: record 0 read, weight 0
-        if (!vb) ib = 0;
-        const float4 ra = __ldg(fpos + ia), rb = __ldg(fpos + ib);
-        const float3 ca = CS::load(fcol, ia), cbv = CS::load(fcol, ib);
-        int ta = ka.tb + __float_as_int(ra.w), tb = kb.tb + __float_as_int(rb.w);
-        const bool wa = va && AFR_CHECK(ta >= 0 && ta < kMaxRows * kMaxRows, dc.derr);
-        const bool wb = vb && AFR_CHECK(tb >= 0 && tb < kMaxRows * kMaxRows, dc.derr);
-        if (!wa) ta = 0;
-        if (!wb) tb = 0;
-        float4 sa = sm.shift[ta], sb = sm.shift[tb];
-        if (!wa) sa = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        if (!wb) sb = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        accumulate<KAHAN>(pc, sa, ra, ca, A);
-        accumulate<KAHAN>(pc, sb, rb, cbv, A);
+    const int origin = (by - R) * kPitch + bx - R;
+    const uint32_t tab = keep(table_at - (uint32_t)origin * 16u);   // + 16 place: the entry of a record's bin
+    auto load = [&](int i) {   // record i + lane (i itself may be negative)
+        const bool ok = AFR_CHECK((uint32_t)(i + lane) < dc.cap + kFramePad, dc.derr);
+        FrameRec r = load_rec(element(frec, ok ? i : 0));   // not ok: another record read, weight 0
+        if (!ok) r.p.w = __int_as_float(-1 - origin);
+        return r;
+    };
+    auto add = [&](const FrameRec &r) {
+        const int place = __float_as_int(r.p.w);
+        const bool ok = AFR_CHECK(place >= origin && place < origin + (2 * R + 2) * kPitch, dc.derr);
+        float4 d = lds4(ok ? tab + (uint32_t)place * 16u : table_at);
+        if (!ok) d = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        accumulate<KAHAN>(pc, d, r, A);
+    };
+    // The last iteration's lanes past the end read on (the frame arrays end in
+    // kFramePad records of padding) and are dropped before they are summed.
+    auto gather = [&](auto one_row) {
+        constexpr bool ONE = decltype(one_row)::value;
+        const uint2 r0 = lds2(rows_at);
+        Cursor k{rows_at, (int)r0.x - lane, (int)r0.y};
+        FrameRec ra, rb;
+        advance<false>(k, 0, lane);
+        ra = load(k.base);
+        int j = 32;
+        for (; j + 32 < (int)total; j += 64) {
+            advance<ONE>(k, j, lane);
+            rb = load(j + k.base);
+            add(ra);
+            advance<ONE>(k, j + 32, lane);
+            ra = load(j + 32 + k.base);
+            add(rb);
+        }
+        if (j < (int)total) {
+            advance<ONE>(k, j, lane);
+            rb = load(j + k.base);
+            add(ra);
+            ra = rb;
+            j += 32;
+        }
+        if (j - 32 + lane < (int)total) add(ra);
+    };
+    if (total) {
+        if (one) gather(std::true_type{});
+        else gather(std::false_type{});
     }
-    if (j < total) {
-        advance(ka, j, sm, span, colofs);
-        uint32_t ia = j + ka.base;
-        const bool va = AFR_CHECK(ia < dc.cap, dc.derr);
-        if (!va) ia = 0;
-        const float4 ra = __ldg(fpos + ia);
-        int ta = ka.tb + __float_as_int(ra.w);
-        const bool wa = va && AFR_CHECK(ta >= 0 && ta < kMaxRows * kMaxRows, dc.derr);
-        if (!wa) ta = 0;
-        float4 sa = sm.shift[ta];
-        if (!wa) sa = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        accumulate<KAHAN>(pc, sa, ra, CS::load(fcol, ia), A);
-    }
+    __syncwarp();
     float vals[16];
 #pragma unroll
     for (int jj = 0; jj < 2; ++jj) {
@@ -491,7 +597,8 @@ __device__ __forceinline__ void filter_block(int W, int H, int Rfix, int bx, int
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
         if (q[0] > 0.f) {
             const float inv = 1.f / q[0];
-            o = make_float4(q[1] * inv, q[2] * inv, q[3] * inv, q[0] * ex2(-fc.z));
+            const float m = lane & 2 ? (lane & 1 ? fc[3].z : fc[2].z) : (lane & 1 ? fc[1].z : fc[0].z);
+            o = make_float4(q[1] * inv, q[2] * inv, q[3] * inv, q[0] * ex2(-m));
         }
         out[(size_t)(by + (lane >> 1)) * W + bx + (lane & 1)] = o;
     }
@@ -500,18 +607,35 @@ __device__ __forceinline__ void filter_block(int W, int H, int Rfix, int bx, int
 
 // Tile of (2 * tbx) x (2 * 32 / tbx) pixels per CTA: 32 blocks of 2x2, four
 // per warp.
-template <int CT, bool KAHAN, bool VAR>
-__global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int tbx, const float4 *__restrict__ fconst,
-                                                   const uint32_t *__restrict__ foff, const float4 *__restrict__ fpos,
-                                                   const void *__restrict__ fcol, float4 *__restrict__ out,
-                                                   DebugCheck dc) {
-    __shared__ QuadSmem smem[kWarps];
-    const int warp = threadIdx.x >> 5;
-    const int tby = 32 / tbx;
+template <bool KAHAN, bool VAR>
+__global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx, const float4 *__restrict__ fconst,
+                                                   const uint32_t *__restrict__ foff, const FrameRec *frec,
+                                                   float4 *__restrict__ out, DebugCheck dc) {
+    __shared__ TileSmem ts;
+    __shared__ DiscTable discs[VAR ? kWarps : 1];
+    const int warp = threadIdx.x >> 5, tw = 2 << ltbx, th = 64 >> ltbx;
+    const int x0 = blockIdx.x * tw, y0 = blockIdx.y * th;
+    frec = keep(frec + (threadIdx.x & 31));
+    const uint32_t table_at = smem_at(discs[VAR ? warp : 0].in), rows_at = smem_at(ts.rows[warp]);
+    int Rt = R, held = -1;
+    float4 fc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (threadIdx.x < kTilePixels) {
+        fc = load_const(threadIdx.x, W, H, x0, y0, tw, fconst);
+        ts.fc[threadIdx.x] = fc;
+    }
+    if (VAR) {   // the tile's largest footprint
+        Rt = 0;
+        for (int r = 1; r <= 8 && __syncthreads_or(__float_as_int(fc.w) >= r && threadIdx.x < kTilePixels); ++r) Rt = r;
+    } else {
+        fill_discs(discs[0], R);
+    }
+    load_offsets(ts, W, H, Rt, x0, y0, tw, th, foff);
+    __syncthreads();
     for (int blk = warp; blk < 32; blk += kWarps) {
-        const int bx = blockIdx.x * 2 * tbx + (blk % tbx) * 2, by = blockIdx.y * 2 * tby + (blk / tbx) * 2;
-        if (bx >= W || by >= H) continue;   // warp-uniform
-        filter_block<CT, KAHAN, VAR>(W, H, R, bx, by, fconst, foff, fpos, fcol, out, smem[warp], dc);
+        const int lx = blk & ((1 << ltbx) - 1), ly = blk >> ltbx;
+        if (x0 + 2 * lx >= W || y0 + 2 * ly >= H) continue;   // warp-uniform
+        filter_block<KAHAN, VAR>(W, H, Rt, x0, y0, tw, lx, ly, frec, out, ts, discs + (VAR ? warp : 0), table_at, held,
+                                 ts.rows[warp], rows_at, dc);
     }
 }
 
@@ -561,13 +685,14 @@ __global__ void __launch_bounds__(256) k_batch_sigma(const BatchCtx *__restrict_
     }
 }
 
-template <int CT, bool KAHAN>
+template <bool KAHAN>
 __global__ void __launch_bounds__(256, 3) k_batch(const BatchCtx *__restrict__ cs, int nctx, uint32_t total,
                                                   uint32_t *queue) {
-    // shared memory: the per-warp tables and two words, so that three CTAs
-    // fit the 132 KB shared-memory carve-out and leave the rest to L1
-    __shared__ QuadSmem smem[kWarps];
+    __shared__ TileSmem ts;
+    __shared__ DiscTable discs;                 // of the current tile's footprint radius
     __shared__ uint32_t item_buf[2];            // current and next claimed tile
+    const uint32_t table_at = smem_at(discs.in), rows_at = smem_at(ts.rows[threadIdx.x >> 5]);
+    int held = -1;
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) item_buf[0] = atomicAdd(queue, 1u);
     __syncthreads();
@@ -582,14 +707,21 @@ __global__ void __launch_bounds__(256, 3) k_batch(const BatchCtx *__restrict__ c
             else hi = mid - 1;
         }
         const BatchCtx &x = cs[lo];
+        const FrameRec *frec = keep(x.frec + (threadIdx.x & 31));
         const uint32_t local = item - x.a0;
         const int band = (int)(local / (uint32_t)x.ntiles_x), tile = (int)(local % (uint32_t)x.ntiles_x);
-        const int tbx = x.tbx, tw = 2 * tbx, th = 2 * (32 / tbx);
+        const int tbx = x.tbx, tw = 2 * tbx, th = 2 * (32 / tbx), x0 = tile * tw, y0 = band * th;
+        // every thread is past the last tile's gather
+        if (threadIdx.x < kTilePixels) ts.fc[threadIdx.x] = load_const(threadIdx.x, x.W, x.H, x0, y0, tw, x.fconst);
+        load_offsets(ts, x.W, x.H, x.R, x0, y0, tw, th, x.foff);
+        if (x.R != held) fill_discs(discs, x.R);
+        held = x.R;
+        __syncthreads();
         for (int blk = warp; blk < 32; blk += kWarps) {
-            const int bx = tile * tw + (blk % tbx) * 2, by = band * th + (blk / tbx) * 2;
-            if (bx >= x.W || by >= x.H) continue;
-            filter_block<CT, KAHAN, false>(x.W, x.H, x.R, bx, by, x.fconst, x.foff, x.fpos, x.fcol, x.out,
-                                           smem[warp], DebugCheck{x.fcap, x.derr});
+            const int lx = blk % tbx, ly = blk / tbx;
+            if (x0 + 2 * lx >= x.W || y0 + 2 * ly >= x.H) continue;
+            filter_block<KAHAN, false>(x.W, x.H, x.R, x0, y0, tw, lx, ly, frec, x.out, ts, &discs, table_at, held,
+                                       ts.rows[warp], rows_at, DebugCheck{x.fcap, x.derr});
         }
         __syncthreads();
     }
@@ -597,16 +729,14 @@ __global__ void __launch_bounds__(256, 3) k_batch(const BatchCtx *__restrict__ c
 
 // ---- adjoint -------------------------------------------------------------------
 
-template <int CT>
 __global__ void __launch_bounds__(128) k_bwd_pixel(int W, int H, int R, int S_, int ntx, float window, float eps,
                                                    AfrParams prm, const float4 *__restrict__ grad,
                                                    const TilePartial *__restrict__ tiles,
                                                    const float2 *__restrict__ sigma, const uint32_t *__restrict__ amin2,
-                                                   const uint32_t *__restrict__ foff, const float4 *__restrict__ fpos,
-                                                   const void *__restrict__ fcol, const float4 *__restrict__ gout,
+                                                   const uint32_t *__restrict__ foff, const FrameRec *__restrict__ frec,
+                                                   const float4 *__restrict__ gout,
                                                    float4 *__restrict__ bg, float4 *__restrict__ bframe,
                                                    float *__restrict__ bparam) {
-    using CS = ColorStore<CT>;
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = blockIdx.y * blockDim.y + threadIdx.y;
     float gp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -628,8 +758,8 @@ __global__ void __launch_bounds__(128) k_bwd_pixel(int W, int H, int R, int S_, 
                 int x0 = max(0, x - hw), x1 = min(W - 1, x + hw);
                 uint32_t e0 = __ldg(foff + (size_t)row * W + x0), e1 = __ldg(foff + (size_t)row * W + x1 + 1);
                 for (uint32_t e = e0; e < e1; ++e) {
-                    float4 r = __ldg(fpos + e);
-                    float3 c = CS::load(fcol, e);
+                    const FrameRec q = load_rec(frec + e);
+                    const float4 r = q.p, c = q.c;
                     float w = ex2(-shifted_exponent(f, r));
                     float ddx = r.x - f.cx, ddy = r.y - f.cy;
                     float d2 = fmaf(ddx, ddx, ddy * ddy);
@@ -680,11 +810,11 @@ __global__ void __launch_bounds__(128) k_bwd_pixel(int W, int H, int R, int S_, 
 // Gradient of each frame record's colour: sum over the pixels whose disc
 // holds the record's bin of (dL/dC_p / S_p) * shifted weight.
 __global__ void __launch_bounds__(256) k_bwd_record(int W, int H, int R, const uint32_t *__restrict__ foff,
-                                                    const float4 *__restrict__ fpos, const float4 *__restrict__ bg,
+                                                    const FrameRec *__restrict__ frec, const float4 *__restrict__ bg,
                                                     const float4 *__restrict__ bframe, float *__restrict__ gcol) {
     uint32_t n = __ldg(foff + (size_t)W * H);
     for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        float4 r = __ldg(fpos + e);
+        float4 r = __ldg(&frec[e].p);
         int qx = (int)floorf(r.x), qy = (int)floorf(r.y);
         float a0 = 0.f, a1 = 0.f, a2 = 0.f;
         for (int dy = -R; dy <= R; ++dy) {
@@ -744,23 +874,21 @@ __global__ void k_bwd_params(const float *__restrict__ part, int nblocks, float 
     }
 }
 
+// Colours rounded to the storage type, then widened as the frame view holds them.
 template <int CT>
 __global__ void k_set_colors(const float *__restrict__ rgb, const uint32_t *__restrict__ foff, int P,
-                             void *__restrict__ fcol) {
+                             FrameRec *__restrict__ frec) {
     uint32_t n = __ldg(foff + P);
     for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        float r = rgb[3 * (size_t)e], g = rgb[3 * (size_t)e + 1], b = rgb[3 * (size_t)e + 2];
-        if (CT == AFR_F32) {
-            reinterpret_cast<float4 *>(fcol)[e] = make_float4(r, g, b, 0.f);
-        } else if (CT == AFR_F16) {
-            reinterpret_cast<ushort4 *>(fcol)[e] = make_ushort4(__half_as_ushort(__float2half_rn(r)),
-                                                                __half_as_ushort(__float2half_rn(g)),
-                                                                __half_as_ushort(__float2half_rn(b)), 0);
-        } else {
-            reinterpret_cast<ushort4 *>(fcol)[e] = make_ushort4(__bfloat16_as_ushort(__float2bfloat16_rn(r)),
-                                                                __bfloat16_as_ushort(__float2bfloat16_rn(g)),
-                                                                __bfloat16_as_ushort(__float2bfloat16_rn(b)), 0);
+        float v[3] = {rgb[3 * (size_t)e], rgb[3 * (size_t)e + 1], rgb[3 * (size_t)e + 2]};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (CT == AFR_F16) v[k] = __half2float(__float2half_rn(v[k]));
+            if (CT == AFR_BF16) v[k] = __bfloat162float(__float2bfloat16_rn(v[k]));
         }
+        float *c = &frec[e].c.x;   // the sequence number beside it stays
+        *reinterpret_cast<float2 *>(c) = make_float2(v[0], v[1]);
+        c[2] = v[2];
     }
 }
 
@@ -799,23 +927,13 @@ cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
     const int tbx = c->tile_bx, tw = 2 * tbx, th = 2 * (32 / tbx);
     dim3 grid((c->W + tw - 1) / tw, (c->H + th - 1) / th);
-#define AFR_FILTER(CT_, K_, V_)                                                                          \
-    k_filter<CT_, K_, V_><<<grid, kQuadBlock, 0, s>>>(c->W, c->H, c->R, tbx, c->fconst, c->foff, c->fpos, c->fcol, \
-                                                      out, dc)
-    switch (c->ct) {
-        case AFR_F32:
-            if (adaptive) AFR_FILTER(AFR_F32, false, true);
-            else AFR_FILTER(AFR_F32, false, false);
-            break;
-        case AFR_F16:
-            if (adaptive) AFR_FILTER(AFR_F16, true, true);
-            else AFR_FILTER(AFR_F16, true, false);
-            break;
-        default:
-            if (adaptive) AFR_FILTER(AFR_BF16, true, true);
-            else AFR_FILTER(AFR_BF16, true, false);
-            break;
-    }
+#define AFR_FILTER(K_, V_) \
+    k_filter<K_, V_><<<grid, kQuadBlock, 0, s>>>(c->W, c->H, c->R, __builtin_ctz(tbx), c->fconst, c->foff, c->frec, out, dc)
+    // colours stored in 16 bits: compensated weight sums
+    if (c->ct == AFR_F32 && adaptive) AFR_FILTER(false, true);
+    else if (c->ct == AFR_F32) AFR_FILTER(false, false);
+    else if (adaptive) AFR_FILTER(true, true);
+    else AFR_FILTER(true, false);
 #undef AFR_FILTER
     return cudaGetLastError();
 }
@@ -825,19 +943,11 @@ cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_c
     dim3 grid((c->W + kFilterBlock.x - 1) / kFilterBlock.x, (c->H + kFilterBlock.y - 1) / kFilterBlock.y);
     float4 *bframe = c->bgrad + c->P;
     const AfrParams &prm = c->recon_params;
-#define AFR_BWD(CT_)                                                                                        \
-    k_bwd_pixel<CT_><<<grid, kFilterBlock, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window,           \
-                                                   c->cfg.eps_grad, prm, c->grad, c->tiles, c->sigma, c->amin2, \
-                                                   c->foff, c->fpos, c->fcol, grad_rgb, c->bgrad, bframe,   \
-                                                   c->bparam)
-    switch (c->ct) {
-        case AFR_F32: AFR_BWD(AFR_F32); break;
-        case AFR_F16: AFR_BWD(AFR_F16); break;
-        default: AFR_BWD(AFR_BF16); break;
-    }
-#undef AFR_BWD
+    k_bwd_pixel<<<grid, kFilterBlock, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, prm,
+                                              c->grad, c->tiles, c->sigma, c->amin2, c->foff, c->frec, grad_rgb,
+                                              c->bgrad, bframe, c->bparam);
     if (grad_col)
-        k_bwd_record<<<grid_for((size_t)c->P * c->b, 256), 256, 0, s>>>(c->W, c->H, c->R, c->foff, c->fpos, c->bgrad,
+        k_bwd_record<<<grid_for((size_t)c->P * c->b, 256), 256, 0, s>>>(c->W, c->H, c->R, c->foff, c->frec, c->bgrad,
                                                                         bframe, grad_col);
     if (grad_prm) k_bwd_params<<<1, 6 * 32, 0, s>>>(c->bparam, (int)(grid.x * grid.y), grad_prm);
     return cudaGetLastError();
@@ -846,9 +956,9 @@ cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_c
 cudaError_t launch_set_frame_colors(AfrContext *c, const float *rgb, cudaStream_t s) {
     int g = grid_for((size_t)c->P * c->b, 256);
     switch (c->ct) {
-        case AFR_F32: k_set_colors<AFR_F32><<<g, 256, 0, s>>>(rgb, c->foff, c->P, c->fcol); break;
-        case AFR_F16: k_set_colors<AFR_F16><<<g, 256, 0, s>>>(rgb, c->foff, c->P, c->fcol); break;
-        default: k_set_colors<AFR_BF16><<<g, 256, 0, s>>>(rgb, c->foff, c->P, c->fcol); break;
+        case AFR_F32: k_set_colors<AFR_F32><<<g, 256, 0, s>>>(rgb, c->foff, c->P, c->frec); break;
+        case AFR_F16: k_set_colors<AFR_F16><<<g, 256, 0, s>>>(rgb, c->foff, c->P, c->frec); break;
+        default: k_set_colors<AFR_BF16><<<g, 256, 0, s>>>(rgb, c->foff, c->P, c->frec); break;
     }
     return cudaGetLastError();
 }
@@ -856,11 +966,8 @@ cudaError_t launch_set_frame_colors(AfrContext *c, const float *rgb, cudaStream_
 cudaError_t launch_batch(int ct, const BatchCtx *cs, int nctx, uint32_t nchunks, uint32_t total, uint32_t *queue,
                          int grid, cudaStream_t s) {
     k_batch_sigma<<<grid_for((size_t)nchunks * 256, 256), 256, 0, s>>>(cs, nctx, nchunks);
-    switch (ct) {
-        case AFR_F32: k_batch<AFR_F32, false><<<grid, kQuadBlock, 0, s>>>(cs, nctx, total, queue); break;
-        case AFR_F16: k_batch<AFR_F16, true><<<grid, kQuadBlock, 0, s>>>(cs, nctx, total, queue); break;
-        default: k_batch<AFR_BF16, true><<<grid, kQuadBlock, 0, s>>>(cs, nctx, total, queue); break;
-    }
+    if (ct == AFR_F32) k_batch<false><<<grid, kQuadBlock, 0, s>>>(cs, nctx, total, queue);
+    else k_batch<true><<<grid, kQuadBlock, 0, s>>>(cs, nctx, total, queue);
     return cudaGetLastError();
 }
 

@@ -14,8 +14,9 @@
 //  place:  thread per frame record, in bin order: the slot of list entry e
 //          is moved again, its rank in the bin is the number of sequence
 //          numbers in the bin's list below its own (sequence numbers are
-//          unique), and it writes (x', y', a^2, bin column), its colour and its
-//          sequence number to the bin's offset + rank. The lanes of a warp
+//          unique), and it writes the 32-byte frame record (x', y', a^2, its bin's
+//          place, its colour in FP32, its sequence number) to the bin's offset +
+//          rank. The lanes of a warp
 //          mostly share a bin, so the rank scans are broadcast reads and the
 //          record writes cover whole sectors; the frame view, and every sum
 //          over it, is deterministic without a reorder pass over the records.
@@ -212,8 +213,7 @@ __global__ void __launch_bounds__(256) k_place(int W, int H, float t_now, Camera
                                                const void *__restrict__ r_col, uint32_t P,
                                                const uint32_t *__restrict__ foff, const uint32_t *__restrict__ flist,
                                                const uint32_t *__restrict__ flseq, uint32_t *__restrict__ fcnt,
-                                               uint32_t *__restrict__ amin2, float4 *__restrict__ fpos,
-                                               void *__restrict__ fcol, uint32_t *__restrict__ fseq,
+                                               uint32_t *__restrict__ amin2, FrameRec *__restrict__ frec,
                                                unsigned long long *__restrict__ dcount, DebugCheck dc, uint32_t nsrc) {
     using CS = ColorStore<CT>;
     uint32_t n = __ldg(foff + P);
@@ -251,9 +251,9 @@ __global__ void __launch_bounds__(256) k_place(int W, int H, float t_now, Camera
         }
         const uint32_t d = beg + rank;
         if (!AFR_CHECK(d < n, dc.derr)) continue;
-        fpos[d] = make_float4(mv.xp, mv.yp, mv.a2, __int_as_float((int)floorf(mv.xp)));
-        reinterpret_cast<typename CS::T *>(fcol)[d] = CS::raw(r_col, i);
-        fseq[d] = sq;
+        const float3 c = CS::load(r_col, i);
+        store_rec(frec + d, {make_float4(mv.xp, mv.yp, mv.a2, bin_place(mv.xp, mv.yp)),
+                             make_float4(c.x, c.y, c.z, __uint_as_float(sq))});
     }
 }
 
@@ -285,7 +285,7 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
 #define AFR_COUNT(F_, C_)                                                                                    \
     k_count<F_, C_><<<g, 256, 0, s>>>(ns, c->b, bshift, c->W, c->H, t_now, cm, wp, state, xy, mo, tt, c->fcnt, \
-                                      c->fseq, c->dcount)
+                                      c->sbin, c->dcount)
     if (fifo && cam) AFR_COUNT(true, true);
     else if (fifo) AFR_COUNT(true, false);
     else if (cam) AFR_COUNT(false, true);
@@ -295,11 +295,10 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     // the list's append cursors start at the bin offsets (a ticket is the entry's place)
     if ((e = cudaMemcpyAsync(c->fcnt, c->foff, sizeof(uint32_t) * c->P, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
         return e;
-    // fseq holds each slot's bin until the placement pass writes the frame
-    k_list<<<g, 256, 0, s>>>(ns, c->fseq, sq, c->fcnt, c->flist, c->flseq, dc);
+    k_list<<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcnt, c->flist, c->flseq, dc);
 #define AFR_PLACE(CT_, F_, C_)                                                                                     \
     k_place<CT_, F_, C_><<<g, 256, 0, s>>>(c->W, c->H, t_now, cm, wp, xy, mo, tt, sq, col, (uint32_t)c->P, c->foff, \
-                                           c->flist, c->flseq, c->fcnt, c->amin2, c->fpos, c->fcol, c->fseq,       \
+                                           c->flist, c->flseq, c->fcnt, c->amin2, c->frec,       \
                                            c->dcount, dc, ns)
 #define AFR_REPROJ(CT_)                                                                                        \
     do {                                                                                                       \
