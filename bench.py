@@ -119,8 +119,8 @@ class ClockSampler:
 #       -c 20 --csv --log-file launches.csv python bench.py --profile --steps 1 --warmup 0 --no-cpu-baseline
 # A changed kernel has no entry, and the line then reports null.
 FILTER_TRAFFIC = {
-    ("6bd769946ab94e7f10cea56098c556932ad8d70a6ece13860732d85d7dbb645e",
-     "63c9dbc321616d713b944b8786da0ab400f22c2b9e448d1eecf7242991f45025"): 0.989e9 + 0.031e9,
+    ("143da3eaaba68891ec3f19dee24844057b28c7a4236973378e26ec4fb99650e3",
+     "3f68b920ff77d63c39515dc2b781f0b724cd643056b182e1da02a77183a9bac6"): 0.988e9 + 0.031e9,
 }
 
 

@@ -163,7 +163,7 @@ struct AfrContext {
     size_t scan_tmp_n = 0;
 
     // backward scratch
-    float4 *bgrad = nullptr;      // [P] per-pixel (g_r/S, g_g/S, g_b/S, valid)
+    float4 *bgrad = nullptr;      // [2 P] planes the adjoint passes share (k_filter.cu: Adjoint)
     float *bparam = nullptr;      // [n_bblocks * 6] per-block parameter-gradient partials
     int n_bblocks = 0;
 

@@ -90,12 +90,6 @@ __device__ __forceinline__ PixelFrame pixel_frame(int x, int y, int W, int H, in
     return f;
 }
 
-__device__ __forceinline__ float shifted_exponent(const PixelFrame &f, float4 r) {
-    float dx = r.x - f.cx, dy = r.y - f.cy;
-    float d2 = fmaf(dx, dx, dy * dy);
-    return fmaf(d2, f.ks, fmaf(r.z, f.kt, -f.m));
-}
-
 // Filter widths of every pixel (unless KEEP: the widths already in the map
 // are used) and the pixel's gather constants for the filter: -ks, -kt, the
 // exponent shift m and the footprint radius (the configured R, or with ADAPT
@@ -247,39 +241,25 @@ __device__ __forceinline__ uint32_t warp_incl_scan_u(uint32_t v) {
     return v;
 }
 
-// Reduces 16 per-lane values across the warp; afterwards lane l holds the
-// total of value ((l>>4)&1)*8 + ((l>>3)&1)*4 + ((l>>2)&1)*2 + ((l>>1)&1)
-// (transposed butterfly: 8 + 4 + 2 + 1 + 1 exchanges).
-__device__ __forceinline__ float warp_reduce16(float (&v)[16]) {
+// Reduces N per-lane values (N a power of two up to 32) across the warp:
+// afterwards lane l holds the total of value l / (32 / N) with its log2(N) bits
+// as they are (a transposed butterfly: N - 1 exchanges, then log2(32 / N)
+// among the lanes that share a value).
+template <int N>
+__device__ __forceinline__ float warp_reduce(float (&v)[N]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        bool hi = lane & 16;
-        float send = hi ? v[k] : v[k + 8];
-        float keep = hi ? v[k + 8] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    for (int n = N / 2, o = 16; n > 0; n >>= 1, o >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int k = 0; k < N / 2; ++k) {
+            if (k >= n) break;
+            const float send = hi ? v[k] : v[k + n], stay = hi ? v[k + n] : v[k];
+            v[k] = stay + __shfl_xor_sync(0xffffffffu, send, o);
+        }
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        bool hi = lane & 8;
-        float send = hi ? v[k] : v[k + 4];
-        float keep = hi ? v[k + 4] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        bool hi = lane & 4;
-        float send = hi ? v[k] : v[k + 2];
-        float keep = hi ? v[k + 2] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    {
-        bool hi = lane & 2;
-        float send = hi ? v[0] : v[1];
-        float keep = hi ? v[1] : v[0];
-        v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-    }
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    for (int o = 16 / N; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     return v[0];
 }
 
@@ -290,40 +270,60 @@ struct PairConsts {
     f2 cy[2];            // (cy_j, cy_j): row centres
     f2 nks[2], nkt[2], m[2];
 };
-struct PairAcc {
-    f2 S[2], C[2], r[2], g[2], b[2];
+// Weights of the block's four pixels for one record. in: 0 for each pixel
+// whose disc holds the record's bin, else -inf; pixel k = 2 j + column in
+// component k.
+struct PairWeights {
+    f2 d2[2], w[2];
 };
 
-// in: 0 for each pixel whose disc holds the record's bin, else -inf; pixel
-// k = 2 j + column in component k.
-template <bool KAHAN>
-__device__ __forceinline__ void accumulate(const PairConsts &pc, float4 in, const FrameRec &q, PairAcc &A) {
+__device__ __forceinline__ PairWeights pair_weights(const PairConsts &pc, float4 in, const FrameRec &q) {
+    PairWeights r;
     const f2 dx = sub2(pk(q.p.x, q.p.x), pc.cx);
     const f2 sx = mul2(dx, dx);
     const f2 y = pk(q.p.y, q.p.y), a2 = pk(q.p.z, q.p.z);
-    const f2 cr = pk(q.c.x, q.c.x), cg = pk(q.c.y, q.c.y), cb = pk(q.c.z, q.c.z);
     const f2 t[2] = {pk(in.x, in.y), pk(in.z, in.w)};
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const f2 dy = sub2(y, pc.cy[j]);
-        const f2 d2 = fma2(dy, dy, sx);
-        const f2 e = fma2(d2, pc.nks[j], fma2(a2, pc.nkt[j], add2(pc.m[j], t[j])));
+        r.d2[j] = fma2(dy, dy, sx);
+        const f2 e = fma2(r.d2[j], pc.nks[j], fma2(a2, pc.nkt[j], add2(pc.m[j], t[j])));
         float e0, e1;
         upk(e, e0, e1);
-        const f2 w = pk(ex2(e0), ex2(e1));
-        if (KAHAN) {
-            const f2 v = sub2(w, A.C[j]);
-            const f2 n = add2(A.S[j], v);
-            A.C[j] = sub2(sub2(n, A.S[j]), v);
-            A.S[j] = n;
-        } else {
-            A.S[j] = add2(A.S[j], w);
-        }
-        A.r[j] = fma2(w, cr, A.r[j]);
-        A.g[j] = fma2(w, cg, A.g[j]);
-        A.b[j] = fma2(w, cb, A.b[j]);
+        r.w[j] = pk(ex2(e0), ex2(e1));
     }
+    return r;
 }
+
+// What the gather sums. Forward: the weights (compensated for 16-bit colour
+// storage) and the weighted colours.
+template <bool KAHAN>
+struct ForwardSums {
+    f2 S[2], C[2], r[2], g[2], b[2];
+    __device__ __forceinline__ ForwardSums() {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) S[j] = C[j] = r[j] = g[j] = b[j] = 0ull;
+    }
+    __device__ __forceinline__ void add(const PairConsts &pc, float4 in, const FrameRec &q) {
+        const PairWeights p = pair_weights(pc, in, q);
+        const f2 cr = pk(q.c.x, q.c.x), cg = pk(q.c.y, q.c.y), cb = pk(q.c.z, q.c.z);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const f2 w = p.w[j];
+            if (KAHAN) {
+                const f2 v = sub2(w, C[j]);
+                const f2 n = add2(S[j], v);
+                C[j] = sub2(sub2(n, S[j]), v);
+                S[j] = n;
+            } else {
+                S[j] = add2(S[j], w);
+            }
+            r[j] = fma2(w, cr, r[j]);
+            g[j] = fma2(w, cg, g[j]);
+            b[j] = fma2(w, cb, b[j]);
+        }
+    }
+};
 
 // Discs of the union box of a 2x2 block at footprint radius R: entry
 // (v, u) = bin row by - R + v, column bx - R + u.
@@ -412,7 +412,7 @@ struct TileSmem {
     float4 fc[kTilePixels];
     uint32_t off[kTileOffsets];
     uint2 rows[kWarps][kMaxRows];
-};
+};   // adjoint kernels run kBwdWarps <= kWarps warps a CTA
 
 // Offsets of the bins of rows y0 - R .. y0 + th + R - 1 at columns x0 - R ..
 // x0 + tw + R (clamped to the row's first and last; rows outside the image
@@ -420,7 +420,7 @@ struct TileSmem {
 __device__ __forceinline__ void load_offsets(TileSmem &t, int W, int H, int R, int x0, int y0, int tw, int th,
                                              const uint32_t *__restrict__ foff) {
     const int cols = tw + 2 * R + 1;
-    for (int r = threadIdx.x >> 5; r < th + 2 * R; r += kWarps) {
+    for (int r = threadIdx.x >> 5; r < th + 2 * R; r += blockDim.x >> 5) {
         const int row = y0 - R + r;
         for (int c = threadIdx.x & 31; c < cols; c += 32) {
             uint32_t v = 0;
@@ -436,17 +436,16 @@ __device__ __forceinline__ float4 load_const(int i, int W, int H, int x0, int y0
     return __ldg(fconst + (size_t)min(y0 + i / tw, H - 1) * W + min(x0 + i % tw, W - 1));
 }
 
-// One 2x2 pixel block by one warp: the block (lx, ly) of the tile at (x0, y0),
-// tw pixels wide, whose offsets were loaded for footprints up to Rt.
+// Sums of one 2x2 pixel block by one warp: the block (lx, ly) of the tile at
+// (x0, y0), tw pixels wide, whose offsets were loaded for footprints up to Rt.
 // VAR: each pixel's footprint radius is read from its gather constants
 // (adaptive footprints); otherwise every pixel uses Rt. table: the warp's own
 // discs (VAR; held says for which radius it was filled last) or the CTA's, at
 // shared address table_at. frec: the frame view from this lane's record on.
-template <bool KAHAN, bool VAR>
-__device__ __forceinline__ void filter_block(int W, int H, int Rt, int x0, int y0, int tw, int lx, int ly,
-                                             const FrameRec *frec, float4 *__restrict__ out, const TileSmem &ts,
-                                             DiscTable *table, uint32_t table_at, int &held, uint2 *rows,
-                                             uint32_t rows_at, const DebugCheck &dc) {
+template <bool VAR, class Sums>
+__device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int lx, int ly, const FrameRec *frec,
+                                             const TileSmem &ts, DiscTable *table, uint32_t table_at, int &held,
+                                             uint2 *rows, uint32_t rows_at, const DebugCheck &dc, Sums &A) {
     const int lane = threadIdx.x & 31;
     const int bx = x0 + 2 * lx, by = y0 + 2 * ly;
     float4 fc[4];
@@ -517,9 +516,6 @@ __device__ __forceinline__ void filter_block(int W, int H, int Rt, int x0, int y
         pc.nkt[j] = pk(fc[2 * j].y, fc[2 * j + 1].y);
         pc.m[j] = pk(fc[2 * j].z, fc[2 * j + 1].z);
     }
-    PairAcc A;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) A.S[j] = A.C[j] = A.r[j] = A.g[j] = A.b[j] = 0ull;
     const int origin = (by - R) * kPitch + bx - R;
     const uint32_t tab = keep(table_at - (uint32_t)origin * 16u);   // + 16 place: the entry of a record's bin
     auto load = [&](int i) {   // record i + lane (i itself may be negative)
@@ -533,7 +529,7 @@ __device__ __forceinline__ void filter_block(int W, int H, int Rt, int x0, int y
         const bool ok = AFR_CHECK(place >= origin && place < origin + (2 * R + 2) * kPitch, dc.derr);
         float4 d = lds4(ok ? tab + (uint32_t)place * 16u : table_at);
         if (!ok) d = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        accumulate<KAHAN>(pc, d, r, A);
+        A.add(pc, d, r);
     };
     // The last iteration's lanes past the end read on (the frame arrays end in
     // kFramePad records of padding) and are dropped before they are summed.
@@ -566,43 +562,40 @@ __device__ __forceinline__ void filter_block(int W, int H, int Rt, int x0, int y
         if (one) gather(std::true_type{});
         else gather(std::false_type{});
     }
-    __syncwarp();
-    float vals[16];
+    __syncwarp();   // the next block overwrites the row table
+}
+
+// Tile pixel of a block that lane k = lane mod 4 stores.
+__device__ __forceinline__ int block_pixel(int tw, int lx, int ly) {
+    return (2 * ly + ((threadIdx.x >> 1) & 1)) * tw + 2 * lx + (threadIdx.x & 1);
+}
+
+// Normalised colours and weight sums of a block's pixels from its sums.
+template <bool KAHAN>
+__device__ __forceinline__ void store_block(const ForwardSums<KAHAN> &A, int W, int H, int bx, int by, float4 fc,
+                                            float4 *__restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    float vals[16];   // sum q of pixel k at q * 4 + k (q: S, r, g, b)
 #pragma unroll
-    for (int jj = 0; jj < 2; ++jj) {
-        float a, b;
-        upk(KAHAN ? sub2(A.S[jj], A.C[jj]) : A.S[jj], a, b);
-        vals[2 * jj] = a;
-        vals[2 * jj + 1] = b;
-        upk(A.r[jj], a, b);
-        vals[4 + 2 * jj] = a;
-        vals[4 + 2 * jj + 1] = b;
-        upk(A.g[jj], a, b);
-        vals[8 + 2 * jj] = a;
-        vals[8 + 2 * jj + 1] = b;
-        upk(A.b[jj], a, b);
-        vals[12 + 2 * jj] = a;
-        vals[12 + 2 * jj + 1] = b;
+    for (int j = 0; j < 2; ++j) {
+        upk(KAHAN ? sub2(A.S[j], A.C[j]) : A.S[j], vals[2 * j], vals[2 * j + 1]);
+        upk(A.r[j], vals[4 + 2 * j], vals[4 + 2 * j + 1]);
+        upk(A.g[j], vals[8 + 2 * j], vals[8 + 2 * j + 1]);
+        upk(A.b[j], vals[12 + 2 * j], vals[12 + 2 * j + 1]);
     }
-    const float tot = warp_reduce16(vals);
-    // value qq*4 + k (qq: S, r, g, b) of pixel k moves to lane k
-    float q[4];
+    const float tot = warp_reduce(vals);
+    float q[4];   // to lane k
 #pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-        const int want = qq * 4 + (lane & 3);
-        const int src = ((want >> 3) & 1) * 16 + ((want >> 2) & 1) * 8 + ((want >> 1) & 1) * 4 + (want & 1) * 2;
-        q[qq] = __shfl_sync(0xffffffffu, tot, src);
-    }
-    if (lane < 4 && bx + (lane & 1) < W && by + (lane >> 1) < H) {
+    for (int i = 0; i < 4; ++i) q[i] = __shfl_sync(0xffffffffu, tot, 2 * (4 * i + (lane & 3)));
+    const int x = bx + (lane & 1), y = by + ((lane >> 1) & 1);
+    if (lane < 4 && x < W && y < H) {
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
         if (q[0] > 0.f) {
             const float inv = 1.f / q[0];
-            const float m = lane & 2 ? (lane & 1 ? fc[3].z : fc[2].z) : (lane & 1 ? fc[1].z : fc[0].z);
-            o = make_float4(q[1] * inv, q[2] * inv, q[3] * inv, q[0] * ex2(-m));
+            o = make_float4(q[1] * inv, q[2] * inv, q[3] * inv, q[0] * ex2(-fc.z));
         }
-        out[(size_t)(by + (lane >> 1)) * W + bx + (lane & 1)] = o;
+        out[(size_t)y * W + x] = o;
     }
-    __syncwarp();
 }
 
 // Tile of (2 * tbx) x (2 * 32 / tbx) pixels per CTA: 32 blocks of 2x2, four
@@ -634,8 +627,10 @@ __global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx
     for (int blk = warp; blk < 32; blk += kWarps) {
         const int lx = blk & ((1 << ltbx) - 1), ly = blk >> ltbx;
         if (x0 + 2 * lx >= W || y0 + 2 * ly >= H) continue;   // warp-uniform
-        filter_block<KAHAN, VAR>(W, H, Rt, x0, y0, tw, lx, ly, frec, out, ts, discs + (VAR ? warp : 0), table_at, held,
-                                 ts.rows[warp], rows_at, dc);
+        ForwardSums<KAHAN> A;
+        gather_block<VAR>(Rt, x0, y0, tw, lx, ly, frec, ts, discs + (VAR ? warp : 0), table_at, held, ts.rows[warp],
+                          rows_at, dc, A);
+        store_block(A, W, H, x0 + 2 * lx, y0 + 2 * ly, ts.fc[block_pixel(tw, lx, ly)], out);
     }
 }
 
@@ -720,127 +715,281 @@ __global__ void __launch_bounds__(256, 3) k_batch(const BatchCtx *__restrict__ c
         for (int blk = warp; blk < 32; blk += kWarps) {
             const int lx = blk % tbx, ly = blk / tbx;
             if (x0 + 2 * lx >= x.W || y0 + 2 * ly >= x.H) continue;
-            filter_block<KAHAN, false>(x.W, x.H, x.R, x0, y0, tw, lx, ly, frec, x.out, ts, &discs, table_at, held,
-                                       ts.rows[warp], rows_at, DebugCheck{x.fcap, x.derr});
+            ForwardSums<KAHAN> A;
+            gather_block<false>(x.R, x0, y0, tw, lx, ly, frec, ts, &discs, table_at, held, ts.rows[warp], rows_at,
+                                DebugCheck{x.fcap, x.derr}, A);
+            store_block(A, x.W, x.H, x0 + 2 * lx, y0 + 2 * ly, ts.fc[block_pixel(tw, lx, ly)], x.out);
         }
         __syncthreads();
     }
 }
 
 // ---- adjoint -------------------------------------------------------------------
+// A pass over the pixels (the same gather as the forward pass, with more sums),
+// then one over the records. Between them, what a record needs of each pixel:
+// a plane of float4 (-ks, -kt, shift, g_r / S) and one of float2 (g_g / S,
+// g_b / S), g the loss gradient of the pixel's colour (0 where it holds no
+// sample).
+struct Adjoint {
+    float4 *k;
+    float2 *g;
+};
 
-__global__ void __launch_bounds__(128) k_bwd_pixel(int W, int H, int R, int S_, int ntx, float window, float eps,
-                                                   AfrParams prm, const float4 *__restrict__ grad,
-                                                   const TilePartial *__restrict__ tiles,
-                                                   const float2 *__restrict__ sigma, const uint32_t *__restrict__ amin2,
-                                                   const uint32_t *__restrict__ foff, const FrameRec *__restrict__ frec,
-                                                   const float4 *__restrict__ gout,
-                                                   float4 *__restrict__ bg, float4 *__restrict__ bframe,
-                                                   float *__restrict__ bparam) {
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
-    float gp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (x < W && y < H) {
-        size_t p = (size_t)y * W + x;
-        float2 sgm = __ldg(sigma + p);
-        PixelFrame f = pixel_frame(x, y, W, H, R, sgm, amin2);
-        float4 g = __ldg(gout + p);
-        if (!f.any) {
-            bg[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-            bframe[p] = make_float4(f.ks, f.kt, f.m, 0.f);
-        } else {
-            float S = 0.f, sc[3] = {0.f, 0.f, 0.f}, Ds = 0.f, dsc[3] = {0.f, 0.f, 0.f}, Dt = 0.f,
-                  dtc[3] = {0.f, 0.f, 0.f};
-            for (int dy = -R; dy <= R; ++dy) {
-                int row = y + dy;
-                if (row < 0 || row >= H) continue;
-                int hw = half_width(R, dy);
-                int x0 = max(0, x - hw), x1 = min(W - 1, x + hw);
-                uint32_t e0 = __ldg(foff + (size_t)row * W + x0), e1 = __ldg(foff + (size_t)row * W + x1 + 1);
-                for (uint32_t e = e0; e < e1; ++e) {
-                    const FrameRec q = load_rec(frec + e);
-                    const float4 r = q.p, c = q.c;
-                    float w = ex2(-shifted_exponent(f, r));
-                    float ddx = r.x - f.cx, ddy = r.y - f.cy;
-                    float d2 = fmaf(ddx, ddx, ddy * ddy);
-                    float ws = w * d2, wt = w * r.z;
-                    S += w;
-                    sc[0] = fmaf(w, c.x, sc[0]); sc[1] = fmaf(w, c.y, sc[1]); sc[2] = fmaf(w, c.z, sc[2]);
-                    Ds += ws; Dt += wt;
-                    dsc[0] = fmaf(ws, c.x, dsc[0]); dsc[1] = fmaf(ws, c.y, dsc[1]); dsc[2] = fmaf(ws, c.z, dsc[2]);
-                    dtc[0] = fmaf(wt, c.x, dtc[0]); dtc[1] = fmaf(wt, c.y, dtc[1]); dtc[2] = fmaf(wt, c.z, dtc[2]);
-                }
-            }
-            float inv = 1.f / S;
-            float gch[3] = {g.x, g.y, g.z};
-            float s3 = sgm.x * sgm.x * sgm.x, t3 = sgm.y * sgm.y * sgm.y;
-            float gs = 0.f, gt = 0.f;
-            for (int ch = 0; ch < 3; ++ch) {
-                float C = sc[ch] * inv;
-                gs = fmaf(gch[ch], (dsc[ch] - C * Ds) * inv / s3, gs);
-                gt = fmaf(gch[ch], (dtc[ch] - C * Dt) * inv / t3, gt);
-            }
-            bg[p] = make_float4(g.x * inv, g.y * inv, g.z * inv, 1.f);
-            bframe[p] = make_float4(f.ks, f.kt, f.m, 1.f);
-            // chain through the width mapping; the widths depend on theta only
-            Widths wd = widths(__ldg(grad + p), tile_volume(x, y, W, H, S_, ntx, window, tiles), eps, prm);
-            if (fmaxf(wd.raw_s, kSigmaSMin) >= prm.clamp_s) gp[2] = gs;
-            else if (wd.raw_s > kSigmaSMin) { gp[0] = gs * wd.es; gp[1] = gs; }
-            if (fmaxf(wd.raw_t, kSigmaTMin) >= prm.clamp_t) gp[5] = gt;
-            else if (wd.raw_t > kSigmaTMin) { gp[3] = gt * wd.et; gp[4] = gt; }
+// With q = g . c (g the loss gradient of the pixel's colour C), the width
+// gradients need, summed over the records: w, w q, w d^2, w d^2 q, w a^2 and
+// w a^2 q: dL/dsigma_s = (sum w d^2 q - (g . C) sum w d^2) / S / sigma_s^3, and
+// the same with a^2 for sigma_t.
+struct AdjointSums {
+    f2 S[2], Q[2], Ds[2], Dsq[2], Dt[2], Dtq[2];
+    f2 g[2][3];
+    __device__ __forceinline__ AdjointSums(const float4 (&go)[4]) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            S[j] = Q[j] = Ds[j] = Dsq[j] = Dt[j] = Dtq[j] = 0ull;
+            g[j][0] = pk(go[2 * j].x, go[2 * j + 1].x);
+            g[j][1] = pk(go[2 * j].y, go[2 * j + 1].y);
+            g[j][2] = pk(go[2 * j].z, go[2 * j + 1].z);
         }
     }
-    // block reduction of the six parameter gradients, then one FP64 partial per block
-    __shared__ float sh[6][4];
-    int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    for (int k = 0; k < 6; ++k) {
-        float v = gp[k];
+    __device__ __forceinline__ void add(const PairConsts &pc, float4 in, const FrameRec &r) {
+        const PairWeights p = pair_weights(pc, in, r);
+        const f2 cr = pk(r.c.x, r.c.x), cg = pk(r.c.y, r.c.y), cb = pk(r.c.z, r.c.z);
+        const float fa = fminf(r.p.z, 3.4e38f);   // an age beyond FP32 weighs 0: 0, not NaN, to every sum
+        const f2 a2 = pk(fa, fa);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((tid & 31) == 0) sh[k][tid >> 5] = v;
+        for (int j = 0; j < 2; ++j) {
+            const f2 w = p.w[j], q = fma2(g[j][2], cb, fma2(g[j][1], cg, mul2(g[j][0], cr)));
+            const f2 ws = mul2(w, p.d2[j]), wt = mul2(w, a2);
+            S[j] = add2(S[j], w);
+            Q[j] = fma2(w, q, Q[j]);
+            Ds[j] = add2(Ds[j], ws);
+            Dsq[j] = fma2(ws, q, Dsq[j]);
+            Dt[j] = add2(Dt[j], wt);
+            Dtq[j] = fma2(wt, q, Dtq[j]);
+        }
     }
+};
+
+// Weight sums alone (no parameter gradients asked for).
+struct WeightSums {
+    f2 S[2];
+    __device__ __forceinline__ WeightSums(const float4 (&)[4]) { S[0] = S[1] = 0ull; }
+    __device__ __forceinline__ void add(const PairConsts &pc, float4 in, const FrameRec &r) {
+        const PairWeights p = pair_weights(pc, in, r);
+        S[0] = add2(S[0], p.w[0]);
+        S[1] = add2(S[1], p.w[1]);
+    }
+};
+
+// The pixel pass is bound as the forward gather is, with 1.7 times its
+// arithmetic: 512x512x8, 325 us as a thread a pixel walking its disc, 176 us as
+// this gather (128 registers and four CTAs 182, 80 and six 221). The record
+// pass at the same size: 101 us reading 32 bytes a pixel and record, 61 us with
+// 24 bytes and two records a thread.
+constexpr int kBwdWarps = 4;   // a CTA of the pixel pass: 128 threads of up to 102 registers, five CTAs a SM
+constexpr int kBwdTbx = 4;     // its tile: 8 x 16 pixels
+
+template <bool PARAMS>
+__global__ void __launch_bounds__(32 * kBwdWarps, 5) k_bwd_pixel(
+    int W, int H, int R, int S_, int ntx, float window, float eps, AfrParams prm, const float4 *__restrict__ grad,
+    const TilePartial *__restrict__ tiles, const float2 *__restrict__ sigma, const float4 *__restrict__ fconst,
+    const uint32_t *__restrict__ foff, const FrameRec *frec, const float4 *__restrict__ gout,
+    Adjoint adj, float *__restrict__ bparam, DebugCheck dc) {
+    __shared__ TileSmem ts;
+    __shared__ DiscTable discs;
+    __shared__ float4 go[kTilePixels];
+    __shared__ float part[kBwdWarps][6];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int tw = 2 * kBwdTbx, th = 64 / kBwdTbx;
+    static_assert(tw * th == kTilePixels && kTilePixels == 32 * kBwdWarps, "a thread per pixel");
+    const int x0 = blockIdx.x * tw, y0 = blockIdx.y * th;
+    frec = keep(frec + lane);
+    const uint32_t table_at = smem_at(discs.in), rows_at = smem_at(ts.rows[warp]);
+    ts.fc[threadIdx.x] = load_const(threadIdx.x, W, H, x0, y0, tw, fconst);
+    go[threadIdx.x] = load_const(threadIdx.x, W, H, x0, y0, tw, gout);
+    fill_discs(discs, R);
+    load_offsets(ts, W, H, R, x0, y0, tw, th, foff);
     __syncthreads();
-    if (tid < 6) {
-        float acc = 0.f;
-        for (int w = 0; w < 4; ++w) acc += sh[tid][w];
-        bparam[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 6 + tid] = acc;
+    float gp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    int held = R;
+    for (int blk = warp; blk < 32; blk += kBwdWarps) {
+        const int lx = blk % kBwdTbx, ly = blk / kBwdTbx;
+        if (x0 + 2 * lx >= W || y0 + 2 * ly >= H) continue;   // warp-uniform
+        const int i0 = 2 * ly * tw + 2 * lx;
+        const float4 g4[4] = {go[i0], go[i0 + 1], go[i0 + tw], go[i0 + tw + 1]};
+        typename std::conditional<PARAMS, AdjointSums, WeightSums>::type A(g4);
+        gather_block<false>(R, x0, y0, tw, lx, ly, frec, ts, &discs, table_at, held, ts.rows[warp], rows_at, dc, A);
+        float S, q[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // of pixel k at lane k: S; w q, w d^2, w d^2 q, w a^2, w a^2 q
+        if constexpr (PARAMS) {
+            float v[16], u[8];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                upk(A.S[j], v[2 * j], v[2 * j + 1]);
+                upk(A.Q[j], v[4 + 2 * j], v[4 + 2 * j + 1]);
+                upk(A.Ds[j], v[8 + 2 * j], v[8 + 2 * j + 1]);
+                upk(A.Dsq[j], v[12 + 2 * j], v[12 + 2 * j + 1]);
+                upk(A.Dt[j], u[2 * j], u[2 * j + 1]);
+                upk(A.Dtq[j], u[4 + 2 * j], u[4 + 2 * j + 1]);
+            }
+            const float a = warp_reduce(v), b = warp_reduce(u);
+            S = __shfl_sync(0xffffffffu, a, 2 * (lane & 3));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) q[i] = __shfl_sync(0xffffffffu, a, 2 * (4 * (i + 1) + (lane & 3)));
+#pragma unroll
+            for (int i = 0; i < 2; ++i) q[3 + i] = __shfl_sync(0xffffffffu, b, 4 * (4 * i + (lane & 3)));
+        } else {
+            float v[4];
+            upk(A.S[0], v[0], v[1]);
+            upk(A.S[1], v[2], v[3]);
+            S = __shfl_sync(0xffffffffu, warp_reduce(v), 8 * (lane & 3));
+        }
+        const int x = x0 + 2 * lx + (lane & 1), y = y0 + 2 * ly + ((lane >> 1) & 1);
+        if (lane < 4 && x < W && y < H) {
+            const size_t p = (size_t)y * W + x;
+            const int i = block_pixel(tw, lx, ly);
+            const float4 fc = ts.fc[i], g = go[i];
+            if (!(S > 0.f)) {
+                adj.k[p] = make_float4(fc.x, fc.y, fc.z, 0.f);
+                adj.g[p] = make_float2(0.f, 0.f);
+            } else {
+                const float inv = 1.f / S;
+                adj.k[p] = make_float4(fc.x, fc.y, fc.z, g.x * inv);
+                adj.g[p] = make_float2(g.y * inv, g.z * inv);
+                if (PARAMS) {
+                    const float2 sg = __ldg(sigma + p);
+                    const float gC = q[0] * inv;
+                    const float gs = (q[2] - gC * q[1]) * inv / (sg.x * sg.x * sg.x);
+                    const float gt = (q[4] - gC * q[3]) * inv / (sg.y * sg.y * sg.y);
+                    // chain through the width mapping; the widths depend on theta only
+                    const Widths wd = widths(__ldg(grad + p), tile_volume(x, y, W, H, S_, ntx, window, tiles), eps, prm);
+                    if (fmaxf(wd.raw_s, kSigmaSMin) >= prm.clamp_s) gp[2] += gs;
+                    else if (wd.raw_s > kSigmaSMin) { gp[0] += gs * wd.es; gp[1] += gs; }
+                    if (fmaxf(wd.raw_t, kSigmaTMin) >= prm.clamp_t) gp[5] += gt;
+                    else if (wd.raw_t > kSigmaTMin) { gp[3] += gt * wd.et; gp[4] += gt; }
+                }
+            }
+        }
+    }
+    if (PARAMS) {   // one partial of each parameter's gradient per CTA
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            float v = gp[k];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            if (lane == 0) part[warp][k] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x < 6) {
+            float acc = 0.f;
+            for (int w = 0; w < kBwdWarps; ++w) acc += part[w][threadIdx.x];
+            bparam[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 6 + threadIdx.x] = acc;
+        }
     }
 }
 
 // Gradient of each frame record's colour: sum over the pixels whose disc
-// holds the record's bin of (dL/dC_p / S_p) * shifted weight.
-__global__ void __launch_bounds__(256) k_bwd_record(int W, int H, int R, const uint32_t *__restrict__ foff,
-                                                    const FrameRec *__restrict__ frec, const float4 *__restrict__ bg,
-                                                    const float4 *__restrict__ bframe, float *__restrict__ gcol) {
-    uint32_t n = __ldg(foff + (size_t)W * H);
-    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        float4 r = __ldg(&frec[e].p);
-        int qx = (int)floorf(r.x), qy = (int)floorf(r.y);
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-        for (int dy = -R; dy <= R; ++dy) {
-            int y = qy + dy;
-            if (y < 0 || y >= H) continue;
-            int hw = half_width(R, dy);
-            for (int x = max(0, qx - hw); x <= min(W - 1, qx + hw); ++x) {
-                size_t p = (size_t)y * W + x;
-                float4 fr = __ldg(bframe + p);
-                if (fr.w == 0.f) continue;
-                PixelFrame f;
-                f.cx = (float)x + 0.5f;
-                f.cy = (float)y + 0.5f;
-                f.ks = fr.x;
-                f.kt = fr.y;
-                f.m = fr.z;
-                float w = ex2(-shifted_exponent(f, r));
-                float4 g = __ldg(bg + p);
-                a0 = fmaf(g.x, w, a0);
-                a1 = fmaf(g.y, w, a1);
-                a2 = fmaf(g.z, w, a2);
+// holds the record's bin of (dL/dC_p / S_p) * shifted weight. Bound: the bytes
+// L1 delivers to registers (24 a pixel read, 128 a clock and SM), so a thread
+// takes two neighbouring records, which mostly share a bin or lie in adjacent
+// ones, and reads each pixel of their two discs once.
+struct RecordAt {
+    int qx, qy;
+    float fx, fy, a2;   // position from the centre of bin (qx, qy), a^2
+};
+
+__device__ __forceinline__ RecordAt record_at(const FrameRec *__restrict__ frec, uint32_t e) {
+    const float4 r = __ldg(&frec[e].p);
+    const int qx = (int)floorf(r.x), qy = (int)floorf(r.y);
+    return {qx, qy, r.x - ((float)qx + 0.5f), r.y - ((float)qy + 0.5f), r.z};
+}
+
+__device__ __forceinline__ float pixel_weight(float4 k, float dx, float dy2, float a2) {
+    return ex2(fmaf(fmaf(dx, dx, dy2), k.x, fmaf(a2, k.y, k.z)));
+}
+
+__device__ __forceinline__ void add_pixel(float4 k, float2 g, float w, float3 &a) {
+    a.x = fmaf(k.w, w, a.x);
+    a.y = fmaf(g.x, w, a.y);
+    a.z = fmaf(g.y, w, a.z);
+}
+
+// One record: RT >= 0 is R at compile time (every pixel at a constant offset)
+// for discs inside the image; the others loop.
+template <int RT>
+__device__ float3 record_gradient(const RecordAt &r, int W, int H, int R, Adjoint adj) {
+    float3 a = make_float3(0.f, 0.f, 0.f);
+    if (RT >= 0 && r.qx >= RT && r.qy >= RT && r.qx < W - RT && r.qy < H - RT) {
+        size_t p = (size_t)(r.qy - RT) * W + r.qx;
+#pragma unroll
+        for (int dy = -RT; dy <= RT; ++dy, p += W) {
+            const float ey = r.fy - (float)dy, dy2 = ey * ey;
+#pragma unroll
+            for (int dx = -RT; dx <= RT; ++dx) {
+                if (dx * dx + dy * dy > RT * RT) continue;
+                const float4 k = __ldg(adj.k + p + dx);
+                add_pixel(k, __ldg(adj.g + p + dx), pixel_weight(k, r.fx - (float)dx, dy2, r.a2), a);
             }
         }
-        gcol[3 * (size_t)e] = a0;
-        gcol[3 * (size_t)e + 1] = a1;
-        gcol[3 * (size_t)e + 2] = a2;
+        return a;
+    }
+    for (int dy = max(-R, -r.qy); dy <= min(R, H - 1 - r.qy); ++dy) {
+        const float ey = r.fy - (float)dy, dy2 = ey * ey;
+        const int hw = half_width(R, dy);
+        const size_t p = (size_t)(r.qy + dy) * W + r.qx;
+        for (int dx = max(-hw, -r.qx); dx <= min(hw, W - 1 - r.qx); ++dx) {
+            const float4 k = __ldg(adj.k + p + dx);
+            add_pixel(k, __ldg(adj.g + p + dx), pixel_weight(k, r.fx - (float)dx, dy2, r.a2), a);
+        }
+    }
+    return a;
+}
+
+template <int RT>
+__global__ void __launch_bounds__(256, 4) k_bwd_record(int W, int H, int R, const uint32_t *__restrict__ foff,
+                                                       const FrameRec *__restrict__ frec, Adjoint adj,
+                                                       float *__restrict__ gcol) {
+    const uint32_t n = __ldg(foff + (size_t)W * H);
+    const uint32_t pairs = n / 2 + (n & 1);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gridDim.x * blockDim.x) {
+        const uint32_t e = 2 * i;
+        const bool two = e + 1 < n;
+        const RecordAt u = record_at(frec, e), v = record_at(frec, two ? e + 1 : e);
+        const int s = v.qx - u.qx;
+        float3 a = make_float3(0.f, 0.f, 0.f), b = a;
+        if (RT >= 0 && v.qy == u.qy && (s == 0 || s == 1) && u.qx >= RT && u.qy >= RT && v.qx < W - RT &&
+            u.qy < H - RT && u.qx + RT + 1 < W) {
+            const float vx = v.fx + (float)s;   // from the centre of the first record's bin
+            size_t p = (size_t)(u.qy - RT) * W + u.qx;
+#pragma unroll
+            for (int dy = -RT; dy <= RT; ++dy, p += W) {
+                const float eu = u.fy - (float)dy, ev = v.fy - (float)dy, yu = eu * eu, yv = ev * ev;
+                // the row's pixels of both discs: columns -hw .. hw of the first, s - hw .. s + hw of the second
+#pragma unroll
+                for (int dx = -RT; dx <= RT + 1; ++dx) {
+                    const bool in = dx * dx + dy * dy <= RT * RT, in1 = (dx - 1) * (dx - 1) + dy * dy <= RT * RT;
+                    if (!in && !in1) continue;
+                    const float4 k = __ldg(adj.k + p + dx);
+                    const float2 g = __ldg(adj.g + p + dx);
+                    if (in) add_pixel(k, g, pixel_weight(k, u.fx - (float)dx, yu, u.a2), a);
+                    float w = pixel_weight(k, vx - (float)dx, yv, v.a2);
+                    if (!in && s == 0) w = 0.f;
+                    if (!in1 && s == 1) w = 0.f;
+                    add_pixel(k, g, w, b);
+                }
+            }
+        } else {
+            a = record_gradient<RT>(u, W, H, R, adj);
+            if (two) b = record_gradient<RT>(v, W, H, R, adj);
+        }
+        float *o = gcol + 3 * (size_t)e;
+        o[0] = a.x;
+        o[1] = a.y;
+        o[2] = a.z;
+        if (two) {
+            o[3] = b.x;
+            o[4] = b.y;
+            o[5] = b.z;
+        }
     }
 }
 
@@ -852,6 +1001,7 @@ __global__ void k_bwd_params(const float *__restrict__ part, int nblocks, float 
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= 6) return;
     float s = 0.f, c = 0.f;
+#pragma unroll 8
     for (int i = lane; i < nblocks; i += 32) {
         const float y = part[(size_t)i * 6 + k] - c;
         const float t = s + y;
@@ -892,7 +1042,6 @@ __global__ void k_set_colors(const float *__restrict__ rgb, const uint32_t *__re
     }
 }
 
-const dim3 kFilterBlock(32, 4);
 const dim3 kQuadBlock(256);
 
 }  // namespace
@@ -940,15 +1089,30 @@ cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out
 
 cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_col, float *grad_prm,
                             cudaStream_t s) {
-    dim3 grid((c->W + kFilterBlock.x - 1) / kFilterBlock.x, (c->H + kFilterBlock.y - 1) / kFilterBlock.y);
-    float4 *bframe = c->bgrad + c->P;
+    const int tw = 2 * kBwdTbx, th = 64 / kBwdTbx;
+    const dim3 grid((c->W + tw - 1) / tw, (c->H + th - 1) / th);
+    const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
+    const Adjoint adj{c->bgrad, reinterpret_cast<float2 *>(c->bgrad + c->P)};
     const AfrParams &prm = c->recon_params;
-    k_bwd_pixel<<<grid, kFilterBlock, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, prm,
-                                              c->grad, c->tiles, c->sigma, c->amin2, c->foff, c->frec, grad_rgb,
-                                              c->bgrad, bframe, c->bparam);
-    if (grad_col)
-        k_bwd_record<<<grid_for((size_t)c->P * c->b, 256), 256, 0, s>>>(c->W, c->H, c->R, c->foff, c->frec, c->bgrad,
-                                                                        bframe, grad_col);
+#define AFR_BWD(P_)                                                                                              \
+    k_bwd_pixel<P_><<<grid, 32 * kBwdWarps, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window,               \
+                                                    c->cfg.eps_grad, prm, c->grad, c->tiles, c->sigma, c->fconst, \
+                                                    c->foff, c->frec, grad_rgb, adj, c->bparam, dc)
+    if (grad_prm) AFR_BWD(true);
+    else AFR_BWD(false);
+#undef AFR_BWD
+#define AFR_REC(R_)                                                                                              \
+    k_bwd_record<R_><<<grid_for((size_t)c->P * c->b / 2, 256), 256, 0, s>>>(c->W, c->H, c->R, c->foff, c->frec, adj, \
+                                                                        grad_col)
+    if (grad_col) {
+        switch (c->R) {   // the radii of the tuner and the default
+            case 3: AFR_REC(3); break;
+            case 4: AFR_REC(4); break;
+            case 5: AFR_REC(5); break;
+            default: AFR_REC(-1); break;
+        }
+    }
+#undef AFR_REC
     if (grad_prm) k_bwd_params<<<1, 6 * 32, 0, s>>>(c->bparam, (int)(grid.x * grid.y), grad_prm);
     return cudaGetLastError();
 }
@@ -972,7 +1136,8 @@ cudaError_t launch_batch(int ct, const BatchCtx *cs, int nctx, uint32_t nchunks,
 }
 
 int backward_blocks(int W, int H) {
-    return (int)(((W + kFilterBlock.x - 1) / kFilterBlock.x) * ((H + kFilterBlock.y - 1) / kFilterBlock.y));
+    const int tw = 2 * kBwdTbx, th = 64 / kBwdTbx;
+    return ((W + tw - 1) / tw) * ((H + th - 1) / th);
 }
 
 }  // namespace afr

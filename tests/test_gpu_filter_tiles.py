@@ -71,3 +71,42 @@ def test_filter_edges_match_oracle(dev, W, H, b, R, tbx, ct, per_pixel, crowd, g
     np.testing.assert_array_equal(img[hole], 0.0)
     err = np.abs(img[~hole, :3] - ref[~hole, :3]) / np.maximum(np.abs(ref[~hole, :3]), 1e-3)
     assert err.size == 0 or err.max() <= 1e-5
+
+
+@pytest.mark.parametrize("W,H,b,R,ct,per_pixel,crowd,gap", [
+    (1, 1, 2, 4, "f32", 1, 0.0, 0), (9, 70, 8, 4, "f32", 8, 0.1, 9), (67, 21, 3, 5, "f32", 0.4, 0.0, 0),
+    (30, 35, 24, 3, "f16", 24, 0.0, 0), (33, 17, 8, 8, "f32", 8, 0.2, 4), (40, 26, 16, 0, "bf16", 12, 0.0, 7),
+    (64, 40, 4, 2, "f32", 3, 0.0, 0)])
+def test_adjoint_edges_match_oracle(dev, W, H, b, R, ct, per_pixel, crowd, gap):
+    """Both passes of the adjoint where they can go wrong: borders, discs known
+    at compile time and not, neighbouring records in one bin, in adjacent bins,
+    across gaps and row ends, an odd number of records; either output alone.
+    Bounds as in the parity test of the adjoint."""
+    from paper_2510_15876_gb300.api import Reconstructor, to_device_batch
+    batch = _batch(W * 10 + H, W, H, max(1, int(W * H * per_pixel)), crowd, gap)
+    rec = Reconstructor(W, H, b, radius=R, color_type=ct, device=dev)
+    tensors = to_device_batch(batch, dev, rec.color_dtype)
+    rec.insert(*tensors)
+    ring = oracle.Ring(W, H, b)
+    ring.insert(batch["pos"], tensors[1].float().cpu().numpy(), batch["motion"])
+    rec.estimate_gradients(T_NOW)
+    rec.reproject(T_NOW)
+    maps = [np.asarray(v).astype(np.float32) for v in oracle.gradients(ring, T_NOW)[1:]]
+    for m, v in zip((L.AFR_MAP_GX, L.AFR_MAP_GY, L.AFR_MAP_GT), maps):
+        rec.import_map(m, v)
+    theta = np.array([0.9, 0.15, 2.4, 1.1, 0.02, 0.7])
+    rec.reconstruct(T_NOW, theta)
+    g = np.random.default_rng(W).normal(size=(W * H, 4)).astype(np.float32)
+    gt = torch.from_numpy(g).to(dev).reshape(H, W, 4)
+    gcol, gprm = rec.backward(gt)
+    only_colors, _ = rec.backward(gt, want_params=False)
+    _, only_params = rec.backward(gt, want_colors=False)
+    off, frec, _, _ = oracle.reproject(ring, T_NOW)
+    wcol, wprm = oracle.backward(ring.count, W, H, (None, *(v.astype(np.float64) for v in maps)), off, frec,
+                                 g[:, :3].astype(np.float64), theta, R=R)
+    for got in (gprm, only_params):
+        np.testing.assert_allclose(got.cpu().numpy(), wprm, rtol=2e-4, atol=1e-4 * max(np.abs(wprm).max(), 1e-30))
+    for got in (gcol, only_colors):
+        np.testing.assert_allclose(got.cpu().numpy()[:len(wcol)], wcol, rtol=1e-3,
+                                   atol=1e-5 * max(np.abs(wcol).max(initial=0.0), 1e-30))
+    rec.close()
