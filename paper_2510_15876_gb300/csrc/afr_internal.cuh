@@ -48,8 +48,8 @@ struct DebugCheck {
 };
 
 // Per-tile partial statistics written by the gradient pass (64 bytes). The
-// luminance moments are FP64 because a tile above 4096 samples merges its
-// warps' moments in FP64; everything else is an integer count or an FP32 sum.
+// luminance moments are summed as double-floats and kept whole in FP64 fields;
+// everything else is an integer count or an FP32 sum.
 struct alignas(16) TilePartial {
     double sw;         // sum of age weights
     double mean;       // weighted mean luminance
@@ -57,7 +57,8 @@ struct alignas(16) TilePartial {
     float sgx, sgy, sgt;   // gradient sums over non-empty pixels
     uint32_t n;        // samples
     uint32_t nonempty; // non-empty pixels
-    uint32_t pad[3];
+    float age;         // sum of the samples' ages max(0, t_now - t)
+    uint32_t pad[2];
 };
 static_assert(sizeof(TilePartial) == 64, "one 64-byte record per tile");
 
@@ -136,9 +137,8 @@ struct AfrContext {
     // maps
     float2 *lbar = nullptr;       // [P] weighted mean luminance as double-float (hi, lo)
     float4 *grad = nullptr;       // [P] (Gx, Gy, Gt, Lbar)
-    float4 *pstat = nullptr;      // [P] (sum w, mean L, M2, Gt)
+    float4 *pstat = nullptr;      // [P] (sum w, M2, Gt, sum of ages)
     float2 *sigma = nullptr;      // [P] (sigma_s, sigma_t)
-    double *tile_terms = nullptr;   // [8 ntiles] per-tile terms of afr_tile_error (64 B a tile)
     float4 *fconst = nullptr;     // [P] gather constants (-ks, -kt, exponent shift m, disc radius as int bits)
     float *cov_r[2] = {nullptr, nullptr};   // [P] footprint radii of adaptive reconstructions (ping-pong)
     int32_t *cov_n = nullptr;     // [P] samples in each pixel's footprint in the last adaptive reconstruction
@@ -146,7 +146,7 @@ struct AfrContext {
     bool cov_init = false;        // the coverage state holds its start values
     bool adaptive_last = false;   // the last reconstruction used adaptive footprints
     uint32_t *amin2 = nullptr;    // [P] float bits of min a^2 per frame bin
-    afr::TilePartial *tiles = nullptr;  // [ntiles]
+    afr::TilePartial *tiles = nullptr;  // [ntiles + 1]; the last holds the samples of all tiles (tile_total)
 
     // frame view
     uint32_t *fcnt = nullptr;     // [P]
@@ -378,6 +378,10 @@ cudaError_t launch_ingest(AfrContext *c, const AfrSampleBatch *batch, uint32_t n
                           cudaStream_t s, cudaEvent_t queues_free = nullptr, bool reset = false);
 cudaError_t launch_fifo_append(AfrContext *c, const AfrSampleBatch *batch, uint32_t n, uint32_t seq0, cudaStream_t s);
 cudaError_t launch_gradients(AfrContext *c, float t_now, cudaStream_t s);
+// Buffered samples of all tiles, counted by the gradient pass.
+inline unsigned long long *tile_total(AfrContext *c) {
+    return reinterpret_cast<unsigned long long *>(c->tiles + c->ntiles);
+}
 cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *cam, cudaStream_t s);
 cudaError_t launch_sigma(AfrContext *c, const AfrParams *prm, bool keep, bool adaptive, cudaStream_t s);
 cudaError_t launch_coverage_init(AfrContext *c, cudaStream_t s);

@@ -1,10 +1,10 @@
 // k_feedback.cu -- sections 4, 4.2 and 6.1: finalise the per-tile records
-// from the partials of the gradient pass (the mean number of empty slots over
-// tiles, then each tile's record with its undersampling measure
-// u = 1 - min(1, m * mean_empty / empty)), and the tile error E with the gain
-// control of section 4.1. Counts are summed as integers and the rest runs in
-// FP32: FP64 issues at 1/64 of the FP32 rate on this part, and every output
-// is FP32.
+// from the partials of the gradient pass (each tile's record with its
+// undersampling measure u = 1 - min(1, m * mean_empty / empty), the mean number
+// of empty slots following from the samples the gradient pass counted), and the
+// tile error E with the gain control of section 4.1. Counts are summed as
+// integers and the rest runs in FP32: FP64 issues at 1/64 of the FP32 rate on
+// this part, and every output is FP32.
 #include "afr_internal.cuh"
 
 namespace afr {
@@ -18,26 +18,16 @@ __device__ __forceinline__ uint32_t tile_area(int t, int W, int H, int S, int nt
     return (uint32_t)(min(S, W - tx * S) * min(S, H - ty * S));
 }
 
-// Every block sums the empty slots of all tiles (an exact integer sum, the
-// same in every block), then writes the records of its own kFinThreads tiles.
+// Mean number of empty slots over the tiles: an exact integer, divided once.
+__device__ __forceinline__ float mean_empty_slots(int W, int H, int b, int ntiles, const unsigned long long *total) {
+    return (float)((unsigned long long)W * H * b - *total) / (float)ntiles;
+}
+
 __global__ void __launch_bounds__(kFinThreads) k_finalize(int W, int H, int S, int ntx, int ntiles, int b, float m,
                                                           const TilePartial *__restrict__ tiles,
+                                                          const unsigned long long *__restrict__ total,
                                                           AfrTileStats *__restrict__ out) {
-    __shared__ unsigned long long sh[kFinThreads / 32];
-    __shared__ float mean_empty;
-    unsigned long long acc = 0ull;
-    for (int t = threadIdx.x; t < ntiles; t += blockDim.x)
-        acc += (unsigned long long)tile_area(t, W, H, S, ntx) * (uint32_t)b - tiles[t].n;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long s = 0ull;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-        mean_empty = (float)s / (float)ntiles;
-    }
-    __syncthreads();
+    const float mean_empty = mean_empty_slots(W, H, b, ntiles, total);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < ntiles) {
         const TilePartial tp = tiles[t];
@@ -54,88 +44,6 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(int W, int H, int S, i
         const float r = empty ? m * mean_empty / (float)empty : 0.f;
         o.u = empty ? 1.f - fminf(r, 1.f) : 0.f;
         out[t] = o;
-    }
-}
-
-// Per-tile terms of the tile error, one block per tile: the sum of sample
-// ages max(0, t_now - t) over the tile's resident samples (the queue's count
-// newest slots of every pixel), then, by one thread, the tile's terms that do
-// not depend on other tiles. A tile row's slots are contiguous (tw pixels x b
-// slots): each thread keeps its slot columns and walks the rows, loading a
-// slot's time beside its pixel's queue state (a warp reads 128 contiguous
-// bytes of times) so that the loads of successive rows overlap. Ages are
-// summed in FP32 over at most 32 rows of one slot column (32 ages, each at
-// most the window); those sums are added as double-float values (TwoSum
-// additions), per thread and by a tree over the block.
-struct alignas(16) TileTerm {
-    float v;           // luminance variance
-    float o;           // occluded share of the tile's slots
-    float inv_empty;   // 1 / empty slots (0 without empty slots)
-    float age;         // mean sample age (unused without samples)
-    float sg, sgt;     // spatial and temporal gradient sums over non-empty pixels
-    uint32_t empty, nonempty, has_samples, pad[3];
-};
-static_assert(sizeof(TileTerm) <= 64, "fits the 64 bytes a tile the context holds");
-
-__global__ void __launch_bounds__(256) k_tile_terms(int W, int H, int S, int ntx, int b, float t_now,
-                                                    const uint32_t *__restrict__ state, const float *__restrict__ r_t,
-                                                    const TilePartial *__restrict__ tiles,
-                                                    const uint32_t *__restrict__ occluded,
-                                                    TileTerm *__restrict__ terms) {
-    __shared__ float2 sh[8];
-    const int tile = blockIdx.x;
-    const int x0 = (tile % ntx) * S, y0 = (tile / ntx) * S;
-    const int tw = min(S, W - x0), th = min(S, H - y0);
-    const int row_slots = tw * b;
-    dfloat d{0.f, 0.f};   // double-float: each chunk's FP32 sum added exactly (TwoSum)
-    for (int k = threadIdx.x; k < row_slots; k += blockDim.x) {
-        const int px = k / b, sl = k - px * b;
-        const size_t p0 = (size_t)y0 * W + x0 + px;
-        for (int r0 = 0; r0 < th; r0 += 32) {
-            const int r1 = min(th, r0 + 32);
-            float acc = 0.f;
-#pragma unroll 8
-            for (int r = r0; r < r1; ++r) {
-                const size_t p = p0 + (size_t)r * W;
-                const uint32_t st = __ldg(state + p);
-                const float t = __ldg(r_t + p * b + sl);
-                int age_rank = (int)(st >> 16) - 1 - sl;
-                if (age_rank < 0) age_rank += b;
-                const float a = t_now - t;
-                acc += (age_rank < (int)(st & 0xFFFFu) && a > 0.f) ? a : 0.f;
-            }
-            d = df_add(d, dfloat{acc, 0.f});
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        d = df_add(d, dfloat{__shfl_xor_sync(0xffffffffu, d.h, o), __shfl_xor_sync(0xffffffffu, d.l, o)});
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = make_float2(d.h, d.l);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        const float2 v = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : make_float2(0.f, 0.f);
-        dfloat xd{v.x, v.y};
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            xd = df_add(xd, dfloat{__shfl_xor_sync(0xffffffffu, xd.h, o), __shfl_xor_sync(0xffffffffu, xd.l, o)});
-        const float x = __fadd_rn(xd.h, xd.l);
-        if (threadIdx.x == 0) {
-            const TilePartial tp = tiles[tile];
-            const uint32_t slots = (uint32_t)(tw * th) * (uint32_t)b, empty = slots - tp.n;
-            const float sw = (float)tp.sw;
-            TileTerm tt;
-            tt.v = sw > 0.f ? (float)tp.m2 / sw : 0.f;
-            tt.o = occluded ? (float)occluded[tile] / (float)slots : 0.f;
-            tt.inv_empty = empty ? 1.f / (float)empty : 0.f;
-            tt.age = tp.n ? x / (float)tp.n : 0.f;
-            tt.sg = 0.5f * (tp.sgx + tp.sgy);
-            tt.sgt = tp.sgt;
-            tt.empty = empty;
-            tt.nonempty = tp.nonempty;
-            tt.has_samples = tp.n ? 1u : 0u;
-            tt.pad[0] = tt.pad[1] = tt.pad[2] = 0u;
-            terms[tile] = tt;
-        }
     }
 }
 
@@ -168,60 +76,67 @@ __device__ __forceinline__ void block_sum(T (&v)[N], T (*sh)[kFbThreads / 32]) {
     __syncthreads();
 }
 
+// A tile's terms of the tile error that follow from its own record.
+struct TileTerm {
+    float v, u, o;   // luminance variance, undersampling measure, occluded share of the tile's slots
+};
+
+__device__ __forceinline__ TileTerm tile_term(const TilePartial &tp, uint32_t slots, float m_mean_empty,
+                                              uint32_t occluded) {
+    TileTerm t;
+    const uint32_t empty = slots - tp.n;
+    const float sw = (float)tp.sw;
+    t.v = sw > 0.f ? (float)tp.m2 / sw : 0.f;
+    // 1 - min(1, m mean_empty / empty), 0 without empty slots: one rounded division,
+    // as in the tile record, so that a tile exactly at the limit gets 0 here too
+    t.u = empty ? 1.f - fminf(m_mean_empty / (float)empty, 1.f) : 0.f;
+    t.o = (float)occluded / (float)slots;
+    return t;
+}
+
 // Sections 6.1 and 4.1: tile error shares and gain control, one block over
-// the per-tile terms. The counts (empty slots, non-empty pixels, tiles with
-// samples) are summed as integers, exactly; the rest are tree sums in FP32.
-__global__ void __launch_bounds__(kFbThreads) k_tile_error(int W, int H, int S, int ntx, int ntiles, float m,
+// the tile records. The sample ages were summed by the gradient pass, which
+// reads the times anyway (a pass over the times of its own took 51 us at
+// 1920x1080x16). Non-empty pixels and tiles with samples are summed as
+// integers, exactly; the rest are tree sums in FP32.
+__global__ void __launch_bounds__(kFbThreads) k_tile_error(int W, int H, int S, int ntx, int ntiles, int b, float m,
                                                            float kappa, float lambda, float importance, float eps,
-                                                           const TileTerm *__restrict__ terms, bool has_occlusion,
+                                                           const TilePartial *__restrict__ tiles,
+                                                           const unsigned long long *__restrict__ total,
+                                                           const uint32_t *__restrict__ occluded,
                                                            float *__restrict__ E, AfrGain *__restrict__ gain) {
-    __shared__ unsigned long long shi[3][kFbThreads / 32];
+    __shared__ unsigned long long shi[2][kFbThreads / 32];
     __shared__ float sh[6][kFbThreads / 32];
-    __shared__ float scal[4];   // m mean_empty, then the weights of v, u, o (one thread divides)
-    unsigned long long cnt[3] = {0ull, 0ull, 0ull};   // empty slots, non-empty pixels, tiles with samples
-    for (int t = threadIdx.x; t < ntiles; t += blockDim.x) {
-        cnt[0] += terms[t].empty;
-        cnt[1] += terms[t].nonempty;
-        cnt[2] += terms[t].has_samples;
-    }
-    block_sum(cnt, shi);
-    if (threadIdx.x == 0) scal[0] = m * ((float)cnt[0] / (float)ntiles);
-    __syncthreads();
-    const float m_mean_empty = scal[0];
-    // u = 1 - min(1, m mean_empty / empty), 0 without empty slots
-    auto undersampling = [&](const TileTerm &tt) {
-        return tt.empty ? 1.f - fminf(m_mean_empty * tt.inv_empty, 1.f) : 0.f;
-    };
+    const float m_mean_empty = m * mean_empty_slots(W, H, b, ntiles, total);
+    unsigned long long cnt[2] = {0ull, 0ull};   // non-empty pixels, tiles with samples
     // sums: v, u, o, spatial gradient, temporal gradient, tile mean ages
     float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int t = threadIdx.x; t < ntiles; t += blockDim.x) {
-        const TileTerm tt = terms[t];
+        const TilePartial tp = tiles[t];
+        const TileTerm tt = tile_term(tp, tile_area(t, W, H, S, ntx) * (uint32_t)b, m_mean_empty, occluded ? occluded[t] : 0u);
+        cnt[0] += tp.nonempty;
+        cnt[1] += tp.n ? 1u : 0u;
         acc[0] += tt.v;
-        acc[1] += undersampling(tt);
+        acc[1] += tt.u;
         acc[2] += tt.o;
-        acc[3] += tt.sg;
-        acc[4] += tt.sgt;
-        acc[5] += tt.has_samples ? tt.age : 0.f;
+        acc[3] += 0.5f * (tp.sgx + tp.sgy);
+        acc[4] += tp.sgt;
+        acc[5] += tp.n ? tp.age / (float)tp.n : 0.f;
     }
+    block_sum(cnt, shi);
     block_sum(acc, sh);
     // E = s (kappa v / sum v + lambda u / sum u + (1 - kappa - lambda) o / sum o)
-    if (threadIdx.x == 0) {
-        scal[1] = acc[0] > 0.f ? kappa / acc[0] : 0.f;
-        scal[2] = acc[1] > 0.f ? lambda / acc[1] : 0.f;
-        scal[3] = has_occlusion && acc[2] > 0.f ? (1.f - kappa - lambda) / acc[2] : 0.f;
-    }
-    __syncthreads();
-    const float wv = scal[1], wu = scal[2], wo = scal[3];
+    const float wv = acc[0] > 0.f ? kappa / acc[0] : 0.f, wu = acc[1] > 0.f ? lambda / acc[1] : 0.f,
+                wo = occluded && acc[2] > 0.f ? (1.f - kappa - lambda) / acc[2] : 0.f;
     for (int t = threadIdx.x; t < ntiles; t += blockDim.x) {
-        const TileTerm tt = terms[t];
-        const int tx = t % ntx, ty = t / ntx;
-        const float A = (float)(min(S, W - tx * S) * min(S, H - ty * S));
-        E[t] = A * (wv * tt.v + wu * undersampling(tt) + wo * tt.o);
+        const uint32_t A = tile_area(t, W, H, S, ntx);
+        const TileTerm tt = tile_term(tiles[t], A * (uint32_t)b, m_mean_empty, occluded ? occluded[t] : 0u);
+        E[t] = (float)A * (wv * tt.v + wu * tt.u + wo * tt.o);
     }
     if (threadIdx.x == 0 && gain) {
-        const float nonempty = (float)cnt[1];
-        const float dcds = cnt[1] ? acc[3] / nonempty : 0.f, dcdt = cnt[1] ? acc[4] / nonempty : 0.f;
-        const float T = cnt[2] ? acc[5] / (float)cnt[2] : 0.f;
+        const float nonempty = (float)cnt[0];
+        const float dcds = cnt[0] ? acc[3] / nonempty : 0.f, dcdt = cnt[0] ? acc[4] / nonempty : 0.f;
+        const float T = cnt[1] ? acc[5] / (float)cnt[1] : 0.f;
         const float Sw = importance * dcdt * T / (dcds > eps ? dcds : eps);
         const float P = (float)W * (float)H;
         float N = Sw > 0.f ? P / (Sw * Sw) : P;
@@ -240,17 +155,14 @@ __global__ void __launch_bounds__(kFbThreads) k_tile_error(int W, int H, int S, 
 
 cudaError_t launch_tile_error(AfrContext *c, float kappa, float lambda, float importance, const uint32_t *occluded,
                               float *E, AfrGain *gain, cudaStream_t s) {
-    TileTerm *terms = reinterpret_cast<TileTerm *>(c->tile_terms);
-    k_tile_terms<<<c->ntiles, 256, 0, s>>>(c->W, c->H, c->S, c->ntx, c->b, c->grads_t, c->r_state, c->r_t, c->tiles,
-                                           occluded, terms);
-    k_tile_error<<<1, kFbThreads, 0, s>>>(c->W, c->H, c->S, c->ntx, c->ntiles, c->cfg.undersample_m, kappa, lambda,
-                                          importance, c->cfg.eps_grad, terms, occluded != nullptr, E, gain);
+    k_tile_error<<<1, kFbThreads, 0, s>>>(c->W, c->H, c->S, c->ntx, c->ntiles, c->b, c->cfg.undersample_m, kappa, lambda,
+                                          importance, c->cfg.eps_grad, c->tiles, tile_total(c), occluded, E, gain);
     return cudaGetLastError();
 }
 
 cudaError_t launch_feedback(AfrContext *c, AfrTileStats *out, cudaStream_t s) {
     k_finalize<<<(c->ntiles + kFinThreads - 1) / kFinThreads, kFinThreads, 0, s>>>(
-        c->W, c->H, c->S, c->ntx, c->ntiles, c->b, c->cfg.undersample_m, c->tiles, out);
+        c->W, c->H, c->S, c->ntx, c->ntiles, c->b, c->cfg.undersample_m, c->tiles, tile_total(c), out);
     return cudaGetLastError();
 }
 

@@ -1,51 +1,86 @@
 // k_gradients.cu -- sections 4 and 4.1 on the deep buffer.
 //
-//  pixel pass   (a group of lanes per pixel, several queue slots each): age
+//  pixel pass   (thread per pixel on queues staged in shared memory): age
 //               weights exp(-3.47 a), weighted mean luminance and its weighted
-//               spread (per-pixel moments for the tile variance), and the
-//               temporal gradient over the queue sorted by time.
+//               spread (per-pixel moments for the tile variance), the sum of
+//               the ages, and the temporal gradient over the queue sorted by
+//               time.
 //  tile pass    (block per tile): G_x, G_y from the four neighbours' means,
-//               the gradient sums and the merged per-pixel moments (FP32, or
-//               FP64 once the tile holds more than 4096 samples).
+//               the gradient and age sums and the tile's luminance moments
+//               (mean first, then the squares about it).
 #include "afr_internal.cuh"
 
 namespace afr {
 namespace {
 
-// Group of L = G / S lanes per pixel (G = queue depth rounded up to a power
-// of two), S queue entries per lane: entry k (0 the newest) sits in lane
-// k mod L, register k / L, so the loads of a warp stay contiguous per pixel and
-// a warp serves 32 S / G pixels; sums, the time sort and the pairwise
-// differences use shuffles within the group.
-template <int L>
-__device__ __forceinline__ float group_sum(float v) {
-#pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, L);
-    return v;
+// ---- pixel pass ------------------------------------------------------------------
+// A warp takes 32 pixels: it copies their times and colours (contiguous in
+// memory) to shared memory with asynchronous 16-byte copies, and then each
+// lane walks one pixel's slots in storage order. Storage order is insertion
+// order turned by the head, so slot s follows slot s - 1 (slot 0 follows slot
+// b - 1) except that slot h, the oldest of a full queue, follows none. Sums do
+// not depend on the order, and consecutive slots are the consecutive samples
+// that the temporal gradient compares when times do not decrease, the usual
+// case; a queue out of time order is sorted (by time, newest first; equal
+// times newest first by insertion) by insertion on slot numbers in shared
+// memory. Sequence numbers are not read: they fall with the insertion rank.
+//
+// Bound: HBM (20 bytes a slot in FP32 colours, 36 a pixel: 5.6 TB/s). A group of
+// lanes a pixel spent the time on shuffles and read the sequence numbers too:
+// 1920x1080x16 227 us, this one 132 us (with a runtime depth, weights kept in
+// shared memory: 156 us; CTAs of two and four warps 135-164 us); 640x480x8 in
+// FP16 32 -> 17 us. Depths 4, 8 and 16 have a kernel of their own, where every
+// slot is at a constant offset and weights and deviations stay in registers.
+//
+// Shared memory of a warp: times (ts words a pixel), colours (cb bytes a
+// pixel), slot order (b bytes a pixel) and, where b is not a compile-time
+// constant, the weights (ts words a pixel; else they stay in registers).
+// Strides are odd multiples of the access size where the copies allow it, so
+// that lanes at one slot do not conflict.
+constexpr int kPixelWarps = 1;
+
+struct PixelLayout {
+    int ts;       // words a pixel of the time and weight areas
+    int cb;       // bytes a pixel of the colour area
+    int bytes;    // of one warp
+};
+
+__host__ __device__ constexpr PixelLayout pixel_layout(int b, int csize, bool weights) {
+    PixelLayout l{};
+    l.ts = (b & 3) == 0 && ((b >> 2) & 1) == 0 ? b + 4 : b;   // 16-byte copies never cross a padded pixel
+    l.cb = (b & 1) == 0 ? csize * b + 16 : csize * b;
+    l.bytes = (32 * ((weights ? 8 : 4) * l.ts + l.cb + b) + 15) & ~15;
+    return l;
 }
 
-// The value of entry k + 1 for each of a lane's entries k = r L + l.
-template <int L, int S, typename V>
-__device__ __forceinline__ void next_entry(const V (&v)[S], V (&nv)[S], int l) {
-#pragma unroll
-    for (int r = 0; r < S; ++r) {
-        const V d = __shfl_down_sync(0xffffffffu, v[r], 1, L);
-        if (r + 1 < S) {
-            const V w = __shfl_sync(0xffffffffu, v[r + 1], 0, L);   // entry (r + 1) L follows entry r L + L - 1
-            nv[r] = l == L - 1 ? w : d;
-        } else {
-            nv[r] = d;
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src, int bytes) {   // bytes < 16: the rest is zero
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// Copies n bytes of 32 pixels' records from src (16-byte aligned) to dst,
+// padding each pixel from `from` to `to` bytes (equal: one linear copy).
+__device__ __forceinline__ void stage(char *dst, const char *src, int n, int from, int to) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(dst);
+    if (from == to) {
+        for (int i = 16 * lane; i < n; i += 512) copy16(d0 + i, src + i, min(16, n - i));
+        return;
+    }
+    const int per = from >> 4, dp = 32 / per, dr = 32 - dp * per;   // chunks a pixel; a step of 32 chunks in (pixels, chunks)
+    int p = lane / per, r = lane - p * per;
+    for (int i = 16 * lane; i < n; i += 512) {
+        copy16(d0 + p * to + 16 * r, src + i, min(16, n - i));
+        p += dp;
+        r += dr;
+        if (r >= per) {
+            r -= per;
+            ++p;
         }
     }
 }
 
-struct Entry {
-    float T, w, cx, cy, cz;
-    uint32_t Q;
-};
-
-__device__ __forceinline__ bool newer(const Entry &a, const Entry &b) {   // descending order by (T, Q)
-    return (a.T > b.T) || (a.T == b.T && a.Q > b.Q);
+__device__ __forceinline__ float lum_diff(float3 a, float3 b) {   // L(a) - L(b) from the colour differences
+    return fmaf(kLumB, __fsub_rn(a.z, b.z), fmaf(kLumG, __fsub_rn(a.y, b.y), kLumR * __fsub_rn(a.x, b.x)));
 }
 
 // Luminance differences carry the gradients: the spatial gradient is a
@@ -59,301 +94,359 @@ __device__ __forceinline__ bool newer(const Entry &a, const Entry &b) {   // des
 // temporal gradient takes each consecutive pair's difference from its colour
 // differences; the age weights, the time steps and the variance moments are
 // FP32.
-template <int CT, int G, int S>
-__global__ void __launch_bounds__(256) k_pixel(int P, int b, float t_now, const uint32_t *__restrict__ state,
-                                               const float *__restrict__ r_t, const uint32_t *__restrict__ r_seq,
-                                               const void *__restrict__ r_col, float2 *__restrict__ lbar,
-                                               float4 *__restrict__ pstat) {
+template <int CT, int B>
+__global__ void __launch_bounds__(32 * kPixelWarps) k_pixel(int P, int b_run, float t_now,
+                                                            const uint32_t *__restrict__ state,
+                                                            const float *__restrict__ r_t,
+                                                            const void *__restrict__ r_col, float2 *__restrict__ lbar,
+                                                            float4 *__restrict__ pstat,
+                                                            unsigned long long *__restrict__ total) {
     using CS = ColorStore<CT>;
-    constexpr int L = G / S;
-    const int l = threadIdx.x & (L - 1);
-    const int groups = (gridDim.x * blockDim.x) / L;
-    // every lane of a warp runs the same number of iterations (P rounded up)
-    const int P_round = (P + (32 / L) - 1) / (32 / L) * (32 / L);
-    for (int p = (blockIdx.x * blockDim.x + threadIdx.x) / L; p < P_round; p += groups) {
-        const bool pix = p < P;
-        const uint32_t st = pix ? __ldg(state + p) : 0u;
-        const int n = (int)(st & 0xFFFFu), h = (int)(st >> 16);
-        Entry E[S];
-        float D[S];
-#pragma unroll
-        for (int r = 0; r < S; ++r) {
-            const int k = r * L + l;
-            E[r] = Entry{-INFINITY, 0.f, 0.f, 0.f, 0.f, 0u};
-            if (k < n) {
-                int s = h - 1 - k;
-                if (s < 0) s += b;
-                const size_t i = (size_t)p * b + s;
-                E[r].T = __ldg(r_t + i);
-                E[r].Q = __ldg(r_seq + i);
-                const float3 c = CS::load(r_col, i);
-                E[r].cx = c.x;
-                E[r].cy = c.y;
-                E[r].cz = c.z;
+    using T4 = typename CS::T;
+    extern __shared__ __align__(16) char smem[];
+    const int b = B ? B : b_run;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const PixelLayout l = pixel_layout(b, (int)sizeof(T4), B == 0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *total = 0ull;   // the tile pass counts the samples
+    const int p0 = (blockIdx.x * kPixelWarps + warp) * 32, np = min(32, P - p0);
+    if (np <= 0) return;
+    char *base = smem + warp * l.bytes;
+    float *ts = reinterpret_cast<float *>(base);
+    char *cs = base + 128 * l.ts;
+    uint8_t *order = reinterpret_cast<uint8_t *>(cs + 32 * l.cb);
+    float *ws = reinterpret_cast<float *>(base + l.bytes - (B ? 0 : 128 * l.ts));
+    const char *src_t = reinterpret_cast<const char *>(r_t + (size_t)p0 * b),
+               *src_c = reinterpret_cast<const char *>(reinterpret_cast<const T4 *>(r_col) + (size_t)p0 * b);
+    if (B && np == 32) {   // whole: constant trip counts, no ends to check
+        stage(base, src_t, 128 * B, 4 * B, 4 * l.ts);
+        stage(cs, src_c, 32 * (int)sizeof(T4) * B, (int)sizeof(T4) * B, l.cb);
+    } else {
+        stage(base, src_t, 4 * np * b, 4 * b, 4 * l.ts);
+        stage(cs, src_c, (int)sizeof(T4) * np * b, (int)sizeof(T4) * b, l.cb);
+    }
+    const int p = p0 + lane;
+    const uint32_t st = lane < np ? __ldg(state + p) : 0u;
+    const int n = (int)(st & 0xFFFFu), h = (int)(st >> 16);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    ts += lane * l.ts;
+    ws += lane * l.ts;
+    const T4 *col = reinterpret_cast<const T4 *>(cs + lane * l.cb);
+    order += lane * b;
+    // live slots: the n before h, cyclically; slots that are the next newer
+    // sample after the slot before them (slot 0 is left to the end)
+    const uint32_t all = 0xFFFFFFFFu >> (32 - b), m = n ? 0xFFFFFFFFu >> (32 - n) : 0u;
+    const uint32_t live = n <= h ? m << (h - n) : ((h ? m >> (n - h) : 0u) | (m << (b + h - n))) & all;
+    const uint32_t follows = live & (live << 1) & ~(1u << h);
+    const int first = h == 0 ? b - 1 : h - 1;   // newest slot
+    const float3 cr = CS::widen(col[first]);
+    float sw = 0.f, swd = 0.f, age = 0.f, num = 0.f, den = 0.f, Tp = 0.f, w0 = 0.f;
+    float3 cp = cr;
+    bool ordered = true;   // times do not decrease
+    float W[B ? B : 1], D[B ? B : 1];
+#pragma unroll(B ? B : 4)
+    for (int s = 0; s < b; ++s) {
+        const float T = ts[s], a = fmaxf(t_now - T, 0.f), w = expf(-kAgeDecay * a);
+        const float3 c = CS::widen(col[s]);
+        const float d = lum_diff(c, cr), dl = fabsf(lum_diff(c, cp));
+        if (B) {
+            W[s] = w;
+            D[s] = d;
+        } else {
+            ws[s] = w;
+        }
+        if (live >> s & 1u) {
+            sw += w;
+            swd += w * d;
+            age += a;
+        }
+        if (follows >> s & 1u) {
+            num += w * dl;
+            den += w * (T - Tp);
+            ordered = ordered && T >= Tp;
+        }
+        if (s == 0) w0 = w;
+        Tp = T;
+        cp = c;
+    }
+    if (live >> (b - 1) & live & (h != 0 ? 1u : 0u)) {   // slot 0 after slot b - 1
+        const float T = ts[0];
+        num += w0 * fabsf(lum_diff(CS::widen(col[0]), cp));
+        den += w0 * (T - Tp);
+        ordered = ordered && T >= Tp;
+    }
+    if (!ordered) {
+        int s = first;
+        for (int k = 0; k < n; ++k) {
+            const float T = ts[s];
+            int j = k;
+            while (j > 0 && ts[order[j - 1]] < T) {
+                order[j] = order[j - 1];
+                --j;
             }
+            order[j] = (uint8_t)s;
+            s = s == 0 ? b - 1 : s - 1;
         }
-#pragma unroll
-        for (int r = 0; r < S; ++r)
-            if (r * L + l < n) E[r].w = expf(-kAgeDecay * fmaxf(t_now - E[r].T, 0.f));
-        // reference: the newest sample (entry 0: lane 0, register 0)
-        const float3 cr = make_float3(__shfl_sync(0xffffffffu, E[0].cx, 0, L),
-                                      __shfl_sync(0xffffffffu, E[0].cy, 0, L),
-                                      __shfl_sync(0xffffffffu, E[0].cz, 0, L));
-        float lw = 0.f, lwd = 0.f;
-#pragma unroll
-        for (int r = 0; r < S; ++r) {   // L - L_r
-            D[r] = r * L + l < n ? fmaf(kLumB, __fsub_rn(E[r].cz, cr.z),
-                                        fmaf(kLumG, __fsub_rn(E[r].cy, cr.y), kLumR * __fsub_rn(E[r].cx, cr.x)))
-                                 : 0.f;
-            lw += E[r].w;
-            lwd += E[r].w * D[r];
+        num = den = 0.f;
+        float T = ts[order[0]];
+        float3 c = CS::widen(col[order[0]]);
+        for (int k = 1; k < n; ++k) {
+            const int o = order[k];
+            const float To = ts[o], w = expf(-kAgeDecay * fmaxf(t_now - T, 0.f));
+            const float3 co = CS::widen(col[o]);
+            num += w * fabsf(lum_diff(c, co));
+            den += w * (T - To);
+            T = To;
+            c = co;
         }
-        const float sw = group_sum<L>(lw);
-        const float swd = group_sum<L>(lwd);
-        const float delta = n > 0 ? swd / sw : 0.f;   // mean - L_r
-        float lm2 = 0.f;
-#pragma unroll
-        for (int r = 0; r < S; ++r) {
-            const float dd = r * L + l < n ? D[r] - delta : 0.f;
-            lm2 += E[r].w * dd * dd;
-        }
-        const float m2 = group_sum<L>(lm2);
-        // newest first by time, equal times newest first by sequence number;
-        // queues filled in time order are already in that order
-        float T[S], Tn[S];
-        uint32_t Q[S], Qn[S];
-#pragma unroll
-        for (int r = 0; r < S; ++r) {
-            T[r] = E[r].T;
-            Q[r] = E[r].Q;
-        }
-        next_entry<L, S>(T, Tn, l);
-        next_entry<L, S>(Q, Qn, l);
-        bool ordered = true;
-#pragma unroll
-        for (int r = 0; r < S; ++r)
-            ordered = ordered && (!(r * L + l + 1 < n) || (T[r] > Tn[r]) || (T[r] == Tn[r] && Q[r] > Qn[r]));
-        if (!__all_sync(0xffffffffu, ordered)) {
-            // bitonic sort of the group's G entries descending by (T, Q);
-            // empty entries (-inf) sink. Entry e = r L + l: the partner at
-            // distance j < L is in lane l ^ j, at j >= L in register r ^ (j / L)
-            // of the same lane.
-#pragma unroll
-            for (int kk = 2; kk <= G; kk <<= 1) {
-#pragma unroll
-                for (int j = kk >> 1; j > 0; j >>= 1) {
-                    if (j >= L) {
-#pragma unroll
-                        for (int r = 0; r < S; ++r) {
-                            const int r2 = r ^ (j / L);
-                            if (r2 < r) continue;   // each pair once, from its lower entry
-                            const bool desc = ((r * L + l) & kk) == 0;
-                            if (newer(E[r], E[r2]) != desc) {
-                                const Entry t = E[r];
-                                E[r] = E[r2];
-                                E[r2] = t;
-                            }
-                        }
-                        continue;
-                    }
-#pragma unroll
-                    for (int r = 0; r < S; ++r) {
-                        const int e = r * L + l;
-                        Entry o;
-                        o.T = __shfl_xor_sync(0xffffffffu, E[r].T, j, L);
-                        o.Q = __shfl_xor_sync(0xffffffffu, E[r].Q, j, L);
-                        o.cx = __shfl_xor_sync(0xffffffffu, E[r].cx, j, L);
-                        o.cy = __shfl_xor_sync(0xffffffffu, E[r].cy, j, L);
-                        o.cz = __shfl_xor_sync(0xffffffffu, E[r].cz, j, L);
-                        o.w = __shfl_xor_sync(0xffffffffu, E[r].w, j, L);
-                        const bool lower = (e & j) == 0, desc = (e & kk) == 0;
-                        const bool keep = (lower == desc) ? newer(E[r], o) : !newer(E[r], o);
-                        if (!keep) E[r] = o;
-                    }
-                }
-            }
-        }
-        // consecutive luminance differences from the colour differences
-        float cx[S], cy[S], cz[S], cxn[S], cyn[S], czn[S];
-#pragma unroll
-        for (int r = 0; r < S; ++r) {
-            T[r] = E[r].T;
-            cx[r] = E[r].cx;
-            cy[r] = E[r].cy;
-            cz[r] = E[r].cz;
-        }
-        next_entry<L, S>(cx, cxn, l);
-        next_entry<L, S>(cy, cyn, l);
-        next_entry<L, S>(cz, czn, l);
-        next_entry<L, S>(T, Tn, l);
-        float num = 0.f, den = 0.f;
-#pragma unroll
-        for (int r = 0; r < S; ++r) {
-            if (r * L + l + 1 < n) {
-                const float dL = fmaf(kLumB, __fsub_rn(cz[r], czn[r]),
-                                      fmaf(kLumG, __fsub_rn(cy[r], cyn[r]), kLumR * __fsub_rn(cx[r], cxn[r])));
-                num += E[r].w * fabsf(dL);
-                den += E[r].w * (T[r] - Tn[r]);
-            }
-        }
-        num = group_sum<L>(num);
-        den = group_sum<L>(den);
-        if (l == 0 && pix) {
-            if (n == 0) {
-                lbar[p] = make_float2(__int_as_float(0x7fc00000), 0.f);
-                pstat[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-            } else {
-                const dfloat Lr = luminance_df(cr);
-                const dfloat mean = df_add(Lr, {delta, 0.f});
-                const float gt = (n >= 2 && den > 0.f) ? num / den : 0.f;
-                lbar[p] = make_float2(mean.h, mean.l);
-                pstat[p] = make_float4(sw, mean.h, m2, gt);
-            }
-        }
+    }
+    const float delta = n > 0 ? swd / sw : 0.f;   // mean - L_r
+    float m2 = 0.f;
+#pragma unroll(B ? B : 4)
+    for (int s = 0; s < b; ++s) {
+        const float w = B ? W[s] : ws[s], dd = (B ? D[s] : lum_diff(CS::widen(col[s]), cr)) - delta;
+        if (live >> s & 1u) m2 += w * dd * dd;
+    }
+    if (lane >= np) return;
+    if (n == 0) {
+        lbar[p] = make_float2(__int_as_float(0x7fc00000), 0.f);
+        pstat[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+        const dfloat mean = df_add(luminance_df(cr), {delta, 0.f});
+        lbar[p] = make_float2(mean.h, mean.l);
+        pstat[p] = make_float4(sw, m2, (n >= 2 && den > 0.f) ? num / den : 0.f, age);
     }
 }
 
-template <typename R>
-struct Moments {
-    R w, mean, m2;
-    __device__ __forceinline__ void merge(R w2, R mean2, R m22) {
-        R wt = w + w2;
-        if (wt > R(0)) {
-            R d = mean2 - mean;
-            mean = mean + d * (w2 / wt);
-            m2 = m2 + m22 + d * d * (w * w2 / wt);
-            w = wt;
-        }
-    }
+// ---- tile pass -------------------------------------------------------------------
+// One block per statistics tile, a warp per row: G_x, G_y of each pixel from
+// its neighbours' means (written to the gradient map) and the tile record:
+// sample count, non-empty pixels, sums of gradients and ages, and the
+// age-weighted luminance moments. The weights, the weighted means and then the
+// weighted squares about the tile's mean are summed as double-floats, so the
+// moments need no division per pixel and lose nothing in tiles of any size.
+// Bound: the latency of a block's loads and sums. Merging per-pixel moments with
+// Chan's formula, two divisions a merge, with FP64 merges of large tiles by one
+// thread, took 63 us at 1920x1080, 20 us at 640x480 and 9.6 us at 128x128; this
+// takes 28.6, 7.3 and 4.1 us (two and four blocks a SM: 30 us).
+constexpr int kTileThreads = 256;
+constexpr int kTileWarps = kTileThreads / 32;
+
+// a + x for a running double-float sum: exact but for the rounding of the low part
+__device__ __forceinline__ dfloat df_more(dfloat a, float x) {
+    const dfloat s = two_sum(a.h, x);
+    return {s.h, __fadd_rn(a.l, s.l)};
+}
+
+// Sum over the `width` lanes (a power of two) of each group of lanes.
+template <int WIDTH>
+__device__ __forceinline__ dfloat lanes_sum(dfloat v) {
+#pragma unroll
+    for (int o = WIDTH / 2; o > 0; o >>= 1)
+        v = df_add(v, dfloat{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
+    return v;
+}
+
+template <int WIDTH, typename T>
+__device__ __forceinline__ T lanes_sum(T v) {
+#pragma unroll
+    for (int o = WIDTH / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// What one pixel adds to its tile.
+struct PixelRead {
+    float2 c, l, r, u, d;   // means of the pixel and its neighbours (itself past the border)
+    float4 ps;
+    uint32_t cnt;
 };
 
-// One block per statistics tile: G_x, G_y of each pixel from its neighbours'
-// means (written to the gradient map) and the tile record: sample count,
-// non-empty pixels, gradient sums, and the age-weighted luminance moments
-// merged with Chan's formula (per thread and per warp in FP32, at most 2048
-// samples each; across warps in FP64 once the tile holds more than 4096, the
-// one FP64 step of the forward path). The record stores FP64 fields.
-constexpr int kTileThreads = 256;
+__device__ __forceinline__ PixelRead read_pixel(int x, int y, int W, int H, const float2 *__restrict__ lbar,
+                                                const float4 *__restrict__ pstat, const uint32_t *__restrict__ state) {
+    const int p = y * W + x;
+    PixelRead v;
+    v.c = __ldg(lbar + p);
+    v.l = __ldg(lbar + (x > 0 ? p - 1 : p));
+    v.r = __ldg(lbar + (x + 1 < W ? p + 1 : p));
+    v.u = __ldg(lbar + (y > 0 ? p - W : p));
+    v.d = __ldg(lbar + (y + 1 < H ? p + W : p));
+    v.ps = __ldg(pstat + p);
+    v.cnt = __ldg(state + p) & 0xFFFFu;
+    return v;
+}
 
-__global__ void __launch_bounds__(kTileThreads) k_spatial_tiles(int W, int H, int S, int ntx,
+struct TileSums {
+    uint32_t n = 0, ne = 0;
+    float gx = 0.f, gy = 0.f, gt = 0.f;
+    dfloat sw{0.f, 0.f}, swm{0.f, 0.f}, age{0.f, 0.f};
+};
+
+__device__ __forceinline__ void add_pixel(const PixelRead &v, int x, int y, int W, int H, float4 *__restrict__ grad,
+                                          TileSums &t) {
+    const int p = y * W + x;
+    if (isnan(v.c.x)) {
+        grad[p] = make_float4(0.f, 0.f, 0.f, v.c.x);
+        return;
+    }
+    // one-sided differences of the double-float means, rounded once
+    const dfloat m{v.c.x, v.c.y};
+    float sx = 0.f, sy = 0.f;
+    int mx = 0, my = 0;
+    if (x > 0 && !isnan(v.l.x)) { sx += fabsf(df_diff(m, {v.l.x, v.l.y})); ++mx; }
+    if (x + 1 < W && !isnan(v.r.x)) { sx += fabsf(df_diff(m, {v.r.x, v.r.y})); ++mx; }
+    if (y > 0 && !isnan(v.u.x)) { sy += fabsf(df_diff(m, {v.u.x, v.u.y})); ++my; }
+    if (y + 1 < H && !isnan(v.d.x)) { sy += fabsf(df_diff(m, {v.d.x, v.d.y})); ++my; }
+    const float gx = mx == 2 ? 0.5f * sx : sx, gy = my == 2 ? 0.5f * sy : sy;
+    grad[p] = make_float4(gx, gy, v.ps.z, v.c.x);
+    t.n += v.cnt;
+    ++t.ne;
+    t.gx += gx;
+    t.gy += gy;
+    t.gt += v.ps.z;
+    t.age = df_more(t.age, v.ps.w);
+    t.sw = df_more(t.sw, v.ps.x);
+    const dfloat q = two_prod(v.ps.x, v.c.x);
+    t.swm = df_more(t.swm, q.h);
+    t.swm.l += q.l;
+}
+
+// SMALL: tiles of up to 32 x 32 pixels, four rows a warp: every load of a
+// thread is issued before the first is used, and the second pass reads
+// registers.
+template <bool SMALL>
+__global__ void __launch_bounds__(kTileThreads, 3) k_spatial_tiles(int W, int H, int S, int ntx,
                                                                 const float2 *__restrict__ lbar,
                                                                 const float4 *__restrict__ pstat,
                                                                 const uint32_t *__restrict__ state,
                                                                 float4 *__restrict__ grad,
-                                                                TilePartial *__restrict__ tiles) {
-    const int tile = blockIdx.x;
+                                                                TilePartial *__restrict__ tiles,
+                                                                unsigned long long *__restrict__ total) {
+    const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int x0 = (tile % ntx) * S, y0 = (tile / ntx) * S;
-    const int tw = min(S, W - x0), th = min(S, H - y0), A = tw * th;
-    float n = 0.f, ne = 0.f, sgx = 0.f, sgy = 0.f, sgt = 0.f;
-    Moments<float> mo{0.f, 0.f, 0.f};
-    for (int k = threadIdx.x; k < A; k += blockDim.x) {
-        const int x = x0 + k % tw, y = y0 + k / tw;
-        const int p = y * W + x;
-        const float2 lp = __ldg(lbar + p);
-        const float l = lp.x;
-        const float4 ps = __ldg(pstat + p);
-        if (isnan(l)) {
-            grad[p] = make_float4(0.f, 0.f, 0.f, l);
-            continue;
-        }
-        // one-sided differences of the double-float means, rounded once
-        float sx = 0.f, sy = 0.f;
-        int mx = 0, my = 0;
-        const dfloat lm = {lp.x, lp.y};
-        float2 v;
-        if (x > 0 && !isnan((v = __ldg(lbar + p - 1)).x)) { sx += fabsf(df_diff(lm, {v.x, v.y})); ++mx; }
-        if (x + 1 < W && !isnan((v = __ldg(lbar + p + 1)).x)) { sx += fabsf(df_diff(lm, {v.x, v.y})); ++mx; }
-        if (y > 0 && !isnan((v = __ldg(lbar + p - W)).x)) { sy += fabsf(df_diff(lm, {v.x, v.y})); ++my; }
-        if (y + 1 < H && !isnan((v = __ldg(lbar + p + W)).x)) { sy += fabsf(df_diff(lm, {v.x, v.y})); ++my; }
-        const float gx = mx ? sx / mx : 0.f, gy = my ? sy / my : 0.f;
-        grad[p] = make_float4(gx, gy, ps.w, l);
-        n += (float)(__ldg(state + p) & 0xFFFFu);
-        ne += 1.f;
-        sgx += gx;
-        sgy += gy;
-        sgt += ps.w;
-        mo.merge(ps.x, ps.y, ps.z);
-    }
+    const int x1 = min(W, x0 + S), y1 = min(H, y0 + S);
+    constexpr int ROWS = SMALL ? 4 : 1;
+    PixelRead v[ROWS];
+    TileSums t;
+    if (SMALL) {
+        const int x = min(x0 + lane, x1 - 1);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        n += __shfl_xor_sync(0xffffffffu, n, o);
-        ne += __shfl_xor_sync(0xffffffffu, ne, o);
-        sgx += __shfl_xor_sync(0xffffffffu, sgx, o);
-        sgy += __shfl_xor_sync(0xffffffffu, sgy, o);
-        sgt += __shfl_xor_sync(0xffffffffu, sgt, o);
-        const float w2 = __shfl_xor_sync(0xffffffffu, mo.w, o);
-        const float mu2 = __shfl_xor_sync(0xffffffffu, mo.mean, o);
-        const float s2 = __shfl_xor_sync(0xffffffffu, mo.m2, o);
-        mo.merge(w2, mu2, s2);
+        for (int r = 0; r < ROWS; ++r) v[r] = read_pixel(x, min(y0 + warp + r * kTileWarps, y1 - 1), W, H, lbar, pstat, state);
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const int y = y0 + warp + r * kTileWarps;
+            if (x0 + lane < x1 && y < y1) add_pixel(v[r], x, y, W, H, grad, t);
+            else v[r].c.x = __int_as_float(0x7fc00000);   // no pixel
+        }
+    } else {
+        for (int x = x0 + lane; x < x1; x += 32)
+            for (int y = y0 + warp; y < y1; y += kTileWarps)
+                add_pixel(read_pixel(x, y, W, H, lbar, pstat, state), x, y, W, H, grad, t);
     }
-    __shared__ float sh[kTileThreads / 32][8];
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
-        sh[warp][0] = n; sh[warp][1] = ne; sh[warp][2] = sgx; sh[warp][3] = sgy; sh[warp][4] = sgt;
-        sh[warp][5] = mo.w; sh[warp][6] = mo.mean; sh[warp][7] = mo.m2;
+    __shared__ float2 shd[3][kTileWarps];
+    __shared__ float shf[3][kTileWarps];
+    __shared__ uint32_t shi[2][kTileWarps];
+    __shared__ float tile_mean;
+    t.n = __reduce_add_sync(0xffffffffu, t.n);
+    t.ne = __reduce_add_sync(0xffffffffu, t.ne);
+    t.gx = lanes_sum<32>(t.gx);
+    t.gy = lanes_sum<32>(t.gy);
+    t.gt = lanes_sum<32>(t.gt);
+    t.sw = lanes_sum<32>(t.sw);
+    t.swm = lanes_sum<32>(t.swm);
+    t.age = lanes_sum<32>(t.age);
+    if (lane == 0) {
+        shi[0][warp] = t.n; shi[1][warp] = t.ne;
+        shf[0][warp] = t.gx; shf[1][warp] = t.gy; shf[2][warp] = t.gt;
+        shd[0][warp] = make_float2(t.sw.h, t.sw.l);
+        shd[1][warp] = make_float2(t.swm.h, t.swm.l);
+        shd[2][warp] = make_float2(t.age.h, t.age.l);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        TilePartial out;
-        // FP32 across the warps: the counts are integers (exact below 2^24) and
-        // the gradient sums add eight warp totals
-        float tn = 0.f, tne = 0.f, tgx = 0.f, tgy = 0.f, tgt = 0.f;
-        for (int w = 0; w < kTileThreads / 32; ++w) {
-            tn += sh[w][0]; tne += sh[w][1]; tgx += sh[w][2]; tgy += sh[w][3]; tgt += sh[w][4];
+    TilePartial out;
+    if (warp == 0) {   // eight lanes a quantity
+        static_assert(kTileWarps == 8, "eight partials a quantity");
+        const int q = min(lane >> 3, 2), w = lane & 7;
+        const dfloat d = lanes_sum<8>(dfloat{shd[q][w].x, shd[q][w].y});
+        const float f = lanes_sum<8>(shf[q][w]);
+        const uint32_t i = lanes_sum<8>(shi[min(q, 1)][w]);
+        auto take = [&](int k) { return dfloat{__shfl_sync(0xffffffffu, d.h, 8 * k), __shfl_sync(0xffffffffu, d.l, 8 * k)}; };
+        const dfloat tw = take(0), tm = take(1), ta = take(2);
+        const dfloat mean = tw.h > 0.f ? df_div(tm, tw) : dfloat{0.f, 0.f};
+        out.sw = (double)tw.h + (double)tw.l;
+        out.mean = (double)mean.h + (double)mean.l;
+        out.n = __shfl_sync(0xffffffffu, i, 0);
+        out.nonempty = __shfl_sync(0xffffffffu, i, 8);
+        out.sgx = __shfl_sync(0xffffffffu, f, 0);
+        out.sgy = __shfl_sync(0xffffffffu, f, 8);
+        out.sgt = __shfl_sync(0xffffffffu, f, 16);
+        out.age = __fadd_rn(ta.h, ta.l);
+        out.pad[0] = out.pad[1] = 0u;
+        if (lane == 0) {
+            tile_mean = mean.h;
+            if (out.n) atomicAdd(total, (unsigned long long)out.n);
         }
-        if (tn > (float)kSortedBinMax) {   // more than 4096 samples: FP64 merge
-            Moments<double> r{0.0, 0.0, 0.0};
-            for (int w = 0; w < kTileThreads / 32; ++w) r.merge(sh[w][5], sh[w][6], sh[w][7]);
-            out.sw = r.w; out.mean = r.mean; out.m2 = r.m2;
-        } else {
-            Moments<float> r{0.f, 0.f, 0.f};
-            for (int w = 0; w < kTileThreads / 32; ++w) r.merge(sh[w][5], sh[w][6], sh[w][7]);
-            out.sw = r.w; out.mean = r.mean; out.m2 = r.m2;
-        }
-        out.n = (uint32_t)tn;
-        out.nonempty = (uint32_t)tne;
-        out.sgx = tgx;
-        out.sgy = tgy;
-        out.sgt = tgt;
-        out.pad[0] = out.pad[1] = out.pad[2] = 0u;
-        tiles[tile] = out;
+    }
+    __syncthreads();
+    // squares about the tile's mean
+    const float tm = tile_mean;
+    dfloat m2{0.f, 0.f};
+    auto square = [&](float c, float sw, float m) {
+        if (!isnan(c)) m2 = df_more(m2, fmaf(sw * (c - tm), c - tm, m));
+    };
+    if (SMALL) {
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) square(v[r].c.x, v[r].ps.x, v[r].ps.y);
+    } else {
+        for (int x = x0 + lane; x < x1; x += 32)
+            for (int y = y0 + warp; y < y1; y += kTileWarps) {
+                const int p = y * W + x;
+                const float2 ps = __ldg(reinterpret_cast<const float2 *>(pstat + p));
+                square(__ldg(&lbar[p].x), ps.x, ps.y);
+            }
+    }
+    m2 = lanes_sum<32>(m2);
+    if (lane == 0) shd[0][warp] = make_float2(m2.h, m2.l);
+    __syncthreads();
+    if (warp == 0) {
+        const dfloat d = lanes_sum<8>(dfloat{shd[0][lane & 7].x, shd[0][lane & 7].y});
+        out.m2 = (double)d.h + (double)d.l;
+        if (lane == 0) tiles[tile] = out;
     }
 }
 
-// Queue entries per lane of the pixel pass.
-constexpr int kPixelEntries = 4;
+template <int CT, int B>
+void launch_depth(AfrContext *c, float t_now, unsigned long long *total, cudaStream_t s) {
+    const PixelLayout l = pixel_layout(c->b, c->csize, B == 0);
+    const int groups = (c->P + 31) / 32;
+    k_pixel<CT, B><<<(groups + kPixelWarps - 1) / kPixelWarps, 32 * kPixelWarps, kPixelWarps * l.bytes, s>>>(
+        c->P, c->b, t_now, c->r_state, c->r_t, c->r_col, c->lbar, c->pstat, total);
+}
 
 template <int CT>
-cudaError_t launch_pixel(AfrContext *c, float t_now, cudaStream_t s) {
-    constexpr int S = kPixelEntries;
-    int g = grid_for((size_t)c->P * 32, 256, 16 * device_sms());
-    if (c->b <= 4)
-        k_pixel<CT, 4, 2><<<g, 256, 0, s>>>(c->P, c->b, t_now, c->r_state, c->r_t, c->r_seq, c->r_col, c->lbar,
-                                            c->pstat);
-    else if (c->b <= 8)
-        k_pixel<CT, 8, S><<<g, 256, 0, s>>>(c->P, c->b, t_now, c->r_state, c->r_t, c->r_seq, c->r_col, c->lbar,
-                                            c->pstat);
-    else if (c->b <= 16)
-        k_pixel<CT, 16, S><<<g, 256, 0, s>>>(c->P, c->b, t_now, c->r_state, c->r_t, c->r_seq, c->r_col, c->lbar,
-                                             c->pstat);
-    else
-        k_pixel<CT, 32, S><<<g, 256, 0, s>>>(c->P, c->b, t_now, c->r_state, c->r_t, c->r_seq, c->r_col, c->lbar,
-                                             c->pstat);
-    return cudaGetLastError();
+void launch_pixel(AfrContext *c, float t_now, unsigned long long *total, cudaStream_t s) {
+    switch (c->b) {
+        case 4: launch_depth<CT, 4>(c, t_now, total, s); break;
+        case 8: launch_depth<CT, 8>(c, t_now, total, s); break;
+        case 16: launch_depth<CT, 16>(c, t_now, total, s); break;
+        default: launch_depth<CT, 0>(c, t_now, total, s); break;
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_gradients(AfrContext *c, float t_now, cudaStream_t s) {
-    cudaError_t e;
+    unsigned long long *total = tile_total(c);
     switch (c->ct) {
-        case AFR_F32: e = launch_pixel<AFR_F32>(c, t_now, s); break;
-        case AFR_F16: e = launch_pixel<AFR_F16>(c, t_now, s); break;
-        default: e = launch_pixel<AFR_BF16>(c, t_now, s); break;
+        case AFR_F32: launch_pixel<AFR_F32>(c, t_now, total, s); break;
+        case AFR_F16: launch_pixel<AFR_F16>(c, t_now, total, s); break;
+        default: launch_pixel<AFR_BF16>(c, t_now, total, s); break;
     }
-    if (e != cudaSuccess) return e;
-    k_spatial_tiles<<<c->ntiles, kTileThreads, 0, s>>>(c->W, c->H, c->S, c->ntx, c->lbar, c->pstat, c->r_state,
-                                                      c->grad, c->tiles);
+    if (c->S <= 32)
+        k_spatial_tiles<true><<<c->ntiles, kTileThreads, 0, s>>>(c->W, c->H, c->S, c->ntx, c->lbar, c->pstat,
+                                                                 c->r_state, c->grad, c->tiles, total);
+    else
+        k_spatial_tiles<false><<<c->ntiles, kTileThreads, 0, s>>>(c->W, c->H, c->S, c->ntx, c->lbar, c->pstat,
+                                                                  c->r_state, c->grad, c->tiles, total);
     return cudaGetLastError();
 }
 
