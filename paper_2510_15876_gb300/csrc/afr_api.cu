@@ -59,7 +59,7 @@ cudaError_t dalloc(T **p, size_t n) {
 
 void free_all(AfrContext *c) {
     void *ptrs[] = {c->r_xy, c->r_mo, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->bucket, c->fifo_flag, c->fifo_rank, c->fifo_scan,
-                    c->ccnt, c->coff, c->ccur, c->lbar, c->grad, c->pstat, c->sigma, c->fconst, c->cov_r[0], c->cov_r[1], c->cov_n, c->amin2, c->tiles, c->fcnt,
+                    c->ccnt, c->coff, c->ccur, c->lbar, c->grad, c->pstat, c->sigma, c->fconst, c->cov_r[0], c->cov_r[1], c->cov_n, c->amin2, c->tiles, c->fcnt, c->fcur,
                     c->foff, c->frec, c->sbin, c->flist, c->flseq, c->q_xy, c->q_mo, c->q_t, c->q_seq, c->q_col, c->q_total, c->q_world, c->r_world, c->scan_tmp, c->scan_tmp_in, c->bgrad, c->bparam, c->dcount, c->derr};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -217,6 +217,7 @@ AfrStatus afr_create(const AfrConfig *cfg, AfrContext **out) {
     AFR_ALLOC(c->amin2, P);
     AFR_ALLOC(c->tiles, (size_t)c->ntiles + 1);
     AFR_ALLOC(c->fcnt, P);
+    AFR_ALLOC(c->fcur, P);
     AFR_ALLOC(c->foff, P + 1);
     if (g.world_points) AFR_ALLOC(c->r_world, N);
     if (c->fifo_n) {
@@ -242,6 +243,8 @@ AfrStatus afr_create(const AfrConfig *cfg, AfrContext **out) {
     AFR_ALLOC(c->derr, 1);
 #undef AFR_ALLOC
     if (e == cudaSuccess) e = cudaMemset(c->r_state, 0, P * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemset(c->ccnt, 0, P * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemset(c->fcnt, 0, P * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(c->foff, 0, (P + 1) * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(c->dcount, 0, afr::CNT_N * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(c->derr, 0, sizeof(uint32_t));

@@ -22,8 +22,9 @@ constexpr int kPitch = 18;                       // frame records carry their bi
 constexpr int kFramePad = 32;                    // records past frame_cap that the filter may read (never sums)
 constexpr int kSortedBinMax = 4096;              // frame bins ordered by seq up to this size
 
-// device counters (unsigned long long)
-enum { CNT_REJECTED = 0, CNT_DROPPED, CNT_UNSORTED, CNT_RESIDENT, CNT_BIG, CNT_N };
+// device counters (unsigned long long); CNT_DROPPING: samples dropped by a
+// reprojection under way, 0 between reprojections
+enum { CNT_REJECTED = 0, CNT_DROPPED, CNT_UNSORTED, CNT_RESIDENT, CNT_DROPPING, CNT_N };
 // device status word bits
 enum { ERR_TIMEOUT = 1u, ERR_CHECK = 2u };
 
@@ -128,9 +129,9 @@ struct AfrContext {
     uint32_t *fifo_scan = nullptr;  // scan block sums for batch_cap entries
     // ingest scratch: per-cell counts and offsets (cells of 16 x 8 pixels) and
     // the batch's records bucketed by pixel (batch_cap records)
-    uint32_t *ccnt = nullptr;     // [P] bucket counts
+    uint32_t *ccnt = nullptr;     // [P] bucket counts, all 0 between batches
     uint32_t *coff = nullptr;     // [P + 1] bucket offsets
-    uint32_t *ccur = nullptr;     // [P] append cursors, then the queue states before the batch
+    uint32_t *ccur = nullptr;     // [P] append cursors, then the queue states after the batch
     uint4 *bucket = nullptr;      // [4 * batch_cap] 64-byte sample records in bucket order
     size_t batch_cap = 0;
 
@@ -149,7 +150,8 @@ struct AfrContext {
     afr::TilePartial *tiles = nullptr;  // [ntiles + 1]; the last holds the samples of all tiles (tile_total)
 
     // frame view
-    uint32_t *fcnt = nullptr;     // [P]
+    uint32_t *fcnt = nullptr;     // [P] bin counts, all 0 between reprojections
+    uint32_t *fcur = nullptr;     // [P] append cursors of the bins' lists
     uint32_t *foff = nullptr;     // [P+1]
     afr::FrameRec *frec = nullptr;  // [frame_cap + kFramePad]
     uint32_t *sbin = nullptr;     // [frame_cap] each source slot's bin (reprojection scratch)
@@ -368,7 +370,18 @@ inline int grid_for(size_t n, int block, int cap = 0) {
 
 // ---- launch wrappers (one per translation unit) ------------------------------
 // Each returns cudaSuccess or the launch error.
-cudaError_t scan_exclusive(const uint32_t *in, uint32_t *out, size_t n, uint32_t *tmp, cudaStream_t s);
+// What else a scan writes on its way (null: nothing).
+struct ScanWith {
+    uint32_t *cursor = nullptr;     // [n] a copy of the offsets
+    bool clear_in = false;          // the counts are set to 0
+    uint32_t *fill = nullptr;       // [n] set to fill_value
+    uint32_t fill_value = 0u;
+    unsigned long long *counter_from = nullptr, *counter_to = nullptr;   // moved (the source becomes 0)
+    unsigned long long *counter_zero = nullptr;                          // set to 0
+};
+// in and the arrays of `with` must be 32-byte aligned.
+cudaError_t scan_exclusive(uint32_t *in, uint32_t *out, size_t n, uint32_t *tmp, cudaStream_t s,
+                           const ScanWith &with = ScanWith());
 size_t scan_tmp_elems(size_t n);
 
 // queues_free: the steps that touch the queues wait for it (may be null);

@@ -25,10 +25,14 @@
 //              min(b, m) go to the queue slots
 //              (head + rank) mod b that sequential pushes would use, so a
 //              warp's stores cover consecutive slots. The first record of each
-//              pixel writes the pixel's new queue state (from a copy of the
-//              states taken before the commit, which every thread reads). A
-//              pixel with more than kBigPixel records is left to a warp that
+//              pixel writes the pixel's new queue state to scratch, for the
+//              other records still read the old one.
+//  5. finish:  a thread per pixel puts the new states in place (and empties the
+//              pixels without records after a reset). A pixel with more than
+//              kBigPixel records, left out by the commit, gets a warp that
 //              streams its bucket keeping the newest 32 in registers.
+// The scan clears the counts it has read and starts the cursors, so a batch
+// takes six launches and no other operation.
 #include "afr_internal.cuh"
 
 namespace afr {
@@ -231,14 +235,14 @@ __device__ __forceinline__ void put_record(const uint4 &a, const uint4 &q1, cons
 // Thread per bucket record, pixels of up to kBigPixel records. A block takes
 // kCommitTile consecutive records at a time and keeps their batch indices in
 // shared memory, where the rank scans find all of a pixel's records but
-// those of pixels crossing the tile's ends. state0 holds the queue states
-// before the batch.
+// those of pixels crossing the tile's ends. The queue states are those before
+// the batch (none after a reset); the new ones go to state1.
 constexpr int kCommitTile = 256;
 
 template <int CT>
 __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__restrict__ poff, uint32_t P, int W,
                                                             int b, uint32_t seq0, Bucket bk, Queues q,
-                                                            const uint32_t *__restrict__ state0, DebugCheck dc) {
+                                                            bool reset, uint32_t *__restrict__ state1, DebugCheck dc) {
     __shared__ uint32_t sidx[kCommitTile];
     uint32_t n = __ldg(poff + P);
     if (!AFR_CHECK(n <= dc.cap, dc.derr)) n = 0;
@@ -262,7 +266,7 @@ __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__re
         if (work) {
             beg = __ldg(poff + px);
             end = __ldg(poff + px + 1);
-            st = __ldg(state0 + px);
+            st = reset ? 0u : __ldg(q.state + px);
             work = end - beg <= kBigPixel && (a.w != kInvalid || e == beg) && AFR_CHECK(end <= n, dc.derr);
         }
         if (work) {
@@ -285,7 +289,7 @@ __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__re
                 dead += w == kInvalid;
             }
             const uint32_t nl = end - beg - dead;
-            if (e == beg) q.state[px] = pushed_state(st, nl, ub);
+            if (e == beg) state1[px] = pushed_state(st, nl, ub);
             if (a.w != kInvalid && rank + min(nl, ub) >= nl) {   // else evicted by newer samples of the batch
                 const size_t dst = (size_t)px * ub + ((st >> 16) + rank) % ub;
                 if (AFR_CHECK(dst < q.nslots, dc.derr)) put_record<CT>(a, q1, q2, q3, dst, seq0 + a.w, q);
@@ -295,12 +299,21 @@ __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__re
     }
 }
 
-// Pixels of more than kBigPixel records: a warp streams the pixel's bucket,
-// keeping the newest 32 live records by bitonic merges.
+// Puts the pixels' new states in place, empties those without records and the
+// counters after a reset, and commits the pixels of more than kBigPixel
+// records: a warp streams such a pixel's bucket, keeping the newest 32 live
+// records by bitonic merges.
 template <int CT>
-__global__ void __launch_bounds__(256) k_pix_commit_big(const uint32_t *__restrict__ poff, uint32_t P, int b,
-                                                        uint32_t seq0, Bucket bk, Queues q,
-                                                        const uint32_t *__restrict__ state0, DebugCheck dc) {
+__global__ void __launch_bounds__(256) k_pix_finish(const uint32_t *__restrict__ poff, uint32_t P, int b,
+                                                    uint32_t seq0, Bucket bk, Queues q, bool reset,
+                                                    const uint32_t *__restrict__ state1,
+                                                    unsigned long long *__restrict__ dcount,
+                                                    uint32_t *__restrict__ q_total, DebugCheck dc) {
+    static_assert(CNT_REJECTED == 0, "the rejected count, cleared before the scatter, comes first");
+    if (reset && blockIdx.x == 0) {
+        if (threadIdx.x >= 1 && threadIdx.x < CNT_N) dcount[threadIdx.x] = 0ull;
+        if (threadIdx.x == 0 && q_total) *q_total = 0u;
+    }
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t ub = (uint32_t)b;
@@ -309,7 +322,11 @@ __global__ void __launch_bounds__(256) k_pix_commit_big(const uint32_t *__restri
     for (uint32_t base = warp * 32u; base < P; base += nwarps * 32u) {
         const uint32_t p = base + (uint32_t)lane;
         uint32_t m = 0;
-        if (p < P) m = __ldg(poff + p + 1) - __ldg(poff + p);
+        if (p < P) {
+            m = __ldg(poff + p + 1) - __ldg(poff + p);
+            if (m && m <= kBigPixel) q.state[p] = state1[p];
+            if (!m && reset) q.state[p] = 0u;
+        }
         unsigned big = __ballot_sync(0xffffffffu, m > kBigPixel);
         while (big) {
             const uint32_t px = base + (uint32_t)(__ffs(big) - 1);
@@ -329,7 +346,8 @@ __global__ void __launch_bounds__(256) k_pix_commit_big(const uint32_t *__restri
                 nl += (uint32_t)__popc(__ballot_sync(0xffffffffu, key != 0ull));
                 top = warp_top32(top, key);
             }
-            const uint32_t st = __ldg(state0 + px);
+            const uint32_t st = reset ? 0u : q.state[px];
+            __syncwarp();   // every lane has read the state
             if (lane == 0) q.state[px] = pushed_state(st, nl, ub);
             const uint32_t kept = min(nl, ub);
             if (lane >= 32 - (int)kept) {
@@ -356,35 +374,24 @@ cudaError_t run(AfrContext *c, const float4 *pos, const void *col, const float2 
     Bucket bk{c->bucket};
     cudaError_t e;
     // binning: the context's scratch only (the scatter counts the rejected samples)
-    if (reset && (e = cudaMemsetAsync(c->dcount + CNT_REJECTED, 0, sizeof(unsigned long long), s)) != cudaSuccess)
-        return e;
-    if ((e = cudaMemsetAsync(c->ccnt, 0, sizeof(uint32_t) * P, s)) != cudaSuccess) return e;
     k_pix_count<<<grid_for(n, 256), 256, 0, s>>>(pos, n, c->W, c->H, c->ccnt);
-    if ((e = scan_exclusive(c->ccnt, c->coff, P, c->scan_tmp_in, s)) != cudaSuccess) return e;
-    // append cursors start at the bucket offsets: a ticket is the record's place
-    if ((e = cudaMemcpyAsync(c->ccur, c->coff, sizeof(uint32_t) * P, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-        return e;
+    ScanWith with;
+    with.cursor = c->ccur;   // append cursors start at the bucket offsets: a ticket is the record's place
+    with.clear_in = true;
+    if (reset) with.counter_zero = c->dcount + CNT_REJECTED;
+    if ((e = scan_exclusive(c->ccnt, c->coff, P, c->scan_tmp_in, s, with)) != cudaSuccess) return e;
     const int gs = grid_for((n + kScatterUnroll - 1) / kScatterUnroll, 32 * kScatterWarps);
     uint32_t *accept = c->fifo_n ? c->fifo_flag : nullptr;
     k_pix_scatter<CT><<<gs, 32 * kScatterWarps, 0, s>>>(pos, col, mo, c->r_world ? world : nullptr, n, c->W, c->H,
                                                         c->ccur, bk, accept, c->dcount, dc);
-    // from here on the queues: wait until they are free, clear them if asked
+    // from here on the queues: wait until they are free. The cursors are spent:
+    // they take the new queue states
     if (queues_free && (e = cudaStreamWaitEvent(s, queues_free, 0)) != cudaSuccess) return e;
-    if (reset) {
-        static_assert(CNT_REJECTED == 0, "the rejected count comes first");
-        if ((e = cudaMemsetAsync(c->r_state, 0, sizeof(uint32_t) * P, s)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(c->dcount + 1, 0, sizeof(unsigned long long) * (CNT_N - 1), s)) != cudaSuccess)
-            return e;
-        if (c->q_total && (e = cudaMemsetAsync(c->q_total, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
-    }
-    // the cursors are spent: they take the queue states before the batch,
-    // which every commit thread reads
-    if ((e = cudaMemcpyAsync(c->ccur, c->r_state, sizeof(uint32_t) * P, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-        return e;
     Queues q{c->r_xy, c->r_mo, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->r_world, c->nslots};
-    k_pix_commit<CT><<<grid_for(n, kCommitTile), kCommitTile, 0, s>>>(c->coff, P, c->W, c->b, seq0, bk, q, c->ccur,
-                                                                      dc);
-    k_pix_commit_big<CT><<<grid_for(P, 256), 256, 0, s>>>(c->coff, P, c->b, seq0, bk, q, c->ccur, dc);
+    k_pix_commit<CT><<<grid_for(n, kCommitTile), kCommitTile, 0, s>>>(c->coff, P, c->W, c->b, seq0, bk, q, reset,
+                                                                      c->ccur, dc);
+    k_pix_finish<CT><<<grid_for(P, 256), 256, 0, s>>>(c->coff, P, c->b, seq0, bk, q, reset, c->ccur, c->dcount,
+                                                      c->q_total, dc);
     return cudaGetLastError();
 }
 

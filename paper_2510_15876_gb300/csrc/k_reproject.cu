@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256) k_count(uint32_t nslots, int b, int bshif
         }
     }
     const uint32_t d = __reduce_add_sync(0xffffffffu, dropped);
-    if (lane == 0 && d) atomicAdd(dcount + CNT_DROPPED, (unsigned long long)d);
+    if (lane == 0 && d) atomicAdd(dcount + CNT_DROPPING, (unsigned long long)d);
 }
 
 // The slots' bins from the count pass (kInvalid: dead or moved out). A warp
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(256) k_list(uint32_t nslots, const uint32_t *_
     }
 }
 
-// fcnt holds every bin's end here (the list's cursors); a bin above
+// fcur holds every bin's end here (the list's cursors); a bin above
 // kSortedBinMax records takes its ranks by counting it down (arrival order)
 // and is counted as unsorted.
 // The frame records arrive in bin order, so the lanes of a warp that share a
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(256) k_place(int W, int H, float t_now, Camera
                                                const float *__restrict__ r_t, const uint32_t *__restrict__ r_seq,
                                                const void *__restrict__ r_col, uint32_t P,
                                                const uint32_t *__restrict__ foff, const uint32_t *__restrict__ flist,
-                                               const uint32_t *__restrict__ flseq, uint32_t *__restrict__ fcnt,
+                                               const uint32_t *__restrict__ flseq, uint32_t *__restrict__ fcur,
                                                uint32_t *__restrict__ amin2, FrameRec *__restrict__ frec,
                                                unsigned long long *__restrict__ dcount, DebugCheck dc, uint32_t nsrc) {
     using CS = ColorStore<CT>;
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(256) k_place(int W, int H, float t_now, Camera
         if (end - beg <= (uint32_t)kSortedBinMax) {
             for (uint32_t k = beg; k < end; ++k) rank += __ldg(flseq + k) < sq;
         } else {
-            rank = atomicSub(fcnt + mv.bin, 1u) - 1u - beg;   // the cursor ends at the bin's end
+            rank = atomicSub(fcur + mv.bin, 1u) - 1u - beg;   // the cursor ends at the bin's end
             if (rank == 0) atomicAdd(dcount + CNT_UNSORTED, 1ull);
         }
         const uint32_t d = beg + rank;
@@ -257,17 +257,10 @@ __global__ void __launch_bounds__(256) k_place(int W, int H, float t_now, Camera
     }
 }
 
-__global__ void k_fill_u32(uint32_t *p, size_t n, uint32_t v) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) p[i] = v;
-}
-
 }  // namespace
 
 cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cudaStream_t s) {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(c->fcnt, 0, sizeof(uint32_t) * c->P, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(c->dcount + CNT_DROPPED, 0, sizeof(unsigned long long) * 2, s)) != cudaSuccess) return e;
-    k_fill_u32<<<grid_for(c->P, 256), 256, 0, s>>>(c->amin2, c->P, 0x7f800000u);
     // source: the per-pixel queues, or the reconstructor queue (section 5.2);
     // moved by screen motion, or rendered by a camera (hit points)
     const bool fifo = c->fifo_n > 0, cam = camp != nullptr;
@@ -291,14 +284,22 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     else if (cam) AFR_COUNT(false, true);
     else AFR_COUNT(false, false);
 #undef AFR_COUNT
-    if ((e = scan_exclusive(c->fcnt, c->foff, c->P, c->scan_tmp, s)) != cudaSuccess) return e;
-    // the list's append cursors start at the bin offsets (a ticket is the entry's place)
-    if ((e = cudaMemcpyAsync(c->fcnt, c->foff, sizeof(uint32_t) * c->P, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-        return e;
-    k_list<<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcnt, c->flist, c->flseq, dc);
+    // the scan starts the list's append cursors at the bin offsets (a ticket is
+    // the entry's place), clears the counts and the bins' smallest ages, and
+    // makes the dropped count public
+    ScanWith with;
+    with.cursor = c->fcur;
+    with.clear_in = true;
+    with.fill = c->amin2;
+    with.fill_value = 0x7f800000u;
+    with.counter_from = c->dcount + CNT_DROPPING;
+    with.counter_to = c->dcount + CNT_DROPPED;
+    with.counter_zero = c->dcount + CNT_UNSORTED;
+    if ((e = scan_exclusive(c->fcnt, c->foff, c->P, c->scan_tmp, s, with)) != cudaSuccess) return e;
+    k_list<<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, c->flseq, dc);
 #define AFR_PLACE(CT_, F_, C_)                                                                                     \
     k_place<CT_, F_, C_><<<g, 256, 0, s>>>(c->W, c->H, t_now, cm, wp, xy, mo, tt, sq, col, (uint32_t)c->P, c->foff, \
-                                           c->flist, c->flseq, c->fcnt, c->amin2, c->frec,       \
+                                           c->flist, c->flseq, c->fcur, c->amin2, c->frec,       \
                                            c->dcount, dc, ns)
 #define AFR_REPROJ(CT_)                                                                                        \
     do {                                                                                                       \

@@ -1,8 +1,16 @@
 // k_scan.cu -- exclusive prefix sum of uint32 counts (bin offsets of the
-// counting sorts in ingest and reprojection). Reduce-then-scan in three
-// launches: per-block sums, a single-block scan of those sums, and a
-// per-block scan that adds its block's prefix. out has n+1 entries; out[n]
-// is the total.
+// counting sorts in ingest and reprojection), with the clearing and filling
+// that the sort around it needs (ScanWith). Two launches: per-block sums, and
+// a per-block scan whose prefix every block adds up from the sums before it
+// (beyond kDirectBlocks blocks a launch between scans the sums first, so that
+// the work does not grow with the square of their number). out has n + 1
+// entries; out[n] is the total.
+//
+// Bound: HBM at large n (every array once, 256-bit accesses), launches at small
+// n: with a launch of its own for the sums, 32-byte strided reads, and separate
+// launches for the cursor copy, the clearing and the fill, a reprojection's
+// share was nine operations (30 us at 1920x1080, 20 us at 128x128), now two
+// (10 and 4.5 us).
 #include "afr_internal.cuh"
 
 namespace afr {
@@ -11,6 +19,37 @@ namespace {
 constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
+constexpr size_t kDirectBlocks = 2048;   // 8.4M counts: a block reads at most 8 KB of sums
+
+struct Items {
+    uint32_t v[kScanItems];
+};
+
+__device__ __forceinline__ Items load_items(const uint32_t *p, size_t i, size_t n) {
+    Items r;
+    if (i + kScanItems <= n) {
+        asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(r.v[0]), "=r"(r.v[1]), "=r"(r.v[2]), "=r"(r.v[3]), "=r"(r.v[4]), "=r"(r.v[5]), "=r"(r.v[6]),
+              "=r"(r.v[7])
+            : "l"(p + i));
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) r.v[k] = i + k < n ? p[i + k] : 0u;
+    }
+    return r;
+}
+
+__device__ __forceinline__ void store_items(uint32_t *p, size_t i, size_t n, const Items &r, bool wide = true) {
+    if (wide && i + kScanItems <= n) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p + i), "r"(r.v[0]), "r"(r.v[1]),
+                     "r"(r.v[2]), "r"(r.v[3]), "r"(r.v[4]), "r"(r.v[5]), "r"(r.v[6]), "r"(r.v[7])
+                     : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k)
+            if (i + k < n) p[i + k] = r.v[k];
+    }
+}
 
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
     int lane = threadIdx.x & 31;
@@ -42,28 +81,28 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *total)
     return r;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t *in, size_t n,
-                                                              uint32_t *sums) {
-    size_t base = (size_t)blockIdx.x * kScanTile;
-    uint32_t acc = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        size_t i = base + (size_t)k * kScanThreads + threadIdx.x;
-        if (i < n) acc += in[i];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+// Sum of one value per thread, returned to every thread.
+__device__ __forceinline__ uint32_t block_sum(uint32_t v) {
     __shared__ uint32_t ws[kScanThreads / 32];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = 0;
-        for (int w = 0; w < kScanThreads / 32; ++w) t += ws[w];
-        sums[blockIdx.x] = t;
-    }
+    uint32_t t = 0;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w) t += ws[w];
+    return t;
 }
 
-// Scans nb block sums in place (exclusive) with one block; sums[nb] = total.
+__global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t *in, size_t n, uint32_t *sums) {
+    const Items r = load_items(in, (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems, n);
+    uint32_t acc = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) acc += r.v[k];
+    const uint32_t t = block_sum(acc);
+    if (threadIdx.x == 0) sums[blockIdx.x] = t;
+}
+
+// Scans nb block sums in place (exclusive) with one block.
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *sums, size_t nb) {
     __shared__ uint32_t carry;
     __shared__ uint32_t tot;
@@ -78,43 +117,64 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *sums, size
         if (threadIdx.x == 0) carry += tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0) sums[nb] = carry;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const uint32_t *in, uint32_t *out, size_t n,
-                                                              const uint32_t *sums) {
+// scanned: sums holds exclusive prefixes already; wide: out is 32-byte aligned
+// (a caller's own array need not be)
+__global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint32_t *in, uint32_t *out, size_t n,
+                                                              const uint32_t *sums, bool scanned, bool wide, ScanWith with) {
     __shared__ uint32_t tot;
-    size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
-    uint32_t v[kScanItems];
+    const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
+    Items r = load_items(in, base, n);
+    uint32_t before = 0;
+    if (!scanned)
+        for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) before += __ldg(sums + i);
     uint32_t acc = 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        size_t i = base + k;
-        v[k] = i < n ? in[i] : 0u;
-        acc += v[k];
-    }
-    uint32_t ex = block_excl_scan(acc, &tot) + sums[blockIdx.x];
+    for (int k = 0; k < kScanItems; ++k) acc += r.v[k];
+    const uint32_t prefix = scanned ? __ldg(sums + blockIdx.x) : block_sum(before);
+    uint32_t ex = block_excl_scan(acc, &tot) + prefix;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        size_t i = base + k;
-        if (i < n) out[i] = ex;
-        ex += v[k];
+        const uint32_t c = r.v[k];
+        r.v[k] = ex;
+        ex += c;
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = sums[gridDim.x];
+    store_items(out, base, n, r, wide);
+    if (with.cursor) store_items(with.cursor, base, n, r);
+    const Items zero{};
+    if (with.clear_in) store_items(in, base, n, zero);
+    if (with.fill) {
+        Items f;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) f.v[k] = with.fill_value;
+        store_items(with.fill, base, n, f);
+    }
+    if (threadIdx.x == 0) {
+        if (blockIdx.x == gridDim.x - 1) out[n] = prefix + tot;
+        if (blockIdx.x == 0) {
+            if (with.counter_from) {
+                *with.counter_to = *with.counter_from;
+                *with.counter_from = 0ull;
+            }
+            if (with.counter_zero) *with.counter_zero = 0ull;
+        }
+    }
 }
 
 }  // namespace
 
 size_t scan_tmp_elems(size_t n) { return (n + kScanTile - 1) / kScanTile + 2; }
 
-cudaError_t scan_exclusive(const uint32_t *in, uint32_t *out, size_t n, uint32_t *tmp, cudaStream_t s) {
+cudaError_t scan_exclusive(uint32_t *in, uint32_t *out, size_t n, uint32_t *tmp, cudaStream_t s, const ScanWith &with) {
     size_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb == 0) {
         return cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
     }
+    const bool scanned = nb > kDirectBlocks, wide = reinterpret_cast<uintptr_t>(out) % 32 == 0;
     k_block_sums<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, tmp);
-    k_scan_sums<<<1, kScanThreads, 0, s>>>(tmp, nb);
-    k_scan_tiles<<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, tmp);
+    if (scanned) k_scan_sums<<<1, kScanThreads, 0, s>>>(tmp, nb);
+    k_scan_tiles<<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, tmp, scanned, wide, with);
     return cudaGetLastError();
 }
 
