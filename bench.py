@@ -119,8 +119,8 @@ class ClockSampler:
 #       -c 20 --csv --log-file launches.csv python bench.py --profile --steps 1 --warmup 0 --no-cpu-baseline
 # A changed kernel has no entry, and the line then reports null.
 FILTER_TRAFFIC = {
-    ("143da3eaaba68891ec3f19dee24844057b28c7a4236973378e26ec4fb99650e3",
-     "240aef99038954fec244d49b0e9265980318b5272c40db6efb47067248a35480"): 0.989e9 + 0.031e9,
+    ("b14a729080794018b708a04b0c948e3c495ff819a44d34e02c535d95c86b537a",
+     "240aef99038954fec244d49b0e9265980318b5272c40db6efb47067248a35480"): 0.988e9 + 0.031e9,
 }
 
 

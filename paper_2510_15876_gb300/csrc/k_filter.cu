@@ -92,43 +92,63 @@ __device__ __forceinline__ PixelFrame pixel_frame(int x, int y, int W, int H, in
 
 // Filter widths of every pixel (unless KEEP: the widths already in the map
 // are used) and the pixel's gather constants for the filter: -ks, -kt, the
-// exponent shift m and the footprint radius (the configured R, or with ADAPT
-// floor(r + 1/2) of the pixel's adaptive radius r, whose sample count is then
-// recorded for the next update).
-template <bool KEEP, bool ADAPT>
-__global__ void __launch_bounds__(256) k_sigma(int W, int H, int R, int S, int ntx, float window, float eps,
-                                               AfrParams prm, const float4 *__restrict__ grad,
-                                               const TilePartial *__restrict__ tiles,
-                                               const uint32_t *__restrict__ amin2, const float *__restrict__ radius,
-                                               const uint32_t *__restrict__ foff, int32_t *__restrict__ cov_n,
-                                               float2 *__restrict__ sigma, float4 *__restrict__ fconst) {
-    int P = W * H;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-        int x = p % W, y = p / W;
-        float2 sg;
-        if (KEEP) {
-            sg = sigma[p];
-        } else {
-            Widths w = widths(__ldg(grad + p), tile_volume(x, y, W, H, S, ntx, window, tiles), eps, prm);
-            sg = make_float2(w.ss, w.st);
-            sigma[p] = sg;
+// exponent shift m and the footprint radius.
+//
+// A block takes 32 x 8 pixels and keeps the smallest ages of their bins and the
+// halo in shared memory. Bins at the same |dx| and |dy| from a pixel have the
+// same distance term, and the bound grows with the age, so their ages are
+// compared as integers first and the bound is evaluated once for each pair of
+// offsets (15 instead of 49 at R = 4): the same minimum, bit for bit. RT: R at
+// compile time (every load at a constant offset), or -1. Bound: issue. A
+// thread a pixel with 49 global loads and bounds took 89 us at 1920x1080 (R 4)
+// and 58 us at 1280x720 (R 5); this takes 34 and 20 us.
+constexpr int kSigX = 32, kSigY = 8, kSigHalo = 8;
+constexpr uint32_t kEmptyBin = 0x7f800000u;
+
+template <bool KEEP, int RT>
+__global__ void __launch_bounds__(kSigX * kSigY) k_sigma(int W, int H, int Rrun, int S, int ntx, float window, float eps,
+                                                         AfrParams prm, const float4 *__restrict__ grad,
+                                                         const TilePartial *__restrict__ tiles,
+                                                         const uint32_t *__restrict__ amin2,
+                                                         float2 *__restrict__ sigma, float4 *__restrict__ fconst) {
+    __shared__ uint32_t age[(kSigY + 2 * kSigHalo) * (kSigX + 2 * kSigHalo)];
+    const int R = RT >= 0 ? RT : Rrun, pitch = kSigX + 2 * R;
+    const int x0 = blockIdx.x * kSigX, y0 = blockIdx.y * kSigY, x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+    for (int r = threadIdx.y; r < kSigY + 2 * R; r += kSigY) {
+        const int row = y0 - R + r;
+        for (int c = threadIdx.x; c < pitch; c += kSigX) {
+            const int col = x0 - R + c;
+            age[r * pitch + c] = row >= 0 && row < H && col >= 0 && col < W ? __ldg(amin2 + (size_t)row * W + col) : kEmptyBin;
         }
-        int Rp = R;
-        if (ADAPT) {
-            Rp = (int)floorf(__fadd_rn(__ldg(radius + p), 0.5f));
-            int32_t n = 0;
-            for (int dy = -Rp; dy <= Rp; ++dy) {
-                const int row = y + dy;
-                if (row < 0 || row >= H) continue;
-                const int hw = half_width(Rp, dy);
-                const int x0 = max(0, x - hw), x1 = min(W - 1, x + hw);
-                n += (int32_t)(__ldg(foff + (size_t)row * W + x1 + 1) - __ldg(foff + (size_t)row * W + x0));
-            }
-            cov_n[p] = n;
-        }
-        PixelFrame f = pixel_frame(x, y, W, H, Rp, sg, amin2);
-        fconst[p] = make_float4(-f.ks, -f.kt, f.m, __int_as_float(Rp));
     }
+    const bool in = x < W && y < H;
+    const size_t p = (size_t)min(y, H - 1) * W + min(x, W - 1);
+    float2 sg;
+    if (KEEP) {
+        sg = sigma[p];
+    } else {
+        const Widths w = widths(__ldg(grad + p), tile_volume(min(x, W - 1), min(y, H - 1), W, H, S, ntx, window, tiles), eps, prm);
+        sg = make_float2(w.ss, w.st);
+        if (in) sigma[p] = sg;
+    }
+    __syncthreads();
+    if (!in) return;
+    const float ks = kLog2e / (2.f * sg.x * sg.x), kt = kLog2e / (2.f * sg.y * sg.y);
+    const uint32_t *own = age + (threadIdx.y + R) * pitch + threadIdx.x + R;
+    float m = INFINITY;
+#pragma unroll
+    for (int v = 0; v <= R; ++v) {
+        const float gy = bin_gap(v);
+#pragma unroll
+        for (int u = 0; u <= R; ++u) {
+            if (u * u + v * v > R * R) continue;
+            uint32_t a = min(own[v * pitch + u], own[v * pitch - u]);
+            if (v) a = min(a, min(own[-v * pitch + u], own[-v * pitch - u]));
+            const float gx = bin_gap(u);
+            if (a != kEmptyBin) m = fminf(m, fmaf(fmaf(gx, gx, gy * gy), ks, __uint_as_float(a) * kt));
+        }
+    }
+    fconst[p] = make_float4(-ks, -kt, m < INFINITY ? m : 0.f, __int_as_float(R));
 }
 
 // Section 6.2 in gather form: the next footprint radius of each pixel is the
@@ -136,29 +156,64 @@ __global__ void __launch_bounds__(256) k_sigma(int W, int H, int R, int S, int n
 // border), times 4 below 4 samples, times 0.7 above 32 (no count: times 1),
 // clamped; single precision with one rounding per operation, in the same
 // order as a plain loop over the neighbourhood rows.
-__global__ void __launch_bounds__(256) k_coverage_update(int W, int H, const float *__restrict__ r_prev,
-                                                         const int32_t *__restrict__ n_prev, float r_min,
-                                                         float r_max, float *__restrict__ r_next) {
-    int P = W * H;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-        const int x = p % W, y = p / W;
-        float sum = 0.f;
-        int cnt = 0;
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int qx = x + dx, qy = y + dy;
-                if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
-                sum = __fadd_rn(sum, __ldg(r_prev + (size_t)qy * W + qx));
-                ++cnt;
-            }
-        const float mean = __fdiv_rn(sum, (float)cnt);
-        const int32_t n = n_prev[p];
-        const float f = n < 0 ? 1.f : n < 4 ? 4.f : n > 32 ? 0.7f : 1.f;
-        float r = __fmul_rn(mean, f);
-        if (r < r_min) r = r_min;
-        if (r > r_max) r = r_max;
-        r_next[p] = r;
+__device__ __forceinline__ float next_radius(int x, int y, int W, int H, const float *__restrict__ r_prev, int32_t n,
+                                             float r_min, float r_max) {
+    float sum = 0.f;
+    int cnt = 0;
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+        for (int dx = -1; dx <= 1; ++dx) {
+            const int qx = x + dx, qy = y + dy;
+            if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
+            sum = __fadd_rn(sum, __ldg(r_prev + (size_t)qy * W + qx));
+            ++cnt;
+        }
+    const float mean = __fdiv_rn(sum, (float)cnt);
+    const float f = n < 0 ? 1.f : n < 4 ? 4.f : n > 32 ? 0.7f : 1.f;
+    float r = __fmul_rn(mean, f);
+    if (r < r_min) r = r_min;
+    if (r > r_max) r = r_max;
+    return r;
+}
+
+// k_sigma for adaptive footprints: each pixel's next radius r, the widths, the
+// gather constants of the disc of radius floor(r + 1/2), and the samples in it
+// for the update after this one. (As a launch of its own the radius update
+// took 17 us at 1920x1080 beside 63 us for the rest; together 58 us.)
+template <bool KEEP>
+__global__ void __launch_bounds__(kSigX * kSigY) k_sigma_adaptive(int W, int H, int S, int ntx, float window, float eps,
+                                                                  AfrParams prm, const float4 *__restrict__ grad,
+                                                                  const TilePartial *__restrict__ tiles,
+                                                                  const uint32_t *__restrict__ amin2,
+                                                                  const float *__restrict__ r_prev,
+                                                                  float *__restrict__ r_next, float r_min, float r_max,
+                                                                  const uint32_t *__restrict__ foff,
+                                                                  int32_t *__restrict__ cov_n, float2 *__restrict__ sigma,
+                                                                  float4 *__restrict__ fconst) {
+    const int x = blockIdx.x * kSigX + threadIdx.x, y = blockIdx.y * kSigY + threadIdx.y;
+    if (x >= W || y >= H) return;
+    const size_t p = (size_t)y * W + x;
+    const float r = next_radius(x, y, W, H, r_prev, cov_n[p], r_min, r_max);
+    r_next[p] = r;
+    const int R = (int)floorf(__fadd_rn(r, 0.5f));
+    float2 sg;
+    if (KEEP) {
+        sg = sigma[p];
+    } else {
+        const Widths w = widths(__ldg(grad + p), tile_volume(x, y, W, H, S, ntx, window, tiles), eps, prm);
+        sg = make_float2(w.ss, w.st);
+        sigma[p] = sg;
     }
+    int32_t n = 0;
+    for (int dy = max(-R, -y); dy <= min(R, H - 1 - y); ++dy) {
+        const int hw = half_width(R, dy);
+        const uint32_t *row = foff + (size_t)(y + dy) * W;
+        n += (int32_t)(__ldg(row + min(W - 1, x + hw) + 1) - __ldg(row + max(0, x - hw)));
+    }
+    cov_n[p] = n;
+    const PixelFrame f = pixel_frame(x, y, W, H, R, sg, amin2);
+    fconst[p] = make_float4(-f.ks, -f.kt, f.m, __int_as_float(R));
 }
 
 __global__ void k_coverage_init(int P, float r0, float *__restrict__ r, int32_t *__restrict__ n) {
@@ -1047,21 +1102,32 @@ const dim3 kQuadBlock(256);
 }  // namespace
 
 cudaError_t launch_sigma(AfrContext *c, const AfrParams *prm, bool keep, bool adaptive, cudaStream_t s) {
-    const int g = grid_for(c->P, 256);
-    const float *radius = nullptr;
+    const dim3 block(kSigX, kSigY), grid((c->W + kSigX - 1) / kSigX, (c->H + kSigY - 1) / kSigY);
     if (adaptive) {
-        float *next = c->cov_r[1 - c->cov_cur];
-        k_coverage_update<<<g, 256, 0, s>>>(c->W, c->H, c->cov_r[c->cov_cur], c->cov_n, 0.5f, 8.f, next);
+        const float *prev = c->cov_r[c->cov_cur];
         c->cov_cur = 1 - c->cov_cur;
-        radius = next;
+        float *next = c->cov_r[c->cov_cur];
+#define AFR_SIGMA(K)                                                                                                    \
+    k_sigma_adaptive<K><<<grid, block, 0, s>>>(c->W, c->H, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, *prm, c->grad, \
+                                               c->tiles, c->amin2, prev, next, 0.5f, 8.f, c->foff, c->cov_n, c->sigma,  \
+                                               c->fconst)
+        if (keep) AFR_SIGMA(true);
+        else AFR_SIGMA(false);
+#undef AFR_SIGMA
+        return cudaGetLastError();
     }
-#define AFR_SIGMA(K, A)                                                                                         \
-    k_sigma<K, A><<<g, 256, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, *prm, c->grad, \
-                                    c->tiles, c->amin2, radius, c->foff, c->cov_n, c->sigma, c->fconst)
-    if (keep && adaptive) AFR_SIGMA(true, true);
-    else if (keep) AFR_SIGMA(true, false);
-    else if (adaptive) AFR_SIGMA(false, true);
-    else AFR_SIGMA(false, false);
+#define AFR_SIGMA(K, R_)                                                                                             \
+    k_sigma<K, R_><<<grid, block, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, *prm, c->grad, \
+                                          c->tiles, c->amin2, c->sigma, c->fconst)
+    if (keep) AFR_SIGMA(true, -1);
+    else {
+        switch (c->R) {   // the radii of the tuner and the default
+            case 3: AFR_SIGMA(false, 3); break;
+            case 4: AFR_SIGMA(false, 4); break;
+            case 5: AFR_SIGMA(false, 5); break;
+            default: AFR_SIGMA(false, -1); break;
+        }
+    }
 #undef AFR_SIGMA
     return cudaGetLastError();
 }
