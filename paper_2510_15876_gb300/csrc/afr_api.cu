@@ -58,9 +58,9 @@ cudaError_t dalloc(T **p, size_t n) {
 }
 
 void free_all(AfrContext *c) {
-    void *ptrs[] = {c->r_xy, c->r_mo, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->bucket, c->fifo_flag, c->fifo_rank, c->fifo_scan,
+    void *ptrs[] = {c->r_xm, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->bucket, c->fifo_flag, c->fifo_rank, c->fifo_scan,
                     c->ccnt, c->coff, c->ccur, c->lbar, c->grad, c->pstat, c->sigma, c->fconst, c->cov_r[0], c->cov_r[1], c->cov_n, c->amin2, c->tiles, c->fcnt, c->fcur,
-                    c->foff, c->frec, c->sbin, c->flist, c->flseq, c->q_xy, c->q_mo, c->q_t, c->q_seq, c->q_col, c->q_total, c->q_world, c->r_world, c->scan_tmp, c->scan_tmp_in, c->bgrad, c->bparam, c->dcount, c->derr};
+                    c->foff, c->frec, c->sbin, c->flist, c->q_xm, c->q_t, c->q_seq, c->q_col, c->q_total, c->q_world, c->r_world, c->scan_tmp, c->scan_tmp_in, c->bgrad, c->bparam, c->dcount, c->derr};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -195,8 +195,7 @@ AfrStatus afr_create(const AfrConfig *cfg, AfrContext **out) {
     size_t P = c->P, N = c->nslots;
 #define AFR_ALLOC(ptr, n)                           \
     if (e == cudaSuccess) e = dalloc(&(ptr), (n));
-    AFR_ALLOC(c->r_xy, N);
-    AFR_ALLOC(c->r_mo, N);
+    AFR_ALLOC(c->r_xm, N);
     AFR_ALLOC(c->r_t, N);
     AFR_ALLOC(c->r_depth, N);
     AFR_ALLOC(c->r_seq, N);
@@ -223,8 +222,7 @@ AfrStatus afr_create(const AfrConfig *cfg, AfrContext **out) {
     if (c->fifo_n) {
         const size_t Q = c->fifo_n;
         if (g.world_points) AFR_ALLOC(c->q_world, Q);
-        AFR_ALLOC(c->q_xy, Q);
-        AFR_ALLOC(c->q_mo, Q);
+        AFR_ALLOC(c->q_xm, Q);
         AFR_ALLOC(c->q_t, Q);
         AFR_ALLOC(c->q_seq, Q);
         if (e == cudaSuccess) e = dmalloc(&c->q_col, Q * c->csize);
@@ -233,8 +231,7 @@ AfrStatus afr_create(const AfrConfig *cfg, AfrContext **out) {
     }
     AFR_ALLOC(c->frec, c->frame_cap + afr::kFramePad);
     AFR_ALLOC(c->sbin, c->frame_cap);
-    AFR_ALLOC(c->flist, c->frame_cap);
-    AFR_ALLOC(c->flseq, c->frame_cap);
+    AFR_ALLOC(c->flist, 2 * c->frame_cap + 4);
     AFR_ALLOC(c->scan_tmp, c->scan_tmp_n);
     AFR_ALLOC(c->scan_tmp_in, c->scan_tmp_n);
     AFR_ALLOC(c->bgrad, 2 * P);
@@ -559,14 +556,13 @@ AfrStatus afr_export_ring(AfrContext *c, int32_t *count_host, float *slot_host, 
     if (!c || !count_host || !slot_host || !seq_host) return AFR_ERR_INVALID_ARG;
     size_t P = c->P, N = c->nslots;
     std::vector<uint32_t> state(P), seq(N);
-    std::vector<float2> xy(N), mo(N);
+    std::vector<float4> xm(N);
     std::vector<float> t(N), depth(N);
     std::vector<unsigned char> col(N * c->csize);
     cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpy(state.data(), c->r_state, P * 4, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(seq.data(), c->r_seq, N * 4, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(xy.data(), c->r_xy, N * 8, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(mo.data(), c->r_mo, N * 8, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(xm.data(), c->r_xm, N * 16, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(t.data(), c->r_t, N * 4, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(depth.data(), c->r_depth, N * 4, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(col.data(), c->r_col, N * c->csize, cudaMemcpyDeviceToHost);
@@ -581,13 +577,13 @@ AfrStatus afr_export_ring(AfrContext *c, int32_t *count_host, float *slot_host, 
             if (s < 0) s += c->b;
             size_t i = p * c->b + s;
             float *o = slot_host + (p * c->b + k) * 9;
-            o[0] = xy[i].x;
-            o[1] = xy[i].y;
+            o[0] = xm[i].x;
+            o[1] = xm[i].y;
             o[2] = t[i];
             o[3] = depth[i];
             widen_colors(c->ct, col.data(), i, o + 4);
-            o[7] = mo[i].x;
-            o[8] = mo[i].y;
+            o[7] = xm[i].z;
+            o[8] = xm[i].w;
             seq_host[p * c->b + k] = seq[i];
         }
     }

@@ -106,8 +106,7 @@ struct AfrContext {
     int csize = 16;           // bytes per stored colour (16 for F32, 8 for 16-bit)
 
     // deep buffer, slot index p*b + s (storage order, circular per pixel)
-    float2 *r_xy = nullptr;
-    float2 *r_mo = nullptr;
+    float4 *r_xm = nullptr;       // x, y and screen motion
     float *r_t = nullptr;
     float *r_depth = nullptr;
     uint32_t *r_seq = nullptr;
@@ -117,7 +116,7 @@ struct AfrContext {
     // ingest scratch
     // reconstructor queue of section 5.2 (fifo_capacity > 0): slot k of N
     size_t fifo_n = 0;
-    float2 *q_xy = nullptr, *q_mo = nullptr;
+    float4 *q_xm = nullptr;
     float *q_t = nullptr;
     uint32_t *q_seq = nullptr;
     void *q_col = nullptr;
@@ -155,8 +154,8 @@ struct AfrContext {
     uint32_t *foff = nullptr;     // [P+1]
     afr::FrameRec *frec = nullptr;  // [frame_cap + kFramePad]
     uint32_t *sbin = nullptr;     // [frame_cap] each source slot's bin (reprojection scratch)
-    uint32_t *flist = nullptr;    // [frame_cap] each bin's source slots, unordered (reprojection scratch)
-    uint32_t *flseq = nullptr;    // [frame_cap] their sequence numbers
+    uint32_t *flist = nullptr;    // [2 frame_cap + 4] reprojection scratch, by bin, unordered: (source slot, sequence
+                                  // number) pairs for the queues, sequence numbers for the reconstructor queue
     size_t frame_cap = 0;
 
     // scan scratch

@@ -54,7 +54,7 @@ struct Bucket {
 
 // Destination planes of the queues (slot p * b + s).
 struct Queues {
-    float2 *xy, *mo;
+    float4 *xm;        // x, y, m_x, m_y
     float *t, *depth;
     uint32_t *seq;
     void *col;
@@ -215,18 +215,17 @@ __device__ __forceinline__ uint32_t pushed_state(uint32_t st, uint32_t m, uint32
 template <int CT>
 __device__ __forceinline__ void put_record(const uint4 &a, const uint4 &q1, const uint4 &q2, const uint4 &q3, size_t dst,
                                            uint32_t seq, const Queues &q) {
-    q.xy[dst] = make_float2(__uint_as_float(a.x), __uint_as_float(a.y));
     q.t[dst] = __uint_as_float(a.z);
     q.depth[dst] = __uint_as_float(q2.y);
     q.seq[dst] = seq;
     if (CT == AFR_F32) {
         reinterpret_cast<float4 *>(q.col)[dst] =
             make_float4(__uint_as_float(q1.x), __uint_as_float(q1.y), __uint_as_float(q1.z), 0.f);
-        q.mo[dst] = make_float2(__uint_as_float(q1.w), __uint_as_float(q2.x));
+        q.xm[dst] = make_float4(__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(q1.w), __uint_as_float(q2.x));
     } else {
         reinterpret_cast<ushort4 *>(q.col)[dst] =
             make_ushort4((unsigned short)(q1.x & 0xFFFFu), (unsigned short)(q1.x >> 16), (unsigned short)q1.y, 0);
-        q.mo[dst] = make_float2(__uint_as_float(q1.z), __uint_as_float(q1.w));
+        q.xm[dst] = make_float4(__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(q1.z), __uint_as_float(q1.w));
     }
     if (q.world)
         q.world[dst] = make_float4(__uint_as_float(q2.z), __uint_as_float(q2.w), __uint_as_float(q3.x), 0.f);
@@ -387,7 +386,7 @@ cudaError_t run(AfrContext *c, const float4 *pos, const void *col, const float2 
     // from here on the queues: wait until they are free. The cursors are spent:
     // they take the new queue states
     if (queues_free && (e = cudaStreamWaitEvent(s, queues_free, 0)) != cudaSuccess) return e;
-    Queues q{c->r_xy, c->r_mo, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->r_world, c->nslots};
+    Queues q{c->r_xm, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->r_world, c->nslots};
     k_pix_commit<CT><<<grid_for(n, kCommitTile), kCommitTile, 0, s>>>(c->coff, P, c->W, c->b, seq0, bk, q, reset,
                                                                       c->ccur, dc);
     k_pix_finish<CT><<<grid_for(P, 256), 256, 0, s>>>(c->coff, P, c->b, seq0, bk, q, reset, c->ccur, c->dcount,
@@ -409,8 +408,8 @@ __global__ void __launch_bounds__(256) k_fifo_append(const float4 *__restrict__ 
                                                      const float2 *__restrict__ mo, uint32_t n,
                                                      const uint32_t *__restrict__ flag,
                                                      const uint32_t *__restrict__ rank, uint32_t seq0, uint32_t N,
-                                                     const uint32_t *__restrict__ total, float2 *__restrict__ q_xy,
-                                                     float2 *__restrict__ q_mo, float *__restrict__ q_t,
+                                                     const uint32_t *__restrict__ total, float4 *__restrict__ q_xm,
+                                                     float *__restrict__ q_t,
                                                      uint32_t *__restrict__ q_seq, void *__restrict__ q_col,
                                                      const float4 *__restrict__ world, float4 *__restrict__ q_world) {
     using CS = ColorStore<CT>;
@@ -419,9 +418,9 @@ __global__ void __launch_bounds__(256) k_fifo_append(const float4 *__restrict__ 
         if (!flag[i] || (uint64_t)rank[i] + N < accepted) continue;
         const uint32_t k = (uint32_t)(((uint64_t)t0 + rank[i]) % N);
         const float4 p = __ldg(pos + i);
-        q_xy[k] = make_float2(p.x, p.y);
+        const float2 m = __ldg(mo + i);
+        q_xm[k] = make_float4(p.x, p.y, m.x, m.y);
         q_t[k] = p.z;
-        q_mo[k] = __ldg(mo + i);
         q_seq[k] = seq0 + i;
         reinterpret_cast<typename CS::T *>(q_col)[k] = CS::raw(col, i);
         if (q_world) {
@@ -443,7 +442,7 @@ cudaError_t run_fifo(AfrContext *c, const float4 *pos, const void *col, const fl
     cudaError_t e = scan_exclusive(c->fifo_flag, c->fifo_rank, n, c->fifo_scan, s);
     if (e != cudaSuccess) return e;
     k_fifo_append<CT><<<g, 256, 0, s>>>(pos, col, mo, n, c->fifo_flag, c->fifo_rank, seq0, (uint32_t)c->fifo_n,
-                                        c->q_total, c->q_xy, c->q_mo, c->q_t, c->q_seq, c->q_col, world,
+                                        c->q_total, c->q_xm, c->q_t, c->q_seq, c->q_col, world,
                                         c->q_world);
     k_fifo_advance<<<1, 1, 0, s>>>(c->fifo_flag, c->fifo_rank, n, c->q_total);
     return cudaGetLastError();

@@ -8,20 +8,29 @@
 //          lanes of a warp grouped by bin with one match instruction).
 //  scan:   bin offsets.
 //  list:   each moved sample (its bin kept by the count pass, 4 bytes a
-//          slot) writes its slot index and its sequence number into its bin's
-//          lists (unordered, 8 bytes a sample), at the ticket its bin's cursor
-//          returns (the cursors start at the bin offsets).
+//          slot) writes its slot index and its sequence number, 8 bytes, into its
+//          bin's list (unordered), at the ticket its bin's cursor returns (the
+//          scan starts the cursors at the bin offsets).
 //  place:  thread per frame record, in bin order: the slot of list entry e
 //          is moved again, its rank in the bin is the number of sequence
 //          numbers in the bin's list below its own (sequence numbers are
 //          unique), and it writes the 32-byte frame record (x', y', a^2, its bin's
 //          place, its colour in FP32, its sequence number) to the bin's offset +
-//          rank. The lanes of a warp
-//          mostly share a bin, so the rank scans are broadcast reads and the
-//          record writes cover whole sectors; the frame view, and every sum
-//          over it, is deterministic without a reorder pass over the records.
-//          Each bin's smallest a^2 (the filter's exponent shift) is the
-//          minimum over the bin's warp segments, one atomic each.
+//          rank. The lanes of a warp mostly share a bin, so the rank scans are
+//          broadcast reads and the record writes whole sectors; the frame view,
+//          and every sum over it, is deterministic without a reorder pass over
+//          the records. Each bin's smallest a^2 (the filter's exponent shift) is
+//          the minimum over the bin's warp segments, one atomic each. Samples of
+//          the reconstructor's queue, which lie in arrival order, are placed
+//          from that order instead (k_place_fifo).
+//
+// Bound: HBM (place), atomic latency (list). 1920x1080x16, FP32 colours: list
+// 191 -> 148 us with one 8-byte entry for two 4-byte ones, place 533 -> 504 us
+// with position and motion in one 16-byte field and 32-byte records; placing
+// from the queues' slot order (no slot in the list, coalesced reads, records
+// written out of order) measured 123 + 562 us, and 30 us more at 1024x1024x8.
+// For the reconstructor's queue that order wins: 1024x1024, 4 samples a pixel,
+// list and place 307 -> 191 us.
 #include "afr_internal.cuh"
 
 namespace afr {
@@ -33,11 +42,11 @@ struct Moved {
     float xp, yp, a2;
 };
 
-__device__ __forceinline__ Moved move_sample(float2 xy, float2 m, float t, float t_now, int W, int H) {
+__device__ __forceinline__ Moved move_sample(float4 xm, float t, float t_now, int W, int H) {
     Moved r;
     float a = __fsub_rn(t_now, t);
-    r.xp = __fadd_rn(xy.x, __fmul_rn(m.x, a));
-    r.yp = __fadd_rn(xy.y, __fmul_rn(m.y, a));
+    r.xp = __fadd_rn(xm.x, __fmul_rn(xm.z, a));
+    r.yp = __fadd_rn(xm.y, __fmul_rn(xm.w, a));
     r.a2 = __fmul_rn(a, a);
     r.ok = r.xp >= 0.f && r.xp < (float)W && r.yp >= 0.f && r.yp < (float)H;
     r.bin = r.ok ? (uint32_t)(int)floorf(r.yp) * (uint32_t)W + (uint32_t)(int)floorf(r.xp) : kInvalid;
@@ -54,15 +63,15 @@ __device__ __forceinline__ float cam_row(const Camera &c, int r, float4 w) {
     return __fadd_rn(v, c.m[4 * r + 3]);
 }
 
-__device__ __forceinline__ Moved move_camera(float4 w, float2 m, float t, float t_now, int W, int H,
+__device__ __forceinline__ Moved move_camera(float4 w, float4 xm, float t, float t_now, int W, int H,
                                              const Camera &cam) {
     Moved r;
     const float cx = cam_row(cam, 0, w), cy = cam_row(cam, 1, w), cw = cam_row(cam, 2, w);
     const float sx = __fmul_rn(__fadd_rn(__fmul_rn(__fdiv_rn(cx, cw), 0.5f), 0.5f), (float)W);
     const float sy = __fmul_rn(__fadd_rn(__fmul_rn(__fdiv_rn(cy, cw), 0.5f), 0.5f), (float)H);
     const float a = __fsub_rn(t_now, t);
-    r.xp = __fadd_rn(sx, __fmul_rn(m.x, a));
-    r.yp = __fadd_rn(sy, __fmul_rn(m.y, a));
+    r.xp = __fadd_rn(sx, __fmul_rn(xm.z, a));
+    r.yp = __fadd_rn(sy, __fmul_rn(xm.w, a));
     r.a2 = __fmul_rn(a, a);
     r.ok = cw > 0.f && r.xp >= 0.f && r.xp < (float)W && r.yp >= 0.f && r.yp < (float)H;
     r.bin = r.ok ? (uint32_t)(int)floorf(r.yp) * (uint32_t)W + (uint32_t)(int)floorf(r.xp) : kInvalid;
@@ -93,8 +102,7 @@ __device__ __forceinline__ bool slot_live(uint32_t st, int s, int b) {
 template <bool FIFO, bool CAM>
 __device__ __forceinline__ bool live_move(uint32_t i, uint32_t nlive, int b, int bshift, int W, int H, float t_now,
                                           const Camera &cam, const float4 *__restrict__ world,
-                                          const uint32_t *__restrict__ state, const float2 *__restrict__ r_xy,
-                                          const float2 *__restrict__ r_mo, const float *__restrict__ r_t, Moved &mv,
+                                          const uint32_t *__restrict__ state, const float4 *__restrict__ r_xm, const float *__restrict__ r_t, Moved &mv,
                                           bool &live) {
     uint32_t p = 0, st = 0;
     int s = 0;
@@ -106,14 +114,12 @@ __device__ __forceinline__ bool live_move(uint32_t i, uint32_t nlive, int b, int
         st = __ldg(state + p);
     }
     float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-    float2 xy = make_float2(0.f, 0.f);
     if (CAM) w = __ldg(world + i);
-    else xy = __ldg(r_xy + i);
-    const float2 m = __ldg(r_mo + i);
+    const float4 xm = __ldg(r_xm + i);
     const float t = __ldg(r_t + i);
     if (!FIFO && !slot_live(st, s, b)) return false;
     live = true;
-    mv = CAM ? move_camera(w, m, t, t_now, W, H, cam) : move_sample(xy, m, t, t_now, W, H);
+    mv = CAM ? move_camera(w, xm, t, t_now, W, H, cam) : move_sample(xm, t, t_now, W, H);
     return mv.ok;
 }
 
@@ -123,8 +129,7 @@ constexpr int kCountRows = 4;
 template <bool FIFO, bool CAM>
 __global__ void __launch_bounds__(256) k_count(uint32_t nslots, int b, int bshift, int W, int H, float t_now,
                                                Camera cam, const float4 *__restrict__ world,
-                                               const uint32_t *__restrict__ state, const float2 *__restrict__ r_xy,
-                                               const float2 *__restrict__ r_mo, const float *__restrict__ r_t,
+                                               const uint32_t *__restrict__ state, const float4 *__restrict__ r_xm, const float *__restrict__ r_t,
                                                uint32_t *__restrict__ fcnt, uint32_t *__restrict__ sbin,
                                                unsigned long long *__restrict__ dcount) {
     const uint32_t nlive = FIFO ? min(__ldg(state), nslots) : 0u;
@@ -140,7 +145,7 @@ __global__ void __launch_bounds__(256) k_count(uint32_t nslots, int b, int bshif
             mv[r].ok = false;
             live[r] = false;
             if (i < nslots)
-                live_move<FIFO, CAM>(i, nlive, b, bshift, W, H, t_now, cam, world, state, r_xy, r_mo, r_t, mv[r],
+                live_move<FIFO, CAM>(i, nlive, b, bshift, W, H, t_now, cam, world, state, r_xm, r_t, mv[r],
                                      live[r]);
         }
 #pragma unroll
@@ -161,9 +166,10 @@ __global__ void __launch_bounds__(256) k_count(uint32_t nslots, int b, int bshif
 // takes kListRows rows of 32 slots at a time and issues every row's ticket
 // atomic before it reads any back, so the atomics' latencies overlap.
 constexpr int kListRows = 8;
+template <bool SLOTS>
 __global__ void __launch_bounds__(256) k_list(uint32_t nslots, const uint32_t *__restrict__ sbin,
-                                              const uint32_t *__restrict__ r_seq, uint32_t *__restrict__ fcur, uint32_t *__restrict__ flist,
-                                              uint32_t *__restrict__ flseq, DebugCheck dc) {
+                                              const uint32_t *__restrict__ r_seq, uint32_t *__restrict__ fcur,
+                                              uint32_t *__restrict__ flist, DebugCheck dc) {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t i0 = warp * 32u * kListRows; i0 < nslots; i0 += nwarps * 32u * kListRows) {
@@ -193,28 +199,33 @@ __global__ void __launch_bounds__(256) k_list(uint32_t nslots, const uint32_t *_
             if (bin[r] == kInvalid) continue;
             const uint32_t at = f + __popc(peers[r] & ((1u << lane) - 1u));
             if (AFR_CHECK(at < dc.cap, dc.derr)) {
-                flist[at] = i;
-                flseq[at] = sq[r];
+                if (SLOTS) reinterpret_cast<uint2 *>(flist)[at] = make_uint2(i, sq[r]);
+                else flist[at] = sq[r];
             }
         }
     }
 }
 
-// fcur holds every bin's end here (the list's cursors); a bin above
-// kSortedBinMax records takes its ranks by counting it down (arrival order)
-// and is counted as unsorted.
+// A record's place in a bin above kSortedBinMax records: fcur holds the bin's
+// end (the list's cursor) and is counted down (arrival order); the bin is
+// counted as unsorted.
+__device__ __forceinline__ uint32_t unsorted_rank(uint32_t *fcur, uint32_t bin, uint32_t beg, unsigned long long *dcount) {
+    const uint32_t rank = atomicSub(fcur + bin, 1u) - 1u - beg;
+    if (rank == 0) atomicAdd(dcount + CNT_UNSORTED, 1ull);
+    return rank;
+}
+
 // The frame records arrive in bin order, so the lanes of a warp that share a
 // bin are one segment: its smallest a^2 goes to amin2 with one atomic (the
 // filter's exponent shift; bit order = value order for a^2 >= 0).
-template <int CT, bool FIFO, bool CAM>
-__global__ void __launch_bounds__(256) k_place(int W, int H, float t_now, Camera cam, const float4 *__restrict__ world,
-                                               const float2 *__restrict__ r_xy, const float2 *__restrict__ r_mo,
-                                               const float *__restrict__ r_t, const uint32_t *__restrict__ r_seq,
-                                               const void *__restrict__ r_col, uint32_t P,
-                                               const uint32_t *__restrict__ foff, const uint32_t *__restrict__ flist,
-                                               const uint32_t *__restrict__ flseq, uint32_t *__restrict__ fcur,
-                                               uint32_t *__restrict__ amin2, FrameRec *__restrict__ frec,
-                                               unsigned long long *__restrict__ dcount, DebugCheck dc, uint32_t nsrc) {
+template <int CT, bool CAM>
+__global__ void __launch_bounds__(256) k_place_queues(int W, int H, float t_now, Camera cam, const float4 *__restrict__ world,
+                                               const float4 *__restrict__ r_xm,
+                                               const float *__restrict__ r_t, const void *__restrict__ r_col, uint32_t P,
+                                               const uint32_t *__restrict__ foff, const uint2 *__restrict__ flist,
+                                               uint32_t *__restrict__ fcur, uint32_t *__restrict__ amin2,
+                                               FrameRec *__restrict__ frec, unsigned long long *__restrict__ dcount,
+                                               DebugCheck dc, uint32_t nsrc) {
     using CS = ColorStore<CT>;
     uint32_t n = __ldg(foff + P);
     if (!AFR_CHECK(n <= dc.cap, dc.derr)) n = 0;
@@ -223,35 +234,94 @@ __global__ void __launch_bounds__(256) k_place(int W, int H, float t_now, Camera
     // warp-uniform trip count: every lane of a warp reaches the match below
     for (uint32_t e0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); e0 < n; e0 += stride) {
         const uint32_t e = e0 + (uint32_t)lane;
-        uint32_t i = 0;
+        uint2 en = make_uint2(0u, 0u);   // slot, sequence number
         bool ok = e < n;
         if (ok) {
-            i = __ldg(flist + e);
-            ok = AFR_CHECK(i < nsrc, dc.derr);
+            en = __ldg(flist + e);
+            ok = AFR_CHECK(en.x < nsrc, dc.derr);
         }
+        const uint32_t i = en.x, sq = en.y;
         Moved mv;
         mv.ok = false;
         mv.bin = kInvalid;
-        if (ok)
-            mv = CAM ? move_camera(__ldg(world + i), __ldg(r_mo + i), __ldg(r_t + i), t_now, W, H, cam)
-                     : move_sample(__ldg(r_xy + i), __ldg(r_mo + i), __ldg(r_t + i), t_now, W, H);
+        typename CS::T col;
+        if (ok) {
+            col = CS::raw(r_col, i);
+            mv = CAM ? move_camera(__ldg(world + i), __ldg(r_xm + i), __ldg(r_t + i), t_now, W, H, cam)
+                     : move_sample(__ldg(r_xm + i), __ldg(r_t + i), t_now, W, H);
+        }
         const uint32_t key = mv.ok ? mv.bin : kInvalid;
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         if (!mv.ok) continue;
         const uint32_t bits = __reduce_min_sync(peers, __float_as_uint(mv.a2));
         if (lane == __ffs(peers) - 1) atomicMin(amin2 + mv.bin, bits);
-        const uint32_t sq = __ldg(flseq + e);
         const uint32_t beg = __ldg(foff + mv.bin), end = __ldg(foff + mv.bin + 1);
         uint32_t rank = 0;
         if (end - beg <= (uint32_t)kSortedBinMax) {
-            for (uint32_t k = beg; k < end; ++k) rank += __ldg(flseq + k) < sq;
+#pragma unroll 4
+            for (uint32_t k = beg; k < end; ++k) rank += __ldg(&flist[k].y) < sq;
         } else {
-            rank = atomicSub(fcur + mv.bin, 1u) - 1u - beg;   // the cursor ends at the bin's end
-            if (rank == 0) atomicAdd(dcount + CNT_UNSORTED, 1ull);
+            rank = unsorted_rank(fcur, mv.bin, beg, dcount);
         }
         const uint32_t d = beg + rank;
         if (!AFR_CHECK(d < n, dc.derr)) continue;
-        const float3 c = CS::load(r_col, i);
+        const float3 c = CS::widen(col);
+        store_rec(frec + d, {make_float4(mv.xp, mv.yp, mv.a2, bin_place(mv.xp, mv.yp)),
+                             make_float4(c.x, c.y, c.z, __uint_as_float(sq))});
+    }
+}
+
+// The reconstructor's queue holds samples in arrival order, anywhere in the
+// image: gathered in bin order, each field of a record cost a sector of its
+// own. So a thread takes a slot, in queue order, and writes its record (one
+// whole sector) where its rank among the bin's sequence numbers puts it, four
+// numbers a load.
+template <int CT, bool CAM>
+__global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int H, float t_now, Camera cam,
+                                                    const float4 *__restrict__ world, const uint32_t *__restrict__ state,
+                                                    const float4 *__restrict__ r_xm,
+                                                    const float *__restrict__ r_t, const uint32_t *__restrict__ r_seq,
+                                                    const void *__restrict__ r_col, const uint32_t *__restrict__ foff,
+                                                    const uint32_t *__restrict__ flist, uint32_t *__restrict__ fcur,
+                                                    uint32_t *__restrict__ amin2, FrameRec *__restrict__ frec,
+                                                    unsigned long long *__restrict__ dcount, DebugCheck dc) {
+    using CS = ColorStore<CT>;
+    const uint32_t nlive = min(__ldg(state), nslots);
+    const int lane = threadIdx.x & 31;
+    const uint32_t stride = gridDim.x * blockDim.x;
+    for (uint32_t i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < nlive; i0 += stride) {
+        const uint32_t i = i0 + (uint32_t)lane;
+        Moved mv;
+        bool live;
+        mv.ok = false;
+        typename CS::T col;
+        uint32_t sq = 0;
+        if (i < nlive) {
+            col = CS::raw(r_col, i);
+            sq = __ldg(r_seq + i);
+            live_move<true, CAM>(i, nlive, 1, 0, W, H, t_now, cam, world, state, r_xm, r_t, mv, live);
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, mv.ok ? mv.bin : kInvalid);
+        if (!mv.ok) continue;
+        const uint32_t beg = __ldg(foff + mv.bin), end = __ldg(foff + mv.bin + 1);
+        const uint32_t bits = __reduce_min_sync(peers, __float_as_uint(mv.a2));
+        if (lane == __ffs(peers) - 1) atomicMin(amin2 + mv.bin, bits);
+        if (!AFR_CHECK(beg < end && end <= dc.cap, dc.derr)) continue;
+        uint32_t rank = 0;
+        const uint32_t len = end - beg;
+        if (len <= (uint32_t)kSortedBinMax) {
+            for (uint32_t k = beg & ~3u; k < end; k += 4) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(flist + k));
+                const uint32_t j = k - beg;   // entries outside the bin wrap past its length or lie beyond it
+                rank += (uint32_t)((j < len) & (v.x < sq)) + (uint32_t)((j + 1u < len) & (v.y < sq)) +
+                        (uint32_t)((j + 2u < len) & (v.z < sq)) + (uint32_t)((j + 3u < len) & (v.w < sq));
+            }
+        } else {
+            rank = unsorted_rank(fcur, mv.bin, beg, dcount);
+        }
+        const uint32_t d = beg + rank;
+        if (!AFR_CHECK(d < end, dc.derr)) continue;
+        const float3 c = CS::widen(col);
         store_rec(frec + d, {make_float4(mv.xp, mv.yp, mv.a2, bin_place(mv.xp, mv.yp)),
                              make_float4(c.x, c.y, c.z, __uint_as_float(sq))});
     }
@@ -267,7 +337,7 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     const Camera cm = cam ? *camp : Camera{};
     const size_t nsrc = fifo ? c->fifo_n : c->nslots;
     const uint32_t *state = fifo ? c->q_total : c->r_state;
-    const float2 *xy = fifo ? c->q_xy : c->r_xy, *mo = fifo ? c->q_mo : c->r_mo;
+    const float4 *xm = fifo ? c->q_xm : c->r_xm;
     const float *tt = fifo ? c->q_t : c->r_t;
     const uint32_t *sq = fifo ? c->q_seq : c->r_seq;
     const void *col = fifo ? c->q_col : c->r_col;
@@ -277,7 +347,7 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     const int bshift = (c->b & (c->b - 1)) == 0 ? __builtin_ctz((unsigned)c->b) : -1;
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
 #define AFR_COUNT(F_, C_)                                                                                    \
-    k_count<F_, C_><<<g, 256, 0, s>>>(ns, c->b, bshift, c->W, c->H, t_now, cm, wp, state, xy, mo, tt, c->fcnt, \
+    k_count<F_, C_><<<g, 256, 0, s>>>(ns, c->b, bshift, c->W, c->H, t_now, cm, wp, state, xm, tt, c->fcnt, \
                                       c->sbin, c->dcount)
     if (fifo && cam) AFR_COUNT(true, true);
     else if (fifo) AFR_COUNT(true, false);
@@ -296,17 +366,21 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     with.counter_to = c->dcount + CNT_DROPPED;
     with.counter_zero = c->dcount + CNT_UNSORTED;
     if ((e = scan_exclusive(c->fcnt, c->foff, c->P, c->scan_tmp, s, with)) != cudaSuccess) return e;
-    k_list<<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, c->flseq, dc);
-#define AFR_PLACE(CT_, F_, C_)                                                                                     \
-    k_place<CT_, F_, C_><<<g, 256, 0, s>>>(c->W, c->H, t_now, cm, wp, xy, mo, tt, sq, col, (uint32_t)c->P, c->foff, \
-                                           c->flist, c->flseq, c->fcur, c->amin2, c->frec,       \
-                                           c->dcount, dc, ns)
-#define AFR_REPROJ(CT_)                                                                                        \
-    do {                                                                                                       \
-        if (fifo && cam) AFR_PLACE(CT_, true, true);                                                           \
-        else if (fifo) AFR_PLACE(CT_, true, false);                                                            \
-        else if (cam) AFR_PLACE(CT_, false, true);                                                             \
-        else AFR_PLACE(CT_, false, false);                                                                     \
+    if (fifo) k_list<false><<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, dc);
+    else k_list<true><<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, dc);
+#define AFR_QUEUES(CT_, C_)                                                                                         \
+    k_place_queues<CT_, C_><<<g, 256, 0, s>>>(c->W, c->H, t_now, cm, wp, xm, tt, col, (uint32_t)c->P, c->foff,    \
+                                              reinterpret_cast<const uint2 *>(c->flist), c->fcur, c->amin2, c->frec, \
+                                              c->dcount, dc, ns)
+#define AFR_FIFO(CT_, C_)                                                                                            \
+    k_place_fifo<CT_, C_><<<g, 256, 0, s>>>(ns, c->W, c->H, t_now, cm, wp, state, xm, tt, sq, col, c->foff, c->flist, \
+                                            c->fcur, c->amin2, c->frec, c->dcount, dc)
+#define AFR_REPROJ(CT_)                       \
+    do {                                      \
+        if (fifo && cam) AFR_FIFO(CT_, true); \
+        else if (fifo) AFR_FIFO(CT_, false);  \
+        else if (cam) AFR_QUEUES(CT_, true);  \
+        else AFR_QUEUES(CT_, false);          \
     } while (0)
     switch (c->ct) {
         case AFR_F32: AFR_REPROJ(AFR_F32); break;
@@ -314,7 +388,8 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
         default: AFR_REPROJ(AFR_BF16); break;
     }
 #undef AFR_REPROJ
-#undef AFR_PLACE
+#undef AFR_QUEUES
+#undef AFR_FIFO
     return cudaGetLastError();
 }
 
