@@ -245,8 +245,11 @@ __global__ void k_coverage_init(int P, float r0, float *__restrict__ r, int32_t 
 // slots, 66% of the L1 data pipe, 1588 warp instructions a block of which 31
 // iterations take 44 each; 24 of the 44 are arithmetic). Records and row
 // offsets in one place each, the shared disc table and the prefetch took the
-// launch at 1920x1080x16 from 1600 to 1115 us (FP32 colours), 1280x720x8 with
-// R = 5 from 607 to 409 us and 640x480x8 in FP16 from 185 to 128 us. The shift
+// launch at 1920x1080x16 from 1600 to 1130 us (FP32 colours), 1280x720x8 with
+// R = 5 from 607 to 407 us and 640x480x8 in FP16 from 185 to 122 us. Adaptive
+// footprints, 1920x1080x16 with most radii at 1: 720 us with a table per block,
+// 617 us keeping a warp's table while the radius stays, 562 us with shared
+// tables of the small radii (the per-warp ones took 41 KB a CTA from L1). The shift
 // table per block (disc + shift, no addition per record) measured 1655 us, its
 // shared memory taken from L1; four CTAs a SM (64 registers, spills) 1183 us;
 // a prefetch two records deep 1413 us (spills); CTAs of 12 or 24 warps
@@ -382,11 +385,12 @@ struct ForwardSums {
 
 // Discs of the union box of a 2x2 block at footprint radius R: entry
 // (v, u) = bin row by - R + v, column bx - R + u.
-struct DiscTable {
-    float4 in[kMaxRows * kPitch];
-};
+constexpr int kTables = 4;   // adaptive footprints: radii 1 .. kTables have a table each
+constexpr int kTableRows = kTables * (kTables + 3);
+__host__ __device__ constexpr int table_row(int R) { return (R - 1) * (R + 2); }   // rows of the tables before R's
+static_assert(table_row(kTables + 1) == kTableRows, "2R + 2 rows each");
 
-__device__ __forceinline__ void fill_discs(DiscTable &t, int R) {
+__device__ __forceinline__ void fill_discs(float4 *in, int R) {
     for (int i = threadIdx.x; i < (2 * R + 2) * kPitch; i += blockDim.x) {
         const int v = i / kPitch - R, u = i % kPitch - R;
         float s[4];
@@ -395,8 +399,21 @@ __device__ __forceinline__ void fill_discs(DiscTable &t, int R) {
             const int du = u - (k & 1), dv = v - (k >> 1);
             s[k] = du * du + dv * dv <= R * R ? 0.f : -INFINITY;
         }
-        t.in[i] = make_float4(s[0], s[1], s[2], s[3]);
+        in[i] = make_float4(s[0], s[1], s[2], s[3]);
     }
+}
+
+// The same for pixels whose radii differ (or have no table), for the bin at
+// place t of the box of radius R.
+__device__ __forceinline__ float4 own_discs(int t, int R, const int (&Rk)[4]) {
+    const int v = t * 57 >> 10, u = t - v * kPitch;   // t / 18 for t < 18 * 18
+    float s[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int du = u - R - (k & 1), dv = v - R - (k >> 1);
+        s[k] = du * du + dv * dv <= Rk[k] * Rk[k] ? 0.f : -INFINITY;
+    }
+    return make_float4(s[0], s[1], s[2], s[3]);
 }
 
 // A value in a register that the assembler cannot compute again from
@@ -485,6 +502,17 @@ __device__ __forceinline__ void load_offsets(TileSmem &t, int W, int H, int R, i
     }
 }
 
+// Asks L2 for the tile's records (rows x cols of offsets) while the first
+// blocks set up: they come from HBM, and a block's few iterations hide little of
+// that (1.5% at R 4, 5% for adaptive footprints).
+__device__ __forceinline__ void prefetch_tile(const TileSmem &t, int cols, int rows, const FrameRec *frec) {
+    for (int r = threadIdx.x >> 5; r < rows; r += blockDim.x >> 5) {
+        const uint32_t end = t.off[r * cols + cols - 1];
+        for (uint32_t i = t.off[r * cols] + 4u * (threadIdx.x & 31); i < end; i += 128u)   // 128-byte lines
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(frec + i));
+    }
+}
+
 // Pixels past the right or bottom edge repeat the edge pixel (never stored).
 __device__ __forceinline__ float4 load_const(int i, int W, int H, int x0, int y0, int tw,
                                              const float4 *__restrict__ fconst) {
@@ -494,13 +522,14 @@ __device__ __forceinline__ float4 load_const(int i, int W, int H, int x0, int y0
 // Sums of one 2x2 pixel block by one warp: the block (lx, ly) of the tile at
 // (x0, y0), tw pixels wide, whose offsets were loaded for footprints up to Rt.
 // VAR: each pixel's footprint radius is read from its gather constants
-// (adaptive footprints); otherwise every pixel uses Rt. table: the warp's own
-// discs (VAR; held says for which radius it was filled last) or the CTA's, at
-// shared address table_at. frec: the frame view from this lane's record on.
+// (adaptive footprints; most neighbouring ones have settled at one radius);
+// otherwise every pixel uses Rt. tables_at: shared address of the disc tables
+// (VAR: of radii 1 .. kTables; else of Rt alone). frec: the frame view from this
+// lane's record on.
 template <bool VAR, class Sums>
 __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int lx, int ly, const FrameRec *frec,
-                                             const TileSmem &ts, DiscTable *table, uint32_t table_at, int &held,
-                                             uint2 *rows, uint32_t rows_at, const DebugCheck &dc, Sums &A) {
+                                             const TileSmem &ts, uint32_t tables_at, uint2 *rows, uint32_t rows_at,
+                                             const DebugCheck &dc, Sums &A) {
     const int lane = threadIdx.x & 31;
     const int bx = x0 + 2 * lx, by = y0 + 2 * ly;
     float4 fc[4];
@@ -508,11 +537,10 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
     for (int k = 0; k < 4; ++k) fc[k] = ts.fc[(2 * ly + (k >> 1)) * tw + 2 * lx + (k & 1)];
     int R = Rt;
     bool same = true;
+    const int Rk[4] = {__float_as_int(fc[0].w), __float_as_int(fc[1].w), __float_as_int(fc[2].w), __float_as_int(fc[3].w)};
     if (VAR) {
-        const int R0 = __float_as_int(fc[0].w), R1 = __float_as_int(fc[1].w), R2 = __float_as_int(fc[2].w),
-                  R3 = __float_as_int(fc[3].w);
-        R = max(max(R0, R1), max(R2, R3));   // the block's largest footprint
-        same = min(min(R0, R1), min(R2, R3)) == R;
+        R = max(max(Rk[0], Rk[1]), max(Rk[2], Rk[3]));   // the block's largest footprint
+        same = min(min(Rk[0], Rk[1]), min(Rk[2], Rk[3])) == R;
     }
     // union rows: lane v (< 2R + 2) takes bin row by - R + v; the union of the
     // four discs' rows is one run of columns [bx - lo, bx + 1 + hi]
@@ -526,9 +554,9 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
             lo = hi = -2;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int dv = v - (k >> 1), Rk = __float_as_int(fc[k].w);
-                if (dv >= -Rk && dv <= Rk) {
-                    const int h = half_width(Rk, dv);
+                const int dv = v - (k >> 1);
+                if (dv >= -Rk[k] && dv <= Rk[k]) {
+                    const int h = half_width(Rk[k], dv);
                     lo = max(lo, h - (k & 1));
                     hi = max(hi, h + (k & 1) - 1);
                 }
@@ -547,19 +575,6 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
     if (lane < 2 * R + 2) rows[lane] = make_uint2(lane == 2 * R + 1 ? 0x7fffffffu : incl, first - (incl - cnt));
     // rows of 32 records or more between the first and the last: an iteration moves a lane at most one row on
     const bool one = __all_sync(0xffffffffu, cnt >= 32u || lane == 0 || lane >= 2 * R + 1);
-    if (VAR && (!same || held != R)) {   // most neighbouring footprints have settled at one radius
-        for (int t = lane; t < (2 * R + 2) * kPitch; t += 32) {
-            const int v = t / kPitch - R, u = t % kPitch - R;
-            float s[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int du = u - (k & 1), dv = v - (k >> 1), Rk = __float_as_int(fc[k].w);
-                s[k] = du * du + dv * dv <= Rk * Rk ? 0.f : -INFINITY;
-            }
-            table->in[t] = make_float4(s[0], s[1], s[2], s[3]);
-        }
-        held = same ? R : -1;
-    }
     __syncwarp();
     PairConsts pc;
     pc.cx = pk((float)bx + 0.5f, (float)bx + 1.5f);
@@ -572,6 +587,8 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
         pc.m[j] = pk(fc[2 * j].z, fc[2 * j + 1].z);
     }
     const int origin = (by - R) * kPitch + bx - R;
+    const bool table = !VAR || (same && R >= 1 && R <= kTables);
+    const uint32_t table_at = tables_at + (VAR && table ? table_row(R) * kPitch * 16u : 0u);
     const uint32_t tab = keep(table_at - (uint32_t)origin * 16u);   // + 16 place: the entry of a record's bin
     auto load = [&](int i) {   // record i + lane (i itself may be negative)
         const bool ok = AFR_CHECK((uint32_t)(i + lane) < dc.cap + kFramePad, dc.derr);
@@ -579,16 +596,18 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
         if (!ok) r.p.w = __int_as_float(-1 - origin);
         return r;
     };
-    auto add = [&](const FrameRec &r) {
+    auto add = [&](const FrameRec &r, auto from_table) {
         const int place = __float_as_int(r.p.w);
         const bool ok = AFR_CHECK(place >= origin && place < origin + (2 * R + 2) * kPitch, dc.derr);
-        float4 d = lds4(ok ? tab + (uint32_t)place * 16u : table_at);
+        float4 d;
+        if constexpr (decltype(from_table)::value) d = lds4(ok ? tab + (uint32_t)place * 16u : table_at);
+        else d = own_discs(place - origin, R, Rk);
         if (!ok) d = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         A.add(pc, d, r);
     };
     // The last iteration's lanes past the end read on (the frame arrays end in
     // kFramePad records of padding) and are dropped before they are summed.
-    auto gather = [&](auto one_row) {
+    auto gather = [&](auto one_row, auto from_table) {
         constexpr bool ONE = decltype(one_row)::value;
         const uint2 r0 = lds2(rows_at);
         Cursor k{rows_at, (int)r0.x - lane, (int)r0.y};
@@ -599,23 +618,28 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
         for (; j + 32 < (int)total; j += 64) {
             advance<ONE>(k, j, lane);
             rb = load(j + k.base);
-            add(ra);
+            add(ra, from_table);
             advance<ONE>(k, j + 32, lane);
             ra = load(j + 32 + k.base);
-            add(rb);
+            add(rb, from_table);
         }
         if (j < (int)total) {
             advance<ONE>(k, j, lane);
             rb = load(j + k.base);
-            add(ra);
+            add(ra, from_table);
             ra = rb;
             j += 32;
         }
-        if (j - 32 + lane < (int)total) add(ra);
+        if (j - 32 + lane < (int)total) add(ra, from_table);
     };
     if (total) {
-        if (one) gather(std::true_type{});
-        else gather(std::false_type{});
+        if (!table) {
+            if constexpr (VAR) gather(std::false_type{}, std::false_type{});
+        } else if (one) {
+            gather(std::true_type{}, std::true_type{});
+        } else {
+            gather(std::false_type{}, std::true_type{});
+        }
     }
     __syncwarp();   // the next block overwrites the row table
 }
@@ -654,37 +678,41 @@ __device__ __forceinline__ void store_block(const ForwardSums<KAHAN> &A, int W, 
 }
 
 // Tile of (2 * tbx) x (2 * 32 / tbx) pixels per CTA: 32 blocks of 2x2, four
-// per warp.
+// per warp; its upper 1 / 2^lsplit for images whose tiles would not fill the GPU.
 template <bool KAHAN, bool VAR>
-__global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx, const float4 *__restrict__ fconst,
+__global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx, int lsplit, const float4 *__restrict__ fconst,
                                                    const uint32_t *__restrict__ foff, const FrameRec *frec,
                                                    float4 *__restrict__ out, DebugCheck dc) {
     __shared__ TileSmem ts;
-    __shared__ DiscTable discs[VAR ? kWarps : 1];
-    const int warp = threadIdx.x >> 5, tw = 2 << ltbx, th = 64 >> ltbx;
+    __shared__ float4 discs[(VAR ? kTableRows : kMaxRows) * kPitch];
+    const int warp = threadIdx.x >> 5, tw = 2 << ltbx, th = 64 >> ltbx >> lsplit, pixels = tw * th;
     const int x0 = blockIdx.x * tw, y0 = blockIdx.y * th;
+    const FrameRec *const frec0 = frec;
     frec = keep(frec + (threadIdx.x & 31));
-    const uint32_t table_at = smem_at(discs[VAR ? warp : 0].in), rows_at = smem_at(ts.rows[warp]);
-    int Rt = R, held = -1;
+    const uint32_t tables_at = smem_at(discs), rows_at = smem_at(ts.rows[warp]);
+    int Rt = R;
     float4 fc = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (threadIdx.x < kTilePixels) {
+    if (threadIdx.x < pixels) {
         fc = load_const(threadIdx.x, W, H, x0, y0, tw, fconst);
         ts.fc[threadIdx.x] = fc;
     }
     if (VAR) {   // the tile's largest footprint
         Rt = 0;
-        for (int r = 1; r <= 8 && __syncthreads_or(__float_as_int(fc.w) >= r && threadIdx.x < kTilePixels); ++r) Rt = r;
+        for (int r = 1; r <= 8 && __syncthreads_or(__float_as_int(fc.w) >= r && threadIdx.x < pixels); ++r) {
+            Rt = r;
+            if (r <= kTables) fill_discs(discs + table_row(r) * kPitch, r);
+        }
     } else {
-        fill_discs(discs[0], R);
+        fill_discs(discs, R);
     }
     load_offsets(ts, W, H, Rt, x0, y0, tw, th, foff);
     __syncthreads();
-    for (int blk = warp; blk < 32; blk += kWarps) {
+    prefetch_tile(ts, tw + 2 * Rt + 1, th + 2 * Rt, frec0);
+    for (int blk = warp; blk < 32 >> lsplit; blk += kWarps) {
         const int lx = blk & ((1 << ltbx) - 1), ly = blk >> ltbx;
         if (x0 + 2 * lx >= W || y0 + 2 * ly >= H) continue;   // warp-uniform
         ForwardSums<KAHAN> A;
-        gather_block<VAR>(Rt, x0, y0, tw, lx, ly, frec, ts, discs + (VAR ? warp : 0), table_at, held, ts.rows[warp],
-                          rows_at, dc, A);
+        gather_block<VAR>(Rt, x0, y0, tw, lx, ly, frec, ts, tables_at, ts.rows[warp], rows_at, dc, A);
         store_block(A, W, H, x0 + 2 * lx, y0 + 2 * ly, ts.fc[block_pixel(tw, lx, ly)], out);
     }
 }
@@ -739,9 +767,9 @@ template <bool KAHAN>
 __global__ void __launch_bounds__(256, 3) k_batch(const BatchCtx *__restrict__ cs, int nctx, uint32_t total,
                                                   uint32_t *queue) {
     __shared__ TileSmem ts;
-    __shared__ DiscTable discs;                 // of the current tile's footprint radius
+    __shared__ float4 discs[kMaxRows * kPitch];   // of the current tile's footprint radius
     __shared__ uint32_t item_buf[2];            // current and next claimed tile
-    const uint32_t table_at = smem_at(discs.in), rows_at = smem_at(ts.rows[threadIdx.x >> 5]);
+    const uint32_t tables_at = smem_at(discs), rows_at = smem_at(ts.rows[threadIdx.x >> 5]);
     int held = -1;
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) item_buf[0] = atomicAdd(queue, 1u);
@@ -771,7 +799,7 @@ __global__ void __launch_bounds__(256, 3) k_batch(const BatchCtx *__restrict__ c
             const int lx = blk % tbx, ly = blk / tbx;
             if (x0 + 2 * lx >= x.W || y0 + 2 * ly >= x.H) continue;
             ForwardSums<KAHAN> A;
-            gather_block<false>(x.R, x0, y0, tw, lx, ly, frec, ts, &discs, table_at, held, ts.rows[warp], rows_at,
+            gather_block<false>(x.R, x0, y0, tw, lx, ly, frec, ts, tables_at, ts.rows[warp], rows_at,
                                 DebugCheck{x.fcap, x.derr}, A);
             store_block(A, x.W, x.H, x0 + 2 * lx, y0 + 2 * ly, ts.fc[block_pixel(tw, lx, ly)], x.out);
         }
@@ -851,7 +879,7 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 5) k_bwd_pixel(
     const uint32_t *__restrict__ foff, const FrameRec *frec, const float4 *__restrict__ gout,
     Adjoint adj, float *__restrict__ bparam, DebugCheck dc) {
     __shared__ TileSmem ts;
-    __shared__ DiscTable discs;
+    __shared__ float4 discs[kMaxRows * kPitch];
     __shared__ float4 go[kTilePixels];
     __shared__ float part[kBwdWarps][6];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -859,21 +887,20 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 5) k_bwd_pixel(
     static_assert(tw * th == kTilePixels && kTilePixels == 32 * kBwdWarps, "a thread per pixel");
     const int x0 = blockIdx.x * tw, y0 = blockIdx.y * th;
     frec = keep(frec + lane);
-    const uint32_t table_at = smem_at(discs.in), rows_at = smem_at(ts.rows[warp]);
+    const uint32_t tables_at = smem_at(discs), rows_at = smem_at(ts.rows[warp]);
     ts.fc[threadIdx.x] = load_const(threadIdx.x, W, H, x0, y0, tw, fconst);
     go[threadIdx.x] = load_const(threadIdx.x, W, H, x0, y0, tw, gout);
     fill_discs(discs, R);
     load_offsets(ts, W, H, R, x0, y0, tw, th, foff);
     __syncthreads();
     float gp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int held = R;
     for (int blk = warp; blk < 32; blk += kBwdWarps) {
         const int lx = blk % kBwdTbx, ly = blk / kBwdTbx;
         if (x0 + 2 * lx >= W || y0 + 2 * ly >= H) continue;   // warp-uniform
         const int i0 = 2 * ly * tw + 2 * lx;
         const float4 g4[4] = {go[i0], go[i0 + 1], go[i0 + tw], go[i0 + tw + 1]};
         typename std::conditional<PARAMS, AdjointSums, WeightSums>::type A(g4);
-        gather_block<false>(R, x0, y0, tw, lx, ly, frec, ts, &discs, table_at, held, ts.rows[warp], rows_at, dc, A);
+        gather_block<false>(R, x0, y0, tw, lx, ly, frec, ts, tables_at, ts.rows[warp], rows_at, dc, A);
         float S, q[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // of pixel k at lane k: S; w q, w d^2, w d^2 q, w a^2, w a^2 q
         if constexpr (PARAMS) {
             float v[16], u[8];
@@ -1140,10 +1167,20 @@ cudaError_t launch_coverage_init(AfrContext *c, cudaStream_t s) {
 cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out, cudaStream_t s) {
     (void)t_now;
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
-    const int tbx = c->tile_bx, tw = 2 * tbx, th = 2 * (32 / tbx);
+    const int tbx = c->tile_bx, tw = 2 * tbx;
+    // Fewer blocks a warp until the CTAs fill the GPU (three a SM) twice over:
+    // 128x128x4 13.8 us with four blocks a warp, 10.4 with one; split further,
+    // the tile's set-up costs more than the fuller last wave gives (640x480x8
+    // FP16 122 us whole, 126 halved, 140 quartered).
+    int lsplit = 0, th = 64 / tbx;
+    const long long want = 2ll * 3 * device_sms();
+    while (lsplit < 2 && th > 2 && (long long)((c->W + tw - 1) / tw) * ((c->H + th - 1) / th) < want) {
+        ++lsplit;
+        th /= 2;
+    }
     dim3 grid((c->W + tw - 1) / tw, (c->H + th - 1) / th);
 #define AFR_FILTER(K_, V_) \
-    k_filter<K_, V_><<<grid, kQuadBlock, 0, s>>>(c->W, c->H, c->R, __builtin_ctz(tbx), c->fconst, c->foff, c->frec, out, dc)
+    k_filter<K_, V_><<<grid, kQuadBlock, 0, s>>>(c->W, c->H, c->R, __builtin_ctz(tbx), lsplit, c->fconst, c->foff, c->frec, out, dc)
     // colours stored in 16 bits: compensated weight sums
     if (c->ct == AFR_F32 && adaptive) AFR_FILTER(false, true);
     else if (c->ct == AFR_F32) AFR_FILTER(false, false);
