@@ -119,7 +119,7 @@ class ClockSampler:
 #       -c 20 --csv --log-file launches.csv python bench.py --profile --steps 1 --warmup 0 --no-cpu-baseline
 # A changed kernel has no entry, and the line then reports null.
 FILTER_TRAFFIC = {
-    ("a214abcfe7df41fdb0f22c804c12a96c2855a337aa0f42f62874059497c77067",
+    ("2735711a19007b1986b05e6fddff655964aed5912e7fc8bea00e12eefa311f7a",
      "be0f05d40096614b19a03e112ad79868d7c1cc4052db9843a7a222a704590814"): 0.989e9 + 0.031e9,
 }
 

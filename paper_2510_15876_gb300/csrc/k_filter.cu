@@ -484,7 +484,7 @@ struct TileSmem {
     float4 fc[kTilePixels];
     uint32_t off[kTileOffsets];
     uint2 rows[kWarps][kMaxRows];
-};   // adjoint kernels run kBwdWarps <= kWarps warps a CTA
+};
 
 // Offsets of the bins of rows y0 - R .. y0 + th + R - 1 at columns x0 - R ..
 // x0 + tw + R (clamped to the row's first and last; rows outside the image
@@ -818,153 +818,130 @@ struct Adjoint {
     float2 *g;
 };
 
-// With q = g . c (g the loss gradient of the pixel's colour C), the width
-// gradients need, summed over the records: w, w q, w d^2, w d^2 q, w a^2 and
-// w a^2 q: dL/dsigma_s = (sum w d^2 q - (g . C) sum w d^2) / S / sigma_s^3, and
-// the same with a^2 for sigma_t.
-struct AdjointSums {
-    f2 S[2], Q[2], Ds[2], Dsq[2], Dt[2], Dtq[2];
-    f2 g[2][3];
-    __device__ __forceinline__ AdjointSums(const float4 (&go)[4]) {
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            S[j] = Q[j] = Ds[j] = Dsq[j] = Dt[j] = Dtq[j] = 0ull;
-            g[j][0] = pk(go[2 * j].x, go[2 * j + 1].x);
-            g[j][1] = pk(go[2 * j].y, go[2 * j + 1].y);
-            g[j][2] = pk(go[2 * j].z, go[2 * j + 1].z);
-        }
-    }
-    __device__ __forceinline__ void add(const PairConsts &pc, float4 in, const FrameRec &r) {
-        const PairWeights p = pair_weights(pc, in, r);
-        const f2 cr = pk(r.c.x, r.c.x), cg = pk(r.c.y, r.c.y), cb = pk(r.c.z, r.c.z);
-        const float fa = fminf(r.p.z, 3.4e38f);   // an age beyond FP32 weighs 0: 0, not NaN, to every sum
-        const f2 a2 = pk(fa, fa);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const f2 w = p.w[j], q = fma2(g[j][2], cb, fma2(g[j][1], cg, mul2(g[j][0], cr)));
-            const f2 ws = mul2(w, p.d2[j]), wt = mul2(w, a2);
-            S[j] = add2(S[j], w);
-            Q[j] = fma2(w, q, Q[j]);
-            Ds[j] = add2(Ds[j], ws);
-            Dsq[j] = fma2(ws, q, Dsq[j]);
-            Dt[j] = add2(Dt[j], wt);
-            Dtq[j] = fma2(wt, q, Dtq[j]);
+// Weighted sums of one pixel over the records of its disc, in frame order. The
+// totals of the width gradients over an image cancel to a small part of their
+// terms, so the terms' rounding shows in them: the order of every sum, here and
+// over the image (32 x 4 pixels a partial), is fixed, whatever a thread or a
+// CTA holds.
+template <bool PARAMS>
+struct PixelSums {
+    float S = 0.f, sc[3] = {0.f, 0.f, 0.f}, Ds = 0.f, dsc[3] = {0.f, 0.f, 0.f}, Dt = 0.f, dtc[3] = {0.f, 0.f, 0.f};
+    // fc: (-ks, -kt, shift); a record outside the disc adds exact zeros
+    __device__ __forceinline__ void add(float4 r, float4 c, float cx, float cy, float4 fc, bool in) {
+        const float ddx = r.x - cx, ddy = r.y - cy;
+        const float d2 = fmaf(ddx, ddx, ddy * ddy);
+        const float e2 = ex2(fmaf(d2, fc.x, fmaf(r.z, fc.y, fc.z))), w = in ? e2 : 0.f;
+        S += w;
+        if (PARAMS) {
+            const float ws = w * d2, wt = in ? w * r.z : 0.f;
+            sc[0] = fmaf(w, c.x, sc[0]); sc[1] = fmaf(w, c.y, sc[1]); sc[2] = fmaf(w, c.z, sc[2]);
+            Ds += ws; Dt += wt;
+            dsc[0] = fmaf(ws, c.x, dsc[0]); dsc[1] = fmaf(ws, c.y, dsc[1]); dsc[2] = fmaf(ws, c.z, dsc[2]);
+            dtc[0] = fmaf(wt, c.x, dtc[0]); dtc[1] = fmaf(wt, c.y, dtc[1]); dtc[2] = fmaf(wt, c.z, dtc[2]);
         }
     }
 };
 
-// Weight sums alone (no parameter gradients asked for).
-struct WeightSums {
-    f2 S[2];
-    __device__ __forceinline__ WeightSums(const float4 (&)[4]) { S[0] = S[1] = 0ull; }
-    __device__ __forceinline__ void add(const PairConsts &pc, float4 in, const FrameRec &r) {
-        const PairWeights p = pair_weights(pc, in, r);
-        S[0] = add2(S[0], p.w[0]);
-        S[1] = add2(S[1], p.w[1]);
-    }
-};
-
-// The pixel pass is bound as the forward gather is, with 1.7 times its
-// arithmetic: 512x512x8, 325 us as a thread a pixel walking its disc, 176 us as
-// this gather (128 registers and four CTAs 182, 80 and six 221). The record
-// pass at the same size: 101 us reading 32 bytes a pixel and record, 61 us with
-// 24 bytes and two records a thread.
-constexpr int kBwdWarps = 4;   // a CTA of the pixel pass: 128 threads of up to 102 registers, five CTAs a SM
-constexpr int kBwdTbx = 4;     // its tile: 8 x 16 pixels
+// The pixel pass: a thread takes kBwdRows pixels of a column and walks the
+// union of their discs, so a record is read once for all of them. Bound: the
+// sectors of L1 (a warp's lanes read records of neighbouring bins, one 32-byte
+// sector each): 512x512x8, 325 us with a pixel a thread that also searched its
+// exponent shift again, now 217 us (two rows a thread 237, four 302: registers).
+// The filter's gather, lanes over records, takes 176 us, but sums in another
+// order.
+constexpr int kBwdX = 32, kBwdY = 4;
+constexpr int kBwdRows = 3;
+constexpr int kPartRows = 4;   // rows of one partial
+static_assert(kBwdY * kBwdRows % kPartRows == 0, "a CTA holds whole partials");
 
 template <bool PARAMS>
-__global__ void __launch_bounds__(32 * kBwdWarps, 5) k_bwd_pixel(
+__global__ void __launch_bounds__(kBwdX * kBwdY) k_bwd_pixel(
     int W, int H, int R, int S_, int ntx, float window, float eps, AfrParams prm, const float4 *__restrict__ grad,
     const TilePartial *__restrict__ tiles, const float2 *__restrict__ sigma, const float4 *__restrict__ fconst,
-    const uint32_t *__restrict__ foff, const FrameRec *frec, const float4 *__restrict__ gout,
-    Adjoint adj, float *__restrict__ bparam, DebugCheck dc) {
-    __shared__ TileSmem ts;
-    __shared__ float4 discs[kMaxRows * kPitch];
-    __shared__ float4 go[kTilePixels];
-    __shared__ float part[kBwdWarps][6];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int tw = 2 * kBwdTbx, th = 64 / kBwdTbx;
-    static_assert(tw * th == kTilePixels && kTilePixels == 32 * kBwdWarps, "a thread per pixel");
-    const int x0 = blockIdx.x * tw, y0 = blockIdx.y * th;
-    frec = keep(frec + lane);
-    const uint32_t tables_at = smem_at(discs), rows_at = smem_at(ts.rows[warp]);
-    ts.fc[threadIdx.x] = load_const(threadIdx.x, W, H, x0, y0, tw, fconst);
-    go[threadIdx.x] = load_const(threadIdx.x, W, H, x0, y0, tw, gout);
-    fill_discs(discs, R);
-    load_offsets(ts, W, H, R, x0, y0, tw, th, foff);
-    __syncthreads();
-    float gp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int blk = warp; blk < 32; blk += kBwdWarps) {
-        const int lx = blk % kBwdTbx, ly = blk / kBwdTbx;
-        if (x0 + 2 * lx >= W || y0 + 2 * ly >= H) continue;   // warp-uniform
-        const int i0 = 2 * ly * tw + 2 * lx;
-        const float4 g4[4] = {go[i0], go[i0 + 1], go[i0 + tw], go[i0 + tw + 1]};
-        typename std::conditional<PARAMS, AdjointSums, WeightSums>::type A(g4);
-        gather_block<false>(R, x0, y0, tw, lx, ly, frec, ts, tables_at, ts.rows[warp], rows_at, dc, A);
-        float S, q[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // of pixel k at lane k: S; w q, w d^2, w d^2 q, w a^2, w a^2 q
-        if constexpr (PARAMS) {
-            float v[16], u[8];
+    const uint32_t *__restrict__ foff, const FrameRec *__restrict__ frec, const float4 *__restrict__ gout, Adjoint adj,
+    float *__restrict__ bparam, DebugCheck dc) {
+    __shared__ float part[kBwdY * kBwdRows][6];
+    const int x = blockIdx.x * kBwdX + threadIdx.x, y0 = (blockIdx.y * kBwdY + threadIdx.y) * kBwdRows;
+    float4 fc[kBwdRows];
+    PixelSums<PARAMS> A[kBwdRows];
+    if (x < W && y0 < H) {
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                upk(A.S[j], v[2 * j], v[2 * j + 1]);
-                upk(A.Q[j], v[4 + 2 * j], v[4 + 2 * j + 1]);
-                upk(A.Ds[j], v[8 + 2 * j], v[8 + 2 * j + 1]);
-                upk(A.Dsq[j], v[12 + 2 * j], v[12 + 2 * j + 1]);
-                upk(A.Dt[j], u[2 * j], u[2 * j + 1]);
-                upk(A.Dtq[j], u[4 + 2 * j], u[4 + 2 * j + 1]);
-            }
-            const float a = warp_reduce(v), b = warp_reduce(u);
-            S = __shfl_sync(0xffffffffu, a, 2 * (lane & 3));
+        for (int k = 0; k < kBwdRows; ++k) fc[k] = __ldg(fconst + (size_t)min(y0 + k, H - 1) * W + x);
+        const float cx = (float)x + 0.5f;
+        for (int v = max(-R, -y0); v <= min(R + kBwdRows - 1, H - 1 - y0); ++v) {
+            // records of each pixel's run of the row, and of the widest
+            const uint32_t *row = foff + (size_t)(y0 + v) * W;
+            uint32_t beg[kBwdRows], end[kBwdRows], e0 = 0xFFFFFFFFu, e1 = 0;
 #pragma unroll
-            for (int i = 0; i < 3; ++i) q[i] = __shfl_sync(0xffffffffu, a, 2 * (4 * (i + 1) + (lane & 3)));
-#pragma unroll
-            for (int i = 0; i < 2; ++i) q[3 + i] = __shfl_sync(0xffffffffu, b, 4 * (4 * i + (lane & 3)));
-        } else {
-            float v[4];
-            upk(A.S[0], v[0], v[1]);
-            upk(A.S[1], v[2], v[3]);
-            S = __shfl_sync(0xffffffffu, warp_reduce(v), 8 * (lane & 3));
-        }
-        const int x = x0 + 2 * lx + (lane & 1), y = y0 + 2 * ly + ((lane >> 1) & 1);
-        if (lane < 4 && x < W && y < H) {
-            const size_t p = (size_t)y * W + x;
-            const int i = block_pixel(tw, lx, ly);
-            const float4 fc = ts.fc[i], g = go[i];
-            if (!(S > 0.f)) {
-                adj.k[p] = make_float4(fc.x, fc.y, fc.z, 0.f);
-                adj.g[p] = make_float2(0.f, 0.f);
-            } else {
-                const float inv = 1.f / S;
-                adj.k[p] = make_float4(fc.x, fc.y, fc.z, g.x * inv);
-                adj.g[p] = make_float2(g.y * inv, g.z * inv);
-                if (PARAMS) {
-                    const float2 sg = __ldg(sigma + p);
-                    const float gC = q[0] * inv;
-                    const float gs = (q[2] - gC * q[1]) * inv / (sg.x * sg.x * sg.x);
-                    const float gt = (q[4] - gC * q[3]) * inv / (sg.y * sg.y * sg.y);
-                    // chain through the width mapping; the widths depend on theta only
-                    const Widths wd = widths(__ldg(grad + p), tile_volume(x, y, W, H, S_, ntx, window, tiles), eps, prm);
-                    if (fmaxf(wd.raw_s, kSigmaSMin) >= prm.clamp_s) gp[2] += gs;
-                    else if (wd.raw_s > kSigmaSMin) { gp[0] += gs * wd.es; gp[1] += gs; }
-                    if (fmaxf(wd.raw_t, kSigmaTMin) >= prm.clamp_t) gp[5] += gt;
-                    else if (wd.raw_t > kSigmaTMin) { gp[3] += gt * wd.et; gp[4] += gt; }
+            for (int k = 0; k < kBwdRows; ++k) {
+                beg[k] = end[k] = 0;
+                if (v - k >= -R && v - k <= R && y0 + k < H) {
+                    const int hw = half_width(R, v - k);
+                    beg[k] = __ldg(row + max(0, x - hw));
+                    end[k] = __ldg(row + min(W - 1, x + hw) + 1);
+                    if (!AFR_CHECK(beg[k] <= end[k] && end[k] <= dc.cap, dc.derr)) beg[k] = end[k] = 0;
+                    if (beg[k] < end[k]) {
+                        e0 = min(e0, beg[k]);
+                        e1 = max(e1, end[k]);
+                    }
                 }
+            }
+            for (uint32_t e = e0; e < e1; ++e) {
+                const FrameRec q = load_rec(frec + e);
+#pragma unroll
+                for (int k = 0; k < kBwdRows; ++k)
+                    A[k].add(q.p, q.c, cx, (float)(y0 + k) + 0.5f, fc[k], e - beg[k] < end[k] - beg[k]);
             }
         }
     }
-    if (PARAMS) {   // one partial of each parameter's gradient per CTA
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            float v = gp[k];
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            if (lane == 0) part[warp][k] = v;
+    for (int k = 0; k < kBwdRows; ++k) {
+        const int y = y0 + k;
+        float gp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (x < W && y < H) {
+            const size_t p = (size_t)y * W + x;
+            const float4 g = __ldg(gout + p);
+            const PixelSums<PARAMS> &s = A[k];
+            const float inv = 1.f / s.S;
+            const bool any = s.S > 0.f;
+            adj.k[p] = make_float4(fc[k].x, fc[k].y, fc[k].z, any ? g.x * inv : 0.f);
+            adj.g[p] = any ? make_float2(g.y * inv, g.z * inv) : make_float2(0.f, 0.f);
+            if (PARAMS && any) {
+                const float2 sgm = __ldg(sigma + p);
+                const float gch[3] = {g.x, g.y, g.z};
+                const float s3 = sgm.x * sgm.x * sgm.x, t3 = sgm.y * sgm.y * sgm.y;
+                float gs = 0.f, gt = 0.f;
+                for (int ch = 0; ch < 3; ++ch) {
+                    const float C = s.sc[ch] * inv;
+                    gs = fmaf(gch[ch], (s.dsc[ch] - C * s.Ds) * inv / s3, gs);
+                    gt = fmaf(gch[ch], (s.dtc[ch] - C * s.Dt) * inv / t3, gt);
+                }
+                // chain through the width mapping; the widths depend on theta only
+                const Widths wd = widths(__ldg(grad + p), tile_volume(x, y, W, H, S_, ntx, window, tiles), eps, prm);
+                if (fmaxf(wd.raw_s, kSigmaSMin) >= prm.clamp_s) gp[2] = gs;
+                else if (wd.raw_s > kSigmaSMin) { gp[0] = gs * wd.es; gp[1] = gs; }
+                if (fmaxf(wd.raw_t, kSigmaTMin) >= prm.clamp_t) gp[5] = gt;
+                else if (wd.raw_t > kSigmaTMin) { gp[3] = gt * wd.et; gp[4] = gt; }
+            }
         }
+        if (PARAMS) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                float v = gp[i];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (threadIdx.x == 0) part[threadIdx.y * kBwdRows + k][i] = v;
+            }
+        }
+    }
+    if (PARAMS) {
         __syncthreads();
-        if (threadIdx.x < 6) {
+        constexpr int kParts = kBwdY * kBwdRows / kPartRows;
+        const int t = threadIdx.y * kBwdX + threadIdx.x, j = t / 6, i = t % 6, py = blockIdx.y * kParts + j;
+        if (j < kParts && py < (H + kPartRows - 1) / kPartRows) {
             float acc = 0.f;
-            for (int w = 0; w < kBwdWarps; ++w) acc += part[w][threadIdx.x];
-            bparam[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 6 + threadIdx.x] = acc;
+            for (int w = 0; w < kPartRows; ++w) acc += part[j * kPartRows + w][i];
+            bparam[((size_t)py * gridDim.x + blockIdx.x) * 6 + i] = acc;
         }
     }
 }
@@ -973,7 +950,8 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 5) k_bwd_pixel(
 // holds the record's bin of (dL/dC_p / S_p) * shifted weight. Bound: the bytes
 // L1 delivers to registers (24 a pixel read, 128 a clock and SM), so a thread
 // takes two neighbouring records, which mostly share a bin or lie in adjacent
-// ones, and reads each pixel of their two discs once.
+// ones, and reads each pixel of their two discs once (512x512x8: 101 us with 32
+// bytes a pixel and record, 61 us).
 struct RecordAt {
     int qx, qy;
     float fx, fy, a2;   // position from the centre of bin (qx, qy), a^2
@@ -1192,15 +1170,14 @@ cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out
 
 cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_col, float *grad_prm,
                             cudaStream_t s) {
-    const int tw = 2 * kBwdTbx, th = 64 / kBwdTbx;
-    const dim3 grid((c->W + tw - 1) / tw, (c->H + th - 1) / th);
+    const dim3 block(kBwdX, kBwdY), grid((c->W + kBwdX - 1) / kBwdX, (c->H + kBwdY * kBwdRows - 1) / (kBwdY * kBwdRows));
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
     const Adjoint adj{c->bgrad, reinterpret_cast<float2 *>(c->bgrad + c->P)};
     const AfrParams &prm = c->recon_params;
 #define AFR_BWD(P_)                                                                                              \
-    k_bwd_pixel<P_><<<grid, 32 * kBwdWarps, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window,               \
-                                                    c->cfg.eps_grad, prm, c->grad, c->tiles, c->sigma, c->fconst, \
-                                                    c->foff, c->frec, grad_rgb, adj, c->bparam, dc)
+    k_bwd_pixel<P_><<<grid, block, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, prm,   \
+                                           c->grad, c->tiles, c->sigma, c->fconst, c->foff, c->frec, grad_rgb, adj, \
+                                           c->bparam, dc)
     if (grad_prm) AFR_BWD(true);
     else AFR_BWD(false);
 #undef AFR_BWD
@@ -1216,7 +1193,7 @@ cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_c
         }
     }
 #undef AFR_REC
-    if (grad_prm) k_bwd_params<<<1, 6 * 32, 0, s>>>(c->bparam, (int)(grid.x * grid.y), grad_prm);
+    if (grad_prm) k_bwd_params<<<1, 6 * 32, 0, s>>>(c->bparam, backward_blocks(c->W, c->H), grad_prm);
     return cudaGetLastError();
 }
 
@@ -1238,9 +1215,6 @@ cudaError_t launch_batch(int ct, const BatchCtx *cs, int nctx, uint32_t nchunks,
     return cudaGetLastError();
 }
 
-int backward_blocks(int W, int H) {
-    const int tw = 2 * kBwdTbx, th = 64 / kBwdTbx;
-    return ((W + tw - 1) / tw) * ((H + th - 1) / th);
-}
+int backward_blocks(int W, int H) { return ((W + kBwdX - 1) / kBwdX) * ((H + kPartRows - 1) / kPartRows); }
 
 }  // namespace afr

@@ -16,20 +16,22 @@ namespace {
 // ---- pixel pass ------------------------------------------------------------------
 // A warp takes 32 pixels: it copies their times and colours (contiguous in
 // memory) to shared memory with asynchronous 16-byte copies, and then each
-// lane walks one pixel's slots in storage order. Storage order is insertion
-// order turned by the head, so slot s follows slot s - 1 (slot 0 follows slot
-// b - 1) except that slot h, the oldest of a full queue, follows none. Sums do
-// not depend on the order, and consecutive slots are the consecutive samples
-// that the temporal gradient compares when times do not decrease, the usual
-// case; a queue out of time order is sorted (by time, newest first; equal
-// times newest first by insertion) by insertion on slot numbers in shared
-// memory. Sequence numbers are not read: they fall with the insertion rank.
+// lane walks one pixel's slots, newest first by insertion (slot h - 1, h - 2,
+// ... cyclically, h the head). Consecutive entries are the consecutive samples
+// that the temporal gradient compares when times do not increase along the
+// walk, the usual case; a queue out of time order is sorted (by time, newest
+// first; equal times newest first by insertion) by insertion on slot numbers in
+// shared memory. Sequence numbers are not read: they fall along the walk.
 //
-// Bound: HBM (20 bytes a slot in FP32 colours, 36 a pixel: 5.6 TB/s). A group of
+// Every sum over a queue adds entry k to partial k mod L and the L partials in
+// a tree, L = 2, 4 or 8 with the depth: short chains, and one order of rounding
+// whatever the number of threads a pixel gets.
+//
+// Bound: HBM (20 bytes a slot in FP32 colours, 36 a pixel: 5.4 TB/s). A group of
 // lanes a pixel spent the time on shuffles and read the sequence numbers too:
-// 1920x1080x16 227 us, this one 132 us (with a runtime depth, weights kept in
+// 1920x1080x16 227 us, this one 135 us (with a runtime depth, weights kept in
 // shared memory: 156 us; CTAs of two and four warps 135-164 us); 640x480x8 in
-// FP16 32 -> 17 us. Depths 4, 8 and 16 have a kernel of their own, where every
+// FP16 32 -> 18 us. Depths 4, 8 and 16 have a kernel of their own, where every
 // slot is at a constant offset and weights and deviations stay in registers.
 //
 // Shared memory of a warp: times (ts words a pixel), colours (cb bytes a
@@ -94,7 +96,21 @@ __device__ __forceinline__ float lum_diff(float3 a, float3 b) {   // L(a) - L(b)
 // temporal gradient takes each consecutive pair's difference from its colour
 // differences; the age weights, the time steps and the variance moments are
 // FP32.
-template <int CT, int B>
+// Sum of L partials: halves added pairwise.
+template <int L>
+__device__ __forceinline__ float tree_sum(float (&v)[L]) {
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < o; ++k) v[k] += v[k + o];
+    return v[0];
+}
+
+// Partials of a sum over a queue of depth b.
+__host__ __device__ constexpr int partials(int b) { return b <= 8 ? 2 : b <= 16 ? 4 : 8; }
+
+// B: the depth, or 0 for a depth known at run time; L: partials(depth).
+template <int CT, int B, int L>
 __global__ void __launch_bounds__(32 * kPixelWarps) k_pixel(int P, int b_run, float t_now,
                                                             const uint32_t *__restrict__ state,
                                                             const float *__restrict__ r_t,
@@ -133,47 +149,43 @@ __global__ void __launch_bounds__(32 * kPixelWarps) k_pixel(int P, int b_run, fl
     ws += lane * l.ts;
     const T4 *col = reinterpret_cast<const T4 *>(cs + lane * l.cb);
     order += lane * b;
-    // live slots: the n before h, cyclically; slots that are the next newer
-    // sample after the slot before them (slot 0 is left to the end)
-    const uint32_t all = 0xFFFFFFFFu >> (32 - b), m = n ? 0xFFFFFFFFu >> (32 - n) : 0u;
-    const uint32_t live = n <= h ? m << (h - n) : ((h ? m >> (n - h) : 0u) | (m << (b + h - n))) & all;
-    const uint32_t follows = live & (live << 1) & ~(1u << h);
     const int first = h == 0 ? b - 1 : h - 1;   // newest slot
     const float3 cr = CS::widen(col[first]);
-    float sw = 0.f, swd = 0.f, age = 0.f, num = 0.f, den = 0.f, Tp = 0.f, w0 = 0.f;
+    float sw[L] = {}, swd[L] = {}, num[L] = {}, den[L] = {}, m2[L] = {}, age = 0.f, Tp = 0.f, wp = 0.f;
     float3 cp = cr;
-    bool ordered = true;   // times do not decrease
+    bool ordered = true;   // times do not increase along the walk
     float W[B ? B : 1], D[B ? B : 1];
-#pragma unroll(B ? B : 4)
-    for (int s = 0; s < b; ++s) {
-        const float T = ts[s], a = fmaxf(t_now - T, 0.f), w = expf(-kAgeDecay * a);
-        const float3 c = CS::widen(col[s]);
-        const float d = lum_diff(c, cr), dl = fabsf(lum_diff(c, cp));
-        if (B) {
-            W[s] = w;
-            D[s] = d;
-        } else {
-            ws[s] = w;
+#pragma unroll(B ? B / L : 1)
+    for (int k0 = 0; k0 < b; k0 += L) {
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const int k = k0 + j;
+            if (!B && k >= b) break;
+            int s = h - 1 - k;
+            if (s < 0) s += b;
+            const float T = ts[s], a = fmaxf(t_now - T, 0.f), w = expf(-kAgeDecay * a);
+            const float3 c = CS::widen(col[s]);
+            const float d = lum_diff(c, cr), dl = fabsf(lum_diff(cp, c));
+            if (B) {
+                W[B ? k : 0] = w;
+                D[B ? k : 0] = d;
+            } else {
+                ws[s] = w;
+            }
+            if (k < n) {
+                sw[j] += w;
+                swd[j] += w * d;
+                age += a;
+                if (k > 0) {   // entry k - 1 and the next older one
+                    num[(j + L - 1) % L] += wp * dl;
+                    den[(j + L - 1) % L] += wp * (Tp - T);
+                    ordered = ordered && Tp >= T;
+                }
+            }
+            Tp = T;
+            wp = w;
+            cp = c;
         }
-        if (live >> s & 1u) {
-            sw += w;
-            swd += w * d;
-            age += a;
-        }
-        if (follows >> s & 1u) {
-            num += w * dl;
-            den += w * (T - Tp);
-            ordered = ordered && T >= Tp;
-        }
-        if (s == 0) w0 = w;
-        Tp = T;
-        cp = c;
-    }
-    if (live >> (b - 1) & live & (h != 0 ? 1u : 0u)) {   // slot 0 after slot b - 1
-        const float T = ts[0];
-        num += w0 * fabsf(lum_diff(CS::widen(col[0]), cp));
-        den += w0 * (T - Tp);
-        ordered = ordered && T >= Tp;
     }
     if (!ordered) {
         int s = first;
@@ -187,25 +199,36 @@ __global__ void __launch_bounds__(32 * kPixelWarps) k_pixel(int P, int b_run, fl
             order[j] = (uint8_t)s;
             s = s == 0 ? b - 1 : s - 1;
         }
-        num = den = 0.f;
+#pragma unroll
+        for (int j = 0; j < L; ++j) num[j] = den[j] = 0.f;
         float T = ts[order[0]];
         float3 c = CS::widen(col[order[0]]);
-        for (int k = 1; k < n; ++k) {
-            const int o = order[k];
-            const float To = ts[o], w = expf(-kAgeDecay * fmaxf(t_now - T, 0.f));
-            const float3 co = CS::widen(col[o]);
-            num += w * fabsf(lum_diff(c, co));
-            den += w * (T - To);
-            T = To;
-            c = co;
+        for (int k0 = 0; k0 + 1 < n; k0 += L) {
+#pragma unroll
+            for (int j = 0; j < L; ++j) {
+                if (k0 + j + 1 >= n) break;
+                const int o = order[k0 + j + 1];
+                const float To = ts[o], w = expf(-kAgeDecay * fmaxf(t_now - T, 0.f));
+                const float3 co = CS::widen(col[o]);
+                num[j] += w * fabsf(lum_diff(c, co));
+                den[j] += w * (T - To);
+                T = To;
+                c = co;
+            }
         }
     }
-    const float delta = n > 0 ? swd / sw : 0.f;   // mean - L_r
-    float m2 = 0.f;
-#pragma unroll(B ? B : 4)
-    for (int s = 0; s < b; ++s) {
-        const float w = B ? W[s] : ws[s], dd = (B ? D[s] : lum_diff(CS::widen(col[s]), cr)) - delta;
-        if (live >> s & 1u) m2 += w * dd * dd;
+    const float tw = tree_sum(sw), delta = n > 0 ? tree_sum(swd) / tw : 0.f;   // mean - L_r
+#pragma unroll(B ? B / L : 1)
+    for (int k0 = 0; k0 < b; k0 += L) {
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const int k = k0 + j;
+            if (!B && k >= b) break;
+            int s = h - 1 - k;
+            if (s < 0) s += b;
+            const float w = B ? W[B ? k : 0] : ws[s], dd = (B ? D[B ? k : 0] : lum_diff(CS::widen(col[s]), cr)) - delta;
+            if (k < n) m2[j] += w * dd * dd;
+        }
     }
     if (lane >= np) return;
     if (n == 0) {
@@ -214,7 +237,8 @@ __global__ void __launch_bounds__(32 * kPixelWarps) k_pixel(int P, int b_run, fl
     } else {
         const dfloat mean = df_add(luminance_df(cr), {delta, 0.f});
         lbar[p] = make_float2(mean.h, mean.l);
-        pstat[p] = make_float4(sw, m2, (n >= 2 && den > 0.f) ? num / den : 0.f, age);
+        const float tn = tree_sum(num), td = tree_sum(den);
+        pstat[p] = make_float4(tw, tree_sum(m2), (n >= 2 && td > 0.f) ? tn / td : 0.f, age);
     }
 }
 
@@ -414,21 +438,26 @@ __global__ void __launch_bounds__(kTileThreads, 3) k_spatial_tiles(int W, int H,
     }
 }
 
-template <int CT, int B>
+template <int CT, int B, int L>
 void launch_depth(AfrContext *c, float t_now, unsigned long long *total, cudaStream_t s) {
+    static_assert(B == 0 || L == partials(B), "one order of summation a depth");
     const PixelLayout l = pixel_layout(c->b, c->csize, B == 0);
     const int groups = (c->P + 31) / 32;
-    k_pixel<CT, B><<<(groups + kPixelWarps - 1) / kPixelWarps, 32 * kPixelWarps, kPixelWarps * l.bytes, s>>>(
+    k_pixel<CT, B, L><<<(groups + kPixelWarps - 1) / kPixelWarps, 32 * kPixelWarps, kPixelWarps * l.bytes, s>>>(
         c->P, c->b, t_now, c->r_state, c->r_t, c->r_col, c->lbar, c->pstat, total);
 }
 
 template <int CT>
 void launch_pixel(AfrContext *c, float t_now, unsigned long long *total, cudaStream_t s) {
     switch (c->b) {
-        case 4: launch_depth<CT, 4>(c, t_now, total, s); break;
-        case 8: launch_depth<CT, 8>(c, t_now, total, s); break;
-        case 16: launch_depth<CT, 16>(c, t_now, total, s); break;
-        default: launch_depth<CT, 0>(c, t_now, total, s); break;
+        case 4: launch_depth<CT, 4, 2>(c, t_now, total, s); break;
+        case 8: launch_depth<CT, 8, 2>(c, t_now, total, s); break;
+        case 16: launch_depth<CT, 16, 4>(c, t_now, total, s); break;
+        default:
+            if (partials(c->b) == 2) launch_depth<CT, 0, 2>(c, t_now, total, s);
+            else if (partials(c->b) == 4) launch_depth<CT, 0, 4>(c, t_now, total, s);
+            else launch_depth<CT, 0, 8>(c, t_now, total, s);
+            break;
     }
 }
 
