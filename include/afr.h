@@ -345,6 +345,18 @@ enum { AFR_RECON_KEEP_SIGMA = 1, AFR_RECON_ADAPTIVE_SUPPORT = 2, AFR_RECON_COVER
 AFR_API AfrStatus afr_reconstruct_ex(AfrContext *ctx, float t_now, const AfrParams *params,
                              uint32_t flags, float *out_rgbw_dev, afr_stream_t stream);
 
+/* One displayed image from the buffered samples, in one call: on side the
+ * afr_estimate_gradients and afr_tile_feedback (to tiles_dev), which wait for
+ * the work issued on stream before the call; on stream the afr_reproject
+ * (afr_reproject_camera with view_proj_host, if not NULL), then, once both
+ * branches are done, afr_reconstruct_ex. reads_done: a CUDA event or NULL;
+ * recorded on stream when both branches are done with the sample buffers,
+ * before the filter. Results, errors and ordering rules as the calls it stands
+ * for; can be captured in a CUDA graph. */
+AFR_API AfrStatus afr_refresh(AfrContext *ctx, float t_now, const float *view_proj_host, const AfrParams *params,
+                              uint32_t flags, float *out_rgbw_dev, AfrTileStats *tiles_dev, afr_stream_t side,
+                              afr_event_t reads_done, afr_stream_t stream);
+
 /* Filter tuning of a context: footprint radius R (0..8; it changes results:
  * the footprint is the integer disc of radius R) and the filter's CTA tile,
  * (2*tile_bx) x (64/tile_bx) pixels with tile_bx in {2, 4, 8, 16} (default 4;

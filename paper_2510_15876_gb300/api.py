@@ -16,21 +16,27 @@ from . import _lib as L
 _COLOR_TYPES = {"f32": L.AFR_F32, "f16": L.AFR_F16, "bf16": L.AFR_BF16}
 _COLOR_DTYPES = {L.AFR_F32: torch.float32, L.AFR_F16: torch.float16, L.AFR_BF16: torch.bfloat16}
 DEFAULT_PARAMS = (1.0, 0.0, 3.0, 1.0, 0.0, 1.0)
+_DEFAULT = L.AfrParams(*DEFAULT_PARAMS)   # the library only reads it
 TILE_FIELDS = ("n", "empty_slots", "mean_L", "var_L", "mean_Gx", "mean_Gy", "mean_Gt", "u")
 
 
 def _stream(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())   # no Stream object (2 us)
 
 
 def _ptr(t: torch.Tensor | None):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
+def _matrix(view_proj):
+    return (ctypes.c_float * 16)(*[float(v) for v in np.asarray(view_proj, np.float32).reshape(16)])
+
+
 def _params(p) -> L.AfrParams:
     if p is None:
-        p = DEFAULT_PARAMS
+        return _DEFAULT
     if isinstance(p, torch.Tensor):
         p = p.detach().to("cpu", torch.float64).tolist()
     return L.AfrParams(*[float(v) for v in p])
@@ -65,7 +71,6 @@ class Reconstructor:
         self._check(self.lib.afr_num_tiles(self.h, ctypes.byref(n)))
         self.n_tiles = n.value
         self._side = None                 # refresh(): stream of the gradient branch
-        self._fork, self._join = torch.cuda.Event(), torch.cuda.Event()
 
     # -- plumbing ------------------------------------------------------------------
     def _check(self, st: int):
@@ -107,8 +112,9 @@ class Reconstructor:
         arrays = [(pos, torch.float32, 4), (color, self.color_dtype, 4), (motion, torch.float32, 2)]
         if world is not None:
             arrays.append((world, torch.float32, 4))
+        device = self.device
         for t, dt, cols in arrays:
-            if t.device != self.device or t.dtype != dt or not t.is_contiguous() or tuple(t.shape) != (n, cols):
+            if t.device != device or t.dtype != dt or not t.is_contiguous() or t.shape != (n, cols):
                 raise ValueError(f"batch tensor must be contiguous {dt} [{n}, {cols}] on {self.device}")
         batch = L.AfrSampleBatch(pos.data_ptr(), color.data_ptr(), motion.data_ptr(),
                                  None if world is None else world.data_ptr())
@@ -128,8 +134,7 @@ class Reconstructor:
     def reproject_camera(self, t_now: float, view_proj, stream=None):
         """Frame view from the stored hit points rendered by the row-major 4x4
         view_proj (section 6.2)."""
-        m = (ctypes.c_float * 16)(*[float(v) for v in np.asarray(view_proj, np.float32).reshape(16)])
-        self._check(self.lib.afr_reproject_camera(self.h, t_now, m, _stream(stream)))
+        self._check(self.lib.afr_reproject_camera(self.h, t_now, _matrix(view_proj), _stream(stream)))
 
     def reconstruct(self, t_now: float = 1.0, params=None, out: torch.Tensor | None = None, flags: int = 0,
                     stream=None) -> torch.Tensor:
@@ -161,8 +166,9 @@ class Reconstructor:
         stream that waits for it overlaps the filter (the filter reads no
         sample buffer). view_proj, if given, reprojects the stored hit points
         with that camera (reproject_camera) instead of the screen motion.
-        Returns (image, tile statistics)."""
-        main = stream if stream is not None else torch.cuda.current_stream(self.device)
+        Returns (image, tile statistics). One native call (afr_refresh): as
+        four, with torch's events between them, it took 36 us of host time."""
+        main = stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(self.device.index)
         if side_stream is None:
             if self._side is None:
                 self._side = torch.cuda.Stream(self.device, priority=-1)
@@ -171,19 +177,14 @@ class Reconstructor:
             tiles = torch.empty((self.n_tiles, 8), dtype=torch.float32, device=self.device)
         if out is None:
             out = torch.empty((self.H, self.W, 4), dtype=torch.float32, device=self.device)
-        self._fork.record(main)
-        side_stream.wait_event(self._fork)
-        self.estimate_gradients(t_now, stream=side_stream)
-        self.tile_feedback(out=tiles, stream=side_stream)
-        self._join.record(side_stream)
-        if view_proj is None:
-            self.reproject(t_now, stream=main)
-        else:
-            self.reproject_camera(t_now, view_proj, stream=main)
-        main.wait_event(self._join)
+        event = None
         if reads_done is not None:
-            reads_done.record(main)
-        self.reconstruct(t_now, params, out, flags, stream=main)
+            if not reads_done.cuda_event:   # torch makes the event when it is first recorded
+                reads_done.record(stream if stream is not None else torch.cuda.current_stream(self.device))
+            event = reads_done.cuda_event
+        self._check(self.lib.afr_refresh(self.h, t_now, None if view_proj is None else _matrix(view_proj),
+                                         ctypes.byref(_params(params)), flags, out.data_ptr(), tiles.data_ptr(),
+                                         side_stream.cuda_stream, event, main))
         return out, tiles
 
     GAIN_KEYS = ("dC_ds", "dC_dt", "mean_age", "tile_width", "tile_count")

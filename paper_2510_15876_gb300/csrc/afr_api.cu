@@ -63,6 +63,8 @@ void free_all(AfrContext *c) {
                     c->foff, c->frec, c->sbin, c->flist, c->q_xm, c->q_t, c->q_seq, c->q_col, c->q_total, c->q_world, c->r_world, c->scan_tmp, c->scan_tmp_in, c->bgrad, c->bparam, c->dcount, c->derr};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    if (c->fork) cudaEventDestroy(c->fork);
+    if (c->join) cudaEventDestroy(c->join);
 }
 
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
@@ -245,6 +247,8 @@ AfrStatus afr_create(const AfrConfig *cfg, AfrContext **out) {
     if (e == cudaSuccess) e = cudaMemset(c->foff, 0, (P + 1) * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(c->dcount, 0, afr::CNT_N * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(c->derr, 0, sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = afr::launch_coverage_init(c, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
@@ -468,6 +472,27 @@ AfrStatus afr_tile_feedback(AfrContext *c, AfrTileStats *out_dev, afr_stream_t s
     cudaError_t e = afr::launch_feedback(c, out_dev, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "afr_tile_feedback");
     return AFR_OK;
+}
+
+AfrStatus afr_refresh(AfrContext *c, float t_now, const float *view_proj, const AfrParams *params, uint32_t flags,
+                      float *out_rgbw_dev, AfrTileStats *tiles_dev, afr_stream_t side, afr_event_t reads_done,
+                      afr_stream_t stream) {
+    Range nvtx_range("afr_refresh");
+    if (!c) return AFR_ERR_INVALID_ARG;
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), g = reinterpret_cast<cudaStream_t>(side);
+    cudaError_t e = cudaEventRecord(c->fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(g, c->fork, 0);
+    if (e != cudaSuccess) return cuda_fail(c, e, "afr_refresh");
+    AfrStatus st = afr_estimate_gradients(c, t_now, side);
+    if (st == AFR_OK) st = afr_tile_feedback(c, tiles_dev, side);
+    if (st != AFR_OK) return st;
+    if ((e = cudaEventRecord(c->join, g)) != cudaSuccess) return cuda_fail(c, e, "afr_refresh");
+    st = view_proj ? afr_reproject_camera(c, t_now, view_proj, stream) : afr_reproject(c, t_now, stream);
+    if (st != AFR_OK) return st;
+    e = cudaStreamWaitEvent(s, c->join, 0);
+    if (e == cudaSuccess && reads_done) e = cudaEventRecord(reinterpret_cast<cudaEvent_t>(reads_done), s);
+    if (e != cudaSuccess) return cuda_fail(c, e, "afr_refresh");
+    return afr_reconstruct_ex(c, t_now, params, flags, out_rgbw_dev, stream);
 }
 
 AfrStatus afr_tile_error(AfrContext *c, float kappa, float lambda, float importance, const uint32_t *occluded_dev,

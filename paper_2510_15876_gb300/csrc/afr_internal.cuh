@@ -182,6 +182,7 @@ struct AfrContext {
     AfrParams recon_params{};
     bool sigma_imported = false;
     int tile_bx = 4;              // filter CTA tile: (2*tile_bx) x (64/tile_bx) pixels (8 x 16 measured fastest at 1080p16)
+    cudaEvent_t fork = nullptr, join = nullptr;   // afr_refresh's two branches
     // filter kernel timing (afr_profile_filter): event pairs, launches recorded
     cudaEvent_t *prof_ev = nullptr;
     bool prof_on = false, prof_capture_hit = false;
