@@ -444,7 +444,7 @@ AfrStatus afr_reconstruct_ex(AfrContext *c, float t_now, const AfrParams *params
         else if (e == cudaSuccess) pair = c->prof_ev + 2 * c->prof_n;
     }
     if (e == cudaSuccess && pair) e = cudaEventRecord(pair[0], s);
-    if (e == cudaSuccess) e = afr::launch_filter(c, t_now, adaptive, reinterpret_cast<float4 *>(out_rgbw_dev), s);
+    if (e == cudaSuccess) e = afr::launch_filter(c, t_now, adaptive, reinterpret_cast<float4 *>(out_rgbw_dev), s, !pair);
     if (e == cudaSuccess && pair) {
         e = cudaEventRecord(pair[1], s);
         ++c->prof_n;
@@ -869,7 +869,7 @@ AfrStatus afr_batch_refresh(AfrBatch *b, float t_now, const AfrParams *params, f
         if (e == cudaSuccess) e = afr::launch_reproject(c, t_now, nullptr, ws);
         if (e == cudaSuccess) e = afr::launch_sigma(c, params, false, false, ws);
         if (e == cudaSuccess)
-            e = afr::launch_filter(c, t_now, false, reinterpret_cast<float4 *>(outs_dev[b->user_index[q]]), ws);
+            e = afr::launch_filter(c, t_now, false, reinterpret_cast<float4 *>(outs_dev[b->user_index[q]]), ws, true);
     }
     for (size_t w = 0; w < b->workers.size() && e == cudaSuccess; ++w) {
         e = cudaEventRecord(b->joined[w], b->workers[w]);
@@ -940,7 +940,7 @@ AfrStatus afr_batch_reconstruct(AfrBatch *b, float t_now, const AfrParams *param
         AfrContext *c = b->ctxs[q];
         e = afr::launch_sigma(c, params, false, false, s);
         if (e == cudaSuccess)
-            e = afr::launch_filter(c, t_now, false, reinterpret_cast<float4 *>(outs_dev[b->user_index[q]]), s);
+            e = afr::launch_filter(c, t_now, false, reinterpret_cast<float4 *>(outs_dev[b->user_index[q]]), s, true);
     }
     const int m = n - b->n_direct;
     if (m > 0) {

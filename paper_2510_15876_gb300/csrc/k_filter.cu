@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(kSigX * kSigY) k_sigma(int W, int H, int Rrun,
                                                          const TilePartial *__restrict__ tiles,
                                                          const uint32_t *__restrict__ amin2,
                                                          float2 *__restrict__ sigma, float4 *__restrict__ fconst) {
+    grid_order();
     __shared__ uint32_t age[(kSigY + 2 * kSigHalo) * (kSigX + 2 * kSigHalo)];
     const int R = RT >= 0 ? RT : Rrun, pitch = kSigX + 2 * R;
     const int x0 = blockIdx.x * kSigX, y0 = blockIdx.y * kSigY, x = x0 + threadIdx.x, y = y0 + threadIdx.y;
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(kSigX * kSigY) k_sigma_adaptive(int W, int H, 
                                                                   const uint32_t *__restrict__ foff,
                                                                   int32_t *__restrict__ cov_n, float2 *__restrict__ sigma,
                                                                   float4 *__restrict__ fconst) {
+    grid_order();
     const int x = blockIdx.x * kSigX + threadIdx.x, y = blockIdx.y * kSigY + threadIdx.y;
     if (x >= W || y >= H) return;
     const size_t p = (size_t)y * W + x;
@@ -683,6 +685,7 @@ template <bool KAHAN, bool VAR>
 __global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx, int lsplit, const float4 *__restrict__ fconst,
                                                    const uint32_t *__restrict__ foff, const FrameRec *frec,
                                                    float4 *__restrict__ out, DebugCheck dc) {
+    grid_order();
     __shared__ TileSmem ts;
     __shared__ float4 discs[(VAR ? kTableRows : kMaxRows) * kPitch];
     const int warp = threadIdx.x >> 5, tw = 2 << ltbx, th = 64 >> ltbx >> lsplit, pixels = tw * th;
@@ -1142,7 +1145,7 @@ cudaError_t launch_coverage_init(AfrContext *c, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out, cudaStream_t s) {
+cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out, cudaStream_t s, bool next) {
     (void)t_now;
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
     const int tbx = c->tile_bx, tw = 2 * tbx;
@@ -1157,8 +1160,15 @@ cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out
         th /= 2;
     }
     dim3 grid((c->W + tw - 1) / tw, (c->H + th - 1) / th);
-#define AFR_FILTER(K_, V_) \
-    k_filter<K_, V_><<<grid, kQuadBlock, 0, s>>>(c->W, c->H, c->R, __builtin_ctz(tbx), lsplit, c->fconst, c->foff, c->frec, out, dc)
+#define AFR_FILTER(K_, V_)                                                                                            \
+    do {                                                                                                              \
+        if (next)                                                                                                     \
+            launch_next(k_filter<K_, V_>, grid, kQuadBlock, 0, s, c->W, c->H, c->R, __builtin_ctz(tbx), lsplit,       \
+                        c->fconst, c->foff, c->frec, out, dc);                                                        \
+        else                                                                                                          \
+            k_filter<K_, V_><<<grid, kQuadBlock, 0, s>>>(c->W, c->H, c->R, __builtin_ctz(tbx), lsplit, c->fconst,     \
+                                                         c->foff, c->frec, out, dc);                                  \
+    } while (0)
     // colours stored in 16 bits: compensated weight sums
     if (c->ct == AFR_F32 && adaptive) AFR_FILTER(false, true);
     else if (c->ct == AFR_F32) AFR_FILTER(false, false);

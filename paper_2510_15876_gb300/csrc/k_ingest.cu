@@ -74,6 +74,7 @@ __device__ __forceinline__ uint32_t pixel_at(float x, float y, int W) {
 
 __global__ void __launch_bounds__(256) k_pix_count(const float4 *__restrict__ pos, uint32_t n, int W, int H,
                                                    uint32_t *__restrict__ pcnt) {
+    grid_order();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float4 p = __ldg(pos + i);
         if (position_ok(p, W, H)) atomicAdd(pcnt + pixel_at(p.x, p.y, W), 1u);
@@ -94,6 +95,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_pix_scatter(
     const float4 *__restrict__ pos, const void *__restrict__ col, const float2 *__restrict__ mo,
     const float4 *__restrict__ world, uint32_t n, int W, int H, uint32_t *__restrict__ pcur, Bucket bk,
     uint32_t *__restrict__ accept, unsigned long long *__restrict__ dcount, DebugCheck dc) {
+    grid_order();
     using CS = ColorStore<CT>;
     __shared__ uint4 stage[kScatterWarps][32][5];   // 80-byte stride: conflict-free 16-byte accesses
     __shared__ uint32_t dest[kScatterWarps][32];
@@ -242,6 +244,7 @@ template <int CT>
 __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__restrict__ poff, uint32_t P, int W,
                                                             int b, uint32_t seq0, Bucket bk, Queues q,
                                                             bool reset, uint32_t *__restrict__ state1, DebugCheck dc) {
+    grid_order();
     __shared__ uint32_t sidx[kCommitTile];
     uint32_t n = __ldg(poff + P);
     if (!AFR_CHECK(n <= dc.cap, dc.derr)) n = 0;
@@ -308,6 +311,7 @@ __global__ void __launch_bounds__(256) k_pix_finish(const uint32_t *__restrict__
                                                     const uint32_t *__restrict__ state1,
                                                     unsigned long long *__restrict__ dcount,
                                                     uint32_t *__restrict__ q_total, DebugCheck dc) {
+    grid_order();
     static_assert(CNT_REJECTED == 0, "the rejected count, cleared before the scatter, comes first");
     if (reset && blockIdx.x == 0) {
         if (threadIdx.x >= 1 && threadIdx.x < CNT_N) dcount[threadIdx.x] = 0ull;
@@ -381,16 +385,17 @@ cudaError_t run(AfrContext *c, const float4 *pos, const void *col, const float2 
     if ((e = scan_exclusive(c->ccnt, c->coff, P, c->scan_tmp_in, s, with)) != cudaSuccess) return e;
     const int gs = grid_for((n + kScatterUnroll - 1) / kScatterUnroll, 32 * kScatterWarps);
     uint32_t *accept = c->fifo_n ? c->fifo_flag : nullptr;
-    k_pix_scatter<CT><<<gs, 32 * kScatterWarps, 0, s>>>(pos, col, mo, c->r_world ? world : nullptr, n, c->W, c->H,
-                                                        c->ccur, bk, accept, c->dcount, dc);
+    launch_next(k_pix_scatter<CT>, dim3(gs), dim3(32 * kScatterWarps), 0, s, pos, col, mo, c->r_world ? world : nullptr, n,
+                c->W, c->H, c->ccur, bk, accept, c->dcount, dc);
     // from here on the queues: wait until they are free. The cursors are spent:
     // they take the new queue states
     if (queues_free && (e = cudaStreamWaitEvent(s, queues_free, 0)) != cudaSuccess) return e;
     Queues q{c->r_xm, c->r_t, c->r_depth, c->r_seq, c->r_col, c->r_state, c->r_world, c->nslots};
-    k_pix_commit<CT><<<grid_for(n, kCommitTile), kCommitTile, 0, s>>>(c->coff, P, c->W, c->b, seq0, bk, q, reset,
-                                                                      c->ccur, dc);
-    k_pix_finish<CT><<<grid_for(P, 256), 256, 0, s>>>(c->coff, P, c->b, seq0, bk, q, reset, c->ccur, c->dcount,
-                                                      c->q_total, dc);
+    const dim3 gc(grid_for(n, kCommitTile)), tc(kCommitTile);
+    if (queues_free) k_pix_commit<CT><<<gc, tc, 0, s>>>(c->coff, P, c->W, c->b, seq0, bk, q, reset, c->ccur, dc);
+    else launch_next(k_pix_commit<CT>, gc, tc, 0, s, c->coff, P, c->W, c->b, seq0, bk, q, reset, c->ccur, dc);
+    launch_next(k_pix_finish<CT>, dim3(grid_for(P, 256)), dim3(256), 0, s, c->coff, P, c->b, seq0, bk, q, reset, c->ccur,
+                c->dcount, c->q_total, dc);
     return cudaGetLastError();
 }
 

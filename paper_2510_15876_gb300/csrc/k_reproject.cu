@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(256) k_count(uint32_t nslots, int b, int bshif
                                                const uint32_t *__restrict__ state, const float4 *__restrict__ r_xm, const float *__restrict__ r_t,
                                                uint32_t *__restrict__ fcnt, uint32_t *__restrict__ sbin,
                                                unsigned long long *__restrict__ dcount) {
+    grid_order();
     const uint32_t nlive = FIFO ? min(__ldg(state), nslots) : 0u;
     const int lane = threadIdx.x & 31;
     uint32_t dropped = 0;
@@ -170,6 +171,7 @@ template <bool SLOTS>
 __global__ void __launch_bounds__(256) k_list(uint32_t nslots, const uint32_t *__restrict__ sbin,
                                               const uint32_t *__restrict__ r_seq, uint32_t *__restrict__ fcur,
                                               uint32_t *__restrict__ flist, DebugCheck dc) {
+    grid_order();
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t i0 = warp * 32u * kListRows; i0 < nslots; i0 += nwarps * 32u * kListRows) {
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(256) k_place_queues(int W, int H, float t_now,
                                                uint32_t *__restrict__ fcur, uint32_t *__restrict__ amin2,
                                                FrameRec *__restrict__ frec, unsigned long long *__restrict__ dcount,
                                                DebugCheck dc, uint32_t nsrc) {
+    grid_order();
     using CS = ColorStore<CT>;
     uint32_t n = __ldg(foff + P);
     if (!AFR_CHECK(n <= dc.cap, dc.derr)) n = 0;
@@ -285,6 +288,7 @@ __global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int 
                                                     const uint32_t *__restrict__ flist, uint32_t *__restrict__ fcur,
                                                     uint32_t *__restrict__ amin2, FrameRec *__restrict__ frec,
                                                     unsigned long long *__restrict__ dcount, DebugCheck dc) {
+    grid_order();
     using CS = ColorStore<CT>;
     const uint32_t nlive = min(__ldg(state), nslots);
     const int lane = threadIdx.x & 31;
@@ -366,14 +370,17 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     with.counter_to = c->dcount + CNT_DROPPED;
     with.counter_zero = c->dcount + CNT_UNSORTED;
     if ((e = scan_exclusive(c->fcnt, c->foff, c->P, c->scan_tmp, s, with)) != cudaSuccess) return e;
+    // Not by launch_next: its blocks then start unevenly and leave the lists out
+    // of slot order, and placing, which gathers in list order, takes 1.1 ms
+    // instead of 0.5 at 1920x1080x16 (3956 -> 4291 us for the step).
     if (fifo) k_list<false><<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, dc);
     else k_list<true><<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, dc);
 #define AFR_QUEUES(CT_, C_)                                                                                         \
-    k_place_queues<CT_, C_><<<g, 256, 0, s>>>(c->W, c->H, t_now, cm, wp, xm, tt, col, (uint32_t)c->P, c->foff,    \
+    launch_next(k_place_queues<CT_, C_>, dim3(g), dim3(256), 0, s, c->W, c->H, t_now, cm, wp, xm, tt, col, (uint32_t)c->P, c->foff,    \
                                               reinterpret_cast<const uint2 *>(c->flist), c->fcur, c->amin2, c->frec, \
                                               c->dcount, dc, ns)
 #define AFR_FIFO(CT_, C_)                                                                                            \
-    k_place_fifo<CT_, C_><<<g, 256, 0, s>>>(ns, c->W, c->H, t_now, cm, wp, state, xm, tt, sq, col, c->foff, c->flist, \
+    launch_next(k_place_fifo<CT_, C_>, dim3(g), dim3(256), 0, s, ns, c->W, c->H, t_now, cm, wp, state, xm, tt, sq, col, c->foff, c->flist, \
                                             c->fcur, c->amin2, c->frec, c->dcount, dc)
 #define AFR_REPROJ(CT_)                       \
     do {                                      \

@@ -94,6 +94,7 @@ __device__ __forceinline__ uint32_t block_sum(uint32_t v) {
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t *in, size_t n, uint32_t *sums) {
+    grid_order();
     const Items r = load_items(in, (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems, n);
     uint32_t acc = 0;
 #pragma unroll
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kScanThreads) k_block_sums(const uint32_t *in,
 
 // Scans nb block sums in place (exclusive) with one block.
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *sums, size_t nb) {
+    grid_order();
     __shared__ uint32_t carry;
     __shared__ uint32_t tot;
     if (threadIdx.x == 0) carry = 0;
@@ -123,6 +125,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *sums, size
 // (a caller's own array need not be)
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint32_t *in, uint32_t *out, size_t n,
                                                               const uint32_t *sums, bool scanned, bool wide, ScanWith with) {
+    grid_order();
     __shared__ uint32_t tot;
     const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
     Items r = load_items(in, base, n);
@@ -172,9 +175,9 @@ cudaError_t scan_exclusive(uint32_t *in, uint32_t *out, size_t n, uint32_t *tmp,
         return cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
     }
     const bool scanned = nb > kDirectBlocks, wide = reinterpret_cast<uintptr_t>(out) % 32 == 0;
-    k_block_sums<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, tmp);
-    if (scanned) k_scan_sums<<<1, kScanThreads, 0, s>>>(tmp, nb);
-    k_scan_tiles<<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, tmp, scanned, wide, with);
+    launch_next(k_block_sums, dim3((unsigned)nb), dim3(kScanThreads), 0, s, in, n, tmp);   // after the caller's counting
+    if (scanned) launch_next(k_scan_sums, dim3(1), dim3(kScanThreads), 0, s, tmp, nb);
+    launch_next(k_scan_tiles, dim3((unsigned)nb), dim3(kScanThreads), 0, s, in, out, n, tmp, scanned, wide, with);
     return cudaGetLastError();
 }
 

@@ -78,3 +78,56 @@ def test_refresh_refuses_what_its_calls_refuse(dev):
     assert err.value.status == L.AFR_ERR_BAD_STATE
     img, _ = a.refresh(1.0)
     assert torch.isfinite(img).all()
+
+
+@pytest.mark.parametrize("w,h,depth,color,fifo", [
+    (1, 1, 2, "f32", 0), (61, 43, 5, "bf16", 0), (640, 360, 8, "f16", 0), (300, 200, 4, "f32", 3 * 300 * 200)])
+def test_overlapped_launches_keep_their_order(dev, w, h, depth, color, fifo):
+    """A step's kernels are launched before the ones they read from have ended
+    (waiting inside), at one block and at many waves: steps issued without a
+    pause, and replayed from a graph, equal steps with a synchronisation after
+    every call, bit for bit, whole state included."""
+    from paper_2510_15876_gb300.api import Reconstructor
+    dtype = {"f32": torch.float32, "f16": torch.float16, "bf16": torch.bfloat16}[color]
+    n = 2 * w * h * depth
+    batches = []
+    for seed in range(3):
+        g = torch.Generator().manual_seed(seed)
+        pos = torch.rand(n, 4, generator=g) * torch.tensor([w, h, 1.0, 1.0])
+        pos[:, 2] = pos[:, 2].sort().values
+        pos[::13, 0] = float("nan")
+        batches.append((pos.to(dev), torch.rand(n, 4, generator=g).to(dev, dtype), torch.randn(n, 2, generator=g).to(dev)))
+
+    def context():
+        rec = Reconstructor(w, h, depth, color_type=color, fifo_capacity=fifo, device=dev)
+        rec.reserve(n)
+        return rec
+
+    plain, graphed, slow = context(), context(), context()
+    outs = []
+    for rec in (plain, graphed):
+        out, tiles = torch.empty((h, w, 4), device=dev), torch.empty((rec.n_tiles, 8), device=dev)
+        outs.append((out, tiles))
+    static = [t.clone() for t in batches[0]]
+    graphed._side = torch.cuda.Stream(dev)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        graphed.insert(*static, reset=True)
+        graphed.refresh(1.0, out=outs[1][0], tiles=outs[1][1])
+    for batch in batches:
+        plain.insert(*batch, reset=True)
+        plain.refresh(1.0, out=outs[0][0], tiles=outs[0][1])
+        for s, t in zip(static, batch):
+            s.copy_(t)
+        graph.replay()
+        slow.reset()
+        for call in (lambda: slow.insert(*batch), lambda: slow.estimate_gradients(1.0), lambda: slow.reproject(1.0)):
+            call()
+            torch.cuda.synchronize()
+        want, want_tiles = slow.reconstruct(1.0), slow.tile_feedback()
+        torch.cuda.synchronize()
+        for out, tiles in outs:
+            assert torch.equal(out, want) and torch.equal(tiles.view(torch.int32), want_tiles.view(torch.int32))
+        for a, b in zip(plain.export_ring(), slow.export_ring()):
+            assert np.array_equal(a, b)
