@@ -863,6 +863,7 @@ __global__ void __launch_bounds__(kBwdX * kBwdY) k_bwd_pixel(
     const TilePartial *__restrict__ tiles, const float2 *__restrict__ sigma, const float4 *__restrict__ fconst,
     const uint32_t *__restrict__ foff, const FrameRec *__restrict__ frec, const float4 *__restrict__ gout, Adjoint adj,
     float *__restrict__ bparam, DebugCheck dc) {
+    grid_order();
     __shared__ float part[kBwdY * kBwdRows][6];
     const int x = blockIdx.x * kBwdX + threadIdx.x, y0 = (blockIdx.y * kBwdY + threadIdx.y) * kBwdRows;
     float4 fc[kBwdRows];
@@ -1011,6 +1012,7 @@ template <int RT>
 __global__ void __launch_bounds__(256, 4) k_bwd_record(int W, int H, int R, const uint32_t *__restrict__ foff,
                                                        const FrameRec *__restrict__ frec, Adjoint adj,
                                                        float *__restrict__ gcol) {
+    grid_order();
     const uint32_t n = __ldg(foff + (size_t)W * H);
     const uint32_t pairs = n / 2 + (n & 1);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gridDim.x * blockDim.x) {
@@ -1061,6 +1063,7 @@ __global__ void __launch_bounds__(256, 4) k_bwd_record(int W, int H, int R, cons
 // the blocks, then the 32 lane sums (value and compensation) added in a fixed
 // order by lane 0.
 __global__ void k_bwd_params(const float *__restrict__ part, int nblocks, float *__restrict__ out) {
+    grid_order();
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= 6) return;
     float s = 0.f, c = 0.f;
@@ -1192,8 +1195,8 @@ cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_c
     else AFR_BWD(false);
 #undef AFR_BWD
 #define AFR_REC(R_)                                                                                              \
-    k_bwd_record<R_><<<grid_for((size_t)c->P * c->b / 2, 256), 256, 0, s>>>(c->W, c->H, c->R, c->foff, c->frec, adj, \
-                                                                        grad_col)
+    launch_next(k_bwd_record<R_>, dim3(grid_for((size_t)c->P * c->b / 2, 256)), dim3(256), 0, s, c->W, c->H, c->R, c->foff, \
+                c->frec, adj, grad_col)
     if (grad_col) {
         switch (c->R) {   // the radii of the tuner and the default
             case 3: AFR_REC(3); break;
@@ -1203,7 +1206,7 @@ cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_c
         }
     }
 #undef AFR_REC
-    if (grad_prm) k_bwd_params<<<1, 6 * 32, 0, s>>>(c->bparam, backward_blocks(c->W, c->H), grad_prm);
+    if (grad_prm) launch_next(k_bwd_params, dim3(1), dim3(6 * 32), 0, s, c->bparam, backward_blocks(c->W, c->H), grad_prm);
     return cudaGetLastError();
 }
 

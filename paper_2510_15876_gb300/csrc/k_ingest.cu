@@ -417,6 +417,7 @@ __global__ void __launch_bounds__(256) k_fifo_append(const float4 *__restrict__ 
                                                      float *__restrict__ q_t,
                                                      uint32_t *__restrict__ q_seq, void *__restrict__ q_col,
                                                      const float4 *__restrict__ world, float4 *__restrict__ q_world) {
+    grid_order();
     using CS = ColorStore<CT>;
     const uint32_t accepted = rank[n - 1] + flag[n - 1], t0 = *total;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -437,6 +438,7 @@ __global__ void __launch_bounds__(256) k_fifo_append(const float4 *__restrict__ 
 
 __global__ void k_fifo_advance(const uint32_t *__restrict__ flag, const uint32_t *__restrict__ rank, uint32_t n,
                                uint32_t *__restrict__ total) {
+    grid_order();
     *total += rank[n - 1] + flag[n - 1];
 }
 
@@ -446,10 +448,9 @@ cudaError_t run_fifo(AfrContext *c, const float4 *pos, const void *col, const fl
     const int g = grid_for(n, 256);
     cudaError_t e = scan_exclusive(c->fifo_flag, c->fifo_rank, n, c->fifo_scan, s);
     if (e != cudaSuccess) return e;
-    k_fifo_append<CT><<<g, 256, 0, s>>>(pos, col, mo, n, c->fifo_flag, c->fifo_rank, seq0, (uint32_t)c->fifo_n,
-                                        c->q_total, c->q_xm, c->q_t, c->q_seq, c->q_col, world,
-                                        c->q_world);
-    k_fifo_advance<<<1, 1, 0, s>>>(c->fifo_flag, c->fifo_rank, n, c->q_total);
+    launch_next(k_fifo_append<CT>, dim3(g), dim3(256), 0, s, pos, col, mo, n, c->fifo_flag, c->fifo_rank, seq0,
+                (uint32_t)c->fifo_n, c->q_total, c->q_xm, c->q_t, c->q_seq, c->q_col, world, c->q_world);
+    launch_next(k_fifo_advance, dim3(1), dim3(1), 0, s, c->fifo_flag, c->fifo_rank, n, c->q_total);
     return cudaGetLastError();
 }
 
