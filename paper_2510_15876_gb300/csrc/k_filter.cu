@@ -849,7 +849,9 @@ struct PixelSums {
 // union of their discs, so a record is read once for all of them. Bound: the
 // sectors of L1 (a warp's lanes read records of neighbouring bins, one 32-byte
 // sector each): 512x512x8, 325 us with a pixel a thread that also searched its
-// exponent shift again, now 217 us (two rows a thread 237, four 302: registers).
+// exponent shift again, 217 us so (two rows a thread 237, four 302: registers),
+// now 207 with the next record loaded ahead and five CTAs a SM (235 when the
+// compiler takes the registers for four).
 // The filter's gather, lanes over records, takes 176 us, but sums in another
 // order.
 constexpr int kBwdX = 32, kBwdY = 4;
@@ -858,7 +860,7 @@ constexpr int kPartRows = 4;   // rows of one partial
 static_assert(kBwdY * kBwdRows % kPartRows == 0, "a CTA holds whole partials");
 
 template <bool PARAMS>
-__global__ void __launch_bounds__(kBwdX * kBwdY) k_bwd_pixel(
+__global__ void __launch_bounds__(kBwdX * kBwdY, 5) k_bwd_pixel(
     int W, int H, int R, int S_, int ntx, float window, float eps, AfrParams prm, const float4 *__restrict__ grad,
     const TilePartial *__restrict__ tiles, const float2 *__restrict__ sigma, const float4 *__restrict__ fconst,
     const uint32_t *__restrict__ foff, const FrameRec *__restrict__ frec, const float4 *__restrict__ gout, Adjoint adj,
@@ -890,8 +892,11 @@ __global__ void __launch_bounds__(kBwdX * kBwdY) k_bwd_pixel(
                     }
                 }
             }
+            if (e0 >= e1) continue;
+            FrameRec next = load_rec(frec + e0);
             for (uint32_t e = e0; e < e1; ++e) {
-                const FrameRec q = load_rec(frec + e);
+                const FrameRec q = next;
+                next = load_rec(frec + e + 1);   // the frame arrays end in padding
 #pragma unroll
                 for (int k = 0; k < kBwdRows; ++k)
                     A[k].add(q.p, q.c, cx, (float)(y0 + k) + 0.5f, fc[k], e - beg[k] < end[k] - beg[k]);
