@@ -169,8 +169,8 @@ AFR_API AfrStatus afr_insert_samples(AfrContext *ctx, const AfrSampleBatch *batc
  *                afr_reset followed by afr_insert_samples would do (the
  *                batch's sequence numbers start at 0).
  *   queues_free  a CUDA event (cudaEvent_t) or NULL. The steps that read or
- *                write the queues (the reset, the copy of the queue states,
- *                the commit, the reconstructor-queue append) first wait for
+ *                write the queues (the reset, the commit, the
+ *                reconstructor-queue append) first wait for
  *                it on the stream; the binning before them (counting, bucket
  *                offsets, the 64-byte bucket records: scratch of this
  *                context) does not. Recorded when the previous image's
