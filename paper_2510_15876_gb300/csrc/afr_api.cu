@@ -136,6 +136,8 @@ cudaError_t launch_resident_count(AfrContext *c, cudaStream_t s) {
 }
 }  // namespace afr
 
+constexpr size_t kBatchAlone = 12u << 20;   // records of a context that takes its turn on one worker stream
+
 struct AfrBatch {
     std::vector<AfrContext *> ctxs;  // queue order (largest first)
     std::vector<int> user_index;     // caller's index of each queue position
@@ -821,11 +823,17 @@ AfrStatus afr_batch_create(AfrContext *const *ctxs, int32_t n, AfrBatch **out) {
     }
     b->grid = 3 * sms;
     // afr_batch_refresh: kBatchWorkers streams, each context on the one with
-    // the least work so far (work ~ its buffered slots), largest first
+    // the least work so far (work ~ its buffered slots), largest first. Contexts
+    // of kBatchAlone slots or more share one: side by side, their list passes
+    // disturb each other's order and the placements gather worse (four of
+    // 1280x720x16 3.54 ms, one after another 3.26; three of 1920x1080x8, 16.6M
+    // slots, 3.24 and 3.23), while smaller ones fill each other's gaps (five of
+    // 1280x720x8, 7.4M slots, 2.37 side by side, 2.52 in turn).
     const int nw = std::min(n, afr::kBatchWorkers);
     std::vector<double> load(nw, 0.0);
     for (int q = 0; q < n; ++q) {
-        const int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+        const bool alone = b->ctxs[q]->frame_cap >= kBatchAlone;
+        const int w = alone ? 0 : (int)(std::min_element(load.begin(), load.end()) - load.begin());
         b->worker_of.push_back(w);
         load[w] += (double)b->ctxs[q]->P * (b->ctxs[q]->b + 8);
     }

@@ -131,3 +131,24 @@ def test_overlapped_launches_keep_their_order(dev, w, h, depth, color, fifo):
             assert torch.equal(out, want) and torch.equal(tiles.view(torch.int32), want_tiles.view(torch.int32))
         for a, b in zip(plain.export_ring(), slow.export_ring()):
             assert np.array_equal(a, b)
+
+
+def test_batch_of_large_and_small_contexts(dev):
+    """Contexts above and below the size that takes its turn on one worker
+    stream: every image equals the calls in series, bit for bit."""
+    from paper_2510_15876_gb300.api import BatchReconstructor, Reconstructor
+    recs = []
+    for seed, (w, h, depth) in enumerate(((1280, 720, 16), (64, 48, 4), (1100, 800, 16), (320, 200, 8))):
+        g = torch.Generator(dev).manual_seed(seed)
+        n = w * h * depth
+        pos = torch.rand(n, 4, generator=g, device=dev) * torch.tensor([w - 0.5, h - 0.5, 1.0, 1.0], device=dev)
+        rec = Reconstructor(w, h, depth, color_type="f16", device=dev)
+        rec.insert(pos, torch.rand(n, 4, generator=g, device=dev).half(), torch.randn(n, 2, generator=g, device=dev))
+        recs.append(rec)
+    got = [img.clone() for img in BatchReconstructor(recs).refresh(1.0)]
+    for rec, img in zip(recs, got):
+        rec.estimate_gradients(1.0)
+        rec.reproject(1.0)
+        want = rec.reconstruct(1.0)
+        torch.cuda.synchronize()
+        assert torch.equal(img, want)
