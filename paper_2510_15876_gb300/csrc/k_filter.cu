@@ -853,33 +853,36 @@ struct PixelSums {
 // now 207 with the next record loaded ahead and five CTAs a SM (235 when the
 // compiler takes the registers for four).
 // The filter's gather, lanes over records, takes 176 us, but sums in another
-// order.
+// order. A small image gets a pixel a thread (the same sums): with three its few
+// CTAs leave most of the GPU idle behind one thread's walk (parameter gradients,
+// 8 deep: 128x128 72 -> 37 us, 256x256 129 -> 103; 352x288, 264 CTAs of three
+// rows, 140 -> 147, so the line lies at one and a half CTAs a SM).
 constexpr int kBwdX = 32, kBwdY = 4;
 constexpr int kBwdRows = 3;
 constexpr int kPartRows = 4;   // rows of one partial
-static_assert(kBwdY * kBwdRows % kPartRows == 0, "a CTA holds whole partials");
+static_assert(kBwdY % kPartRows == 0, "a CTA holds whole partials");
 
-template <bool PARAMS>
+template <bool PARAMS, int ROWS>
 __global__ void __launch_bounds__(kBwdX * kBwdY, 5) k_bwd_pixel(
     int W, int H, int R, int S_, int ntx, float window, float eps, AfrParams prm, const float4 *__restrict__ grad,
     const TilePartial *__restrict__ tiles, const float2 *__restrict__ sigma, const float4 *__restrict__ fconst,
     const uint32_t *__restrict__ foff, const FrameRec *__restrict__ frec, const float4 *__restrict__ gout, Adjoint adj,
     float *__restrict__ bparam, DebugCheck dc) {
     grid_order();
-    __shared__ float part[kBwdY * kBwdRows][6];
-    const int x = blockIdx.x * kBwdX + threadIdx.x, y0 = (blockIdx.y * kBwdY + threadIdx.y) * kBwdRows;
-    float4 fc[kBwdRows];
-    PixelSums<PARAMS> A[kBwdRows];
+    __shared__ float part[kBwdY * ROWS][6];
+    const int x = blockIdx.x * kBwdX + threadIdx.x, y0 = (blockIdx.y * kBwdY + threadIdx.y) * ROWS;
+    float4 fc[ROWS];
+    PixelSums<PARAMS> A[ROWS];
     if (x < W && y0 < H) {
 #pragma unroll
-        for (int k = 0; k < kBwdRows; ++k) fc[k] = __ldg(fconst + (size_t)min(y0 + k, H - 1) * W + x);
+        for (int k = 0; k < ROWS; ++k) fc[k] = __ldg(fconst + (size_t)min(y0 + k, H - 1) * W + x);
         const float cx = (float)x + 0.5f;
-        for (int v = max(-R, -y0); v <= min(R + kBwdRows - 1, H - 1 - y0); ++v) {
+        for (int v = max(-R, -y0); v <= min(R + ROWS - 1, H - 1 - y0); ++v) {
             // records of each pixel's run of the row, and of the widest
             const uint32_t *row = foff + (size_t)(y0 + v) * W;
-            uint32_t beg[kBwdRows], end[kBwdRows], e0 = 0xFFFFFFFFu, e1 = 0;
+            uint32_t beg[ROWS], end[ROWS], e0 = 0xFFFFFFFFu, e1 = 0;
 #pragma unroll
-            for (int k = 0; k < kBwdRows; ++k) {
+            for (int k = 0; k < ROWS; ++k) {
                 beg[k] = end[k] = 0;
                 if (v - k >= -R && v - k <= R && y0 + k < H) {
                     const int hw = half_width(R, v - k);
@@ -898,13 +901,13 @@ __global__ void __launch_bounds__(kBwdX * kBwdY, 5) k_bwd_pixel(
                 const FrameRec q = next;
                 next = load_rec(frec + e + 1);   // the frame arrays end in padding
 #pragma unroll
-                for (int k = 0; k < kBwdRows; ++k)
+                for (int k = 0; k < ROWS; ++k)
                     A[k].add(q.p, q.c, cx, (float)(y0 + k) + 0.5f, fc[k], e - beg[k] < end[k] - beg[k]);
             }
         }
     }
 #pragma unroll
-    for (int k = 0; k < kBwdRows; ++k) {
+    for (int k = 0; k < ROWS; ++k) {
         const int y = y0 + k;
         float gp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (x < W && y < H) {
@@ -939,13 +942,13 @@ __global__ void __launch_bounds__(kBwdX * kBwdY, 5) k_bwd_pixel(
                 float v = gp[i];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (threadIdx.x == 0) part[threadIdx.y * kBwdRows + k][i] = v;
+                if (threadIdx.x == 0) part[threadIdx.y * ROWS + k][i] = v;
             }
         }
     }
     if (PARAMS) {
         __syncthreads();
-        constexpr int kParts = kBwdY * kBwdRows / kPartRows;
+        constexpr int kParts = kBwdY * ROWS / kPartRows;
         const int t = threadIdx.y * kBwdX + threadIdx.x, j = t / 6, i = t % 6, py = blockIdx.y * kParts + j;
         if (j < kParts && py < (H + kPartRows - 1) / kPartRows) {
             float acc = 0.f;
@@ -1188,16 +1191,21 @@ cudaError_t launch_filter(AfrContext *c, float t_now, bool adaptive, float4 *out
 
 cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_col, float *grad_prm,
                             cudaStream_t s) {
-    const dim3 block(kBwdX, kBwdY), grid((c->W + kBwdX - 1) / kBwdX, (c->H + kBwdY * kBwdRows - 1) / (kBwdY * kBwdRows));
+    const auto bands = [&](int rows) { return (c->H + kBwdY * rows - 1) / (kBwdY * rows); };
+    const int cols = (c->W + kBwdX - 1) / kBwdX;
+    const int rows = (long long)cols * bands(kBwdRows) < 3ll * device_sms() / 2 ? 1 : kBwdRows;
+    const dim3 block(kBwdX, kBwdY), grid(cols, bands(rows));
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
     const Adjoint adj{c->bgrad, reinterpret_cast<float2 *>(c->bgrad + c->P)};
     const AfrParams &prm = c->recon_params;
-#define AFR_BWD(P_)                                                                                              \
-    k_bwd_pixel<P_><<<grid, block, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, prm,   \
+#define AFR_BWD(P_, N_)                                                                                          \
+    k_bwd_pixel<P_, N_><<<grid, block, 0, s>>>(c->W, c->H, c->R, c->S, c->ntx, c->cfg.window, c->cfg.eps_grad, prm,   \
                                            c->grad, c->tiles, c->sigma, c->fconst, c->foff, c->frec, grad_rgb, adj, \
                                            c->bparam, dc)
-    if (grad_prm) AFR_BWD(true);
-    else AFR_BWD(false);
+    if (grad_prm && rows == 1) AFR_BWD(true, 1);
+    else if (grad_prm) AFR_BWD(true, kBwdRows);
+    else if (rows == 1) AFR_BWD(false, 1);
+    else AFR_BWD(false, kBwdRows);
 #undef AFR_BWD
 #define AFR_REC(R_)                                                                                              \
     launch_next(k_bwd_record<R_>, dim3(grid_for((size_t)c->P * c->b / 2, 256)), dim3(256), 0, s, c->W, c->H, c->R, c->foff, \
