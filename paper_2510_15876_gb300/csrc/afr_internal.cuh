@@ -239,7 +239,9 @@ __device__ __forceinline__ float bin_place(float xp, float yp) {
     return __int_as_float((int)floorf(yp) * kPitch + (int)floorf(xp));
 }
 
-// 256-bit accesses of a frame record (read-only path for the load)
+// 256-bit accesses of a frame record. The load takes the read-only path and may
+// be scheduled freely: no kernel that the filter's passes overlap writes records
+// (they are placed before k_sigma and k_bwd_pixel, ordinary launches).
 __device__ __forceinline__ FrameRec load_rec(const FrameRec *r) {
     FrameRec v;
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -396,6 +398,20 @@ inline void launch_next(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem
 __device__ __forceinline__ void grid_order() {
     asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
 }
+
+// Memory that the kernel launched just before writes. A kernel started by
+// launch_next may be resident while that happens, so for its lifetime the
+// memory is not read-only: it is read with ordinary loads, which neither the
+// compiler nor the read-only path can take from before grid_order's wait
+// (no __ldg, no __restrict__). What kernels further back wrote is complete
+// before a kernel becomes resident, for it is launched only when every block of
+// its predecessor is past its own wait; the read-only path may serve that.
+template <typename T>
+struct Fresh {
+    const T *p;
+    __host__ __device__ Fresh(const T *q) : p(q) {}
+    __device__ __forceinline__ const T &operator[](size_t i) const { return p[i]; }
+};
 
 // ---- launch wrappers (one per translation unit) ------------------------------
 // Each returns cudaSuccess or the launch error.

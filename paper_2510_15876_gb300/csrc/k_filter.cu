@@ -517,8 +517,8 @@ __device__ __forceinline__ void prefetch_tile(const TileSmem &t, int cols, int r
 
 // Pixels past the right or bottom edge repeat the edge pixel (never stored).
 __device__ __forceinline__ float4 load_const(int i, int W, int H, int x0, int y0, int tw,
-                                             const float4 *__restrict__ fconst) {
-    return __ldg(fconst + (size_t)min(y0 + i / tw, H - 1) * W + min(x0 + i % tw, W - 1));
+                                             Fresh<float4> fconst) {
+    return fconst[(size_t)min(y0 + i / tw, H - 1) * W + min(x0 + i % tw, W - 1)];
 }
 
 // Sums of one 2x2 pixel block by one warp: the block (lx, ly) of the tile at
@@ -682,7 +682,7 @@ __device__ __forceinline__ void store_block(const ForwardSums<KAHAN> &A, int W, 
 // Tile of (2 * tbx) x (2 * 32 / tbx) pixels per CTA: 32 blocks of 2x2, four
 // per warp; its upper 1 / 2^lsplit for images whose tiles would not fill the GPU.
 template <bool KAHAN, bool VAR>
-__global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx, int lsplit, const float4 *__restrict__ fconst,
+__global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx, int lsplit, Fresh<float4> fconst,
                                                    const uint32_t *__restrict__ foff, const FrameRec *frec,
                                                    float4 *__restrict__ out, DebugCheck dc) {
     grid_order();
@@ -819,6 +819,10 @@ __global__ void __launch_bounds__(256, 3) k_batch(const BatchCtx *__restrict__ c
 struct Adjoint {
     float4 *k;
     float2 *g;
+};
+struct AdjointRead {   // for the pass launched just after
+    Fresh<float4> k;
+    Fresh<float2> g;
 };
 
 // Weighted sums of one pixel over the records of its disc, in frame order. The
@@ -988,7 +992,7 @@ __device__ __forceinline__ void add_pixel(float4 k, float2 g, float w, float3 &a
 // One record: RT >= 0 is R at compile time (every pixel at a constant offset)
 // for discs inside the image; the others loop.
 template <int RT>
-__device__ float3 record_gradient(const RecordAt &r, int W, int H, int R, Adjoint adj) {
+__device__ float3 record_gradient(const RecordAt &r, int W, int H, int R, AdjointRead adj) {
     float3 a = make_float3(0.f, 0.f, 0.f);
     if (RT >= 0 && r.qx >= RT && r.qy >= RT && r.qx < W - RT && r.qy < H - RT) {
         size_t p = (size_t)(r.qy - RT) * W + r.qx;
@@ -998,8 +1002,8 @@ __device__ float3 record_gradient(const RecordAt &r, int W, int H, int R, Adjoin
 #pragma unroll
             for (int dx = -RT; dx <= RT; ++dx) {
                 if (dx * dx + dy * dy > RT * RT) continue;
-                const float4 k = __ldg(adj.k + p + dx);
-                add_pixel(k, __ldg(adj.g + p + dx), pixel_weight(k, r.fx - (float)dx, dy2, r.a2), a);
+                const float4 k = adj.k[p + dx];
+                add_pixel(k, adj.g[p + dx], pixel_weight(k, r.fx - (float)dx, dy2, r.a2), a);
             }
         }
         return a;
@@ -1009,8 +1013,8 @@ __device__ float3 record_gradient(const RecordAt &r, int W, int H, int R, Adjoin
         const int hw = half_width(R, dy);
         const size_t p = (size_t)(r.qy + dy) * W + r.qx;
         for (int dx = max(-hw, -r.qx); dx <= min(hw, W - 1 - r.qx); ++dx) {
-            const float4 k = __ldg(adj.k + p + dx);
-            add_pixel(k, __ldg(adj.g + p + dx), pixel_weight(k, r.fx - (float)dx, dy2, r.a2), a);
+            const float4 k = adj.k[p + dx];
+            add_pixel(k, adj.g[p + dx], pixel_weight(k, r.fx - (float)dx, dy2, r.a2), a);
         }
     }
     return a;
@@ -1018,7 +1022,7 @@ __device__ float3 record_gradient(const RecordAt &r, int W, int H, int R, Adjoin
 
 template <int RT>
 __global__ void __launch_bounds__(256, 4) k_bwd_record(int W, int H, int R, const uint32_t *__restrict__ foff,
-                                                       const FrameRec *__restrict__ frec, Adjoint adj,
+                                                       const FrameRec *__restrict__ frec, AdjointRead adj,
                                                        float *__restrict__ gcol) {
     grid_order();
     const uint32_t n = __ldg(foff + (size_t)W * H);
@@ -1041,8 +1045,8 @@ __global__ void __launch_bounds__(256, 4) k_bwd_record(int W, int H, int R, cons
                 for (int dx = -RT; dx <= RT + 1; ++dx) {
                     const bool in = dx * dx + dy * dy <= RT * RT, in1 = (dx - 1) * (dx - 1) + dy * dy <= RT * RT;
                     if (!in && !in1) continue;
-                    const float4 k = __ldg(adj.k + p + dx);
-                    const float2 g = __ldg(adj.g + p + dx);
+                    const float4 k = adj.k[p + dx];
+                    const float2 g = adj.g[p + dx];
                     if (in) add_pixel(k, g, pixel_weight(k, u.fx - (float)dx, yu, u.a2), a);
                     float w = pixel_weight(k, vx - (float)dx, yv, v.a2);
                     if (!in && s == 0) w = 0.f;
@@ -1070,7 +1074,7 @@ __global__ void __launch_bounds__(256, 4) k_bwd_record(int W, int H, int R, cons
 // parameter, each lane a compensated (Kahan) FP32 sum over a strided share of
 // the blocks, then the 32 lane sums (value and compensation) added in a fixed
 // order by lane 0.
-__global__ void k_bwd_params(const float *__restrict__ part, int nblocks, float *__restrict__ out) {
+__global__ void k_bwd_params(Fresh<float> part, int nblocks, float *__restrict__ out) {
     grid_order();
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= 6) return;
@@ -1209,7 +1213,7 @@ cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_c
 #undef AFR_BWD
 #define AFR_REC(R_)                                                                                              \
     launch_next(k_bwd_record<R_>, dim3(grid_for((size_t)c->P * c->b / 2, 256)), dim3(256), 0, s, c->W, c->H, c->R, c->foff, \
-                c->frec, adj, grad_col)
+                c->frec, AdjointRead{adj.k, adj.g}, grad_col)
     if (grad_col) {
         switch (c->R) {   // the radii of the tuner and the default
             case 3: AFR_REC(3); break;

@@ -52,6 +52,9 @@ struct Bucket {
     uint4 *r;    // [NP * batch_cap]
 };
 
+// Batch index of record k.
+__device__ __forceinline__ uint32_t batch_index(const Bucket &bk, uint32_t k) { return bk.r[(size_t)NP * k].w; }
+
 // Destination planes of the queues (slot p * b + s).
 struct Queues {
     float4 *xm;        // x, y, m_x, m_y
@@ -237,7 +240,8 @@ __device__ __forceinline__ void put_record(const uint4 &a, const uint4 &q1, cons
 // kCommitTile consecutive records at a time and keeps their batch indices in
 // shared memory, where the rank scans find all of a pixel's records but
 // those of pixels crossing the tile's ends. The queue states are those before
-// the batch (none after a reset); the new ones go to state1.
+// the batch (none after a reset); the new ones go to state1. The records are
+// what the scatter, launched just before, writes: ordinary loads (Fresh).
 constexpr int kCommitTile = 256;
 
 template <int CT>
@@ -249,15 +253,14 @@ __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__re
     uint32_t n = __ldg(poff + P);
     if (!AFR_CHECK(n <= dc.cap, dc.derr)) n = 0;
     const uint32_t ub = (uint32_t)b;
-    const uint32_t *ridx = reinterpret_cast<const uint32_t *>(bk.r) + 3;   // batch index of record k: ridx[16 k]
     for (uint32_t t0 = blockIdx.x * (uint32_t)kCommitTile; t0 < n; t0 += gridDim.x * (uint32_t)kCommitTile) {
         const uint32_t e = t0 + threadIdx.x, t1 = min(t0 + (uint32_t)kCommitTile, n);
         uint4 a = make_uint4(0u, 0u, 0u, kInvalid), q1 = a, q2 = a, q3 = a;
         if (e < n) {
-            a = __ldg(bk.r + (size_t)NP * e);
-            q1 = __ldg(bk.r + (size_t)NP * e + 1);
-            q2 = __ldg(bk.r + (size_t)NP * e + 2);
-            if (q.world) q3 = __ldg(bk.r + (size_t)NP * e + 3);
+            a = bk.r[(size_t)NP * e];
+            q1 = bk.r[(size_t)NP * e + 1];
+            q2 = bk.r[(size_t)NP * e + 2];
+            if (q.world) q3 = bk.r[(size_t)NP * e + 3];
         }
         sidx[threadIdx.x] = a.w;
         __syncthreads();
@@ -276,7 +279,7 @@ __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__re
             uint32_t rank = 0, dead = 0;
             const uint32_t s0 = max(beg, t0), s1 = min(end, t1);
             for (uint32_t k = beg; k < min(end, t0); ++k) {
-                const uint32_t w = __ldg(ridx + (size_t)16 * k);
+                const uint32_t w = batch_index(bk, k);
                 rank += w < a.w;
                 dead += w == kInvalid;
             }
@@ -286,7 +289,7 @@ __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__re
                 dead += w == kInvalid;
             }
             for (uint32_t k = max(beg, t1); k < end; ++k) {
-                const uint32_t w = __ldg(ridx + (size_t)16 * k);
+                const uint32_t w = batch_index(bk, k);
                 rank += w < a.w;
                 dead += w == kInvalid;
             }
@@ -308,7 +311,7 @@ __global__ void __launch_bounds__(kCommitTile) k_pix_commit(const uint32_t *__re
 template <int CT>
 __global__ void __launch_bounds__(256) k_pix_finish(const uint32_t *__restrict__ poff, uint32_t P, int b,
                                                     uint32_t seq0, Bucket bk, Queues q, bool reset,
-                                                    const uint32_t *__restrict__ state1,
+                                                    Fresh<uint32_t> state1,
                                                     unsigned long long *__restrict__ dcount,
                                                     uint32_t *__restrict__ q_total, DebugCheck dc) {
     grid_order();
@@ -320,7 +323,6 @@ __global__ void __launch_bounds__(256) k_pix_finish(const uint32_t *__restrict__
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t ub = (uint32_t)b;
-    const uint32_t *ridx = reinterpret_cast<const uint32_t *>(bk.r) + 3;
     const uint32_t n = __ldg(poff + P);
     for (uint32_t base = warp * 32u; base < P; base += nwarps * 32u) {
         const uint32_t p = base + (uint32_t)lane;
@@ -343,7 +345,7 @@ __global__ void __launch_bounds__(256) k_pix_finish(const uint32_t *__restrict__
                 const uint32_t k = k0 + (uint32_t)lane;
                 unsigned long long key = 0ull;
                 if (k < end) {
-                    const uint32_t w = __ldg(ridx + (size_t)16 * k);
+                    const uint32_t w = batch_index(bk, k);
                     if (w != kInvalid) key = ((unsigned long long)(w + 1u) << 32) | k;
                 }
                 nl += (uint32_t)__popc(__ballot_sync(0xffffffffu, key != 0ull));
@@ -357,11 +359,11 @@ __global__ void __launch_bounds__(256) k_pix_finish(const uint32_t *__restrict__
                 const uint32_t k = (uint32_t)top, rank = nl - 32u + (uint32_t)lane;   // position in insertion order
                 const size_t dst = (size_t)px * ub + ((st >> 16) + rank) % ub;
                 if (AFR_CHECK(dst < q.nslots && k < end, dc.derr)) {
-                    const uint4 a = __ldg(bk.r + (size_t)NP * k);
-                    const uint4 q1 = __ldg(bk.r + (size_t)NP * k + 1);
-                    const uint4 q2 = __ldg(bk.r + (size_t)NP * k + 2);
+                    const uint4 a = bk.r[(size_t)NP * k];
+                    const uint4 q1 = bk.r[(size_t)NP * k + 1];
+                    const uint4 q2 = bk.r[(size_t)NP * k + 2];
                     uint4 q3 = make_uint4(0u, 0u, 0u, 0u);
-                    if (q.world) q3 = __ldg(bk.r + (size_t)NP * k + 3);
+                    if (q.world) q3 = bk.r[(size_t)NP * k + 3];
                     put_record<CT>(a, q1, q2, q3, dst, seq0 + a.w, q);
                 }
             }
@@ -412,7 +414,7 @@ template <int CT>
 __global__ void __launch_bounds__(256) k_fifo_append(const float4 *__restrict__ pos, const void *__restrict__ col,
                                                      const float2 *__restrict__ mo, uint32_t n,
                                                      const uint32_t *__restrict__ flag,
-                                                     const uint32_t *__restrict__ rank, uint32_t seq0, uint32_t N,
+                                                     Fresh<uint32_t> rank, uint32_t seq0, uint32_t N,
                                                      const uint32_t *__restrict__ total, float4 *__restrict__ q_xm,
                                                      float *__restrict__ q_t,
                                                      uint32_t *__restrict__ q_seq, void *__restrict__ q_col,

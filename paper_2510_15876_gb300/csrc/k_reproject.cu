@@ -224,7 +224,7 @@ template <int CT, bool CAM>
 __global__ void __launch_bounds__(256) k_place_queues(int W, int H, float t_now, Camera cam, const float4 *__restrict__ world,
                                                const float4 *__restrict__ r_xm,
                                                const float *__restrict__ r_t, const void *__restrict__ r_col, uint32_t P,
-                                               const uint32_t *__restrict__ foff, const uint2 *__restrict__ flist,
+                                               const uint32_t *__restrict__ foff, Fresh<uint2> flist,
                                                uint32_t *__restrict__ fcur, uint32_t *__restrict__ amin2,
                                                FrameRec *__restrict__ frec, unsigned long long *__restrict__ dcount,
                                                DebugCheck dc, uint32_t nsrc) {
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256) k_place_queues(int W, int H, float t_now,
         uint2 en = make_uint2(0u, 0u);   // slot, sequence number
         bool ok = e < n;
         if (ok) {
-            en = __ldg(flist + e);
+            en = flist[e];
             ok = AFR_CHECK(en.x < nsrc, dc.derr);
         }
         const uint32_t i = en.x, sq = en.y;
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(256) k_place_queues(int W, int H, float t_now,
         uint32_t rank = 0;
         if (end - beg <= (uint32_t)kSortedBinMax) {
 #pragma unroll 4
-            for (uint32_t k = beg; k < end; ++k) rank += __ldg(&flist[k].y) < sq;
+            for (uint32_t k = beg; k < end; ++k) rank += flist[k].y < sq;
         } else {
             rank = unsorted_rank(fcur, mv.bin, beg, dcount);
         }
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int 
                                                     const float4 *__restrict__ r_xm,
                                                     const float *__restrict__ r_t, const uint32_t *__restrict__ r_seq,
                                                     const void *__restrict__ r_col, const uint32_t *__restrict__ foff,
-                                                    const uint32_t *__restrict__ flist, uint32_t *__restrict__ fcur,
+                                                    Fresh<uint32_t> flist, uint32_t *__restrict__ fcur,
                                                     uint32_t *__restrict__ amin2, FrameRec *__restrict__ frec,
                                                     unsigned long long *__restrict__ dcount, DebugCheck dc) {
     grid_order();
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int 
         const uint32_t len = end - beg;
         if (len <= (uint32_t)kSortedBinMax) {
             for (uint32_t k = beg & ~3u; k < end; k += 4) {
-                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(flist + k));
+                const uint4 v = *reinterpret_cast<const uint4 *>(&flist[k]);
                 const uint32_t j = k - beg;   // entries outside the bin wrap past its length or lie beyond it
                 rank += (uint32_t)((j < len) & (v.x < sq)) + (uint32_t)((j + 1u < len) & (v.y < sq)) +
                         (uint32_t)((j + 2u < len) & (v.z < sq)) + (uint32_t)((j + 3u < len) & (v.w < sq));

@@ -28,10 +28,11 @@ struct Items {
 __device__ __forceinline__ Items load_items(const uint32_t *p, size_t i, size_t n) {
     Items r;
     if (i + kScanItems <= n) {
-        asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
             : "=r"(r.v[0]), "=r"(r.v[1]), "=r"(r.v[2]), "=r"(r.v[3]), "=r"(r.v[4]), "=r"(r.v[5]), "=r"(r.v[6]),
               "=r"(r.v[7])
-            : "l"(p + i));
+            : "l"(p + i)
+            : "memory");   // not before grid_order's wait
     } else {
 #pragma unroll
         for (int k = 0; k < kScanItems; ++k) r.v[k] = i + k < n ? p[i + k] : 0u;
@@ -124,18 +125,18 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *sums, size
 // scanned: sums holds exclusive prefixes already; wide: out is 32-byte aligned
 // (a caller's own array need not be)
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint32_t *in, uint32_t *out, size_t n,
-                                                              const uint32_t *sums, bool scanned, bool wide, ScanWith with) {
+                                                              Fresh<uint32_t> sums, bool scanned, bool wide, ScanWith with) {
     grid_order();
     __shared__ uint32_t tot;
     const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
     Items r = load_items(in, base, n);
     uint32_t before = 0;
     if (!scanned)
-        for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) before += __ldg(sums + i);
+        for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) before += sums[i];
     uint32_t acc = 0;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) acc += r.v[k];
-    const uint32_t prefix = scanned ? __ldg(sums + blockIdx.x) : block_sum(before);
+    const uint32_t prefix = scanned ? sums[blockIdx.x] : block_sum(before);
     uint32_t ex = block_excl_scan(acc, &tot) + prefix;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
