@@ -352,7 +352,8 @@ AFR_API AfrStatus afr_reconstruct_ex(AfrContext *ctx, float t_now, const AfrPara
  * branches are done, afr_reconstruct_ex. reads_done: a CUDA event or NULL;
  * recorded on stream when both branches are done with the sample buffers,
  * before the filter. Results, errors and ordering rules as the calls it stands
- * for; can be captured in a CUDA graph. */
+ * for, but every argument is checked first: a refused call launches nothing and
+ * leaves the context as it was. Can be captured in a CUDA graph. */
 AFR_API AfrStatus afr_refresh(AfrContext *ctx, float t_now, const float *view_proj_host, const AfrParams *params,
                               uint32_t flags, float *out_rgbw_dev, AfrTileStats *tiles_dev, afr_stream_t side,
                               afr_event_t reads_done, afr_stream_t stream);

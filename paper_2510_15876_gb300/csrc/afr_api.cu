@@ -366,10 +366,52 @@ AfrStatus afr_insert_samples_ex(AfrContext *c, const AfrSampleBatch *batch, uint
                        reinterpret_cast<cudaStream_t>(stream));
 }
 
+// What the arguments of each call are refused for, before it does anything
+// (afr_refresh asks for all the calls it stands for first).
+static AfrStatus check_gradients(AfrContext *c, float t_now) {
+    if (!std::isfinite(t_now)) return fail(c, AFR_ERR_INVALID_ARG, "afr_estimate_gradients: t_now not finite");
+    return AFR_OK;
+}
+
+static AfrStatus check_feedback(AfrContext *c, const AfrTileStats *out_dev) {
+    if (!out_dev) return fail(c, AFR_ERR_INVALID_ARG, "afr_tile_feedback: null output");
+    return AFR_OK;
+}
+
+static AfrStatus check_reproject(AfrContext *c, float t_now) {
+    if (!std::isfinite(t_now)) return fail(c, AFR_ERR_INVALID_ARG, "afr_reproject: t_now not finite");
+    return AFR_OK;
+}
+
+static AfrStatus check_camera(AfrContext *c, float t_now, const float *view_proj) {
+    if (!std::isfinite(t_now) || !view_proj)
+        return fail(c, AFR_ERR_INVALID_ARG, "afr_reproject_camera: t_now not finite or null matrix");
+    for (int k = 0; k < 16; ++k)
+        if (!std::isfinite(view_proj[k])) return fail(c, AFR_ERR_INVALID_ARG, "afr_reproject_camera: matrix not finite");
+    if (!c->r_world) return fail(c, AFR_ERR_BAD_STATE, "afr_reproject_camera: context stores no world points");
+    return AFR_OK;
+}
+
+static bool params_ok(const AfrParams *p) {
+    const float v[6] = {p->alpha_s, p->beta_s, p->clamp_s, p->alpha_t, p->beta_t, p->clamp_t};
+    for (float f : v)
+        if (!std::isfinite(f)) return false;
+    return p->clamp_s > 0.f && p->clamp_t > 0.f;
+}
+
+static AfrStatus check_reconstruct(AfrContext *c, const AfrParams *params, uint32_t flags, const float *out_rgbw_dev) {
+    if (!params || !out_rgbw_dev || !aligned(out_rgbw_dev, 16))
+        return fail(c, AFR_ERR_INVALID_ARG, "afr_reconstruct: null or misaligned pointer");
+    if (!params_ok(params)) return fail(c, AFR_ERR_INVALID_ARG, "afr_reconstruct: parameters not finite/positive");
+    if (flags & ~(uint32_t)(AFR_RECON_KEEP_SIGMA | AFR_RECON_ADAPTIVE_SUPPORT | AFR_RECON_COVERAGE_RESET))
+        return fail(c, AFR_ERR_INVALID_ARG, "afr_reconstruct_ex: unknown flag");
+    return AFR_OK;
+}
+
 AfrStatus afr_estimate_gradients(AfrContext *c, float t_now, afr_stream_t stream) {
     Range nvtx_range("afr_estimate_gradients");
     if (!c) return AFR_ERR_INVALID_ARG;
-    if (!std::isfinite(t_now)) return fail(c, AFR_ERR_INVALID_ARG, "afr_estimate_gradients: t_now not finite");
+    if (const AfrStatus st = check_gradients(c, t_now)) return st;
     cudaError_t e = afr::launch_gradients(c, t_now, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "afr_estimate_gradients");
     c->grads_valid = true;
@@ -381,11 +423,7 @@ AfrStatus afr_estimate_gradients(AfrContext *c, float t_now, afr_stream_t stream
 AfrStatus afr_reproject_camera(AfrContext *c, float t_now, const float *view_proj, afr_stream_t stream) {
     Range nvtx_range("afr_reproject_camera");
     if (!c) return AFR_ERR_INVALID_ARG;
-    if (!std::isfinite(t_now) || !view_proj)
-        return fail(c, AFR_ERR_INVALID_ARG, "afr_reproject_camera: t_now not finite or null matrix");
-    for (int k = 0; k < 16; ++k)
-        if (!std::isfinite(view_proj[k])) return fail(c, AFR_ERR_INVALID_ARG, "afr_reproject_camera: matrix not finite");
-    if (!c->r_world) return fail(c, AFR_ERR_BAD_STATE, "afr_reproject_camera: context stores no world points");
+    if (const AfrStatus st = check_camera(c, t_now, view_proj)) return st;
     afr::Camera cam;
     for (int k = 0; k < 4; ++k) {
         cam.m[k] = view_proj[k];           // row 0
@@ -403,7 +441,7 @@ AfrStatus afr_reproject_camera(AfrContext *c, float t_now, const float *view_pro
 AfrStatus afr_reproject(AfrContext *c, float t_now, afr_stream_t stream) {
     Range nvtx_range("afr_reproject");
     if (!c) return AFR_ERR_INVALID_ARG;
-    if (!std::isfinite(t_now)) return fail(c, AFR_ERR_INVALID_ARG, "afr_reproject: t_now not finite");
+    if (const AfrStatus st = check_reproject(c, t_now)) return st;
     cudaError_t e = afr::launch_reproject(c, t_now, nullptr, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "afr_reproject");
     c->frame_valid = true;
@@ -412,24 +450,13 @@ AfrStatus afr_reproject(AfrContext *c, float t_now, afr_stream_t stream) {
     return AFR_OK;
 }
 
-static bool params_ok(const AfrParams *p) {
-    const float v[6] = {p->alpha_s, p->beta_s, p->clamp_s, p->alpha_t, p->beta_t, p->clamp_t};
-    for (float f : v)
-        if (!std::isfinite(f)) return false;
-    return p->clamp_s > 0.f && p->clamp_t > 0.f;
-}
-
 AfrStatus afr_reconstruct_ex(AfrContext *c, float t_now, const AfrParams *params, uint32_t flags,
                              float *out_rgbw_dev, afr_stream_t stream) {
     Range nvtx_range("afr_reconstruct_ex");
     if (!c) return AFR_ERR_INVALID_ARG;
-    if (!params || !out_rgbw_dev || !aligned(out_rgbw_dev, 16))
-        return fail(c, AFR_ERR_INVALID_ARG, "afr_reconstruct: null or misaligned pointer");
-    if (!params_ok(params)) return fail(c, AFR_ERR_INVALID_ARG, "afr_reconstruct: parameters not finite/positive");
+    if (const AfrStatus st = check_reconstruct(c, params, flags, out_rgbw_dev)) return st;
     bool keep = (flags & AFR_RECON_KEEP_SIGMA) != 0;
     const bool adaptive = (flags & AFR_RECON_ADAPTIVE_SUPPORT) != 0;
-    if (flags & ~(uint32_t)(AFR_RECON_KEEP_SIGMA | AFR_RECON_ADAPTIVE_SUPPORT | AFR_RECON_COVERAGE_RESET))
-        return fail(c, AFR_ERR_INVALID_ARG, "afr_reconstruct_ex: unknown flag");
     if (!c->frame_valid || c->frame_t != t_now)
         return fail(c, AFR_ERR_BAD_STATE, "afr_reconstruct: call afr_reproject for this t_now first");
     if (!keep && (!c->grads_valid || c->grads_t != t_now))
@@ -469,7 +496,7 @@ AfrStatus afr_reconstruct(AfrContext *c, float t_now, const AfrParams *params, f
 AfrStatus afr_tile_feedback(AfrContext *c, AfrTileStats *out_dev, afr_stream_t stream) {
     Range nvtx_range("afr_tile_feedback");
     if (!c) return AFR_ERR_INVALID_ARG;
-    if (!out_dev) return fail(c, AFR_ERR_INVALID_ARG, "afr_tile_feedback: null output");
+    if (const AfrStatus st = check_feedback(c, out_dev)) return st;
     if (!c->grads_valid) return fail(c, AFR_ERR_BAD_STATE, "afr_tile_feedback: call afr_estimate_gradients first");
     cudaError_t e = afr::launch_feedback(c, out_dev, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "afr_tile_feedback");
@@ -481,17 +508,24 @@ AfrStatus afr_refresh(AfrContext *c, float t_now, const float *view_proj, const 
                       afr_stream_t stream) {
     Range nvtx_range("afr_refresh");
     if (!c) return AFR_ERR_INVALID_ARG;
+    // everything that can be refused is, before anything is launched
+    AfrStatus st = check_gradients(c, t_now);
+    if (st == AFR_OK) st = check_feedback(c, tiles_dev);
+    if (st == AFR_OK) st = view_proj ? check_camera(c, t_now, view_proj) : check_reproject(c, t_now);
+    if (st == AFR_OK) st = check_reconstruct(c, params, flags, out_rgbw_dev);
+    if (st != AFR_OK) return st;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), g = reinterpret_cast<cudaStream_t>(side);
     cudaError_t e = cudaEventRecord(c->fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(g, c->fork, 0);
     if (e != cudaSuccess) return cuda_fail(c, e, "afr_refresh");
-    AfrStatus st = afr_estimate_gradients(c, t_now, side);
+    st = afr_estimate_gradients(c, t_now, side);
     if (st == AFR_OK) st = afr_tile_feedback(c, tiles_dev, side);
+    if (st == AFR_OK)
+        st = view_proj ? afr_reproject_camera(c, t_now, view_proj, stream) : afr_reproject(c, t_now, stream);
+    // whatever failed, stream waits for what side was given
+    e = cudaEventRecord(c->join, g);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->join, 0);
     if (st != AFR_OK) return st;
-    if ((e = cudaEventRecord(c->join, g)) != cudaSuccess) return cuda_fail(c, e, "afr_refresh");
-    st = view_proj ? afr_reproject_camera(c, t_now, view_proj, stream) : afr_reproject(c, t_now, stream);
-    if (st != AFR_OK) return st;
-    e = cudaStreamWaitEvent(s, c->join, 0);
     if (e == cudaSuccess && reads_done) e = cudaEventRecord(reinterpret_cast<cudaEvent_t>(reads_done), s);
     if (e != cudaSuccess) return cuda_fail(c, e, "afr_refresh");
     return afr_reconstruct_ex(c, t_now, params, flags, out_rgbw_dev, stream);

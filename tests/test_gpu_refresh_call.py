@@ -80,6 +80,60 @@ def test_refresh_refuses_what_its_calls_refuse(dev):
     assert torch.isfinite(img).all()
 
 
+def test_a_refused_refresh_launches_nothing(dev):
+    """After a refusal both streams are idle, so nothing still reads the queues
+    or writes the tile records when the caller's next batch arrives, and a
+    capture that a refusal happened in goes on."""
+    import ctypes
+    from paper_2510_15876_gb300.api import Reconstructor
+    w, h, depth, n = 1024, 768, 8, 1 << 21
+    batches = []
+    for seed in range(2):
+        g = torch.Generator(dev).manual_seed(seed)
+        pos = torch.rand(n, 4, generator=g, device=dev) * torch.tensor([w - 0.5, h - 0.5, 1.0, 1.0], device=dev)
+        batches.append((pos, torch.rand(n, 4, generator=g, device=dev), torch.randn(n, 2, generator=g, device=dev)))
+    rec, fresh = Reconstructor(w, h, depth, device=dev), Reconstructor(w, h, depth, device=dev)
+    rec.reserve(n)
+    rec._side = torch.cuda.Stream(dev, priority=-1)
+    main = torch.cuda.current_stream(dev)
+    out, tiles = torch.empty((h, w, 4), device=dev), torch.empty((rec.n_tiles, 8), device=dev)
+    default = L.AfrParams(1.0, 0.0, 3.0, 1.0, 0.0, 1.0)
+
+    def native(params=default, flags=0, image=out, stats=tiles):
+        st = rec.lib.afr_refresh(rec.h, 1.0, None, ctypes.byref(params), flags, image.data_ptr() if image is not None else None,
+                                 stats.data_ptr() if stats is not None else None, rec._side.cuda_stream, None, main.cuda_stream)
+        if st != L.AFR_OK:
+            raise L.AfrError(st, "refused")
+
+    calls = [lambda: rec.refresh(float("nan")), lambda: rec.refresh(1.0, params=(1, 0, -3, 1, 0, 1)),
+             lambda: rec.refresh(1.0, flags=64), lambda: rec.refresh(1.0, view_proj=np.full((4, 4), np.inf)),
+             lambda: rec.refresh(1.0, view_proj=VP), lambda: native(image=None), lambda: native(stats=None),
+             lambda: native(image=out.view(-1)[1:])]
+    fresh.insert(*batches[1])
+    want, want_tiles = fresh.refresh(1.0)
+    for call in calls:
+        rec.insert(*batches[0], reset=True)
+        torch.cuda.synchronize()
+        with pytest.raises(L.AfrError):
+            call()
+        assert rec._side.query() and main.query()
+        rec.insert(*batches[1], reset=True)
+        rec.refresh(1.0, out=out, tiles=tiles)
+        torch.cuda.synchronize()
+        assert torch.equal(out, want) and torch.equal(tiles.view(torch.int32), want_tiles.view(torch.int32))
+    graph = torch.cuda.CUDAGraph()
+    out.zero_(), tiles.zero_()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        for kw in (dict(view_proj=VP), dict(flags=64)):
+            with pytest.raises(L.AfrError):
+                rec.refresh(1.0, out=out, tiles=tiles, **kw)
+        rec.refresh(1.0, out=out, tiles=tiles)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and torch.equal(tiles.view(torch.int32), want_tiles.view(torch.int32))
+
+
 @pytest.mark.parametrize("w,h,depth,color,fifo", [
     (1, 1, 2, "f32", 0), (61, 43, 5, "bf16", 0), (640, 360, 8, "f16", 0), (300, 200, 4, "f32", 3 * 300 * 200)])
 def test_overlapped_launches_keep_their_order(dev, w, h, depth, color, fifo):
