@@ -595,7 +595,7 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
     auto load = [&](int i) {   // record i + lane (i itself may be negative)
         const bool ok = AFR_CHECK((uint32_t)(i + lane) < dc.cap + kFramePad, dc.derr);
         FrameRec r = load_rec(element(frec, ok ? i : 0));   // not ok: another record read, weight 0
-        if (!ok) r.p.w = __int_as_float(-1 - origin);
+        if (!ok) r.p.w = __int_as_float(origin - 1);   // a place before the box
         return r;
     };
     auto add = [&](const FrameRec &r, auto from_table) {
