@@ -506,10 +506,11 @@ __device__ __forceinline__ void load_offsets(TileSmem &t, int W, int H, int R, i
 
 // Asks L2 for the tile's records (rows x cols of offsets) while the first
 // blocks set up: they come from HBM, and a block's few iterations hide little of
-// that (1.5% at R 4, 5% for adaptive footprints).
-__device__ __forceinline__ void prefetch_tile(const TileSmem &t, int cols, int rows, const FrameRec *frec) {
+// that (1.5% at R 4, 5% for adaptive footprints). Nothing past the cap records
+// of the frame view is asked for, whatever the offsets say.
+__device__ __forceinline__ void prefetch_tile(const TileSmem &t, int cols, int rows, const FrameRec *frec, uint32_t cap) {
     for (int r = threadIdx.x >> 5; r < rows; r += blockDim.x >> 5) {
-        const uint32_t end = t.off[r * cols + cols - 1];
+        const uint32_t end = min(t.off[r * cols + cols - 1], cap);
         for (uint32_t i = t.off[r * cols] + 4u * (threadIdx.x & 31); i < end; i += 128u)   // 128-byte lines
             asm volatile("prefetch.global.L2 [%0];" ::"l"(frec + i));
     }
@@ -710,7 +711,7 @@ __global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx
     }
     load_offsets(ts, W, H, Rt, x0, y0, tw, th, foff);
     __syncthreads();
-    prefetch_tile(ts, tw + 2 * Rt + 1, th + 2 * Rt, frec0);
+    prefetch_tile(ts, tw + 2 * Rt + 1, th + 2 * Rt, frec0, dc.cap);
     for (int blk = warp; blk < 32 >> lsplit; blk += kWarps) {
         const int lx = blk & ((1 << ltbx) - 1), ly = blk >> ltbx;
         if (x0 + 2 * lx >= W || y0 + 2 * ly >= H) continue;   // warp-uniform

@@ -79,15 +79,16 @@ def test_inconsistent_frame_view_reaches_the_device_checks(dev):
     rec.close()
 
 
-def test_records_out_of_range_have_no_weight_in_any_block(dev):
-    """Every bin points past the records: each guarded read is replaced by
+@pytest.mark.parametrize("past", [64, 1 << 30])
+def test_records_out_of_range_have_no_weight_in_any_block(dev, past):
+    """Every bin points past the records, a little or far: each guarded read is replaced by
     another record's with weight 0, the image's first block (whose footprint box
     starts at negative rows and columns) included."""
     lib = L.load_debug()
     W, H, b = 20, 10, 4
     rec = _filled(dev, lib, W, H, b, seed=2)
     off, _, _ = rec.export_frame()
-    bad = np.ascontiguousarray((off.astype(np.int64) + W * H * b + 64).astype(np.uint32))
+    bad = np.ascontiguousarray((off.astype(np.int64) + W * H * b + past).astype(np.uint32))
     assert lib.afr_debug_set_frame_offsets(rec.h, bad.ctypes.data) == L.AFR_OK
     img = rec.reconstruct(1.0)
     assert rec.status() == L.AFR_ERR_DEVICE_CHECK
