@@ -308,6 +308,7 @@ struct TileSums {
 __device__ __forceinline__ void add_pixel(const PixelRead &v, int x, int y, int W, int H, float4 *__restrict__ grad,
                                           TileSums &t) {
     const int p = y * W + x;
+    t.age = df_more(t.age, v.ps.w);   // of every buffered sample, too old for any weight or not
     if (isnan(v.c.x)) {
         grad[p] = make_float4(0.f, 0.f, 0.f, v.c.x);
         return;
@@ -327,7 +328,6 @@ __device__ __forceinline__ void add_pixel(const PixelRead &v, int x, int y, int 
     t.gx += gx;
     t.gy += gy;
     t.gt += v.ps.z;
-    t.age = df_more(t.age, v.ps.w);
     t.sw = df_more(t.sw, v.ps.x);
     const dfloat q = two_prod(v.ps.x, v.c.x);
     t.swm = df_more(t.swm, q.h);
