@@ -278,6 +278,11 @@ __device__ __forceinline__ T lanes_sum(T v) {
     return v;
 }
 
+// The weights of samples 25 time units old and more are below the least normal
+// number, and their products with the means would keep a few bits only. A power
+// of two changes no other bit of the sums.
+constexpr float kWeightScale = 4294967296.f;   // 2^32
+
 // What one pixel adds to its tile.
 struct PixelRead {
     float2 c, l, r, u, d;   // means of the pixel and its neighbours (itself past the border)
@@ -328,8 +333,9 @@ __device__ __forceinline__ void add_pixel(const PixelRead &v, int x, int y, int 
     t.gx += gx;
     t.gy += gy;
     t.gt += v.ps.z;
-    t.sw = df_more(t.sw, v.ps.x);
-    const dfloat q = two_prod(v.ps.x, v.c.x);
+    const float w = v.ps.x * kWeightScale;
+    t.sw = df_more(t.sw, w);
+    const dfloat q = two_prod(w, v.c.x);
     t.swm = df_more(t.swm, q.h);
     t.swm.l += q.l;
 }
@@ -396,7 +402,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) k_spatial_tiles(int W, int H,
         auto take = [&](int k) { return dfloat{__shfl_sync(0xffffffffu, d.h, 8 * k), __shfl_sync(0xffffffffu, d.l, 8 * k)}; };
         const dfloat tw = take(0), tm = take(1), ta = take(2);
         const dfloat mean = tw.h > 0.f ? df_div(tm, tw) : dfloat{0.f, 0.f};
-        out.sw = (double)tw.h + (double)tw.l;
+        out.sw = ((double)tw.h + (double)tw.l) / kWeightScale;
         out.mean = (double)mean.h + (double)mean.l;
         out.n = __shfl_sync(0xffffffffu, i, 0);
         out.nonempty = __shfl_sync(0xffffffffu, i, 8);

@@ -1,7 +1,8 @@
 """Samples too old for their weights in single precision (exp(-3.47 a) is below
 the least normal number from a = 25 and 0 from a = 30): the gain control's mean
 age counts the ages of all buffered samples, those of pixels left without a
-weight included, over the samples of the tile records."""
+weight included, over the samples of the tile records; a tile's mean luminance
+is good to single precision while any of its weights is left."""
 import numpy as np
 import pytest
 import torch
@@ -44,4 +45,22 @@ def test_mean_age_counts_every_buffered_sample(dev, S):
     _, gain = rec.tile_error()
     want = ((64.0 * tiles.sum(2) + 1.0 * n) / n).mean()
     np.testing.assert_allclose(gain["mean_age"], want, rtol=1e-5)
+    rec.close()
+
+
+@pytest.mark.parametrize("S,age", [(2, 29.0), (2, 27.0), (8, 29.0), (32, 28.0), (34, 29.0), (2, 1.0)])
+def test_tile_mean_of_samples_with_tiny_weights(dev, S, age):
+    """One sample a pixel and all of one age: the weights are equal, so the mean
+    is the plain mean. Bound: the FP32 luminances and the result, 2^-24 each, and
+    the reference's own rounding of the colours, within 4 of those."""
+    from paper_2510_15876_gb300.api import decode_tiles
+    W, H = 6 * S, 5 * S
+    y, x = (v.reshape(-1) for v in np.mgrid[0:H, 0:W])
+    L = np.random.default_rng(S).uniform(0.1, 1.0, W * H).astype(np.float32)
+    rec = _rec(dev, W, H, S, x, y, np.zeros(W * H), L)
+    rec.estimate_gradients(age)
+    got = decode_tiles(rec.tile_feedback())
+    assert (got["n"] == S * S).all()
+    want = L.astype(np.float64).reshape(5, S, 6, S).mean((1, 3)).reshape(-1)
+    np.testing.assert_allclose(got["mean_L"], want, rtol=4 * 2.0 ** -24)
     rec.close()
