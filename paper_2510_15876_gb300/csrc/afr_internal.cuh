@@ -23,8 +23,9 @@ constexpr int kFramePad = 32;                    // records past frame_cap that 
 constexpr int kSortedBinMax = 4096;              // frame bins ordered by seq up to this size
 
 // device counters (unsigned long long); CNT_DROPPING: samples dropped by a
-// reprojection under way, 0 between reprojections
-enum { CNT_REJECTED = 0, CNT_DROPPED, CNT_UNSORTED, CNT_RESIDENT, CNT_DROPPING, CNT_N };
+// reprojection under way, 0 between reprojections; CNT_CROWDED: 1 if the last
+// reprojection of the reconstructor's queue found a crowded bin
+enum { CNT_REJECTED = 0, CNT_DROPPED, CNT_UNSORTED, CNT_RESIDENT, CNT_DROPPING, CNT_CROWDED, CNT_N };
 // device status word bits
 enum { ERR_TIMEOUT = 1u, ERR_CHECK = 2u };
 
@@ -155,7 +156,7 @@ struct AfrContext {
     afr::FrameRec *frec = nullptr;  // [frame_cap + kFramePad]
     uint32_t *sbin = nullptr;     // [frame_cap] each source slot's bin (reprojection scratch)
     uint32_t *flist = nullptr;    // [2 frame_cap + 4] reprojection scratch, by bin, unordered: (source slot, sequence
-                                  // number) pairs for the queues, sequence numbers for the reconstructor queue
+                                  // number) pairs for the queues, arrival ranks for the reconstructor queue
     size_t frame_cap = 0;
 
     // scan scratch
@@ -423,6 +424,8 @@ struct ScanWith {
     uint32_t fill_value = 0u;
     unsigned long long *counter_from = nullptr, *counter_to = nullptr;   // moved (the source becomes 0)
     unsigned long long *counter_zero = nullptr;                          // set to 0
+    unsigned long long *crowded = nullptr;                               // set to 1 if a count is above crowded_from
+    uint32_t crowded_from = 0u;
 };
 // in and the arrays of `with` must be 32-byte aligned.
 cudaError_t scan_exclusive(uint32_t *in, uint32_t *out, size_t n, uint32_t *tmp, cudaStream_t s,

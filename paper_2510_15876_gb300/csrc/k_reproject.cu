@@ -22,7 +22,8 @@
 //          the records. Each bin's smallest a^2 (the filter's exponent shift) is
 //          the minimum over the bin's warp segments, one atomic each. Samples of
 //          the reconstructor's queue, which lie in arrival order, are placed
-//          from that order instead (k_place_fifo).
+//          from that order instead (k_place_fifo), those of crowded bins by
+//          sorting the bin (place_crowded).
 //
 // Bound: HBM (place), atomic latency (list). 1920x1080x16, FP32 colours: list
 // 191 -> 148 us with one 8-byte entry for two 4-byte ones, place 533 -> 504 us
@@ -123,6 +124,17 @@ __device__ __forceinline__ bool live_move(uint32_t i, uint32_t nlive, int b, int
     return mv.ok;
 }
 
+// The reconstructor's queue of N slots holds the samples in the order of their
+// arrival, which is that of their sequence numbers: slot of the oldest sample
+// (total: samples it has taken), a slot's arrival rank, and the way back.
+__device__ __forceinline__ uint32_t oldest_slot(uint32_t total, uint32_t N) { return total > N ? total % N : 0u; }
+__device__ __forceinline__ uint32_t arrival_rank(uint32_t i, uint32_t oldest, uint32_t N) {
+    return i >= oldest ? i - oldest : i + (N - oldest);
+}
+__device__ __forceinline__ uint32_t ranked_slot(uint32_t rank, uint32_t oldest, uint32_t N) {
+    return rank < N - oldest ? rank + oldest : rank - (N - oldest);
+}
+
 // A warp takes kCountRows rows of 32 slots at a time, their loads issued
 // together.
 constexpr int kCountRows = 4;
@@ -133,6 +145,7 @@ __global__ void __launch_bounds__(256) k_count(uint32_t nslots, int b, int bshif
                                                uint32_t *__restrict__ fcnt, uint32_t *__restrict__ sbin,
                                                unsigned long long *__restrict__ dcount) {
     grid_order();
+    if (FIFO && blockIdx.x == 0 && threadIdx.x == 0) dcount[CNT_CROWDED] = 0ull;   // the scan sets it
     const uint32_t nlive = FIFO ? min(__ldg(state), nslots) : 0u;
     const int lane = threadIdx.x & 31;
     uint32_t dropped = 0;
@@ -166,12 +179,15 @@ __global__ void __launch_bounds__(256) k_count(uint32_t nslots, int b, int bshif
 // The slots' bins from the count pass (kInvalid: dead or moved out). A warp
 // takes kListRows rows of 32 slots at a time and issues every row's ticket
 // atomic before it reads any back, so the atomics' latencies overlap.
+// FIFO: the entry is the sample's arrival rank, which orders the bin as the
+// sequence number does and names the slot as well.
 constexpr int kListRows = 8;
-template <bool SLOTS>
+template <bool FIFO>
 __global__ void __launch_bounds__(256) k_list(uint32_t nslots, const uint32_t *__restrict__ sbin,
-                                              const uint32_t *__restrict__ r_seq, uint32_t *__restrict__ fcur,
-                                              uint32_t *__restrict__ flist, DebugCheck dc) {
+                                              const uint32_t *__restrict__ r_seq, const uint32_t *__restrict__ state,
+                                              uint32_t *__restrict__ fcur, uint32_t *__restrict__ flist, DebugCheck dc) {
     grid_order();
+    const uint32_t oldest = FIFO ? oldest_slot(__ldg(state), nslots) : 0u;
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t i0 = warp * 32u * kListRows; i0 < nslots; i0 += nwarps * 32u * kListRows) {
@@ -184,7 +200,7 @@ __global__ void __launch_bounds__(256) k_list(uint32_t nslots, const uint32_t *_
             sq[r] = 0;
             if (i < nslots) {
                 bin[r] = __ldg(sbin + i);
-                sq[r] = __ldg(r_seq + i);
+                sq[r] = FIFO ? arrival_rank(i, oldest, nslots) : __ldg(r_seq + i);
             }
         }
 #pragma unroll
@@ -201,8 +217,8 @@ __global__ void __launch_bounds__(256) k_list(uint32_t nslots, const uint32_t *_
             if (bin[r] == kInvalid) continue;
             const uint32_t at = f + __popc(peers[r] & ((1u << lane) - 1u));
             if (AFR_CHECK(at < dc.cap, dc.derr)) {
-                if (SLOTS) reinterpret_cast<uint2 *>(flist)[at] = make_uint2(i, sq[r]);
-                else flist[at] = sq[r];
+                if (FIFO) flist[at] = sq[r];
+                else reinterpret_cast<uint2 *>(flist)[at] = make_uint2(i, sq[r]);
             }
         }
     }
@@ -277,8 +293,74 @@ __global__ void __launch_bounds__(256) k_place_queues(int W, int H, float t_now,
 // The reconstructor's queue holds samples in arrival order, anywhere in the
 // image: gathered in bin order, each field of a record cost a sector of its
 // own. So a thread takes a slot, in queue order, and writes its record (one
-// whole sector) where its rank among the bin's sequence numbers puts it, four
-// numbers a load.
+// whole sector) where its place among the bin's arrival ranks puts it, four
+// ranks a load. Every lane walks another list, so that only pays while the lists
+// are short; longer ones are left to place_crowded.
+constexpr uint32_t kCrowded = 64;
+
+// Bins of kCrowded + 1 to kSortedBinMax records of the reconstructor's queue: a
+// block takes one at a time, sorts its arrival ranks in shared memory and
+// gathers the samples in that order. Neighbouring bins go to different blocks,
+// for crowds are local. Two million samples in 2,700 bins (some 800 each) take
+// 272 us with the rest of the reprojection; a thread a slot took 1147, gathering in
+// bin order 413.
+struct CrowdSmem {
+    uint32_t ranks[kSortedBinMax];
+    uint32_t found[256], n;
+};
+
+template <int CT, bool CAM>
+__device__ __forceinline__ void place_crowded(CrowdSmem &sm, uint32_t nslots, uint32_t oldest, int W, int H, float t_now,
+                                              const Camera &cam, const float4 *__restrict__ world,
+                                              const float4 *__restrict__ r_xm, const float *__restrict__ r_t,
+                                              const uint32_t *__restrict__ r_seq, const void *__restrict__ r_col,
+                                              const uint32_t *__restrict__ foff, const Fresh<uint32_t> &flist,
+                                              FrameRec *__restrict__ frec, const DebugCheck &dc) {
+    using CS = ColorStore<CT>;
+    const uint32_t P = (uint32_t)W * (uint32_t)H, G = gridDim.x;
+    for (uint32_t q0 = blockIdx.x; q0 < P; q0 += G * blockDim.x) {   // bins q0, q0 + G, ...
+        if (threadIdx.x == 0) sm.n = 0;
+        __syncthreads();
+        const unsigned long long q = q0 + (unsigned long long)threadIdx.x * G;
+        if (q < P) {
+            const uint32_t len = __ldg(foff + q + 1) - __ldg(foff + q);
+            if (len > kCrowded && len <= (uint32_t)kSortedBinMax) sm.found[atomicAdd(&sm.n, 1u)] = (uint32_t)q;
+        }
+        __syncthreads();
+        const uint32_t nf = sm.n;
+        for (uint32_t f = 0; f < nf; ++f) {
+            const uint32_t bin = sm.found[f], beg = __ldg(foff + bin), end = __ldg(foff + bin + 1);
+            const uint32_t len = AFR_CHECK(end <= dc.cap, dc.derr) ? end - beg : 0u;
+            uint32_t n2 = 2 * kCrowded;
+            while (n2 < len) n2 *= 2;
+            for (uint32_t k = threadIdx.x; k < n2; k += blockDim.x) sm.ranks[k] = k < len ? flist[beg + k] : kInvalid;
+            for (uint32_t k = 2; k <= n2; k *= 2)
+                for (uint32_t j = k / 2; j > 0; j /= 2) {   // bitonic, ascending
+                    __syncthreads();
+                    for (uint32_t t = threadIdx.x; t < n2 / 2; t += blockDim.x) {
+                        const uint32_t i = 2 * t - (t & (j - 1));
+                        const uint32_t a = sm.ranks[i], b = sm.ranks[i + j];
+                        if ((a > b) == ((i & k) == 0)) {
+                            sm.ranks[i] = b;
+                            sm.ranks[i + j] = a;
+                        }
+                    }
+                }
+            __syncthreads();
+            for (uint32_t r = threadIdx.x; r < len; r += blockDim.x) {
+                const uint32_t i = ranked_slot(sm.ranks[r], oldest, nslots);
+                if (!AFR_CHECK(i < nslots, dc.derr)) continue;
+                const Moved mv = CAM ? move_camera(__ldg(world + i), __ldg(r_xm + i), __ldg(r_t + i), t_now, W, H, cam)
+                                     : move_sample(__ldg(r_xm + i), __ldg(r_t + i), t_now, W, H);
+                const float3 c = CS::widen(CS::raw(r_col, i));
+                store_rec(frec + beg + r, {make_float4(mv.xp, mv.yp, mv.a2, bin_place(mv.xp, mv.yp)),
+                                           make_float4(c.x, c.y, c.z, __uint_as_float(__ldg(r_seq + i)))});
+            }
+            __syncthreads();   // the next bin overwrites the ranks
+        }
+    }
+}
+
 template <int CT, bool CAM>
 __global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int H, float t_now, Camera cam,
                                                     const float4 *__restrict__ world, const uint32_t *__restrict__ state,
@@ -290,7 +372,7 @@ __global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int 
                                                     unsigned long long *__restrict__ dcount, DebugCheck dc) {
     grid_order();
     using CS = ColorStore<CT>;
-    const uint32_t nlive = min(__ldg(state), nslots);
+    const uint32_t nlive = min(__ldg(state), nslots), oldest = oldest_slot(__ldg(state), nslots);
     const int lane = threadIdx.x & 31;
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < nlive; i0 += stride) {
@@ -312,14 +394,16 @@ __global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int 
         if (lane == __ffs(peers) - 1) atomicMin(amin2 + mv.bin, bits);
         if (!AFR_CHECK(beg < end && end <= dc.cap, dc.derr)) continue;
         uint32_t rank = 0;
-        const uint32_t len = end - beg;
-        if (len <= (uint32_t)kSortedBinMax) {
+        const uint32_t len = end - beg, mine = arrival_rank(i, oldest, nslots);
+        if (len <= kCrowded) {
             for (uint32_t k = beg & ~3u; k < end; k += 4) {
                 const uint4 v = *reinterpret_cast<const uint4 *>(&flist[k]);
                 const uint32_t j = k - beg;   // entries outside the bin wrap past its length or lie beyond it
-                rank += (uint32_t)((j < len) & (v.x < sq)) + (uint32_t)((j + 1u < len) & (v.y < sq)) +
-                        (uint32_t)((j + 2u < len) & (v.z < sq)) + (uint32_t)((j + 3u < len) & (v.w < sq));
+                rank += (uint32_t)((j < len) & (v.x < mine)) + (uint32_t)((j + 1u < len) & (v.y < mine)) +
+                        (uint32_t)((j + 2u < len) & (v.z < mine)) + (uint32_t)((j + 3u < len) & (v.w < mine));
             }
+        } else if (len <= (uint32_t)kSortedBinMax) {
+            continue;
         } else {
             rank = unsorted_rank(fcur, mv.bin, beg, dcount);
         }
@@ -329,6 +413,9 @@ __global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int 
         store_rec(frec + d, {make_float4(mv.xp, mv.yp, mv.a2, bin_place(mv.xp, mv.yp)),
                              make_float4(c.x, c.y, c.z, __uint_as_float(sq))});
     }
+    __shared__ CrowdSmem crowd;
+    if (dcount[CNT_CROWDED])
+        place_crowded<CT, CAM>(crowd, nslots, oldest, W, H, t_now, cam, world, r_xm, r_t, r_seq, r_col, foff, flist, frec, dc);
 }
 
 }  // namespace
@@ -369,12 +456,16 @@ cudaError_t launch_reproject(AfrContext *c, float t_now, const Camera *camp, cud
     with.counter_from = c->dcount + CNT_DROPPING;
     with.counter_to = c->dcount + CNT_DROPPED;
     with.counter_zero = c->dcount + CNT_UNSORTED;
+    if (fifo) {
+        with.crowded = c->dcount + CNT_CROWDED;
+        with.crowded_from = kCrowded;
+    }
     if ((e = scan_exclusive(c->fcnt, c->foff, c->P, c->scan_tmp, s, with)) != cudaSuccess) return e;
     // Not by launch_next: its blocks then start unevenly and leave the lists out
     // of slot order, and placing, which gathers in list order, takes 1.1 ms
     // instead of 0.5 at 1920x1080x16 (3956 -> 4291 us for the step).
-    if (fifo) k_list<false><<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, dc);
-    else k_list<true><<<g, 256, 0, s>>>(ns, c->sbin, sq, c->fcur, c->flist, dc);
+    if (fifo) k_list<true><<<g, 256, 0, s>>>(ns, c->sbin, sq, state, c->fcur, c->flist, dc);
+    else k_list<false><<<g, 256, 0, s>>>(ns, c->sbin, sq, state, c->fcur, c->flist, dc);
 #define AFR_QUEUES(CT_, C_)                                                                                         \
     launch_next(k_place_queues<CT_, C_>, dim3(g), dim3(256), 0, s, c->W, c->H, t_now, cm, wp, xm, tt, col, (uint32_t)c->P, c->foff,    \
                                               reinterpret_cast<const uint2 *>(c->flist), c->fcur, c->amin2, c->frec, \

@@ -133,9 +133,12 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint32_t *in, uint3
     uint32_t before = 0;
     if (!scanned)
         for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) before += sums[i];
-    uint32_t acc = 0;
+    uint32_t acc = 0, most = 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) acc += r.v[k];
+    for (int k = 0; k < kScanItems; ++k) {
+        acc += r.v[k];
+        most = max(most, r.v[k]);
+    }
     const uint32_t prefix = scanned ? sums[blockIdx.x] : block_sum(before);
     uint32_t ex = block_excl_scan(acc, &tot) + prefix;
 #pragma unroll
@@ -144,6 +147,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(uint32_t *in, uint3
         r.v[k] = ex;
         ex += c;
     }
+    if (with.crowded && most > with.crowded_from) *with.crowded = 1ull;
     store_items(out, base, n, r, wide);
     if (with.cursor) store_items(with.cursor, base, n, r);
     const Items zero{};
