@@ -298,16 +298,60 @@ __global__ void __launch_bounds__(256) k_place_queues(int W, int H, float t_now,
 // are short; longer ones are left to place_crowded.
 constexpr uint32_t kCrowded = 64;
 
-// Bins of kCrowded + 1 to kSortedBinMax records of the reconstructor's queue: a
-// block takes one at a time, sorts its arrival ranks in shared memory and
-// gathers the samples in that order. Neighbouring bins go to different blocks,
-// for crowds are local. Two million samples in 2,700 bins (some 800 each) take
-// 272 us with the rest of the reprojection; a thread a slot took 1147, gathering in
-// bin order 413.
+// Bins of kCrowded + 1 to kSortedBinMax records of the reconstructor's queue: the
+// bin's arrival ranks are sorted in shared memory and its samples gathered in
+// that order, by a warp up to kWarpBin records, else by a block. Neighbouring
+// bins go to different blocks, for crowds are local.
+// A reprojection of two million samples in 2,700 bins (some 800 each): 276 us;
+// walking the lists 1147, gathering everything in bin order 413 to 447. 256x256
+// with 32, 48, 64 and 96 samples a pixel: 158, 266, 393 and 597 us; gathering in
+// bin order 158, 247, 349, 579, walking the lists 170, 304, 456, 650. Lines at 16,
+// 24 and 32 records measured 184 to 201, 288, 392 and 613.
+constexpr uint32_t kWarpBin = 512;
+constexpr int kFifoWarps = 8;
+static_assert(kFifoWarps * kWarpBin <= (uint32_t)kSortedBinMax, "a warp sorts in its share of the block's ranks");
+
 struct CrowdSmem {
     uint32_t ranks[kSortedBinMax];
-    uint32_t found[256], n;
+    uint32_t found[32 * kFifoWarps], n;
 };
+
+// Threads t, t + T, ... of T sort and place the bin whose list entries are beg .. beg + len - 1.
+template <int CT, bool CAM, class Sync>
+__device__ __forceinline__ void place_sorted(uint32_t *ranks, uint32_t t, uint32_t T, Sync sync, uint32_t beg, uint32_t len,
+                                             uint32_t nslots, uint32_t oldest, int W, int H, float t_now,
+                                             const Camera &cam, const float4 *__restrict__ world,
+                                             const float4 *__restrict__ r_xm, const float *__restrict__ r_t,
+                                             const uint32_t *__restrict__ r_seq, const void *__restrict__ r_col,
+                                             const Fresh<uint32_t> &flist, FrameRec *__restrict__ frec, const DebugCheck &dc) {
+    using CS = ColorStore<CT>;
+    uint32_t n2 = 32;
+    while (n2 < len) n2 *= 2;
+    for (uint32_t k = t; k < n2; k += T) ranks[k] = k < len ? flist[beg + k] : kInvalid;
+    for (uint32_t k = 2; k <= n2; k *= 2)
+        for (uint32_t j = k / 2; j > 0; j /= 2) {   // bitonic, ascending
+            sync();
+            for (uint32_t c = t; c < n2 / 2; c += T) {
+                const uint32_t i = 2 * c - (c & (j - 1));
+                const uint32_t a = ranks[i], b = ranks[i + j];
+                if ((a > b) == ((i & k) == 0)) {
+                    ranks[i] = b;
+                    ranks[i + j] = a;
+                }
+            }
+        }
+    sync();
+    for (uint32_t r = t; r < len; r += T) {
+        const uint32_t i = ranked_slot(ranks[r], oldest, nslots);
+        if (!AFR_CHECK(i < nslots, dc.derr)) continue;
+        const Moved mv = CAM ? move_camera(__ldg(world + i), __ldg(r_xm + i), __ldg(r_t + i), t_now, W, H, cam)
+                             : move_sample(__ldg(r_xm + i), __ldg(r_t + i), t_now, W, H);
+        const float3 c = CS::widen(CS::raw(r_col, i));
+        store_rec(frec + beg + r, {make_float4(mv.xp, mv.yp, mv.a2, bin_place(mv.xp, mv.yp)),
+                                   make_float4(c.x, c.y, c.z, __uint_as_float(__ldg(r_seq + i)))});
+    }
+    sync();   // the next bin overwrites the ranks
+}
 
 template <int CT, bool CAM>
 __device__ __forceinline__ void place_crowded(CrowdSmem &sm, uint32_t nslots, uint32_t oldest, int W, int H, float t_now,
@@ -316,9 +360,8 @@ __device__ __forceinline__ void place_crowded(CrowdSmem &sm, uint32_t nslots, ui
                                               const uint32_t *__restrict__ r_seq, const void *__restrict__ r_col,
                                               const uint32_t *__restrict__ foff, const Fresh<uint32_t> &flist,
                                               FrameRec *__restrict__ frec, const DebugCheck &dc) {
-    using CS = ColorStore<CT>;
-    const uint32_t P = (uint32_t)W * (uint32_t)H, G = gridDim.x;
-    for (uint32_t q0 = blockIdx.x; q0 < P; q0 += G * blockDim.x) {   // bins q0, q0 + G, ...
+    const uint32_t P = (uint32_t)W * (uint32_t)H, G = gridDim.x, T = 32 * kFifoWarps, warp = threadIdx.x >> 5;
+    for (uint32_t q0 = blockIdx.x; q0 < P; q0 += G * T) {   // bins q0, q0 + G, ...
         if (threadIdx.x == 0) sm.n = 0;
         __syncthreads();
         const unsigned long long q = q0 + (unsigned long long)threadIdx.x * G;
@@ -328,41 +371,22 @@ __device__ __forceinline__ void place_crowded(CrowdSmem &sm, uint32_t nslots, ui
         }
         __syncthreads();
         const uint32_t nf = sm.n;
-        for (uint32_t f = 0; f < nf; ++f) {
-            const uint32_t bin = sm.found[f], beg = __ldg(foff + bin), end = __ldg(foff + bin + 1);
-            const uint32_t len = AFR_CHECK(end <= dc.cap, dc.derr) ? end - beg : 0u;
-            uint32_t n2 = 2 * kCrowded;
-            while (n2 < len) n2 *= 2;
-            for (uint32_t k = threadIdx.x; k < n2; k += blockDim.x) sm.ranks[k] = k < len ? flist[beg + k] : kInvalid;
-            for (uint32_t k = 2; k <= n2; k *= 2)
-                for (uint32_t j = k / 2; j > 0; j /= 2) {   // bitonic, ascending
-                    __syncthreads();
-                    for (uint32_t t = threadIdx.x; t < n2 / 2; t += blockDim.x) {
-                        const uint32_t i = 2 * t - (t & (j - 1));
-                        const uint32_t a = sm.ranks[i], b = sm.ranks[i + j];
-                        if ((a > b) == ((i & k) == 0)) {
-                            sm.ranks[i] = b;
-                            sm.ranks[i + j] = a;
-                        }
-                    }
-                }
-            __syncthreads();
-            for (uint32_t r = threadIdx.x; r < len; r += blockDim.x) {
-                const uint32_t i = ranked_slot(sm.ranks[r], oldest, nslots);
-                if (!AFR_CHECK(i < nslots, dc.derr)) continue;
-                const Moved mv = CAM ? move_camera(__ldg(world + i), __ldg(r_xm + i), __ldg(r_t + i), t_now, W, H, cam)
-                                     : move_sample(__ldg(r_xm + i), __ldg(r_t + i), t_now, W, H);
-                const float3 c = CS::widen(CS::raw(r_col, i));
-                store_rec(frec + beg + r, {make_float4(mv.xp, mv.yp, mv.a2, bin_place(mv.xp, mv.yp)),
-                                           make_float4(c.x, c.y, c.z, __uint_as_float(__ldg(r_seq + i)))});
-            }
-            __syncthreads();   // the next bin overwrites the ranks
-        }
+        const auto place = [&](uint32_t *ranks, uint32_t t, uint32_t threads, auto sync, uint32_t f, bool block) {
+            const uint32_t beg = __ldg(foff + sm.found[f]), end = __ldg(foff + sm.found[f] + 1), len = end - beg;
+            if (block == (len <= kWarpBin) || !AFR_CHECK(end <= dc.cap, dc.derr)) return;   // uniform over the threads
+            place_sorted<CT, CAM>(ranks, t, threads, sync, beg, len, nslots, oldest, W, H, t_now, cam, world, r_xm, r_t,
+                                  r_seq, r_col, flist, frec, dc);
+        };
+        for (uint32_t f = warp; f < nf; f += kFifoWarps)
+            place(sm.ranks + warp * kWarpBin, threadIdx.x & 31, 32, [] { __syncwarp(); }, f, false);
+        __syncthreads();
+        for (uint32_t f = 0; f < nf; ++f) place(sm.ranks, threadIdx.x, T, [] { __syncthreads(); }, f, true);
+        __syncthreads();   // the next bins' count overwrites this one's
     }
 }
 
 template <int CT, bool CAM>
-__global__ void __launch_bounds__(256) k_place_fifo(uint32_t nslots, int W, int H, float t_now, Camera cam,
+__global__ void __launch_bounds__(32 * kFifoWarps) k_place_fifo(uint32_t nslots, int W, int H, float t_now, Camera cam,
                                                     const float4 *__restrict__ world, const uint32_t *__restrict__ state,
                                                     const float4 *__restrict__ r_xm,
                                                     const float *__restrict__ r_t, const uint32_t *__restrict__ r_seq,

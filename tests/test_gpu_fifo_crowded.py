@@ -1,9 +1,9 @@
 """The reconstructor's queue with crowded bins: bins at the edges of the length
-that a thread places (64), of a block's steps (256 threads, four ranks each, four
-ranks a load) and of the sorted range (4096), queues that have wrapped and not, a
-camera, 16-bit colours; the frame view bit for bit against the oracle, crowded
-and uncrowded reprojections in turn. Bins above 4096 records hold the same
-records in any order."""
+that a thread places (64), that a warp sorts (512) and of the sorted range
+(4096), around powers of two, queues that have wrapped and not, a camera, 16-bit
+colours; the frame view bit for bit against the oracle, crowded and uncrowded
+reprojections in turn. Bins above 4096 records hold the same records in any
+order."""
 import numpy as np
 import pytest
 import torch
@@ -59,7 +59,7 @@ def test_crowded_bins_match_oracle(dev, W, H, N, ct):
     from paper_2510_15876_gb300.api import Reconstructor, to_device_batch
     rng = np.random.default_rng(N)
     rec, fifo = Reconstructor(W, H, 2, color_type=ct, fifo_capacity=N, device=dev), oracle.Fifo(W, H, N)
-    lengths = [64, 65, 66, 63, 255, 256, 257, 1023, 1024, 1025, 1100, 130, 3, 4300]
+    lengths = [64, 65, 66, 63, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 1100, 130, 3, 4300]
     seen = set()
     for crowd, spread in ((lengths, 500), ([], W * H // 2), (lengths[::-1], 100), ([70] * 200, 0), ([4090, 5000], 2000)):
         batch = _batch(rng, W, H, crowd, spread) if crowd or spread else None
