@@ -251,7 +251,10 @@ __global__ void k_coverage_init(int P, float r0, float *__restrict__ r, int32_t 
 // R = 5 from 607 to 407 us and 640x480x8 in FP16 from 185 to 122 us. Adaptive
 // footprints, 1920x1080x16 with most radii at 1: 720 us with a table per block,
 // 617 us keeping a warp's table while the radius stays, 562 us with shared
-// tables of the small radii (the per-warp ones took 41 KB a CTA from L1). The shift
+// tables of the small radii (the per-warp ones took 41 KB a CTA from L1); with one
+// more for a tile's largest radius above those, 640x480x32 at radius 8 takes 1366
+// us instead of 1693 (a table per block: 1310). The adaptive form spills 40 to 44
+// bytes at its 80 registers, the fixed one 8 to 12. The shift
 // table per block (disc + shift, no addition per record) measured 1655 us, its
 // shared memory taken from L1; four CTAs a SM (64 registers, spills) 1183 us;
 // a prefetch two records deep 1413 us (spills); CTAs of 12 or 24 warps
@@ -387,7 +390,7 @@ struct ForwardSums {
 
 // Discs of the union box of a 2x2 block at footprint radius R: entry
 // (v, u) = bin row by - R + v, column bx - R + u.
-constexpr int kTables = 4;   // adaptive footprints: radii 1 .. kTables have a table each
+constexpr int kTables = 4;   // adaptive footprints: radii 1 .. kTables have a table each, a tile's largest radius above them one more
 constexpr int kTableRows = kTables * (kTables + 3);
 __host__ __device__ constexpr int table_row(int R) { return (R - 1) * (R + 2); }   // rows of the tables before R's
 static_assert(table_row(kTables + 1) == kTableRows, "2R + 2 rows each");
@@ -405,8 +408,8 @@ __device__ __forceinline__ void fill_discs(float4 *in, int R) {
     }
 }
 
-// The same for pixels whose radii differ (or have no table), for the bin at
-// place t of the box of radius R.
+// The same for pixels whose radii differ, for the bin at place t of the box of
+// radius R.
 __device__ __forceinline__ float4 own_discs(int t, int R, const int (&Rk)[4]) {
     const int v = t * 57 >> 10, u = t - v * kPitch;   // t / 18 for t < 18 * 18
     float s[4];
@@ -527,8 +530,8 @@ __device__ __forceinline__ float4 load_const(int i, int W, int H, int x0, int y0
 // VAR: each pixel's footprint radius is read from its gather constants
 // (adaptive footprints; most neighbouring ones have settled at one radius);
 // otherwise every pixel uses Rt. tables_at: shared address of the disc tables
-// (VAR: of radii 1 .. kTables; else of Rt alone). frec: the frame view from this
-// lane's record on.
+// (VAR: of radii 1 .. kTables, then of Rt if it is larger; else of Rt alone). frec:
+// the frame view from this lane's record on.
 template <bool VAR, class Sums>
 __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int lx, int ly, const FrameRec *frec,
                                              const TileSmem &ts, uint32_t tables_at, uint2 *rows, uint32_t rows_at,
@@ -590,8 +593,8 @@ __device__ __forceinline__ void gather_block(int Rt, int x0, int y0, int tw, int
         pc.m[j] = pk(fc[2 * j].z, fc[2 * j + 1].z);
     }
     const int origin = (by - R) * kPitch + bx - R;
-    const bool table = !VAR || (same && R >= 1 && R <= kTables);
-    const uint32_t table_at = tables_at + (VAR && table ? table_row(R) * kPitch * 16u : 0u);
+    const bool table = !VAR || (same && R >= 1 && (R <= kTables || R == Rt));
+    const uint32_t table_at = tables_at + (VAR && table ? table_row(min(R, kTables + 1)) * kPitch * 16u : 0u);
     const uint32_t tab = keep(table_at - (uint32_t)origin * 16u);   // + 16 place: the entry of a record's bin
     auto load = [&](int i) {   // record i + lane (i itself may be negative)
         const bool ok = AFR_CHECK((uint32_t)(i + lane) < dc.cap + kFramePad, dc.derr);
@@ -688,7 +691,7 @@ __global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx
                                                    float4 *__restrict__ out, DebugCheck dc) {
     grid_order();
     __shared__ TileSmem ts;
-    __shared__ float4 discs[(VAR ? kTableRows : kMaxRows) * kPitch];
+    __shared__ float4 discs[(VAR ? kTableRows + kMaxRows : kMaxRows) * kPitch];
     const int warp = threadIdx.x >> 5, tw = 2 << ltbx, th = 64 >> ltbx >> lsplit, pixels = tw * th;
     const int x0 = blockIdx.x * tw, y0 = blockIdx.y * th;
     const FrameRec *const frec0 = frec;
@@ -706,6 +709,7 @@ __global__ void __launch_bounds__(256, 3) k_filter(int W, int H, int R, int ltbx
             Rt = r;
             if (r <= kTables) fill_discs(discs + table_row(r) * kPitch, r);
         }
+        if (Rt > kTables) fill_discs(discs + kTableRows * kPitch, Rt);
     } else {
         fill_discs(discs, R);
     }

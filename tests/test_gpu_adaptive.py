@@ -103,3 +103,23 @@ def test_fixed_footprint_unaffected_and_backward_guard(dev):
     again = rec.reconstruct(T_NOW)
     assert torch.equal(again, ref)
     rec.backward(torch.ones((H, W, 4), device=dev))     # allowed again after a fixed reconstruction
+
+
+@pytest.mark.parametrize("R", [1, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("W,H,b,ct", [(67, 45, 12, "f32"), (33, 70, 5, "f16")])
+def test_first_adaptive_image_has_the_configured_discs(dev, R, W, H, b, ct):
+    """After a reset every footprint has the configured radius, with a disc table
+    of its own up to 4 and the tile's one above: the plain image, bit for bit."""
+    from paper_2510_15876_gb300.api import Reconstructor
+    g = torch.Generator(dev).manual_seed(R)
+    rec = Reconstructor(W, H, b, radius=R, color_type=ct, device=dev)
+    n = 2 * W * H * b
+    pos = torch.rand(n, 4, generator=g, device=dev) * torch.tensor([W - 0.01, H - 0.01, 1.0, 1.0], device=dev)
+    pos[:, 2] = pos[:, 2].sort().values
+    rec.insert(pos, torch.rand(n, 4, generator=g, device=dev).to(rec.color_dtype), torch.randn(n, 2, generator=g, device=dev))
+    rec.estimate_gradients(1.0)
+    rec.reproject(1.0)
+    want = rec.reconstruct(1.0)
+    got = rec.reconstruct(1.0, flags=L.AFR_RECON_ADAPTIVE_SUPPORT | L.AFR_RECON_COVERAGE_RESET)
+    assert torch.equal(got, want)
+    rec.close()
