@@ -865,7 +865,9 @@ struct PixelSums {
 // order. A small image gets a pixel a thread (the same sums): with three its few
 // CTAs leave most of the GPU idle behind one thread's walk (parameter gradients,
 // 8 deep: 128x128 72 -> 37 us, 256x256 129 -> 103; 352x288, 264 CTAs of three
-// rows, 140 -> 147, so the line lies at one and a half CTAs a SM).
+// rows, 140 -> 147, so the line lies at one and a half CTAs a SM). So do the radii 0
+// and 1, whose rows share no record or few: 512x512x8 29 -> 24 and 55 -> 52 us,
+// 1024x768x4 77 -> 64 and 112 -> 97 (at radius 2 three rows are faster from depth 4 on).
 constexpr int kBwdX = 32, kBwdY = 4;
 constexpr int kBwdRows = 3;
 constexpr int kPartRows = 4;   // rows of one partial
@@ -1232,7 +1234,7 @@ cudaError_t launch_backward(AfrContext *c, const float4 *grad_rgb, float *grad_c
                             cudaStream_t s) {
     const auto bands = [&](int rows) { return (c->H + kBwdY * rows - 1) / (kBwdY * rows); };
     const int cols = (c->W + kBwdX - 1) / kBwdX;
-    const int rows = (long long)cols * bands(kBwdRows) < 3ll * device_sms() / 2 ? 1 : kBwdRows;
+    const int rows = c->R <= 1 || (long long)cols * bands(kBwdRows) < 3ll * device_sms() / 2 ? 1 : kBwdRows;
     const dim3 block(kBwdX, kBwdY), grid(cols, bands(rows));
     const DebugCheck dc{(uint32_t)c->frame_cap, c->derr};
     const Adjoint adj{c->bgrad, reinterpret_cast<float2 *>(c->bgrad + c->P)};
