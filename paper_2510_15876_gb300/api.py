@@ -26,6 +26,11 @@ def _stream(stream=None) -> int:
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())   # no Stream object (2 us)
 
 
+def _capturing(stream) -> bool:
+    with torch.cuda.stream(stream):
+        return torch.cuda.is_current_stream_capturing()
+
+
 def _ptr(t: torch.Tensor | None):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -179,13 +184,34 @@ class Reconstructor:
             out = torch.empty((self.H, self.W, 4), dtype=torch.float32, device=self.device)
         event = None
         if reads_done is not None:
+            on = stream if stream is not None else torch.cuda.current_stream(self.device)
+            if _capturing(on):   # an external event is recorded by a graph node, which torch's record alone makes
+                self._refresh_in_calls(t_now, out, tiles, params, flags, on, side_stream, reads_done, view_proj)
+                return out, tiles
             if not reads_done.cuda_event:   # torch makes the event when it is first recorded
-                reads_done.record(stream if stream is not None else torch.cuda.current_stream(self.device))
+                reads_done.record(on)
             event = reads_done.cuda_event
         self._check(self.lib.afr_refresh(self.h, t_now, None if view_proj is None else _matrix(view_proj),
                                          ctypes.byref(_params(params)), flags, out.data_ptr(), tiles.data_ptr(),
                                          side_stream.cuda_stream, event, main))
         return out, tiles
+
+    def _refresh_in_calls(self, t_now, out, tiles, params, flags, main, side, reads_done, view_proj):
+        fork, join = torch.cuda.Event(), torch.cuda.Event()
+        fork.record(main)
+        side.wait_event(fork)
+        try:
+            self.estimate_gradients(t_now, stream=side)
+            self.tile_feedback(out=tiles, stream=side)
+            if view_proj is None:
+                self.reproject(t_now, stream=main)
+            else:
+                self.reproject_camera(t_now, view_proj, stream=main)
+        finally:
+            join.record(side)
+            main.wait_event(join)
+        reads_done.record(main)
+        self.reconstruct(t_now, params, out, flags, stream=main)
 
     GAIN_KEYS = ("dC_ds", "dC_dt", "mean_age", "tile_width", "tile_count")
 

@@ -80,6 +80,42 @@ def test_refresh_refuses_what_its_calls_refuse(dev):
     assert torch.isfinite(img).all()
 
 
+@pytest.mark.parametrize("camera", [False, True])
+def test_captured_refresh_records_an_external_event_at_every_replay(dev, camera):
+    """reads_done made with external=True is recorded by a node of the graph, as
+    by torch's own record between the calls: after a replay it has a time, between
+    that of an event before the refresh and that of one after it. One without the
+    flag orders streams inside the capture."""
+    a, s = _filled(dev), _filled(dev)
+    out, tiles = torch.empty((H, W, 4), device=dev), torch.empty((a.n_tiles, 8), device=dev)
+    kw = dict(out=out, tiles=tiles, view_proj=VP if camera else None)
+    a._side = torch.cuda.Stream(dev)
+    before, done, after = (torch.cuda.Event(enable_timing=True, external=True) for _ in range(3))
+    inside, other = torch.cuda.Event(), torch.cuda.Stream(dev)
+    flag = torch.zeros(1, device=dev)
+    done.record()   # as a pipeline does before its first image: the event exists
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        main = torch.cuda.current_stream(dev)
+        before.record(main)
+        a.refresh(1.0, reads_done=done, **kw)
+        after.record(main)
+        a.refresh(1.0, reads_done=inside, **kw)
+        other.wait_event(inside)
+        with torch.cuda.stream(other):
+            flag.add_(1)
+        main.wait_stream(other)
+    for k in range(2):
+        graph.replay()
+        torch.cuda.synchronize()
+        assert done.query() and 0 < before.elapsed_time(done) <= before.elapsed_time(after)
+        assert flag.item() == k + 1
+    want, want_tiles = s.refresh(1.0, view_proj=VP if camera else None)
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and torch.equal(tiles.view(torch.int32), want_tiles.view(torch.int32))
+
+
 def test_a_refused_refresh_launches_nothing(dev):
     """After a refusal both streams are idle, so nothing still reads the queues
     or writes the tile records when the caller's next batch arrives, and a
