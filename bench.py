@@ -119,8 +119,8 @@ class ClockSampler:
 #       -c 20 --csv --log-file launches.csv python bench.py --profile --steps 1 --warmup 0 --no-cpu-baseline
 # A changed kernel has no entry, and the line then reports null.
 FILTER_TRAFFIC = {
-    ("ae244bb8771123929683c9b2558fa68bc4362a0969ad05f926180d2e7a19bba8",
-     "fd33035b9c3af08892ade33cb43da58342913577528cd19e6fbc2422473b9cea"): 0.989e9 + 0.031e9,
+    ("e36f9c27298bbac8c03317e27c0ea89b5a14320081db1875b447d24ab7979fe0",
+     "78b1db33d948f865e0434fa1614f959600d5e6eabedc4ade7322543bf6279e39"): 0.989e9 + 0.031e9,
 }
 
 
@@ -146,7 +146,7 @@ def stage_bytes(P, n_batch, resident, frame, csize, ntiles):
     x, y, mx, my (16 B), t (4), depth (4), seq (4) and its colour; a frame
     record is 32 bytes (x', y', a^2, bin, r, g, b, seq)."""
     ingest = n_batch * (16 + csize + 8) + resident * (16 + 4 + 4 + 4 + csize) + P * 8
-    grads = resident * (4 + 4 + csize) + P * (4 + 4 + 16 + 4 + 16) + ntiles * 64
+    grads = resident * (4 + csize) + P * (4 + 4 + 16 + 4 + 16) + ntiles * 64
     reproj = resident * (16 + 4 + 4 + csize) + frame * 32 + P * 12
     recon = frame * 32 + P * (16 + 8 + 4 + 8 + 16)
     feedback = ntiles * (64 + 32)

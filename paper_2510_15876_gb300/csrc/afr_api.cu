@@ -859,10 +859,13 @@ AfrStatus afr_batch_create(AfrContext *const *ctxs, int32_t n, AfrBatch **out) {
     // afr_batch_refresh: kBatchWorkers streams, each context on the one with
     // the least work so far (work ~ its buffered slots), largest first. Contexts
     // of kBatchAlone slots or more share one: side by side, their list passes
-    // disturb each other's order and the placements gather worse (four of
-    // 1280x720x16 3.54 ms, one after another 3.26; three of 1920x1080x8, 16.6M
-    // slots, 3.24 and 3.23), while smaller ones fill each other's gaps (five of
-    // 1280x720x8, 7.4M slots, 2.37 side by side, 2.52 in turn). Contexts with a
+    // disturb each other's order and the placements gather worse (side by side
+    // and in turn, ms: eight of 1280x720x16 8.8 and 8.17, four 3.54 and 3.26, with
+    // six of 640x480x8 beside three 4.26 and 4.20; two of 1920x1080x16 4.53 and
+    // 4.47), while smaller ones fill each other's gaps (five of 1280x720x8, 7.4M
+    // slots, 2.37 and 2.52). For two or three alone it can cost a little: two of
+    // 1280x720x16 1.99 and 2.04, two of 1920x1080x8 2.45 and 2.56, three 3.79 and
+    // 3.84. Contexts with a
     // reconstructor queue place in that queue's order, which nothing disturbs: by
     // its capacity, four of 256x256 with room for 16M samples took 385 us in turn,
     // 286 side by side.

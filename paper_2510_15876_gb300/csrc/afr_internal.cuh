@@ -127,8 +127,8 @@ struct AfrContext {
     uint32_t *fifo_flag = nullptr;  // [batch_cap] 1 for an accepted sample
     uint32_t *fifo_rank = nullptr;  // [batch_cap + 1] exclusive scan of fifo_flag, then the total
     uint32_t *fifo_scan = nullptr;  // scan block sums for batch_cap entries
-    // ingest scratch: per-cell counts and offsets (cells of 16 x 8 pixels) and
-    // the batch's records bucketed by pixel (batch_cap records)
+    // ingest scratch: per-pixel counts and offsets, and the batch's records
+    // bucketed by pixel (batch_cap records)
     uint32_t *ccnt = nullptr;     // [P] bucket counts, all 0 between batches
     uint32_t *coff = nullptr;     // [P + 1] bucket offsets
     uint32_t *ccur = nullptr;     // [P] append cursors, then the queue states after the batch
@@ -376,9 +376,9 @@ inline int grid_for(size_t n, int block, int cap = 0) {
 // first statement of every kernel of such a chain, holds them until the grids
 // before it are complete and their writes visible (so each link also waits for
 // all links before). Only between two kernels of one call with nothing between
-// them on the stream. Each link saves 1 to 3 us: a 128x128x4 step 75 -> 59 us,
-// 640x480x8 in FP16 261 -> 242, 1024x1024x8 with a camera 736 -> 714,
-// 1920x1080x16 3956 -> 3938. Not everywhere: see k_list's launch; and waiting
+// them on the stream. Each link saves 1 to 3 us: a 128x128x4 step 76 -> 60 us,
+// 640x480x8 in FP16 266 -> 243, 1024x1024x8 with a camera 730 -> 715,
+// 1920x1080x16 3956 -> 3924. Not everywhere: see k_list's launch; and waiting
 // blocks of the gradient branch keep the other branch's out (k_spatial_tiles
 // launched so: +4 us at 640x480x8).
 template <class... P, class... A>

@@ -859,8 +859,9 @@ struct PixelSums {
 // sectors of L1 (a warp's lanes read records of neighbouring bins, one 32-byte
 // sector each): 512x512x8, 325 us with a pixel a thread that also searched its
 // exponent shift again, 217 us so (two rows a thread 237, four 302: registers),
-// now 207 with the next record loaded ahead and five CTAs a SM (235 when the
-// compiler takes the registers for four).
+// 207 with the next record loaded ahead and five CTAs a SM (235 when the
+// compiler takes the registers for four), 211 with the check for sums that are not
+// finite.
 // The filter's gather, lanes over records, takes 176 us, but sums in another
 // order. A small image gets a pixel a thread (the same sums): with three its few
 // CTAs leave most of the GPU idle behind one thread's walk (parameter gradients,
@@ -1140,6 +1141,9 @@ __global__ void k_bwd_params(Fresh<float> part, int nblocks, float *__restrict__
 }
 
 // Colours rounded to the storage type, then widened as the frame view holds them.
+// Bound: HBM, twelve of the 32 bytes of every record, so each is read and written
+// whole: 1280x720x8 83 us, where a plane of colours alone took 36. (A
+// reconstruction, which follows and reads all 32, went from 562 to 346 us there.)
 template <int CT>
 __global__ void k_set_colors(const float *__restrict__ rgb, const uint32_t *__restrict__ foff, int P,
                              FrameRec *__restrict__ frec) {
